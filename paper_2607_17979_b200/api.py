@@ -3,7 +3,9 @@
 Every function takes torch CUDA tensors, checks dtype / contiguity / device,
 and passes raw device pointers and the current CUDA stream to the entry point
 of the same name.  Nothing is computed here, and there is no fallback: if the
-compiled library is missing the import fails.
+compiled library is missing the import fails.  The calls of a serving loop
+(decode, gate, prefill) do that in the native module ``_binding``
+(``binding/binding.cpp``), the others through ctypes.
 """
 from __future__ import annotations
 
@@ -35,29 +37,14 @@ if not os.path.exists(LIB_PATH):
         "(nvcc, sm_100a). There is no CPU or PyTorch fallback for the gated delta rule kernels.")
 
 _lib = ctypes.CDLL(LIB_PATH)
+from . import _binding  # noqa: E402  (after torch and the library it links against)
 _P, _I, _F, _Z = ctypes.c_void_p, ctypes.c_int32, ctypes.c_float, ctypes.c_size_t
-_lib.gdn_decode.restype = ctypes.c_int
-_lib.gdn_decode.argtypes = [_P] * 8 + [_I] * 6 + [_F, _P, _P]
 _lib.gdn_prefill_workspace_bytes.restype = _Z
-_lib.gdn_decode_multi.restype = ctypes.c_int
-_lib.gdn_decode_multi.argtypes = [_P] * 8 + [_I] * 7 + [_F, _I, _P, _P]
-_lib.gdn_gate.restype = ctypes.c_int
-_lib.gdn_gate.argtypes = [_P] * 6 + [_I, _I, _P]
 _lib.gdn_state_transpose.restype = ctypes.c_int
 _lib.gdn_state_transpose.argtypes = [_P, _P] + [_I] * 5 + [_P, _P]
 _lib.gdn_prefill_workspace_bytes.argtypes = [_I] * 7
-_lib.gdn_prefill.restype = ctypes.c_int
-_lib.gdn_prefill.argtypes = [_P] * 10 + [_I] * 9 + [_F, _P, _Z, _P, _P]
-_lib.gdn_prefill_chunked.restype = ctypes.c_int
-_lib.gdn_prefill_chunked.argtypes = _lib.gdn_prefill.argtypes
-_lib.gdn_prefill_fused.restype = ctypes.c_int
-_lib.gdn_prefill_fused.argtypes = _lib.gdn_prefill.argtypes
 _lib.gdn_prefill_route.restype = ctypes.c_int
 _lib.gdn_prefill_route.argtypes = [_I] * 6
-_lib.gdn_prefill_stream.restype = ctypes.c_int
-_lib.gdn_prefill_stream.argtypes = _lib.gdn_prefill.argtypes
-_lib.gdn_prefill_overlap.restype = ctypes.c_int
-_lib.gdn_prefill_overlap.argtypes = _lib.gdn_prefill.argtypes + [_I]
 _lib.gdn_prefill_recurrent.restype = ctypes.c_int
 _lib.gdn_prefill_recurrent.argtypes = [_P] * 10 + [_I] * 7 + [_F, _P, _P]
 _lib.gdn_prefill_static.restype = ctypes.c_int
@@ -113,15 +100,7 @@ def _stream():
 
 def gdn_decode(q, k, v, g, beta, state_pool, slot_idx, o, scale, dev_status=None):
     """One decode step, state_pool updated in place, o written.  Shapes as in gdn.h."""
-    B, Hqk, dk = q.shape
-    _, Hv, dv = v.shape
-    rc = _lib.gdn_decode(
-        _dev(q, torch.bfloat16, "q"), _dev(k, torch.bfloat16, "k"), _dev(v, torch.bfloat16, "v"),
-        _dev(g, torch.float32, "g"), _dev(beta, torch.float32, "beta"),
-        _dev(state_pool, torch.float32, "state_pool"),
-        _dev(slot_idx, torch.int32, "slot_idx", True), _dev(o, torch.bfloat16, "o"),
-        B, Hqk, Hv, dk, dv, state_pool.shape[0], float(scale),
-        _dev(dev_status, torch.int32, "dev_status", True), _stream())
+    rc = _binding.decode(q, k, v, g, beta, state_pool, slot_idx, o, scale, dev_status)
     if rc != 0:
         raise GdnError(rc, "gdn_decode")
 
@@ -134,26 +113,15 @@ def gdn_decode_multi(q, k, v, g, beta, state_pool, slot_idx, o, scale, state_lay
                      dev_status=None):
     """L new tokens per sequence in one call (q [B,L,Hqk,128], v/o [B,L,Hv,128], g/beta [B,L,Hv]);
     ``state_layout`` STATE_VK = tiles [dv][dk], STATE_KV = tiles [dk][dv]."""
-    B, L, Hqk, dk = q.shape
-    _, _, Hv, dv = v.shape
-    rc = _lib.gdn_decode_multi(
-        _dev(q, torch.bfloat16, "q"), _dev(k, torch.bfloat16, "k"), _dev(v, torch.bfloat16, "v"),
-        _dev(g, torch.float32, "g"), _dev(beta, torch.float32, "beta"),
-        _dev(state_pool, torch.float32, "state_pool"),
-        _dev(slot_idx, torch.int32, "slot_idx", True), _dev(o, torch.bfloat16, "o"),
-        B, L, Hqk, Hv, dk, dv, state_pool.shape[0], float(scale), int(state_layout),
-        _dev(dev_status, torch.int32, "dev_status", True), _stream())
+    rc = _binding.decode_multi(q, k, v, g, beta, state_pool, slot_idx, o, scale, state_layout,
+                               dev_status)
     if rc != 0:
         raise GdnError(rc, "gdn_decode_multi")
 
 
 def gdn_gate(a, b, A_log, dt_bias, g, beta):
     """g = -exp(A_log) * softplus(a + dt_bias), beta = sigmoid(b); a, b bf16 [T, Hv]."""
-    T, Hv = a.shape
-    rc = _lib.gdn_gate(_dev(a, torch.bfloat16, "a"), _dev(b, torch.bfloat16, "b"),
-                       _dev(A_log, torch.float32, "A_log"), _dev(dt_bias, torch.float32, "dt_bias"),
-                       _dev(g, torch.float32, "g"), _dev(beta, torch.float32, "beta"), T, Hv,
-                       _stream())
+    rc = _binding.gate(a, b, A_log, dt_bias, g, beta)
     if rc != 0:
         raise GdnError(rc, "gdn_gate")
 
@@ -172,6 +140,7 @@ def gdn_state_transpose(state_pool, slot_idx=None, n=None, dev_status=None):
 
 
 ROUTES = {0: "none", 1: "recurrent", 2: "chunked", 3: "fused", 4: "stream", 5: "overlap"}
+_ROUTE_CODES = {"auto": 0, "chunked": 2, "fused": 3, "stream": 4, "overlap": 5}
 
 
 def gdn_prefill_route(T, N, max_seqlen_hint, Hv, sm_count=148, cooperative_launch=True) -> str:
@@ -192,23 +161,9 @@ def gdn_prefill(q, k, v, g, beta, cu_seqlens, init_state, final_state, slot_idx,
     launches), "fused" = gdn_prefill_fused (one cooperative launch), "stream" = gdn_prefill_stream
     (three launches, persistent state pass), "overlap" = gdn_prefill_overlap (the intra-chunk work
     in two parts around the state pass; ``split_permille`` is its last argument)."""
-    T, Hqk, dk = q.shape
-    _, Hv, dv = v.shape
-    N = cu_seqlens.shape[0] - 1
-    fn = {"auto": _lib.gdn_prefill, "chunked": _lib.gdn_prefill_chunked,
-          "fused": _lib.gdn_prefill_fused, "stream": _lib.gdn_prefill_stream,
-          "overlap": _lib.gdn_prefill_overlap}[route]
-    extra = (int(split_permille),) if route == "overlap" else ()
-    rc = fn(
-        _dev(q, torch.bfloat16, "q"), _dev(k, torch.bfloat16, "k"), _dev(v, torch.bfloat16, "v"),
-        _dev(g, torch.float32, "g"), _dev(beta, torch.float32, "beta"),
-        _dev(cu_seqlens, torch.int32, "cu_seqlens"),
-        _dev(init_state, torch.float32, "init_state", True),
-        _dev(final_state, torch.float32, "final_state"),
-        _dev(slot_idx, torch.int32, "slot_idx", True), _dev(o, torch.bfloat16, "o"),
-        T, N, int(max_seqlen_hint), Hqk, Hv, dk, dv, int(chunk), final_state.shape[0],
-        float(scale), _dev(workspace, torch.uint8, "workspace"), workspace.numel(),
-        _dev(dev_status, torch.int32, "dev_status", True), _stream(), *extra)
+    rc = _binding.prefill(_ROUTE_CODES[route], q, k, v, g, beta, cu_seqlens, init_state, final_state,
+                          slot_idx, o, scale, workspace, max_seqlen_hint, chunk, dev_status,
+                          split_permille)
     if rc != 0:
         raise GdnError(rc, "gdn_prefill")
 
