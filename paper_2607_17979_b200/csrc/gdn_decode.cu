@@ -12,7 +12,9 @@
 // With p_k = S_old.k and p_q = S_old.q per row (two 8-lane shuffle sums):
 //   u = alpha p_k,  w = beta (v_j - u),  S_new = alpha S_old + w k,
 //   o_j = scale (alpha p_q + w (k.q)).
+// Launched as a programmatic dependent: its CTAs are set up while the kernel before it drains.
 #include "gdn_common.cuh"
+#include "gdn_sm100.cuh"
 
 namespace gdn {
 
@@ -45,6 +47,8 @@ decode_kernel(const DecodeParams p) {
     const int warp = threadIdx.x >> 5;
     const int sub = lane & 7;        // which 16-column share of the row
     const int rsel = lane >> 3;      // which of the pass's four rows
+    sm100::pdl_launch_dependents();
+    sm100::pdl_wait();
 
     __nv_bfloat16* o_row = p.o + (static_cast<size_t>(i) * p.Hv + hv) * kD;
     const int slot = p.slot_idx ? p.slot_idx[i] : i;
@@ -114,11 +118,10 @@ cudaError_t launch_decode(const DecodeParams& p, cudaStream_t stream) {
     // times as many SMs (the state rows are independent)
     DeviceInfo di;
     const int sms = device_info(&di) == cudaSuccess ? di.sms : 148;
-    if (units < 2LL * sms)
-        decode_kernel<1><<<static_cast<unsigned>(units * 4), kDecodeThreads, 0, stream>>>(p);
-    else   // half tiles at three CTAs per SM: measured 0.5-1 % faster than whole tiles at two
-        decode_kernel<2><<<static_cast<unsigned>(units * 2), kDecodeThreads, 0, stream>>>(p);
-    return cudaGetLastError();
+    const bool few = units < 2LL * sms;
+    // half tiles at three CTAs per SM: measured 0.5-1 % faster than whole tiles at two
+    return launch_dependent(few ? decode_kernel<1> : decode_kernel<2>,
+                            dim3(static_cast<unsigned>(units * (few ? 4 : 2))), dim3(kDecodeThreads), 0, stream, p);
 }
 
 }  // namespace gdn
