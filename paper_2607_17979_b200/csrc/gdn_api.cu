@@ -135,11 +135,14 @@ size_t gdn_prefill_workspace_bytes(int32_t T, int32_t N, int32_t Hqk, int32_t Hv
     return gdn::workspace_layout(T, N, Hv).total;
 }
 
-int gdn_prefill_recurrent(const void* q, const void* k, const void* v, const float* g,
-                          const float* beta, const int32_t* cu_seqlens, const float* init_state,
-                          float* final_state, const int32_t* slot_idx, void* o,
-                          int32_t T, int32_t N, int32_t Hqk, int32_t Hv, int32_t dk, int32_t dv,
-                          int32_t num_slots, float scale, int32_t* dev_status, void* stream) {
+}  // extern "C"
+
+namespace {
+int prefill_recurrent_impl(const void* q, const void* k, const void* v, const float* g, const float* beta,
+                           const int32_t* cu_seqlens, const float* init_state, float* final_state,
+                           const int32_t* slot_idx, void* o, int32_t T, int32_t N, int32_t Hqk, int32_t Hv,
+                           int32_t dk, int32_t dv, int32_t num_slots, float scale, int32_t longest,
+                           int32_t* dev_status, void* stream) {
     const int rc = check_prefill(q, k, v, g, beta, cu_seqlens, init_state, final_state, o,
                                  T, N, Hqk, Hv, dk, dv, num_slots);
     if (rc != GDN_OK || T == 0 || N == 0) return rc;
@@ -152,7 +155,19 @@ int gdn_prefill_recurrent(const void* q, const void* k, const void* v, const flo
     p.o = static_cast<__nv_bfloat16*>(o);
     p.T = T; p.N = N; p.Hqk = Hqk; p.Hv = Hv; p.num_slots = num_slots; p.scale = scale;
     p.dev_status = dev_status;
-    return cuda_status(gdn::launch_prefill_recurrent(p, static_cast<cudaStream_t>(stream)));
+    return cuda_status(gdn::launch_prefill_recurrent(p, longest, static_cast<cudaStream_t>(stream)));
+}
+}  // namespace
+
+extern "C" {
+
+int gdn_prefill_recurrent(const void* q, const void* k, const void* v, const float* g,
+                          const float* beta, const int32_t* cu_seqlens, const float* init_state,
+                          float* final_state, const int32_t* slot_idx, void* o,
+                          int32_t T, int32_t N, int32_t Hqk, int32_t Hv, int32_t dk, int32_t dv,
+                          int32_t num_slots, float scale, int32_t* dev_status, void* stream) {
+    return prefill_recurrent_impl(q, k, v, g, beta, cu_seqlens, init_state, final_state, slot_idx, o, T, N,
+                                  Hqk, Hv, dk, dv, num_slots, scale, T, dev_status, stream);
 }
 
 namespace {
@@ -295,9 +310,10 @@ int gdn_prefill(const void* q, const void* k, const void* v, const float* g, con
         if (workspace_bytes < gdn_prefill_workspace_bytes(T, N, Hqk, Hv, dk, dv, chunk))
             return check_heads(Hqk, Hv, dk, dv) != GDN_OK ? check_heads(Hqk, Hv, dk, dv)
                                                           : GDN_ERR_WORKSPACE;
-        return gdn_prefill_recurrent(q, k, v, g, beta, cu_seqlens, init_state, final_state,
-                                     slot_idx, o, T, N, Hqk, Hv, dk, dv, num_slots, scale,
-                                     dev_status, stream);
+        const int32_t longest = (max_seqlen_hint > 0 && max_seqlen_hint < T) ? max_seqlen_hint : T;
+        return prefill_recurrent_impl(q, k, v, g, beta, cu_seqlens, init_state, final_state,
+                                      slot_idx, o, T, N, Hqk, Hv, dk, dv, num_slots, scale, longest,
+                                      dev_status, stream);
     }
     const PrefillRoute route = route_id == GDN_ROUTE_FUSED     ? kRouteFused
                                : route_id == GDN_ROUTE_STREAM  ? kRouteStream

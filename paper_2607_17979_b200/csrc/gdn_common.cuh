@@ -70,7 +70,8 @@ cudaError_t launch_gate(const __nv_bfloat16* a, const __nv_bfloat16* b, const fl
                         cudaStream_t stream);
 cudaError_t launch_state_transpose(float* pool, const int32_t* slot_idx, int32_t n, int32_t Hv,
                                    int32_t num_slots, int32_t* dev_status, cudaStream_t stream);
-cudaError_t launch_prefill_recurrent(const PrefillParams& p, cudaStream_t stream);
+// longest: a bound on the longest sequence (picks the block size, never the results)
+cudaError_t launch_prefill_recurrent(const PrefillParams& p, int longest, cudaStream_t stream);
 
 __device__ __forceinline__ void report(int32_t* dev_status, int bit) {
     if (dev_status) atomicOr(dev_status, bit);

@@ -1,0 +1,487 @@
+// A block of up to 16 consecutive tokens of the gated delta rule applied to a state tile (or a
+// share of its dv rows) held in registers: multi-token decode and the short-prompt prefill.
+//
+// The block is unrolled over its first state S0 (D_ij = product of alpha over tokens j+1..i, D_i over
+// tokens 0..i):
+//     w_i = beta_i (v_i - D_i S0 k_i) - sum_{j<i}  beta_i D_ij (k_i.k_j) w_j
+//     o_i = scale (D_i S0 q_i + sum_{j<=i} D_ij (q_i.k_j) w_j)
+//     S   = D_L S0 + sum_j D_Lj w_j k_j^T
+// so the 2L products with S0 are one small GEMM, the token-to-token part is a triangular solve per row
+// whose coefficients depend on the tokens only, and the state is touched twice per block instead
+// of twice per token.  The decays are products of alphas, never differences of their logarithms'
+// sums, so no gate range loses accuracy.
+//
+// What bounds it: applied token by token on the CUDA cores a tile cost 860 cycles per token and SM
+// (shared-memory reads of k and q and the cross-lane sums as much as the multiply-adds), against
+// 5900 cycles for the tile's HBM traffic, and the two did not overlap well: 52 / 73 / 121 us at L =
+// 4 / 8 / 16 (B = 64, 32 v-heads, floor 42).  Both state GEMMs here are mma.sync with M = 16 rows
+// per warp; the state in fp32 is the accumulator fragment of the update, and the same registers,
+// split EXACTLY into three bf16 terms (8 + 8 + 8 bits), are the A operand of the products with k and
+// q, which are bf16 in memory: no operand is rounded and every sum is fp32.  (w is split the same
+// way.)  tcgen05 would need the split terms in TMEM and a 128-row tile per instruction: a detour
+// through two more memories for a kernel whose floor is the tile's HBM traffic.
+//
+// Fragment map (m16n8k16): lane = 4 g + t; a warp holds 64 state values per lane, s[m][n][c], c = {fragment
+// row g: columns 2t, 2t+1; row g + 8: the same} of 8-column block n of row tile m.
+//   Tiles [dv][dk]: a warp owns 16 dv rows over all 128 dk: one row tile, row g = dv 2 g, row g + 8 = 2 g + 1.
+//     The 16 columns of a k-step are permuted so that a lane's four are one float4: column 8 b + 2 t + e of
+//     k-step j is dk 16 j + 4 t + 2 b + e.
+//   Tiles [dk][dv]: a pair of warps owns 32 dv, each over half of the dk, so that a warp load covers
+//     128-byte pieces of the dv rows (64-byte pieces: 51 us where these take 44, L = 1): two row tiles,
+//     rows g, g + 8 of tile m = dv 4 g + 2 m, + 1; the columns in dk order.  The two warps' partial
+//     products meet in shared memory, each solves one of the row tiles.
+// k and q are staged in fragment column order.
+#pragma once
+#include "gdn_common.cuh"
+
+namespace gdn {
+
+constexpr int kBlockTokens = 16;
+static_assert(kBlockTokens >= kDecodeMaxTokens, "a multi-token decode is one block");
+
+// What the tokens of a block are and where their rows lie.
+struct TokenRows {
+    const __nv_bfloat16 *q, *k, *v;      // first token's row of this head
+    const float *g, *beta;
+    __nv_bfloat16* o;
+    size_t qk_stride, v_stride, g_stride;      // elements from one token to the next
+    int count;                                 // 1..kMax
+    float scale;
+};
+
+// kMax: 4, 8 or 16 tokens the arrays and loops are made for.
+template <bool kTransposed, int kWarps, int kMax> struct TokenBlock {
+    static constexpr int kRows = 16 * kWarps;          // dv rows of the CTA
+    static constexpr int kTiles = kTransposed ? 2 : 1; // row tiles of a warp
+    static constexpr int kPitch = kD + 16;             // bf16
+    static constexpr int kXPitch = 16 * kTiles + 4;    // floats: conflict-free for the fragment's (2t, g)
+    __nv_bfloat16 kq[2 * kMax][kPitch];                // rows 0.. k, kMax.. q
+    __nv_bfloat16 v[kMax][kRows];
+    float x[kWarps][2][kMax][kXPitch];                 // [kind][token][row]: S0 k / S0 q, then D_Lt w_t in kind 0
+    float coef[2][kMax][kMax];                         // [kind][j][i], see the solve
+    float decay[kMax + 1][kMax];                       // [j][i] = D_ij; row kMax: D_i
+    float beta[kMax];
+};
+
+__device__ __forceinline__ uint32_t bf16x2(const float lo, const float hi) {
+    uint32_t r;
+    asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(r) : "f"(hi), "f"(lo));
+    return r;
+}
+// (a, b) -> three packed bf16 pairs whose sum is exact
+__device__ __forceinline__ void split3(float a, float b, uint32_t& h, uint32_t& m, uint32_t& l) {
+    h = bf16x2(a, b);
+    a -= __uint_as_float(h << 16);
+    b -= __uint_as_float(h & 0xffff0000u);
+    m = bf16x2(a, b);
+    l = bf16x2(a - __uint_as_float(m << 16), b - __uint_as_float(m & 0xffff0000u));
+}
+template <bool kTrans> __device__ __forceinline__ void ldmatrix_x4(uint32_t (&r)[4], const void* p) {
+    const uint32_t a = static_cast<uint32_t>(__cvta_generic_to_shared(p));
+    if constexpr (kTrans)
+        asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];"
+                     : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(a) : "memory");
+    else
+        asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];"
+                     : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(a) : "memory");
+}
+__device__ __forceinline__ void mma_k16(float (&c)[4], const uint32_t (&a)[4], const uint32_t b0, const uint32_t b1) {
+    asm(
+        "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, "
+        "{%0,%1,%2,%3};"
+        : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
+        : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+}
+__device__ __forceinline__ void mma_k8(float (&c)[4], const uint32_t a0, const uint32_t a1, const uint32_t b0) {
+    asm(
+        "mma.sync.aligned.m16n8k8.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5}, {%6}, {%0,%1,%2,%3};"
+        : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
+        : "r"(a0), "r"(a1), "r"(b0));
+}
+
+// Which dv rows and dk columns of the tile the warp holds: first dv row, first dk.
+template <bool kTransposed> __device__ __forceinline__ int warp_row0(const int row_base) {
+    const int warp = threadIdx.x >> 5;
+    return row_base + (kTransposed ? 32 * (warp >> 1) : 16 * warp);
+}
+template <bool kTransposed> __device__ __forceinline__ int warp_col0() {
+    return kTransposed ? 64 * ((threadIdx.x >> 5) & 1) : 0;
+}
+
+// Streaming accesses: a tile is read and written once.
+// (volatile: the order of the loads is meant)
+__device__ __forceinline__ float4 ldcs4(const float* p) {
+    float4 r;
+    asm volatile("ld.global.cs.v4.f32 {%0,%1,%2,%3}, [%4];" : "=f"(r.x), "=f"(r.y), "=f"(r.z), "=f"(r.w) : "l"(p));
+    return r;
+}
+template <bool kTransposed> using State = float[kTransposed ? 2 : 1][kTransposed ? 8 : 16][4];
+
+template <bool kTransposed>
+__device__ __forceinline__ void load_state(State<kTransposed>& s, const float* tile, const int row_base) {
+    const int g = (threadIdx.x & 31) >> 2, t = threadIdx.x & 3;
+    const int row0 = warp_row0<kTransposed>(row_base);
+    if constexpr (!kTransposed) {
+        const float* p = tile + (row0 + 2 * g) * kD + 4 * t;
+#pragma unroll
+        for (int j = 0; j < 8; ++j)
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const float4 x = ldcs4(p + h * kD + 16 * j);
+                s[0][2 * j][2 * h] = x.x;
+                s[0][2 * j][2 * h + 1] = x.y;
+                s[0][2 * j + 1][2 * h] = x.z;
+                s[0][2 * j + 1][2 * h + 1] = x.w;
+            }
+    } else {
+        // A fragment's lane order would send the eight lanes of a quarter warp to four rows; so a warp
+        // reads its four rows of 128 bytes in address order (lane 8 r + c: piece c of row r) and every
+        // lane fetches its piece (row t, piece g) from the lane that has it.
+        const int lane = threadIdx.x & 31;
+        const float* p = tile + (warp_col0<true>() + 2 * (lane >> 3)) * kD + row0 + 4 * (lane & 7);
+#pragma unroll
+        for (int n = 0; n < 8; ++n)
+#pragma unroll
+            for (int e = 0; e < 2; ++e) {
+                const float4 x = ldcs4(p + (8 * n + e) * kD);
+                s[0][n][e] = x.x;
+                s[0][n][2 + e] = x.y;
+                s[1][n][e] = x.z;
+                s[1][n][2 + e] = x.w;
+            }
+    }
+}
+// (apart from the loads: the first exchange waits for data)
+__device__ __forceinline__ void exchange_state(float (&s)[2][8][4], const int src_lane) {
+#pragma unroll
+    for (int n = 0; n < 8; ++n)
+#pragma unroll
+        for (int m = 0; m < 2; ++m)
+#pragma unroll
+            for (int c = 0; c < 4; ++c) s[m][n][c] = __shfl_sync(0xffffffffu, s[m][n][c], src_lane);
+}
+template <bool kTransposed>
+__device__ __forceinline__ void store_state(const State<kTransposed>& s, float* tile, const int row_base) {
+    const int g = (threadIdx.x & 31) >> 2, t = threadIdx.x & 3;
+    const int row0 = warp_row0<kTransposed>(row_base);
+    if constexpr (!kTransposed) {
+        float* p = tile + (row0 + 2 * g) * kD + 4 * t;
+#pragma unroll
+        for (int j = 0; j < 8; ++j)
+#pragma unroll
+            for (int h = 0; h < 2; ++h)
+                __stcs(reinterpret_cast<float4*>(p + h * kD + 16 * j),
+                       make_float4(s[0][2 * j][2 * h], s[0][2 * j][2 * h + 1], s[0][2 * j + 1][2 * h],
+                                   s[0][2 * j + 1][2 * h + 1]));
+    } else {
+        const int lane = threadIdx.x & 31;
+        float* p = tile + (warp_col0<true>() + 2 * (lane >> 3)) * kD + row0 + 4 * (lane & 7);
+#pragma unroll
+        for (int n = 0; n < 8; ++n)
+#pragma unroll
+            for (int e = 0; e < 2; ++e)
+                __stcs(reinterpret_cast<float4*>(p + (8 * n + e) * kD),
+                       make_float4(s[0][n][e], s[0][n][2 + e], s[1][n][e], s[1][n][2 + e]));
+    }
+}
+
+// The tokens' rows on their way to shared memory, in registers: loaded BEFORE the tile, so that they do
+// not queue behind its bytes and everything staged from them is ready when the tile lands.
+template <bool kTransposed, int kWarps, int kMax> struct TokenLoads {
+    static constexpr int kThreads = kWarps * 32;
+    static constexpr int kKq = 2 * kMax * (kD / 8);                          // 16-byte pieces of k and q
+    static constexpr int kV = kMax * (TokenBlock<kTransposed, kWarps, kMax>::kRows / 8);  // ... of v
+    uint4 kq[(kKq + kThreads - 1) / kThreads], v[(kV + kThreads - 1) / kThreads];
+    float g, beta;
+};
+__device__ __forceinline__ uint4 ld_piece(const __nv_bfloat16* p) {
+    uint4 r;
+    asm volatile("ld.global.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(r.x), "=r"(r.y), "=r"(r.z), "=r"(r.w) : "l"(p));
+    return r;
+}
+__device__ __forceinline__ float ld_scalar(const float* p) {
+    float r;
+    asm volatile("ld.global.f32 %0, [%1];" : "=f"(r) : "l"(p));
+    return r;
+}
+template <bool kTransposed, int kWarps, int kMax>
+__device__ __forceinline__ void load_tokens(TokenLoads<kTransposed, kWarps, kMax>& ld, const TokenRows& t, const int row_base) {
+    using L = TokenLoads<kTransposed, kWarps, kMax>;
+    const int tid = threadIdx.x;
+    ld.g = ld.beta = 0.f;
+    if (tid < t.count) {
+        ld.g = ld_scalar(t.g + tid * t.g_stride);
+        ld.beta = ld_scalar(t.beta + tid * t.g_stride);
+    }
+#pragma unroll
+    for (int it = 0; it < (L::kKq + L::kThreads - 1) / L::kThreads; ++it) {
+        const int idx = tid + it * L::kThreads, row = idx >> 4, tok = row & (kMax - 1);
+        ld.kq[it] = make_uint4(0u, 0u, 0u, 0u);                 // rows past the count are zero
+        if (idx < L::kKq && tok < t.count)
+            ld.kq[it] = ld_piece((row < kMax ? t.k : t.q) + tok * t.qk_stride + (idx & 15) * 8);
+    }
+    constexpr int kPieces = TokenBlock<kTransposed, kWarps, kMax>::kRows / 8;
+#pragma unroll
+    for (int it = 0; it < (L::kV + L::kThreads - 1) / L::kThreads; ++it) {
+        const int idx = tid + it * L::kThreads, tok = idx / kPieces;
+        ld.v[it] = make_uint4(0u, 0u, 0u, 0u);
+        if (idx < L::kV && tok < t.count)
+            ld.v[it] = ld_piece(t.v + tok * t.v_stride + row_base + (idx - tok * kPieces) * 8);
+    }
+}
+
+// Tokens -> shared memory, decays; then the solve's coefficients.  Two CTA barriers, both passed
+// while the tile's loads are in flight.
+template <bool kTransposed, int kWarps, int kMax>
+__device__ __forceinline__ void stage_block(const TokenRows& t, TokenBlock<kTransposed, kWarps, kMax>& st,
+                                            const TokenLoads<kTransposed, kWarps, kMax>& ld) {
+    using L = TokenLoads<kTransposed, kWarps, kMax>;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    if (warp == 0) {       // decays: lane j < kMax walks D_ij down i, lane kMax walks D_i
+        float alpha = 1.f;
+        if (lane < t.count) {
+            alpha = expf(ld.g);
+            st.beta[lane] = ld.beta;
+        }
+        float d = lane < kMax ? 0.f : 1.f;
+#pragma unroll
+        for (int i = 0; i < kMax; ++i) {
+            const float a = __shfl_sync(0xffffffffu, alpha, i);
+            d = i == lane ? 1.f : d * a;
+            if (lane <= kMax) st.decay[lane][i] = d;
+        }
+    }
+#pragma unroll
+    for (int it = 0; it < (L::kKq + L::kThreads - 1) / L::kThreads; ++it) {
+        const int idx = tid + it * L::kThreads, row = idx >> 4, piece = idx & 15;
+        if (L::kKq % L::kThreads != 0 && idx >= L::kKq) break;
+        const uint4 raw = ld.kq[it];
+        if (kTransposed) {
+            *reinterpret_cast<uint4*>(&st.kq[row][piece * 8]) = raw;
+        } else {           // fragment column order
+            __nv_bfloat16* dst = &st.kq[row][(piece >> 1) * 16 + (piece & 1) * 4];
+            *reinterpret_cast<uint2*>(dst) = make_uint2(raw.x, raw.z);
+            *reinterpret_cast<uint2*>(dst + 8) = make_uint2(raw.y, raw.w);
+        }
+    }
+#pragma unroll
+    for (int it = 0; it < (L::kV + L::kThreads - 1) / L::kThreads; ++it) {
+        const int idx = tid + it * L::kThreads;
+        if (L::kV % L::kThreads != 0 && idx >= L::kV) break;
+        *reinterpret_cast<uint4*>(&st.v[0][0] + idx * 8) = ld.v[it];
+    }
+    __syncthreads();
+
+    // k.k and q.k of the block's tokens: 16 fragment rows are 16 k or q rows (kMax = 16: one warp each),
+    // k then q (8), or k, q and nothing (4)
+    if (warp < (kMax == 16 ? 2 : 1)) {
+        const int g = lane >> 2, t4 = lane & 3;
+        constexpr int kN = kMax == 16 ? 2 : 1;
+        float c[kN][4];
+#pragma unroll
+        for (auto& r : c) r[0] = r[1] = r[2] = r[3] = 0.f;
+        const int arow = kMax == 4 ? lane & 7 : 16 * warp + (lane & 15);
+        const int brow = (lane & 7) + (kMax == 16 ? 8 * (lane >> 4) : 0);
+#pragma unroll
+        for (int ks = 0; ks < 8; ++ks) {
+            uint32_t a[4], b[4];
+            ldmatrix_x4<false>(a, &st.kq[arow][16 * ks + 8 * (lane >> 4)]);
+            ldmatrix_x4<false>(b, &st.kq[brow][16 * ks + 8 * ((lane >> 3) & 1)]);
+#pragma unroll
+            for (int nb = 0; nb < kN; ++nb) mma_k16(c[nb], a, b[2 * nb], b[2 * nb + 1]);
+        }
+#pragma unroll
+        for (int nb = 0; nb < kN; ++nb)
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                const int row = 16 * warp + g + 8 * (e >> 1), j = 8 * nb + 2 * t4 + (e & 1);
+                const int kind = row / kMax, i = row & (kMax - 1);
+                if (kind < 2 && j < kMax) {
+                    const bool keep = i < t.count && (kind == 0 ? j < i : j <= i);
+                    const float f = kind == 0 ? -st.beta[i] : t.scale;
+                    st.coef[kind][j][i] = keep ? f * st.decay[j][i] * c[nb][e] : 0.f;
+                }
+            }
+    }
+    __syncthreads();
+}
+
+// The staged block on the state in registers.  Barriers of the warp only (tiles [dk][dv]: of the pair).
+template <bool kTransposed, int kWarps, int kMax>
+__device__ __forceinline__ void apply_block(const TokenRows& t, TokenBlock<kTransposed, kWarps, kMax>& st,
+                                            State<kTransposed>& s, const int row_base) {
+    using Block = TokenBlock<kTransposed, kWarps, kMax>;
+    constexpr int kTiles = Block::kTiles, kSteps = 8 / kTiles;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int g = lane >> 2, t4 = lane & 3;
+    const int count = t.count;
+    const int col0 = warp_col0<kTransposed>();
+    static_assert(!kTransposed || kWarps == 2 || kWarps == 4, "one or two pairs of warps");
+    auto group_sync = [warp] {
+        if constexpr (!kTransposed) __syncwarp();
+        else if (kWarps == 2 || warp < 2) asm volatile("bar.sync 1, 64;" ::: "memory");
+        else asm volatile("bar.sync 2, 64;" ::: "memory");
+    };
+
+    // S0 K^T, S0 Q^T: the staged rows are the N dimension, eight at a time
+    constexpr int kN = 2 * kMax / 8;
+    constexpr int kSets = kTiles == 2 ? 1 : kN == 1 ? 3 : kN == 2 ? 2 : 1;     // accumulators per split term: shorter chains
+    if constexpr (kTransposed) exchange_state(s, 8 * t4 + g);       // address order -> fragment order
+    float c[kTiles][kN][kSets][4];
+#pragma unroll
+    for (auto& m : c)
+#pragma unroll
+        for (auto& n : m)
+#pragma unroll
+            for (auto& r : n) r[0] = r[1] = r[2] = r[3] = 0.f;
+    uint32_t b[4];                                // (kN = 1 only)
+#pragma unroll
+    for (int j = 0; j < kSteps; ++j) {
+        uint32_t a[kTiles][3][4];
+#pragma unroll
+        for (int m = 0; m < kTiles; ++m)
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {         // a0, a1: rows g, g + 8 of block b = 0; a2, a3: of b = 1
+                const float* y = &s[m][2 * j + (e >> 1)][2 * (e & 1)];
+                split3(y[0], y[1], a[m][0][e], a[m][1][e], a[m][2][e]);
+            }
+        if constexpr (kN == 1) {
+            // 32 columns of the eight rows: one load for two k-steps
+            if ((j & 1) == 0) ldmatrix_x4<false>(b, &st.kq[lane & 7][col0 + 16 * j + 8 * (lane >> 3)]);
+#pragma unroll
+            for (int sp = 0; sp < 3; ++sp)
+#pragma unroll
+                for (int m = 0; m < kTiles; ++m)
+                    mma_k16(c[m][0][sp % kSets], a[m][sp], b[2 * (j & 1)], b[2 * (j & 1) + 1]);
+        } else {
+            uint32_t bn[kN / 2][4];
+#pragma unroll
+            for (int n = 0; n < kN / 2; ++n)      // 16 columns of sixteen rows
+                ldmatrix_x4<false>(bn[n], &st.kq[16 * n + (lane & 7) + 8 * (lane >> 4)]
+                                                [col0 + 16 * j + 8 * ((lane >> 3) & 1)]);
+#pragma unroll
+            for (int sp = 0; sp < 3; ++sp)
+#pragma unroll
+                for (int m = 0; m < kTiles; ++m)
+#pragma unroll
+                    for (int n = 0; n < kN; ++n)
+                        mma_k16(c[m][n][sp % kSets], a[m][sp], bn[n >> 1][2 * (n & 1)], bn[n >> 1][2 * (n & 1) + 1]);
+        }
+    }
+#pragma unroll
+    for (int m = 0; m < kTiles; ++m)
+#pragma unroll
+        for (int n = 0; n < kN; ++n)
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                const int col = 8 * n + 2 * t4 + (e & 1);
+                float v = c[m][n][0][e];
+                if constexpr (kSets > 1) v += c[m][n][1][e];
+                if constexpr (kSets > 2) v += c[m][n][2][e];
+                st.x[warp][col / kMax][col & (kMax - 1)][16 * m + g + 8 * (e >> 1)] = v;
+            }
+    group_sync();
+
+    // Solve: lane (kind, row) carries w_i (kind 0) or o_i (kind 1) of its row, right-looking.
+    const int kind = lane >> 4;
+    const int tile = kTransposed ? warp & 1 : 0;             // the row tile this warp solves
+    const int row = 16 * tile + (lane & 15);
+    const int local_row = kTransposed ? 32 * (warp >> 1) + 4 * (lane & 7) + 2 * tile + ((lane & 15) >> 3)
+                                      : 16 * warp + 2 * (lane & 7) + ((lane & 15) >> 3);
+    const int xw = kTransposed ? warp & ~1 : warp;           // where the pair's (the warp's) sums and w live
+    float acc[kMax];
+#pragma unroll
+    for (int i = 0; i < kMax; ++i) {
+        acc[i] = 0.f;
+        if (i < count) {
+            float y = st.x[xw][kind][i][row];
+            if constexpr (kTransposed) y += st.x[xw + 1][kind][i][row];
+            y *= st.decay[kMax][i];
+            acc[i] = kind == 0 ? st.beta[i] * (__bfloat162float(st.v[i][local_row]) - y) : t.scale * y;
+        }
+    }
+    __syncwarp();                                 // (the rows this warp rewrites below are read by it alone)
+    const float* coef = &st.coef[kind][0][0];
+    __nv_bfloat16* o_row = t.o + row_base + local_row;
+#pragma unroll
+    for (int j = 0; j < kMax; ++j) {
+        float wj = 0.f;
+        if (j < count) {
+            const float w = __shfl_sync(0xffffffffu, acc[j], lane & 15);
+#pragma unroll
+            for (int i4 = (j / 4) * 4; i4 < kMax; i4 += 4) {
+                const float4 cf = *reinterpret_cast<const float4*>(coef + j * kMax + i4);
+                if (i4 >= j) acc[i4] = fmaf(cf.x, w, acc[i4]);
+                if (i4 + 1 >= j) acc[i4 + 1] = fmaf(cf.y, w, acc[i4 + 1]);
+                if (i4 + 2 >= j) acc[i4 + 2] = fmaf(cf.z, w, acc[i4 + 2]);
+                if (i4 + 3 >= j) acc[i4 + 3] = fmaf(cf.w, w, acc[i4 + 3]);
+            }
+            wj = w * st.decay[j][count - 1];
+            if (kind == 1) o_row[j * t.v_stride] = __float2bfloat16(acc[j]);
+        }
+        if (kind == 0) st.x[xw][0][j][row] = wj;
+    }
+    group_sync();
+
+    // S = D_L S0 + sum_j (D_Lj w_j) k_j^T
+    const float last = st.decay[kMax][count - 1];
+    // A operand: w's split terms over the 16 token columns of an instruction: 16 tokens of one term (kMax =
+    // 16: three instructions), 8 of the first and of the second, the third by itself in one with
+    // 8 columns (8), or 4 of each of the three (4: one instruction); B repeats k's rows alike
+    constexpr int kA = kMax == 16 ? 3 : kMax == 8 ? 2 : 1;
+    uint32_t a[kTiles][kA][4];
+#pragma unroll
+    for (int m = 0; m < kTiles; ++m)
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {             // rows g, g + 8; this lane's tokens 2t, 2t+1
+            const int r = 16 * m + g + 8 * h;
+            if constexpr (kMax == 16) {
+#pragma unroll
+                for (int e = 0; e < 2; ++e)
+                    split3(st.x[xw][0][2 * t4 + 8 * e][r], st.x[xw][0][2 * t4 + 8 * e + 1][r], a[m][0][2 * e + h],
+                           a[m][1][2 * e + h], a[m][2][2 * e + h]);
+            } else if constexpr (kMax == 8) {
+                split3(st.x[xw][0][2 * t4][r], st.x[xw][0][2 * t4 + 1][r], a[m][0][h], a[m][0][2 + h], a[m][1][h]);
+            } else {
+                uint32_t hi, mid, lo;
+                split3(st.x[xw][0][2 * (t4 & 1)][r], st.x[xw][0][2 * (t4 & 1) + 1][r], hi, mid, lo);
+                a[m][0][h] = t4 < 2 ? hi : mid;
+                a[m][0][2 + h] = t4 < 2 ? lo : 0u;
+            }
+        }
+#pragma unroll
+    for (int n0 = 0; n0 < 2 * kSteps; n0 += 4) {  // four 8-column blocks of independent accumulators at a time
+        // tokens x columns, transposed on the way in
+        uint32_t bn[kMax == 16 ? 2 : 1][4];
+        if constexpr (kMax == 16) {
+#pragma unroll
+            for (int h = 0; h < 2; ++h)
+                ldmatrix_x4<true>(bn[h], &st.kq[lane & 15][col0 + 8 * (n0 + 2 * h + (lane >> 4))]);
+        } else {
+            ldmatrix_x4<true>(bn[0], &st.kq[lane & (kMax - 1)][col0 + 8 * (n0 + (lane >> 3))]);
+        }
+#pragma unroll
+        for (int n = 0; n < 4; ++n)
+#pragma unroll
+            for (int m = 0; m < kTiles; ++m)
+#pragma unroll
+                for (float& y : s[m][n0 + n]) y *= last;
+#pragma unroll
+        for (int i = kA - 1; i >= 0; --i)         // small terms first
+#pragma unroll
+            for (int n = 0; n < 4; ++n)
+#pragma unroll
+                for (int m = 0; m < kTiles; ++m) {
+                    float(&d)[4] = s[m][n0 + n];
+                    if constexpr (kMax == 16)
+                        mma_k16(d, a[m][i], bn[n >> 1][2 * (n & 1)], bn[n >> 1][2 * (n & 1) + 1]);
+                    else if (kMax == 8 && i == 1)
+                        mma_k8(d, a[m][1][0], a[m][1][1], bn[0][n]);
+                    else
+                        mma_k16(d, a[m][0], bn[0][n], bn[0][n]);
+                }
+    }
+    if constexpr (kTransposed) exchange_state(s, 4 * (lane & 7) + (lane >> 3));      // and back
+}
+
+}  // namespace gdn
