@@ -198,12 +198,28 @@ __device__ __forceinline__ void solve_merge_64(float* sA, const int nb, const in
     }
 }
 
-// Lane 0 polls the mbarrier (bounded), the other lanes block at the warp barrier instead of
-// competing for issue slots; returns the same verdict on every lane.
-__device__ __forceinline__ bool warp_wait(uint64_t* bar, uint32_t parity) {
-    int ok = 1;
-    if ((threadIdx.x & 31) == 0) ok = mbar_wait(bar, parity) ? 1 : 0;
-    return __shfl_sync(0xffffffffu, ok, 0) != 0;
+// bounded wait that also gives up as soon as another role has flagged an abort.  `reason` is what a
+// wait that runs out writes into the flag: 1 = an error (reported as a timeout), 2 = give up
+// without an error (the caller's work is finished by a later launch).
+__device__ __forceinline__ bool wait_or_abort(uint64_t* bar, uint32_t parity, volatile int* abort_flag,
+                                              const int reason = 1) {
+    for (uint32_t i = 0; i < kSpinLimit; ++i) {
+        if (mbar_try_wait(bar, parity)) return true;
+        if ((i & 255u) == 255u && *abort_flag) return false;
+    }
+    if (*abort_flag == 0) *abort_flag = reason;      // keep an earlier, different reason
+    return false;
+}
+
+// Same, for a whole converged warp: every lane polls, so the instruction stays warp-wide and the
+// verdict is the same on every lane.  (Polling by lane 0 and broadcasting the verdict costs a divergent
+// branch and a shuffle: a wait on a completed barrier took 140 cycles instead of 4, and a waiting
+// warp saw an arrival after 183 instead of 62.)
+__device__ __forceinline__ bool warp_wait_or_abort(uint64_t* bar, uint32_t parity, volatile int* abort_flag,
+                                                   const int reason = 1) {
+    const bool ok = wait_or_abort(bar, parity, abort_flag, reason);
+    __syncwarp();
+    return ok;
 }
 
 // The intra-chunk quantities of one (chunk, v-head) item, computed by a group of 256 threads
@@ -277,7 +293,10 @@ __device__ __forceinline__ bool intra_item(const TensorMaps& maps, const Prefill
         if (lane == 0) dec[kChunk] = ex2_approx(bC * kLog2e);
     }
     sync();
-    // On a timeout: flag it and let thread 0 drain what it has in flight; the caller unwinds.
+    // Every warp polls the barriers it needs itself.  A wait that runs out flags the item and the group
+    // goes on to its next barrier, behind which everyone leaves together; thread 0 drains what it has
+    // in flight and the caller unwinds.
+    volatile int* abortp = &st.abort_flag;
     auto bail = [&](bool stores_pending) {
         if (tid == 0) {
             report(p.dev_status, kDevTimeout);
@@ -285,27 +304,23 @@ __device__ __forceinline__ bool intra_item(const TensorMaps& maps, const Prefill
         }
     };
 
-    if (warp == 0 && !warp_wait(&st.bar_tma, par1)) st.abort_flag = 1;      // one warp polls, the rest block
-    sync();
-    if (st.abort_flag) { bail(false); return false; }
-    tc_fence_after_sync();
-
     const uint32_t tG = tmem, tW = tmem, tU = tmem + 64;     // W reuses the Gram columns
     const uint32_t sQK = smem_u32(smem + kI_QK);
-    if (tid == 0) {
+    // Tensor-core instructions are issued by warp 0, converged, one elected lane each (issuing eight
+    // from a single-lane branch takes 500 cycles instead of 180).
+    if (warp == 0 && warp_wait_or_abort(&st.bar_tma, par1, abortp)) {
+        tc_fence_after_sync();
         // [Q;K] (128 x 128, K-major) times K^T: lanes 0-63 = q.k, lanes 64-127 = k.k
         const uint32_t idesc = make_idesc_bf16(128, 64, false, false);
+        const uint64_t dA = make_sdesc_sw128(sQK, 16, 1024), dB = make_sdesc_sw128(sQK + 8192, 16, 1024);
 #pragma unroll
         for (int ks = 0; ks < 8; ++ks) {
             const uint32_t off = (ks >> 2) * 16384 + (ks & 3) * 32;
-            mma_ss(tG, make_sdesc_sw128(sQK + off, 16, 1024),
-                   make_sdesc_sw128(sQK + 8192 + off, 16, 1024), idesc, ks > 0);
+            if (elect_one()) mma_ss(tG, sdesc_advance(dA, off), sdesc_advance(dB, off), idesc, ks > 0);
         }
-        mma_commit(&st.bar_mma);
+        if (elect_one()) mma_commit(&st.bar_mma);
     }
-    if (warp == 0 && !warp_wait(&st.bar_mma, par3)) st.abort_flag = 1;
-    sync();
-    if (st.abort_flag) { bail(false); return false; }
+    warp_wait_or_abort(&st.bar_mma, par3, abortp);
     tc_fence_after_sync();
 
     const uint32_t lane_base = static_cast<uint32_t>((warp & 3) * 32) << 16;
@@ -366,6 +381,7 @@ __device__ __forceinline__ bool intra_item(const TensorMaps& maps, const Prefill
     }
     tc_fence_before_sync();
     sync();
+    if (st.abort_flag) { bail(false); return false; }
     // Two jobs side by side: warps 0-1 invert the two diagonal 32x32 blocks of I + A (serial
     // forward substitutions and two small products each, all inside the warp), warps 2-7 scale
     // the Q rows by scale * e^{b_r} in place (the Gram product has consumed Q): the Qg image.
@@ -400,58 +416,50 @@ __device__ __forceinline__ bool intra_item(const TensorMaps& maps, const Prefill
     }
     sync();
 
-    uint32_t tu_lo[2][4];    // T diag(beta) - bf16(T diag(beta)), parked until T_w is dead
-    {   // T (fp32, row-major) -> bf16 B operands T diag(beta e^b), T diag(beta) (hi, lo)
+    // T (fp32, row-major) -> bf16 B operands T diag(beta e^b), T diag(beta) (hi, lo).  A thread takes four
+    // columns of every 16th row: its column factors stay in registers and both the reads of T and
+    // the writes of the images cover whole 128-byte rows (eight columns a thread conflicted twice
+    // over on every access: a quarter of this kernel's shared-memory cycles).
+    uint32_t tu_lo[4][2];    // T diag(beta) - bf16(T diag(beta)), parked until T_w is dead
+    const int icol = tid & 15, irow = tid >> 4;
+    auto image_offset = [&](int it) { return sw128_offset(irow + 16 * it, icol >> 1) + 8u * (icol & 1); };
+    {
+        const float4 fg = *reinterpret_cast<const float4*>(st.s_bg + 4 * icol);
+        const float4 fb = *reinterpret_cast<const float4*>(st.s_beta + 4 * icol);
 #pragma unroll
-        for (int it = 0; it < 2; ++it) {
-            const int idx = tid + it * kIntraThreads;          // 512 pieces of 8 columns
-            const int r = idx >> 3, c8 = idx & 7;
-            const float4 t0 = *reinterpret_cast<const float4*>(sA + r * kLdA + 8 * c8);
-            const float4 t1 = *reinterpret_cast<const float4*>(sA + r * kLdA + 8 * c8 + 4);
-            const float4 g0 = *reinterpret_cast<const float4*>(st.s_bg + 8 * c8);
-            const float4 g1 = *reinterpret_cast<const float4*>(st.s_bg + 8 * c8 + 4);
-            const float4 e0 = *reinterpret_cast<const float4*>(st.s_beta + 8 * c8);
-            const float4 e1 = *reinterpret_cast<const float4*>(st.s_beta + 8 * c8 + 4);
-            const float tv[8] = {t0.x, t0.y, t0.z, t0.w, t1.x, t1.y, t1.z, t1.w};
-            const float gv[8] = {g0.x, g0.y, g0.z, g0.w, g1.x, g1.y, g1.z, g1.w};
-            const float ev[8] = {e0.x, e0.y, e0.z, e0.w, e1.x, e1.y, e1.z, e1.w};
-            uint32_t w[4], hi[4];
-#pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                w[j] = pack_bf16(tv[2 * j] * gv[2 * j], tv[2 * j + 1] * gv[2 * j + 1]);
-                const float u0 = tv[2 * j] * ev[2 * j], u1 = tv[2 * j + 1] * ev[2 * j + 1];
-                hi[j] = pack_bf16(u0, u1);
-                tu_lo[it][j] = pack_bf16(u0 - __uint_as_float(hi[j] << 16),
-                                         u1 - __uint_as_float(hi[j] & 0xffff0000u));
-            }
-            const uint32_t off = sw128_offset(r, c8);
-            *reinterpret_cast<uint4*>(smem + kI_Tw + off) = make_uint4(w[0], w[1], w[2], w[3]);
-            *reinterpret_cast<uint4*>(smem + kI_Tu + off) = make_uint4(hi[0], hi[1], hi[2], hi[3]);
+        for (int it = 0; it < 4; ++it) {
+            const float4 t = *reinterpret_cast<const float4*>(sA + (irow + 16 * it) * kLdA + 4 * icol);
+            const float u0 = t.x * fb.x, u1 = t.y * fb.y, u2 = t.z * fb.z, u3 = t.w * fb.w;
+            const uint32_t h0 = pack_bf16(u0, u1), h1 = pack_bf16(u2, u3);
+            tu_lo[it][0] = pack_bf16(u0 - __uint_as_float(h0 << 16), u1 - __uint_as_float(h0 & 0xffff0000u));
+            tu_lo[it][1] = pack_bf16(u2 - __uint_as_float(h1 << 16), u3 - __uint_as_float(h1 & 0xffff0000u));
+            const uint32_t off = image_offset(it);
+            *reinterpret_cast<uint2*>(smem + kI_Tw + off) =
+                make_uint2(pack_bf16(t.x * fg.x, t.y * fg.y), pack_bf16(t.z * fg.z, t.w * fg.w));
+            *reinterpret_cast<uint2*>(smem + kI_Tu + off) = make_uint2(h0, h1);
         }
     }
     fence_proxy_async_smem();
     sync();
 
     const uint32_t sV = smem_u32(smem + kI_V);
-    if (tid == 0) {
-        // V into the space the solve has left; meanwhile W^T (dk x r) = K^T T_w^T with the raw K
-        // tile read MN-major
+    if (tid == 0) {      // V into the space the solve has left
         mbar_expect_tx(&st.bar_v, 16384);
         tma_load_2d(smem + kI_V, &maps.v, hv * kD, ci.t0, &st.bar_v);
         tma_load_2d(smem + kI_V + 8192, &maps.v, hv * kD + 64, ci.t0, &st.bar_v);
-        const uint32_t idesc = make_idesc_bf16(128, 64, true, false);
-        const uint32_t sTw = smem_u32(smem + kI_Tw);
+    }
+    __syncwarp();
+    const uint32_t idesc_t = make_idesc_bf16(128, 64, true, false);
+    if (warp == 0) {     // meanwhile W^T (dk x r) = K^T T_w^T with the raw K tile read MN-major
+        const uint64_t dK = make_sdesc_sw128(sQK + 8192, 16384, 1024), dT = make_sdesc_sw128(smem_u32(smem + kI_Tw), 16, 1024);
         // columns of T_w and T_u past the chunk's length are zero: their k-steps are left out
 #pragma unroll
         for (int ks = 0; ks < 4; ++ks)
-            if (ks * 16 < ci.len)
-                mma_ss(tW, make_sdesc_sw128(sQK + 8192 + ks * 2048, 16384, 1024),
-                       make_sdesc_sw128(sTw + ks * 32, 16, 1024), idesc, ks > 0);
-        mma_commit(&st.bar_mma);
+            if (ks * 16 < ci.len && elect_one())
+                mma_ss(tW, sdesc_advance(dK, ks * 2048), sdesc_advance(dT, ks * 32), idesc_t, ks > 0);
+        if (elect_one()) mma_commit(&st.bar_mma);
     }
-    if (warp == 0 && !warp_wait(&st.bar_mma, par3 ^ 1u)) st.abort_flag = 1;
-    sync();
-    if (st.abort_flag) { bail(false); return false; }      // nothing of thread 0's stores is pending here
+    warp_wait_or_abort(&st.bar_mma, par3 ^ 1u, abortp);
     tc_fence_after_sync();
 
     const int d = (warp & 3) * 32 + (tid & 31);   // TMEM lane of this thread: a dk / dv index
@@ -478,39 +486,34 @@ __device__ __forceinline__ bool intra_item(const TensorMaps& maps, const Prefill
     }
     // the product that read T_w has retired: its place takes the remainder of T diag(beta)
 #pragma unroll
-    for (int it = 0; it < 2; ++it) {
-        const int idx = tid + it * kIntraThreads;
-        *reinterpret_cast<uint4*>(smem + kI_TuLo + sw128_offset(idx >> 3, idx & 7)) =
-            make_uint4(tu_lo[it][0], tu_lo[it][1], tu_lo[it][2], tu_lo[it][3]);
-    }
+    for (int it = 0; it < 4; ++it)
+        *reinterpret_cast<uint2*>(smem + kI_TuLo + image_offset(it)) = make_uint2(tu_lo[it][0], tu_lo[it][1]);
     fence_proxy_async_smem();
     tc_fence_before_sync();
-    if (warp == 0 && !warp_wait(&st.bar_v, par1)) st.abort_flag = 1;        // V has landed
     sync();
-    if (st.abort_flag) { bail(false); return false; }
-    tc_fence_after_sync();
+    if (st.abort_flag) { bail(false); return false; }      // nothing of thread 0's stores is pending here
     if (tid == 0) {
         bulk_store(rec + kRecW, smem + kI_QK + 8192, 8192);
         bulk_store(rec + kRecW + 8192, smem + kI_QK + 24576, 8192);
         bulk_commit();
-        // U~^T (dv x r) = V^T T_u^T with T_u = hi + lo
-        const uint32_t idesc = make_idesc_bf16(128, 64, true, false);
-        const uint32_t sTu = smem_u32(smem + kI_Tu), sTuLo = smem_u32(smem + kI_TuLo);
-#pragma unroll
-        for (int ks = 0; ks < 4; ++ks)
-            if (ks * 16 < ci.len)
-                mma_ss(tU, make_sdesc_sw128(sV + ks * 2048, 8192, 1024),
-                       make_sdesc_sw128(sTu + ks * 32, 16, 1024), idesc, ks > 0);
-#pragma unroll
-        for (int ks = 0; ks < 4; ++ks)
-            if (ks * 16 < ci.len)
-                mma_ss(tU, make_sdesc_sw128(sV + ks * 2048, 8192, 1024),
-                       make_sdesc_sw128(sTuLo + ks * 32, 16, 1024), idesc, true);
-        mma_commit(&st.bar_mma);
     }
-    if (warp == 0 && !warp_wait(&st.bar_mma, par3)) st.abort_flag = 1;
-    sync();
-    if (st.abort_flag) { bail(true); return false; }
+    __syncwarp();
+    if (warp == 0 && warp_wait_or_abort(&st.bar_v, par1, abortp)) {        // V has landed
+        tc_fence_after_sync();
+        // U~^T (dv x r) = V^T T_u^T with T_u = hi + lo
+        const uint64_t dV = make_sdesc_sw128(sV, 8192, 1024);
+        const uint64_t dH = make_sdesc_sw128(smem_u32(smem + kI_Tu), 16, 1024), dL = make_sdesc_sw128(smem_u32(smem + kI_TuLo), 16, 1024);
+#pragma unroll
+        for (int ks = 0; ks < 4; ++ks)
+            if (ks * 16 < ci.len && elect_one())
+                mma_ss(tU, sdesc_advance(dV, ks * 2048), sdesc_advance(dH, ks * 32), idesc_t, ks > 0);
+#pragma unroll
+        for (int ks = 0; ks < 4; ++ks)
+            if (ks * 16 < ci.len && elect_one())
+                mma_ss(tU, sdesc_advance(dV, ks * 2048), sdesc_advance(dL, ks * 32), idesc_t, true);
+        if (elect_one()) mma_commit(&st.bar_mma);
+    }
+    warp_wait_or_abort(&st.bar_mma, par3, abortp);
     tc_fence_after_sync();
 
     {   // U~^T[d][32 tokens] -> record, [token group][dv][4 tokens] fp32
@@ -530,6 +533,7 @@ __device__ __forceinline__ bool intra_item(const TensorMaps& maps, const Prefill
     }
     tc_fence_before_sync();
     sync();
+    if (st.abort_flag) { bail(true); return false; }
     if (tid == 0) bulk_wait_read_all();
     return true;
 }
@@ -542,30 +546,6 @@ constexpr uint32_t kS_Out = 2 * kStageBytes;   // o staging [64 tokens][128 dv] 
 // TMEM columns
 constexpr uint32_t kT_D1 = 0, kT_Y = 64 /* two tiles of 64 */, kT_D4 = 192, kT_S = 320, kT_U = 384,
                    kT_Us = 416, kT_UsLo = 448;
-
-// bounded wait that also gives up as soon as another role has flagged an abort.  `reason` is what a
-// wait that runs out writes into the flag: 1 = an error (reported as a timeout), 2 = give up
-// without an error (the caller's work is finished by a later launch).
-__device__ __forceinline__ bool wait_or_abort(uint64_t* bar, uint32_t parity, volatile int* abort_flag,
-                                              const int reason = 1) {
-    for (uint32_t i = 0; i < kSpinLimit; ++i) {
-        if (mbar_try_wait(bar, parity)) return true;
-        if ((i & 255u) == 255u && *abort_flag) return false;
-    }
-    if (*abort_flag == 0) *abort_flag = reason;      // keep an earlier, different reason
-    return false;
-}
-
-// Same, for a whole converged warp: every lane polls, so the instruction stays warp-wide and the
-// verdict is the same on every lane.  (Polling by lane 0 and broadcasting the verdict costs a divergent
-// branch and a shuffle: a wait on a completed barrier took 140 cycles instead of 4, and a waiting
-// warp saw an arrival after 183 instead of 62.)
-__device__ __forceinline__ bool warp_wait_or_abort(uint64_t* bar, uint32_t parity, volatile int* abort_flag,
-                                                   const int reason = 1) {
-    const bool ok = wait_or_abort(bar, parity, abort_flag, reason);
-    __syncwarp();
-    return ok;
-}
 
 
 }  // namespace gdn
