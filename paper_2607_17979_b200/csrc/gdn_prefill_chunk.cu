@@ -136,7 +136,8 @@ bool make_token_map(CUtensorMap* m, const void* base, int64_t rows, int64_t cols
 bool make_prefill_tensor_maps(TensorMaps* maps, const PrefillParams& p) {
     return make_token_map(&maps->q, p.q, p.T, static_cast<int64_t>(p.Hqk) * kD) &&
            make_token_map(&maps->k, p.k, p.T, static_cast<int64_t>(p.Hqk) * kD) &&
-           make_token_map(&maps->v, p.v, p.T, static_cast<int64_t>(p.Hv) * kD);
+           make_token_map(&maps->v, p.v, p.T, static_cast<int64_t>(p.Hv) * kD) &&
+           make_token_map(&maps->o, p.o, p.T, static_cast<int64_t>(p.Hv) * kD);
 }
 
 bool prefill_tables_inline(const ChunkedParams& cp) {

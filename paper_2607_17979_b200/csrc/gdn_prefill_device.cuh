@@ -29,9 +29,9 @@ constexpr uint32_t kIntraSmem = kI_End + 1024;         // + alignment slack
 static_assert(kI_End % 1024 == 0 && 64 * kLdA * 4 >= 16384, "V tile must fit over A");
 
 struct TensorMaps {
-    CUtensorMap q, k, v;
+    CUtensorMap q, k, v, o;
 };
-// Host side: 2-D maps over the packed q, k, v (64 x 64 boxes, 128B swizzle); false on failure.
+// Host side: 2-D maps over the packed q, k, v, o (64 x 64 boxes, 128B swizzle); false on failure.
 bool make_prefill_tensor_maps(TensorMaps* maps, const PrefillParams& p);
 // Launch of the intra-chunk kernel over every (chunk, v-head) item of the batch.
 // inline_tables: no table-building launch went before; every CTA finds its chunk from cu_seqlens and
@@ -201,23 +201,40 @@ __device__ __forceinline__ void solve_merge_64(float* sA, const int nb, const in
 // bounded wait that also gives up as soon as another role has flagged an abort.  `reason` is what a
 // wait that runs out writes into the flag: 1 = an error (reported as a timeout), 2 = give up
 // without an error (the caller's work is finished by a later launch).
+// kSleepNs: pause between polls.  Polls take issue slots and shared-memory cycles from whatever is being
+// waited for, so every wait but the shortest pauses.
+template <int kSleepNs = 0>
 __device__ __forceinline__ bool wait_or_abort(uint64_t* bar, uint32_t parity, volatile int* abort_flag,
                                               const int reason = 1) {
     for (uint32_t i = 0; i < kSpinLimit; ++i) {
         if (mbar_try_wait(bar, parity)) return true;
+        if (kSleepNs) __nanosleep(kSleepNs);
         if ((i & 255u) == 255u && *abort_flag) return false;
     }
     if (*abort_flag == 0) *abort_flag = reason;      // keep an earlier, different reason
     return false;
 }
 
+// Barrier `kId` over kThreads threads; the AND of their arguments.
+template <int kId, int kThreads> __device__ __forceinline__ bool group_all(const bool mine) {
+    uint32_t r;
+    asm volatile(
+        "{\n\t.reg .pred p, q;\n\tsetp.ne.u32 q, %1, 0;\n\t"
+        "bar.red.and.pred p, %2, %3, q;\n\tselp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(r)
+        : "r"(static_cast<uint32_t>(mine)), "n"(kId), "n"(kThreads)
+        : "memory");
+    return r != 0;
+}
+
 // Same, for a whole converged warp: every lane polls, so the instruction stays warp-wide and the
 // verdict is the same on every lane.  (Polling by lane 0 and broadcasting the verdict costs a divergent
 // branch and a shuffle: a wait on a completed barrier took 140 cycles instead of 4, and a waiting
 // warp saw an arrival after 183 instead of 62.)
+template <int kSleepNs = 0>
 __device__ __forceinline__ bool warp_wait_or_abort(uint64_t* bar, uint32_t parity, volatile int* abort_flag,
                                                    const int reason = 1) {
-    const bool ok = wait_or_abort(bar, parity, abort_flag, reason);
+    const bool ok = wait_or_abort<kSleepNs>(bar, parity, abort_flag, reason);
     __syncwarp();
     return ok;
 }

@@ -7,9 +7,10 @@
 // The one-CTA-per-unit state kernel pays, for every unit, a launch slot, barrier and TMEM set-up,
 // the first record's memory latency and the tail of its last chunk; with thousands of short
 // units (many short sequences) that overhead is longer than the chunk steps themselves.  Here
-//   * warp 13 (loader) copies records and K tiles in unit order, running up to two chunks ahead
-//     of the consumers and straight across unit boundaries (in the fused launch it first waits
-//     for each record's flag);
+//   * warps 13-15 (loaders) copy records and K tiles in unit order, running up to two chunks ahead
+//     of the consumers and straight across unit boundaries (in the fused launch they first wait for
+//     each record's flag); a stage is released in three parts and each warp refills one, so that no
+//     part waits behind another's release or flag;
 //   * warp 12 (issuer) issues every tcgen05.mma;
 //   * warps 0-7 (chain) carry the dependent chain  U = U~ - S W^T  ->  D4 = (U decayed)^T K  ->
 //     S = e^{b_C} S + D4  and nothing else; U~ is already in the accumulator of S W^T when the
@@ -39,7 +40,7 @@ constexpr int kSEpiThreads = kSEpiWarps * 32;
 constexpr int kSOutWarp0 = 8;                 // warps 8-11: output rows (one per TMEM lane quadrant)
 constexpr int kSOutThreads = 128;
 constexpr int kSIssueWarp = 12;               // warp 12: tcgen05.mma issue
-constexpr int kSLoadWarp = 13;                // warp 13: record and K-tile copies (14, 15 spare)
+constexpr int kSLoadWarp = 13;                // warps 13-15: record and K-tile copies, one part of a stage each
 constexpr int kStreamThreads = 512;
 constexpr uint32_t kStreamSmem = 2 * kStageBytes + 16384 + 1024;
 
@@ -109,7 +110,7 @@ __device__ __forceinline__ void state_stream_role(const TensorMaps& maps, const 
     __shared__ uint64_t bar_full[2], bar_free_a[2], bar_free_b[2], bar_free_c[2], bar_y[2],
         bar_d1, bar_d4, bar_s, bar_u;
     __shared__ int abort_flag;
-    __shared__ uint32_t armed_chunks;     // chunks of the CTA's stream whose copies the loader has started
+    __shared__ uint32_t armed_chunks;     // chunks of the CTA's stream whose copies a loader has started
     // kGated == 2 waits for records of a launch that may not be running beside this one: there no
     // wait that runs out is an error, whichever role it happens in (the loader's own wait for a
     // flag is the shortest, but the limits are counted in polls, not in time): the units this CTA
@@ -125,8 +126,8 @@ __device__ __forceinline__ void state_stream_role(const TensorMaps& maps, const 
     (void)done_w;
 
     if (tid == 0) {
-        mbar_init(&bar_full[0], 1);
-        mbar_init(&bar_full[1], 1);
+        mbar_init(&bar_full[0], 3);      // one arrival (and its bytes) per loading warp
+        mbar_init(&bar_full[1], 3);
         // A stage is released in three parts as its readers finish with them, so that the next
         // record's copies start up to half a chunk step earlier (one chunk step of look-ahead is
         // shorter than a cold 74 KB copy): W and Qg once S W^T and S Qg^T have retired, U~ and the
@@ -170,8 +171,10 @@ __device__ __forceinline__ void state_stream_role(const TensorMaps& maps, const 
     // chain warps take 256 x 16.
     if (warp >= kSIssueWarp) {
     reg_dealloc<64>();
-    if (warp == kSLoadWarp) {
-        // ===================== loader: records and K tiles, in stream order
+    if (warp >= kSLoadWarp) {
+        // ===================== loaders: records and K tiles, in stream order
+        const int part = warp - kSLoadWarp;
+        uint64_t* const bar_free = part == 0 ? bar_free_a : part == 1 ? bar_free_b : bar_free_c;
         if (lane == 0) {
             const size_t rec_stride = static_cast<size_t>(p.Hv) * kRecBytes;
             const uint32_t* flags = reinterpret_cast<const uint32_t*>(ws + lay.flags);
@@ -228,23 +231,27 @@ __device__ __forceinline__ void state_stream_role(const TensorMaps& maps, const 
                         // below; one here would also wait for this thread's copies in flight (3 %
                         // of a long sequence's run time).
                     }
-                    if (g >= 2 && !wait_or_abort(&bar_free_a[st], par_free, abortp, kWaitReason)) { live = false; break; }
-                    armed_chunks = g + 1;
-                    mbar_expect_tx(&bar_full[st], kRecBytes + 16384);
-                    bulk_load(base + kS_Rec + kRecW, rec + kRecW, kRecP - kRecW, &bar_full[st]);
-                    if (g >= 2 && !wait_or_abort(&bar_free_b[st], par_free, abortp, kWaitReason)) { live = false; break; }
-                    bulk_load(base + kS_Rec + kRecU, rec + kRecU, kRecBytes - kRecU, &bar_full[st]);
-                    if (g >= 2 && !wait_or_abort(&bar_free_c[st], par_free, abortp, kWaitReason)) { live = false; break; }
-                    bulk_load(base + kS_Rec + kRecP, rec + kRecP, kRecU - kRecP, &bar_full[st]);
-                    tma_load_2d(base + kS_K, &maps.k, u.hqk * kD, u.seq_t0 + j * kChunk, &bar_full[st]);
-                    tma_load_2d(base + kS_K + 8192, &maps.k, u.hqk * kD + 64, u.seq_t0 + j * kChunk,
-                                &bar_full[st]);
+                    if (g >= 2 && !wait_or_abort<40>(&bar_free[st], par_free, abortp, kWaitReason)) { live = false; break; }
+                    atomicMax(&armed_chunks, g + 1);
+                    if (part == 0) {
+                        mbar_expect_tx(&bar_full[st], kRecP - kRecW);
+                        bulk_load(base + kS_Rec + kRecW, rec + kRecW, kRecP - kRecW, &bar_full[st]);
+                    } else if (part == 1) {
+                        mbar_expect_tx(&bar_full[st], kRecBytes - kRecU);
+                        bulk_load(base + kS_Rec + kRecU, rec + kRecU, kRecBytes - kRecU, &bar_full[st]);
+                    } else {
+                        const int tok = u.seq_t0 + j * kChunk;
+                        mbar_expect_tx(&bar_full[st], kRecU - kRecP + 16384);
+                        bulk_load(base + kS_Rec + kRecP, rec + kRecP, kRecU - kRecP, &bar_full[st]);
+                        tma_load_2d(base + kS_K, &maps.k, u.hqk * kD, tok, &bar_full[st]);
+                        tma_load_2d(base + kS_K + 8192, &maps.k, u.hqk * kD + 64, tok, &bar_full[st]);
+                    }
                 }
                 gc += u.nc;
             }
         }
         __syncwarp();
-    } else if (warp == kSIssueWarp) {
+    } else {
         // ===================== issuer: tensor-core instructions
         {   // the whole warp runs this warp-uniform code; one elected lane executes each tcgen05 instruction
             const uint32_t id64 = make_idesc_bf16(128, 64, false, false);
@@ -347,7 +354,8 @@ __device__ __forceinline__ void state_stream_role(const TensorMaps& maps, const 
             }
         };
         bool ok = true;
-        auto await = [&](uint64_t* bar, uint32_t parity) {   // bounded wait + tcgen05 fence
+        // Bounded wait + tcgen05 fence
+        auto await = [&](uint64_t* bar, uint32_t parity) {
             if (ok && !warp_wait_or_abort(bar, parity, abortp, kWaitReason)) ok = false;
             tc_fence_after_sync();
         };
@@ -452,9 +460,11 @@ __device__ __forceinline__ void state_stream_role(const TensorMaps& maps, const 
                             S[c0 + 16 + jj] = fmaf(gC, S[c0 + 16 + jj], __uint_as_float(xb[jj]));
                         }
                     }
-                    if (!last) {
-                        store_state_bf16();          // the next chunk's A operand
-                    } else {
+                    if (!last) store_state_bf16();   // the next chunk's A operand
+                }
+                if (last) {
+                    ok = group_all<2, kSEpiThreads>(ok);     // nothing of a unit is written after a failed wait
+                    if (ok) {
 #pragma unroll
                         for (int j4 = 0; j4 < 64; j4 += 4)
                             *reinterpret_cast<float4*>(p.final_state + tile_off + j4) =
@@ -479,7 +489,6 @@ __device__ __forceinline__ void state_stream_role(const TensorMaps& maps, const 
         const uint32_t olane = static_cast<uint32_t>(q4 * 32) << 16;
         const int ot = tid - kSOutWarp0 * 32;
         const size_t tok_stride = static_cast<size_t>(p.Hv) * kD;
-        __nv_bfloat16* sO = reinterpret_cast<__nv_bfloat16*>(smem + kS_Out);
         auto out_sync = [] { asm volatile("bar.sync 1, %0;" ::"n"(kSOutThreads) : "memory"); };
         bool ok = true;
         // U~ (fp32, 32 KB per chunk) reaches the chain through the accumulator of S W^T: this group
@@ -489,19 +498,21 @@ __device__ __forceinline__ void state_stream_role(const TensorMaps& maps, const 
         const int odv = q4 * 32 + lane;
         auto preload = [&](uint32_t gq) {       // chunk gq of the CTA's stream -> accumulator
             const int sq = gq & 1;
-            if (ok && !warp_wait_or_abort(&bar_full[sq], (gq >> 1) & 1u, abortp, kWaitReason)) ok = false;
+            if (ok && !warp_wait_or_abort<40>(&bar_full[sq], (gq >> 1) & 1u, abortp, kWaitReason)) ok = false;
             if (ok) {
                 const float4* sU = reinterpret_cast<const float4*>(smem + sq * kStageBytes + kS_Rec + kRecU);
 #pragma unroll
-                for (int c0 = 0; c0 < 64; c0 += 16) {
-                    uint32_t r[16];
+                for (int c0 = 0; c0 < 64; c0 += 32) {       // eight reads in flight
+                    uint32_t r[2][16];
 #pragma unroll
-                    for (int q = 0; q < 4; ++q) {
+                    for (int q = 0; q < 8; ++q) {
                         const float4 v = sU[((c0 >> 2) + q) * kD + odv];
-                        r[4 * q] = __float_as_uint(v.x); r[4 * q + 1] = __float_as_uint(v.y);
-                        r[4 * q + 2] = __float_as_uint(v.z); r[4 * q + 3] = __float_as_uint(v.w);
+                        uint32_t(&x)[16] = r[q >> 2];
+                        x[4 * (q & 3)] = __float_as_uint(v.x); x[4 * (q & 3) + 1] = __float_as_uint(v.y);
+                        x[4 * (q & 3) + 2] = __float_as_uint(v.z); x[4 * (q & 3) + 3] = __float_as_uint(v.w);
                     }
-                    tmem_st16(tmem + kT_D1 + olane + c0, r);
+                    tmem_st16(tmem + kT_D1 + olane + c0, r[0]);
+                    tmem_st16(tmem + kT_D1 + olane + c0 + 16, r[1]);
                 }
             }
             tmem_wait_st();
@@ -526,7 +537,7 @@ __device__ __forceinline__ void state_stream_role(const TensorMaps& maps, const 
 #pragma unroll 1
                 for (int k = preloaded ? 1 : 0; k < 2; ++k) {
                     if (k == 1) {
-                        if (ok && !warp_wait_or_abort(&bar_u, g & 1u, abortp, kWaitReason)) ok = false;
+                        if (ok && !warp_wait_or_abort<40>(&bar_u, g & 1u, abortp, kWaitReason)) ok = false;
                         tc_fence_after_sync();
                         if (!ahead) break;
                     }
@@ -534,53 +545,56 @@ __device__ __forceinline__ void state_stream_role(const TensorMaps& maps, const 
                 }
                 preloaded = ahead;
                 // every warp runs both group barriers of every chunk, also after a failed wait
-                if (ok && !warp_wait_or_abort(&bar_y[buf], (g >> 1) & 1u, abortp, kWaitReason)) ok = false;
+                if (ot == 0) bulk_wait_read_all();       // the last chunk's rows have left the staging tile
+                out_sync();
+                if (ok && !warp_wait_or_abort<40>(&bar_y[buf], (g >> 1) & 1u, abortp, kWaitReason)) ok = false;
                 tc_fence_after_sync();
-                // The Y tile (lanes = dv, columns = tokens) is read as accumulator fragments, rounded
-                // in pairs and stored transposed, 8 dv of one token per 16 bytes, into a [token][dv]
-                // tile of two 128B-swizzled halves of 64 dv: 2 loads, 32 conversions and 8 stores
-                // per thread instead of 64 scalar conversions and 64 two-byte stores (what these
-                // warps issue comes out of the chain warps' issue slots).
-                uint32_t pa[16], pb[16];     // packed pairs: lanes 0-15 / 16-31 of the quadrant
-                if (ok) {
-                    const uint32_t tY = tmem + kT_Y + buf * 64;
-                    uint32_t y[32];
-                    tmem_ld_16x256b_x8(tY + olane, y);
-                    tmem_wait_ld();
-#pragma unroll
-                    for (int i = 0; i < 16; ++i)
-                        pa[i] = pack_bf16(__uint_as_float(y[2 * i]), __uint_as_float(y[2 * i + 1]));
-                    tmem_ld_16x256b_x8(tY + olane + (16u << 16), y);
-                    tmem_wait_ld();
-#pragma unroll
-                    for (int i = 0; i < 16; ++i)
-                        pb[i] = pack_bf16(__uint_as_float(y[2 * i]), __uint_as_float(y[2 * i + 1]));
-                }
+                // The tile (lanes = dv, columns = tokens) is read as accumulator fragments (lane 4 x + t holds
+                // columns 8 i + 2 t, + 1), rounded in pairs and stored transposed, 8 dv of one token per 16
+                // bytes, into a [token][dv] tile of two 128B-swizzled halves of 64 dv (what these warps
+                // issue comes out of the chain warps' issue slots).
                 if (ok) {
                     const int dv0 = q4 * 32 + 8 * (lane >> 3);         // the 8 dv this lane's address covers
-                    const uint32_t dst = smem_u32(sO) + (dv0 >> 6) * 8192;
+                    const uint32_t dst = smem_u32(smem + kS_Out) + (dv0 >> 6) * 8192;
 #pragma unroll
-                    for (int i = 0; i < 8; ++i)
-                        stmatrix_x4_trans(dst + sw128_offset(8 * i + (lane & 7), (dv0 & 63) >> 3),
-                                          pa[2 * i], pa[2 * i + 1], pb[2 * i], pb[2 * i + 1]);
-                }
-                out_sync();
-                if (ok) {
-                    const int len = min(kChunk, u.seq_len - j * kChunk);
-                    __nv_bfloat16* og = p.o + (static_cast<size_t>(u.seq_t0 + j * kChunk) * p.Hv + u.hv) * kD;
-                    const uint8_t* src = reinterpret_cast<const uint8_t*>(sO) + ((ot & 15) >> 3) * 8192;
+                    for (int c = 0; c < 2; ++c) {        // 32 columns at a time
+                        uint32_t pk[2][8];               // packed pairs: lanes 0-15 / 16-31 of the quadrant
 #pragma unroll
-                    for (int it = 0; it < 8; ++it) {
-                        const int row = it * 8 + (ot >> 4), piece = ot & 15;
-                        if (row < len)
-                            *reinterpret_cast<uint4*>(og + row * tok_stride + piece * 8) =
-                                *reinterpret_cast<const uint4*>(src + sw128_offset(row, piece & 7));
+                        for (int h = 0; h < 2; ++h) {
+                            uint32_t y1[16];
+                            tmem_ld_16x256b_x4(tmem + kT_Y + buf * 64 + olane + (static_cast<uint32_t>(h) << 20) + 32 * c, y1);
+                            tmem_wait_ld();
+#pragma unroll
+                            for (int i = 0; i < 8; ++i)
+                                pk[h][i] = pack_bf16(__uint_as_float(y1[2 * i]), __uint_as_float(y1[2 * i + 1]));
+                        }
+#pragma unroll
+                        for (int i = 0; i < 4; ++i)
+                            stmatrix_x4_trans(dst + sw128_offset(8 * (4 * c + i) + (lane & 7), (dv0 & 63) >> 3),
+                                              pk[0][2 * i], pk[0][2 * i + 1], pk[1][2 * i], pk[1][2 * i + 1]);
                     }
                 }
+                fence_proxy_async_smem();
                 out_sync();
+                const int len = min(kChunk, u.seq_len - j * kChunk), tok = u.seq_t0 + j * kChunk;
+                if (len == kChunk) {
+                    if (ot == 0 && ok) {     // two tiled copies (16-byte loops of the group's threads took 960 cycles)
+                        tma_store_2d(&maps.o, u.hv * kD, tok, smem + kS_Out);
+                        tma_store_2d(&maps.o, u.hv * kD + 64, tok, smem + kS_Out + 8192);
+                        bulk_commit();
+                    }
+                } else if (ok) {             // a ragged tail: the rows behind it are another sequence's
+                    const int piece = ot & 15;
+                    const uint8_t* src = smem + kS_Out + (piece >> 3) * 8192;
+                    __nv_bfloat16* og = p.o + (static_cast<size_t>(tok) * p.Hv + u.hv) * kD + piece * 8;
+                    for (int row = ot >> 4; row < len; row += 8)
+                        *reinterpret_cast<uint4*>(og + row * tok_stride) =
+                            *reinterpret_cast<const uint4*>(src + sw128_offset(row, piece & 7));
+                }
             }
             gc += u.nc;
         }
+        if (ot == 0) bulk_wait_all();        // before the CTA's shared memory goes away
     }
 
     tc_fence_before_sync();
@@ -588,7 +602,7 @@ __device__ __forceinline__ void state_stream_role(const TensorMaps& maps, const 
     if (abort_flag != 0 && warp == kSIssueWarp && lane == 0) {
         if (abort_flag == 1) report(p.dev_status, kDevTimeout);     // 2: a record not produced yet, no error
         // let copies already in flight land before the CTA's shared memory goes away: the last two
-        // chunks the loader started, each on its stage's barrier at that chunk's own parity
+        // chunks a loader started, each on its stage's barrier at that chunk's own parity
         const uint32_t armed = *reinterpret_cast<volatile uint32_t*>(&armed_chunks);
         for (uint32_t back = 1; back <= 2 && back <= armed; ++back) {
             const uint32_t gq = armed - back;
