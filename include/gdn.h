@@ -334,7 +334,7 @@ int gdn_prefill_recurrent(const void* q, const void* k, const void* v,
  * workspace_bytes; inputs and outputs are still the caller's buffers.
  *   - A batch needing more scratch than the array holds
  *     (gdn_prefill_workspace_bytes(...) > GDN_STATIC_WORKSPACE_BYTES) returns
- *     GDN_ERR_LIMIT and nothing is launched.  The scratch is 74 240 bytes per
+ *     GDN_ERR_LIMIT and nothing is launched.  The scratch is 74 496 bytes per
  *     chunk slot and v-head plus small tables, so with Hv = 32 the array covers
  *     14 chunk slots (floor(T/64) + N <= 14), e.g. 768 tokens in 2 sequences.
  *   - The call itself allocates and frees nothing.  The first call on each

@@ -96,6 +96,17 @@ __device__ __forceinline__ float dot4(const float4& a, const float4& b, float ac
     return acc;
 }
 
+// Packed pair of fp32 multiply-adds (one issue slot for two): a * b + c.
+__device__ __forceinline__ float2 fma2(const float2 a, const float2 b, const float2 c) {
+    unsigned long long d;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;"
+        : "=l"(d)
+        : "l"(*reinterpret_cast<const unsigned long long*>(&a)),
+          "l"(*reinterpret_cast<const unsigned long long*>(&b)),
+          "l"(*reinterpret_cast<const unsigned long long*>(&c)));
+    return *reinterpret_cast<float2*>(&d);
+}
+
 // sum over the 8 lanes that share a state row (lanes differing in bits 0..2)
 __device__ __forceinline__ float sum8(float x) {
     x += __shfl_xor_sync(0xffffffffu, x, 1);

@@ -18,6 +18,11 @@ prefill_intra_kernel(const __grid_constant__ TensorMaps maps, const PrefillParam
     const int c = blockIdx.x;
     const int hv = blockIdx.y;
     pdl_launch_dependents();
+    if (threadIdx.x == 0) {         // (before the wait: a first use would fetch them in front of the tiles)
+        prefetch_tensormap(&maps.q);
+        prefetch_tensormap(&maps.k);
+        prefetch_tensormap(&maps.v);
+    }
     pdl_wait();                     // the chunk table is the previous kernel's
     ChunkInfo ci;
     if constexpr (kInlineTable) {
@@ -89,7 +94,7 @@ prefill_intra_kernel(const __grid_constant__ TensorMaps maps, const PrefillParam
     __syncthreads();
     tc_fence_after_sync();
     const uint32_t tmem = tmem_base_s;
-    intra_item(maps, p, rec, ci, hqk, hv, smem, st, tmem, tid, [] { __syncthreads(); });
+    intra_item<false>(maps, p, rec, ci, hqk, hv, smem, st, tmem, tid, [] { __syncthreads(); });
     tc_fence_before_sync();
     __syncthreads();
     if (warp == 0) tmem_dealloc(tmem, kIntraTmemCols);

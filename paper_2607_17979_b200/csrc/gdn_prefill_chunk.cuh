@@ -7,7 +7,7 @@
 //   P_ri =        e^{b_r-b_i} (q_r.k_i)  (i <= r)
 //   W  = T diag(beta e^b) K   (C x dk),   U~ = T diag(beta) V   (C x dv)
 //   U  = U~ - W S0^T
-//   O  = scale ( diag(e^b) Q S0^T + P U )  =  scale ( Qg S0^T + P U ),  Qg = diag(e^b) Q
+//   O  = scale ( diag(e^b) Q S0^T + P U )
 //   S' = e^{b_C} S0 + U^T diag(e^{b_C-b}) K
 //
 // Three launches: a prep kernel builds the chunk table from cu_seqlens; the
@@ -24,21 +24,27 @@
 namespace gdn {
 
 // One record per (chunk, v-head), written by the intra-chunk kernel in exactly the
-// byte image the state-pass kernel wants in shared memory (one linear bulk copy):
+// byte image the state-pass kernel wants in shared memory (linear bulk copies):
 //   [0, 16384)      W   as one MN-major 128B-swizzled tile [128 dk][64 tokens] bf16 (a row per dk)
-//   [16384, 32768)  Qg  = diag(e^b) Q as two K-major 128B-swizzled halves [64 tokens][64 dk] bf16
-//                   (the output's first term S0 Qg^T)
-//   [32768, 40960)  P   as one K-major 128B-swizzled tile   [64 r][64 i]      bf16
+//   [16384, 32768)  Qg  = diag(scale e^b) Q as two K-major 128B-swizzled halves [64 tokens][64 dk] bf16:
+//                   only where kScaledQ
+//   [32768, 40960)  P   as one K-major 128B-swizzled tile   [64 r][64 i]      bf16, scale folded in
 //   [40960, 73728)  U~  as [16 token-groups][128 dv][4 tokens] fp32
 //   [73728, 73984)  e^{b_C - b_c} for c = 0..63, fp32 (rows past the chunk's length hold 1)
-//   [73984, 74240)  e^{b_C} in the first float, rest unused
+//   [73984, 74240)  scale e^{b_r} for r = 0..63, fp32
+//   [74240, 74496)  e^{b_C} in the first float, rest unused
+// The output's first term is diag(scale e^b) Q S0^T.  kScaledQ: the record carries Qg, both terms meet in
+// one accumulator.  Otherwise the state pass loads the raw Q tile and scales the rows of the product:
+// the intra-chunk kernel saves a pass over Q and a fifth of its writes and can load V early (4
+// sequences, 7680 tokens: 98 -> 89 us), the state pass pays with a second accumulator to read.
 constexpr uint32_t kRecW = 0;
 constexpr uint32_t kRecQg = 16384;
 constexpr uint32_t kRecP = 32768;
 constexpr uint32_t kRecU = 40960;
 constexpr uint32_t kRecDecay = 73728;
-constexpr uint32_t kRecGammaC = 73984;
-constexpr uint32_t kRecBytes = 74240;
+constexpr uint32_t kRecEb = 73984;
+constexpr uint32_t kRecGammaC = 74240;
+constexpr uint32_t kRecBytes = 74496;
 
 // Small batches of at most this many sequences need no table-building launch: the intra-chunk
 // kernel finds its chunks from cu_seqlens itself and writes the per-sequence tables for the state pass.

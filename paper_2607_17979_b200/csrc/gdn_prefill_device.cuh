@@ -13,20 +13,20 @@ constexpr uint32_t kIntraTmemCols = 128;    // the Gram accumulator, then W^T in
 constexpr int kLdA = 68;               // row stride (floats) of the fp32 A / T matrix
 // Shared memory map (bytes from a 1024-aligned base).  Regions are reused as their contents die
 // so that four CTAs fit on an SM:
-//   R1  Q/K tiles.  Q half 0 -> Qg image (stored early) -> T_w -> T_u(lo);
-//       Q half 1 -> Qg image -> T_u(hi);  K halves -> W image.
-//   R2  A, then T, in fp32 -> V tile (loaded after the solve).
+//   R1  Q/K tiles.  Q halves (-> Qg image, stored early) -> V tile, loaded once the Gram product (or
+//       the store) has read Q;  K halves -> W image.
+//   R2  A, then T, in fp32 -> T_w -> T_u(lo);  T_u(hi).
 // The P image goes straight from registers to the record; T_u(lo) waits in registers until the
 // product that reads T_w has retired.
 constexpr uint32_t kI_QK = 0;          // 2 halves x [128 rows x 128 B]: rows 0-63 Q, 64-127 K
-constexpr uint32_t kI_Tw = 0;          // over Q half 0: T diag(beta e^b) [64 r x 64 i] bf16, K-major
-constexpr uint32_t kI_TuLo = 0;        // ... and later the bf16 remainder of T diag(beta)
-constexpr uint32_t kI_Tu = 16384;      // over Q half 1: T diag(beta) rounded to bf16
+constexpr uint32_t kI_V = 0;           // over Q: 2 halves x [64 x 128 B], 16384 apart
 constexpr uint32_t kI_A = 32768;       // A, then T in place: fp32 [64][kLdA]
-constexpr uint32_t kI_V = 32768;       // over A: 2 halves x [64 x 128 B]
+constexpr uint32_t kI_Tw = kI_A;       // over A: T diag(beta e^b) [64 r x 64 i] bf16, K-major
+constexpr uint32_t kI_TuLo = kI_A;     // ... and later the bf16 remainder of T diag(beta)
+constexpr uint32_t kI_Tu = kI_A + 8192;                // T diag(beta) rounded to bf16
 constexpr uint32_t kI_End = kI_A + 64 * kLdA * 4;      // 50176
 constexpr uint32_t kIntraSmem = kI_End + 1024;         // + alignment slack
-static_assert(kI_End % 1024 == 0 && 64 * kLdA * 4 >= 16384, "V tile must fit over A");
+static_assert(kI_End % 1024 == 0 && 64 * kLdA * 4 >= 16384, "the T images must fit over A");
 
 struct TensorMaps {
     CUtensorMap q, k, v, o;
@@ -99,7 +99,6 @@ struct IntraStatics {
     alignas(16) float s_b2[kChunk];    // b_r log2(e): inclusive log-decay prefix
     alignas(16) float s_beta[kChunk];  // beta_r (0 past the chunk's length)
     alignas(16) float s_bg[kChunk];    // beta_r e^{b_r}
-    alignas(16) float s_eb[kChunk];    // e^{b_r}
 };
 
 // T = (I + A)^{-1} for the strictly lower-triangular 64x64 A in sA (fp32, row-major, stride kLdA),
@@ -239,12 +238,13 @@ __device__ __forceinline__ bool warp_wait_or_abort(uint64_t* bar, uint32_t parit
     return ok;
 }
 
+// kScaledQ: whether the record carries the scaled Q (gdn_prefill_chunk.cuh).
 // The intra-chunk quantities of one (chunk, v-head) item, computed by a group of 256 threads
 // (tid = 0..255 within the group; its warps must be CTA warps 0-3 mod 4 aligned, because a warp
 // reaches TMEM lanes 32 (warp % 4) ...).  `smem` is the group's 1024-aligned slice of kI_End
 // bytes, `tmem` its 128 TMEM columns, `sync` a barrier over exactly the group.  Writes the item's
 // record; returns false after a bounded wait gave up (status word set, nothing left in flight).
-template <class Sync>
+template <bool kScaledQ, class Sync>
 __device__ __forceinline__ bool intra_item(const TensorMaps& maps, const PrefillParams& p,
                                            uint8_t* rec, const ChunkInfo ci, const int hqk,
                                            const int hv, uint8_t* smem, IntraStatics& st,
@@ -265,16 +265,12 @@ __device__ __forceinline__ bool intra_item(const TensorMaps& maps, const Prefill
             fence_barrier_init();
         }
         st.abort_flag = 0;
-        // Q and K first: everything below overlaps their flight (V comes later, over dead data)
+        // Q and K first: everything below overlaps their flight (V comes later, over Q)
         mbar_expect_tx(&st.bar_tma, 32768);
         tma_load_2d(smem + kI_QK, &maps.q, hqk * kD, ci.t0, &st.bar_tma);
         tma_load_2d(smem + kI_QK + 8192, &maps.k, hqk * kD, ci.t0, &st.bar_tma);
         tma_load_2d(smem + kI_QK + 16384, &maps.q, hqk * kD + 64, ci.t0, &st.bar_tma);
         tma_load_2d(smem + kI_QK + 24576, &maps.k, hqk * kD + 64, ci.t0, &st.bar_tma);
-        // V has no room in shared memory until the solve is over; fetch it into L2 meanwhile, so
-        // that its load then is not a DRAM round trip in front of the U~ product
-        tma_prefetch_2d(&maps.v, hv * kD, ci.t0);
-        tma_prefetch_2d(&maps.v, hv * kD + 64, ci.t0);
     }
     if (warp == 1) {
         // inclusive prefix sum of the log gates over the chunk (two tokens per lane); rows past
@@ -301,22 +297,23 @@ __device__ __forceinline__ bool intra_item(const TensorMaps& maps, const Prefill
         st.s_b2[2 * lane] = b0 * kLog2e; st.s_b2[2 * lane + 1] = b1 * kLog2e;
         st.s_beta[2 * lane] = be0; st.s_beta[2 * lane + 1] = be1;
         const float e0 = ex2_approx(b0 * kLog2e), e1 = ex2_approx(b1 * kLog2e);
-        st.s_eb[2 * lane] = e0; st.s_eb[2 * lane + 1] = e1;
         st.s_bg[2 * lane] = be0 * e0; st.s_bg[2 * lane + 1] = be1 * e1;
-        // decay vector of the record: e^{b_C - b_c}, then e^{b_C}
-        float* dec = reinterpret_cast<float*>(rec + kRecDecay);
-        dec[2 * lane] = ex2_approx((bC - b0) * kLog2e);
-        dec[2 * lane + 1] = ex2_approx((bC - b1) * kLog2e);
-        if (lane == 0) dec[kChunk] = ex2_approx(bC * kLog2e);
+        // the record's vectors: e^{b_C - b_c}, scale e^{b_r}, and e^{b_C}
+        *reinterpret_cast<float2*>(rec + kRecDecay + 8 * lane) =
+            make_float2(ex2_approx((bC - b0) * kLog2e), ex2_approx((bC - b1) * kLog2e));
+        *reinterpret_cast<float2*>(rec + kRecEb + 8 * lane) = make_float2(p.scale * e0, p.scale * e1);
+        if (lane == 0) *reinterpret_cast<float*>(rec + kRecGammaC) = ex2_approx(bC * kLog2e);
     }
     sync();
     // Every warp polls the barriers it needs itself.  A wait that runs out flags the item and the group
     // goes on to its next barrier, behind which everyone leaves together; thread 0 drains what it has
     // in flight and the caller unwinds.
     volatile int* abortp = &st.abort_flag;
+    bool v_started = false;         // (thread 0's)
     auto bail = [&](bool stores_pending) {
         if (tid == 0) {
             report(p.dev_status, kDevTimeout);
+            if (v_started) mbar_wait(&st.bar_v, par1, 1u << 12);
             if (stores_pending) bulk_wait_read_all();
         }
     };
@@ -337,8 +334,16 @@ __device__ __forceinline__ bool intra_item(const TensorMaps& maps, const Prefill
         }
         if (elect_one()) mma_commit(&st.bar_mma);
     }
-    warp_wait_or_abort(&st.bar_mma, par3, abortp);
+    const bool gram_ok = warp_wait_or_abort(&st.bar_mma, par3, abortp);
     tc_fence_after_sync();
+    auto load_v = [&] {             // thread 0, once Q is dead
+        v_started = true;
+        mbar_expect_tx(&st.bar_v, 16384);
+        tma_load_2d(smem + kI_V, &maps.v, hv * kD, ci.t0, &st.bar_v);
+        tma_load_2d(smem + kI_V + 16384, &maps.v, hv * kD + 64, ci.t0, &st.bar_v);
+    };
+    if (!kScaledQ && tid == 0 && gram_ok) load_v();
+    __syncwarp();
 
     const uint32_t lane_base = static_cast<uint32_t>((warp & 3) * 32) << 16;
     float* sA = reinterpret_cast<float*>(smem + kI_A);
@@ -350,14 +355,15 @@ __device__ __forceinline__ bool intra_item(const TensorMaps& maps, const Prefill
         const int r = row & 63;
         const bool is_p = row < 64;
         const float br2 = st.s_b2[r];
-        const float rowscale = is_p ? p.scale : st.s_beta[r];      // the output scale rides on P and Qg
+        const float rowscale = is_p ? p.scale : st.s_beta[r];      // the output scale rides on P
         const int limit = is_p ? r : r - 1;              // keep columns i <= limit
 #pragma unroll
         for (int step = 0; step < 2; ++step) {
             const int cbase = colhalf * 32 + step * 16;
             float val[16];
             // a 16-column block that lies wholly above the diagonal for every row of the warp is
-            // zero (warp-uniform test: no accumulator read, no exponentials)
+            // zero (warp-uniform test: no accumulator read, no exponentials), one that lies wholly
+            // below it needs no mask
             if (cbase > (row & 32) + 31) {
 #pragma unroll
                 for (int jj = 0; jj < 16; ++jj) val[jj] = 0.f;
@@ -370,12 +376,12 @@ __device__ __forceinline__ bool intra_item(const TensorMaps& maps, const Prefill
                     const float4 bb = *reinterpret_cast<const float4*>(st.s_b2 + cbase + 4 * q4);
                     const float bv[4] = {bb.x, bb.y, bb.z, bb.w};
 #pragma unroll
-                    for (int e = 0; e < 4; ++e) {
-                        const int jj = 4 * q4 + e;
-                        const bool keep = cbase + jj <= limit;
-                        const float dec = ex2_approx(keep ? br2 - bv[e] : 0.f);   // e^{b_r - b_i}
-                        val[jj] = keep ? rowscale * dec * __uint_as_float(x[jj]) : 0.f;
-                    }
+                    for (int e = 0; e < 4; ++e)          // times e^{b_r - b_i} (above the diagonal: discarded)
+                        val[4 * q4 + e] = rowscale * __uint_as_float(x[4 * q4 + e]) * ex2_approx(br2 - bv[e]);
+                }
+                if (cbase + 15 >= (row & 32)) {
+#pragma unroll
+                    for (int jj = 0; jj < 16; ++jj) val[jj] = cbase + jj <= limit ? val[jj] : 0.f;
                 }
             }
             if (is_p) {
@@ -399,18 +405,17 @@ __device__ __forceinline__ bool intra_item(const TensorMaps& maps, const Prefill
     tc_fence_before_sync();
     sync();
     if (st.abort_flag) { bail(false); return false; }
-    // Two jobs side by side: warps 0-1 invert the two diagonal 32x32 blocks of I + A (serial
-    // forward substitutions and two small products each, all inside the warp), warps 2-7 scale
-    // the Q rows by scale * e^{b_r} in place (the Gram product has consumed Q): the Qg image.
+    // Warps 0-1 invert the two diagonal 32x32 blocks of I + A (serial forward substitutions and two
+    // small products each, all inside the warp), then warps 4-7 the block below them.
     if (warp < 2) {
         solve_blocks_16_32(sA, warp, tid & 31, ci.len);
-    } else {
+    } else if constexpr (kScaledQ) {
+        // beside them the others scale the Q rows by scale * e^{b_r} in place: the Qg image
 #pragma unroll 2
         for (int idx = tid - 64; idx < 1024; idx += kIntraThreads - 64) {      // 1024 16-byte pieces
-            const int halfq = idx >> 9, rem = idx & 511;
-            const int r = rem >> 3;
-            uint4* ptr = reinterpret_cast<uint4*>(smem + kI_QK + halfq * 16384 + rem * 16);
-            const float f = st.s_eb[r] * p.scale;
+            const int rem = idx & 511;
+            uint4* ptr = reinterpret_cast<uint4*>(smem + kI_QK + (idx >> 9) * 16384 + rem * 16);
+            const float f = ex2_approx(st.s_b2[rem >> 3]) * p.scale;
             uint4 w = *ptr;
             w.x = scale_bf16x2(w.x, f); w.y = scale_bf16x2(w.y, f);
             w.z = scale_bf16x2(w.z, f); w.w = scale_bf16x2(w.w, f);
@@ -419,18 +424,17 @@ __device__ __forceinline__ bool intra_item(const TensorMaps& maps, const Prefill
         fence_proxy_async_smem();
     }
     sync();
-    if (tid == 0) {
-        // Qg is final: store it now.  The T_w / T_u images are written over it next: wait for the
-        // bulk store's reads (not for its writes to land) meanwhile.
+    if (kScaledQ && tid == 0) {     // Qg is final: store it, and fetch V over it once the store has read it
         bulk_store(rec + kRecQg, smem + kI_QK, 8192);
         bulk_store(rec + kRecQg + 8192, smem + kI_QK + 16384, 8192);
         bulk_commit();
         bulk_wait_read_all();
-    } else if (warp >= 4 && ci.len > 32) {
-        // (rows past the length are zero: nothing to do then).  Barrier ids 4.. are this routine's:
-        // one per group of 256 threads of the CTA.
-        solve_merge_64(sA, warp - 4, tid & 31, 4 + (static_cast<int>(threadIdx.x) >> 8));
+        load_v();
     }
+    // (rows past the length are zero: nothing to do then).  Barrier ids 4.. are this routine's: one per
+    // group of 256 threads of the CTA.
+    if (warp >= 4 && ci.len > 32)
+        solve_merge_64(sA, warp - 4, tid & 31, 4 + (static_cast<int>(threadIdx.x) >> 8));
     sync();
 
     // T (fp32, row-major) -> bf16 B operands T diag(beta e^b), T diag(beta) (hi, lo).  A thread takes four
@@ -443,6 +447,7 @@ __device__ __forceinline__ bool intra_item(const TensorMaps& maps, const Prefill
     {
         const float4 fg = *reinterpret_cast<const float4*>(st.s_bg + 4 * icol);
         const float4 fb = *reinterpret_cast<const float4*>(st.s_beta + 4 * icol);
+        uint32_t tw[4][2], tu[4][2];
 #pragma unroll
         for (int it = 0; it < 4; ++it) {
             const float4 t = *reinterpret_cast<const float4*>(sA + (irow + 16 * it) * kLdA + 4 * icol);
@@ -450,24 +455,24 @@ __device__ __forceinline__ bool intra_item(const TensorMaps& maps, const Prefill
             const uint32_t h0 = pack_bf16(u0, u1), h1 = pack_bf16(u2, u3);
             tu_lo[it][0] = pack_bf16(u0 - __uint_as_float(h0 << 16), u1 - __uint_as_float(h0 & 0xffff0000u));
             tu_lo[it][1] = pack_bf16(u2 - __uint_as_float(h1 << 16), u3 - __uint_as_float(h1 & 0xffff0000u));
+            tu[it][0] = h0; tu[it][1] = h1;
+            tw[it][0] = pack_bf16(t.x * fg.x, t.y * fg.y);
+            tw[it][1] = pack_bf16(t.z * fg.z, t.w * fg.w);
+        }
+        sync();              // T has been read: the images take its place
+#pragma unroll
+        for (int it = 0; it < 4; ++it) {
             const uint32_t off = image_offset(it);
-            *reinterpret_cast<uint2*>(smem + kI_Tw + off) =
-                make_uint2(pack_bf16(t.x * fg.x, t.y * fg.y), pack_bf16(t.z * fg.z, t.w * fg.w));
-            *reinterpret_cast<uint2*>(smem + kI_Tu + off) = make_uint2(h0, h1);
+            *reinterpret_cast<uint2*>(smem + kI_Tw + off) = make_uint2(tw[it][0], tw[it][1]);
+            *reinterpret_cast<uint2*>(smem + kI_Tu + off) = make_uint2(tu[it][0], tu[it][1]);
         }
     }
     fence_proxy_async_smem();
     sync();
 
     const uint32_t sV = smem_u32(smem + kI_V);
-    if (tid == 0) {      // V into the space the solve has left
-        mbar_expect_tx(&st.bar_v, 16384);
-        tma_load_2d(smem + kI_V, &maps.v, hv * kD, ci.t0, &st.bar_v);
-        tma_load_2d(smem + kI_V + 8192, &maps.v, hv * kD + 64, ci.t0, &st.bar_v);
-    }
-    __syncwarp();
     const uint32_t idesc_t = make_idesc_bf16(128, 64, true, false);
-    if (warp == 0) {     // meanwhile W^T (dk x r) = K^T T_w^T with the raw K tile read MN-major
+    if (warp == 0) {     // W^T (dk x r) = K^T T_w^T with the raw K tile read MN-major
         const uint64_t dK = make_sdesc_sw128(sQK + 8192, 16384, 1024), dT = make_sdesc_sw128(smem_u32(smem + kI_Tw), 16, 1024);
         // columns of T_w and T_u past the chunk's length are zero: their k-steps are left out
 #pragma unroll
@@ -518,7 +523,7 @@ __device__ __forceinline__ bool intra_item(const TensorMaps& maps, const Prefill
     if (warp == 0 && warp_wait_or_abort(&st.bar_v, par1, abortp)) {        // V has landed
         tc_fence_after_sync();
         // U~^T (dv x r) = V^T T_u^T with T_u = hi + lo
-        const uint64_t dV = make_sdesc_sw128(sV, 8192, 1024);
+        const uint64_t dV = make_sdesc_sw128(sV, 16384, 1024);
         const uint64_t dH = make_sdesc_sw128(smem_u32(smem + kI_Tu), 16, 1024), dL = make_sdesc_sw128(smem_u32(smem + kI_TuLo), 16, 1024);
 #pragma unroll
         for (int ks = 0; ks < 4; ++ks)
@@ -556,9 +561,11 @@ __device__ __forceinline__ bool intra_item(const TensorMaps& maps, const Prefill
 }
 
 constexpr uint32_t kStateTmemCols = 512;
-constexpr uint32_t kS_Rec = 0;                 // record image (74240 B, padded to 74752)
+constexpr uint32_t kS_Rec = 0;                 // record image (74496 B, padded to 74752)
+constexpr uint32_t kS_Q = kRecQg;              // Q tile in Qg's place, 2 halves [64 x 128 B]
 constexpr uint32_t kS_K = 74752;               // K tile, 2 halves [64 x 128 B]
-constexpr uint32_t kStageBytes = 74752 + 16384;                 // 91136
+constexpr uint32_t kStageBytes = kS_K + 16384;                  // 91136
+static_assert(kRecBytes <= kS_K && kS_K % 1024 == 0, "tiles are 1024-byte aligned");
 constexpr uint32_t kS_Out = 2 * kStageBytes;   // o staging [64 tokens][128 dv] bf16
 // TMEM columns
 constexpr uint32_t kT_D1 = 0, kT_Y = 64 /* two tiles of 64 */, kT_D4 = 192, kT_S = 320, kT_U = 384,

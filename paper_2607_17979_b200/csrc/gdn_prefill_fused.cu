@@ -326,7 +326,7 @@ __device__ __forceinline__ void fused_intra_role(const TensorMaps& maps, const P
         const ChunkInfo ci = chunks[c];
         const size_t slot = static_cast<size_t>(c) * p.Hv + hv;
         uint8_t* rec = ws + lay.records + slot * kRecBytes;
-        const bool ok = intra_item(maps, p, rec, ci, hv / G, hv, gsmem, st, tmem, gtid, gsync, n_done);
+        const bool ok = intra_item<true>(maps, p, rec, ci, hv / G, hv, gsmem, st, tmem, gtid, gsync, n_done);
         ++n_done;
         // publish: every thread's own stores first, then the bulk stores, then the flag
         __threadfence();

@@ -63,7 +63,7 @@ prefill_intra_first_kernel(const __grid_constant__ TensorMaps maps, const Prefil
     __syncthreads();
     tc_fence_after_sync();
     const uint32_t tmem = tmem_base_s;
-    intra_item(maps, p, rec, ci, hv / (p.Hv / p.Hqk), hv, smem, st, tmem, tid, [] { __syncthreads(); });
+    intra_item<false>(maps, p, rec, ci, hv / (p.Hv / p.Hqk), hv, smem, st, tmem, tid, [] { __syncthreads(); });
     tc_fence_before_sync();
     __syncthreads();
     if (warp == 0) tmem_dealloc(tmem, kIntraTmemCols);
@@ -110,7 +110,7 @@ prefill_intra_second_kernel(const __grid_constant__ TensorMaps maps, const Prefi
             const ChunkInfo ci = chunks[c];
             const size_t slot = static_cast<size_t>(c) * p.Hv + hv;
             uint8_t* rec = ws + lay.records + slot * kRecBytes;
-            const bool ok = intra_item(maps, p, rec, ci, hv / G, hv, smem, st, tmem, tid,
+            const bool ok = intra_item<false>(maps, p, rec, ci, hv / G, hv, smem, st, tmem, tid,
                                        [] { __syncthreads(); }, n_done);
             ++n_done;
             // publish: every thread's own stores first, then the bulk stores, then the flag

@@ -16,7 +16,7 @@
 //     S = e^{b_C} S + D4  and nothing else; U~ is already in the accumulator of S W^T when the
 //     product runs (negated B operand), so the chain warps read U itself;
 //   * warps 8-11 (output) put U~ of the next chunk into that accumulator and turn
-//     Y = S Qg^T + U P^T into o rows one chunk behind.  Whatever these warps issue comes out of
+//     Y = diag(scale e^b) (Q S^T) + P U into o rows one chunk behind.  Whatever these warps issue comes out of
 //     the chain warps' issue slots, so the rows are made with few instructions (fragment loads,
 //     paired conversions, transposing matrix stores).
 // The CTA is compiled for 512 threads (128 registers); the chain warps take 144 registers each
@@ -108,7 +108,7 @@ __device__ __forceinline__ void state_stream_role(const TensorMaps& maps, const 
                                                   uint8_t* smem, const uint32_t tmem, const int cta,
                                                   const int n_ctas) {
     __shared__ uint64_t bar_full[2], bar_free_a[2], bar_free_b[2], bar_free_c[2], bar_y[2],
-        bar_d1, bar_d4, bar_s, bar_u;
+        bar_y_read, bar_d1, bar_d4, bar_s, bar_u;
     __shared__ int abort_flag;
     __shared__ uint32_t armed_chunks;     // chunks of the CTA's stream whose copies a loader has started
     // kGated == 2 waits for records of a launch that may not be running beside this one: there no
@@ -116,6 +116,7 @@ __device__ __forceinline__ void state_stream_role(const TensorMaps& maps, const 
     // flag is the shortest, but the limits are counted in polls, not in time): the units this CTA
     // has not finished are left to the last launch, which reports real failures.
     constexpr int kWaitReason = kGated == 2 ? 2 : 1;
+    constexpr bool kScaledQ = kGated == 1;      // the records of the fused launch carry the scaled Q
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int half = (warp >> 2) & 1;                 // which half of the columns this thread owns
     const int dv = (warp & 3) * 32 + lane;            // TMEM lane = state row
@@ -130,7 +131,7 @@ __device__ __forceinline__ void state_stream_role(const TensorMaps& maps, const 
         mbar_init(&bar_full[1], 3);
         // A stage is released in three parts as its readers finish with them, so that the next
         // record's copies start up to half a chunk step earlier (one chunk step of look-ahead is
-        // shorter than a cold 74 KB copy): W and Qg once S W^T and S Qg^T have retired, U~ and the
+        // shorter than a cold copy): W and Q once S W^T and S Q^T have retired, U~ and the
         // decay vector once every chain warp has read them, P and the K tile once U P^T and the
         // state product have retired.
         for (int st = 0; st < 2; ++st) {
@@ -140,13 +141,14 @@ __device__ __forceinline__ void state_stream_role(const TensorMaps& maps, const 
         }
         mbar_init(&bar_d1, 1);
         mbar_init(&bar_d4, 1);
+        mbar_init(&bar_y_read, kSOutThreads / 32);      // (raw Q) the output warps have read S Q^T and U P^T
         mbar_init(&bar_y[0], 1);      // one per Y tile: with a single barrier the output warps could
         mbar_init(&bar_y[1], 1);      // find it two phases ahead, which a parity wait cannot tell
         // bar_s: everything the chunk's first product needs is in TMEM: the bf16 state (one arrival
         // per chain warp) and U~ in the accumulator (one per output warp).  The output warps copy
-        // U~ only after they have seen the record land and have read the Y tile of two chunks
-        // ago, so this one wait also tells the issuing warp that the record is in shared memory
-        // and that the Y tile may be overwritten.
+        // U~ only after they have seen the record land and have read Y of two chunks ago, so this one
+        // wait also tells the issuing warp that the record is in shared memory (and, with scaled Q, that
+        // the Y tile may be overwritten).
         mbar_init(&bar_s, kSEpiWarps + kSOutThreads / 32);
         mbar_init(&bar_u, kSEpiWarps);
         abort_flag = 0;
@@ -233,14 +235,20 @@ __device__ __forceinline__ void state_stream_role(const TensorMaps& maps, const 
                     }
                     if (g >= 2 && !wait_or_abort<40>(&bar_free[st], par_free, abortp, kWaitReason)) { live = false; break; }
                     atomicMax(&armed_chunks, g + 1);
+                    const int tok = u.seq_t0 + j * kChunk;
                     if (part == 0) {
                         mbar_expect_tx(&bar_full[st], kRecP - kRecW);
-                        bulk_load(base + kS_Rec + kRecW, rec + kRecW, kRecP - kRecW, &bar_full[st]);
+                        if constexpr (kScaledQ) {
+                            bulk_load(base + kS_Rec + kRecW, rec + kRecW, kRecP - kRecW, &bar_full[st]);
+                        } else {
+                            bulk_load(base + kS_Rec + kRecW, rec + kRecW, kRecQg - kRecW, &bar_full[st]);
+                            tma_load_2d(base + kS_Q, &maps.q, u.hqk * kD, tok, &bar_full[st]);
+                            tma_load_2d(base + kS_Q + 8192, &maps.q, u.hqk * kD + 64, tok, &bar_full[st]);
+                        }
                     } else if (part == 1) {
                         mbar_expect_tx(&bar_full[st], kRecBytes - kRecU);
                         bulk_load(base + kS_Rec + kRecU, rec + kRecU, kRecBytes - kRecU, &bar_full[st]);
                     } else {
-                        const int tok = u.seq_t0 + j * kChunk;
                         mbar_expect_tx(&bar_full[st], kRecU - kRecP + 16384);
                         bulk_load(base + kS_Rec + kRecP, rec + kRecP, kRecU - kRecP, &bar_full[st]);
                         tma_load_2d(base + kS_K, &maps.k, u.hqk * kD, tok, &bar_full[st]);
@@ -279,7 +287,9 @@ __device__ __forceinline__ void state_stream_role(const TensorMaps& maps, const 
                     const int st = g & 1;
                     const uint64_t w = st ? dW1 : dW0, qg = st ? dQ1 : dQ0, pp = st ? dP1 : dP0,
                                    kk = st ? dK1 : dK0;
-                    const uint32_t tY = tmem + kT_Y + st * 64;
+                    // Y.  Scaled Q: both terms in one of two tiles.  Raw Q: a tile for each term.
+                    const uint32_t tY1 = tmem + kT_Y + (kScaledQ ? 64 * st : 0);
+                    const uint32_t tY2 = tmem + kT_Y + (kScaledQ ? 64 * st : 64);
                     if (!wait_or_abort(&bar_s, g & 1u, abortp, kWaitReason)) {      // record landed, bf16 S and U~ in TMEM
                         live = false;
                         break;
@@ -296,16 +306,22 @@ __device__ __forceinline__ void state_stream_role(const TensorMaps& maps, const 
                     if (elect_one()) mma_ts_c<true>(tD1, tS + 48, sdesc_advance(w, 12288), id64mn);
                     if (elect_one()) mma_ts_c<true>(tD1, tS + 56, sdesc_advance(w, 14336), id64mn);
                     if (elect_one()) mma_commit(&bar_d1);
-                    // Y = S Qg^T  (off the chain) overwrites the tile the output warps read two chunks ago
-                    if (elect_one()) mma_ts_c<false>(tY, tS, qg, id64);
-                    if (elect_one()) mma_ts_c<true>(tY, tS + 8, sdesc_advance(qg, 32), id64);
-                    if (elect_one()) mma_ts_c<true>(tY, tS + 16, sdesc_advance(qg, 64), id64);
-                    if (elect_one()) mma_ts_c<true>(tY, tS + 24, sdesc_advance(qg, 96), id64);
-                    if (elect_one()) mma_ts_c<true>(tY, tS + 32, sdesc_advance(qg, 8192), id64);
-                    if (elect_one()) mma_ts_c<true>(tY, tS + 40, sdesc_advance(qg, 8192 + 32), id64);
-                    if (elect_one()) mma_ts_c<true>(tY, tS + 48, sdesc_advance(qg, 8192 + 64), id64);
-                    if (elect_one()) mma_ts_c<true>(tY, tS + 56, sdesc_advance(qg, 8192 + 96), id64);
-                    if (elect_one()) mma_commit(&bar_free_a[st]);                          // W and Qg have been read
+                    // S Q^T  (off the chain) overwrites the tile the output warps read two chunks ago (raw Q: one
+                    // chunk ago)
+                    if (!kScaledQ && g > 0 && !wait_or_abort(&bar_y_read, (g - 1) & 1u, abortp, kWaitReason)) {
+                        live = false;
+                        break;
+                    }
+                    if (!kScaledQ) tc_fence_after_sync();
+                    if (elect_one()) mma_ts_c<false>(tY1, tS, qg, id64);
+                    if (elect_one()) mma_ts_c<true>(tY1, tS + 8, sdesc_advance(qg, 32), id64);
+                    if (elect_one()) mma_ts_c<true>(tY1, tS + 16, sdesc_advance(qg, 64), id64);
+                    if (elect_one()) mma_ts_c<true>(tY1, tS + 24, sdesc_advance(qg, 96), id64);
+                    if (elect_one()) mma_ts_c<true>(tY1, tS + 32, sdesc_advance(qg, 8192), id64);
+                    if (elect_one()) mma_ts_c<true>(tY1, tS + 40, sdesc_advance(qg, 8192 + 32), id64);
+                    if (elect_one()) mma_ts_c<true>(tY1, tS + 48, sdesc_advance(qg, 8192 + 64), id64);
+                    if (elect_one()) mma_ts_c<true>(tY1, tS + 56, sdesc_advance(qg, 8192 + 96), id64);
+                    if (elect_one()) mma_commit(&bar_free_a[st]);                          // W and Q have been read
                     if (!wait_or_abort(&bar_u, g & 1u, abortp, kWaitReason)) {         // U operands in TMEM
                         live = false;
                         break;
@@ -321,11 +337,11 @@ __device__ __forceinline__ void state_stream_role(const TensorMaps& maps, const 
                     if (elect_one()) mma_ts_c<true>(tD4, tmem + kT_UsLo + 16, sdesc_advance(kk, 4096), id128mn);
                     if (elect_one()) mma_ts_c<true>(tD4, tmem + kT_UsLo + 24, sdesc_advance(kk, 6144), id128mn);
                     if (elect_one()) mma_commit(&bar_d4);
-                    // Y += U P^T
-                    if (elect_one()) mma_ts_c<true>(tY, tmem + kT_U, pp, id64);
-                    if (elect_one()) mma_ts_c<true>(tY, tmem + kT_U + 8, sdesc_advance(pp, 32), id64);
-                    if (elect_one()) mma_ts_c<true>(tY, tmem + kT_U + 16, sdesc_advance(pp, 64), id64);
-                    if (elect_one()) mma_ts_c<true>(tY, tmem + kT_U + 24, sdesc_advance(pp, 96), id64);
+                    // U P^T
+                    if (elect_one()) mma_ts_c<kScaledQ>(tY2, tmem + kT_U, pp, id64);
+                    if (elect_one()) mma_ts_c<true>(tY2, tmem + kT_U + 8, sdesc_advance(pp, 32), id64);
+                    if (elect_one()) mma_ts_c<true>(tY2, tmem + kT_U + 16, sdesc_advance(pp, 64), id64);
+                    if (elect_one()) mma_ts_c<true>(tY2, tmem + kT_U + 24, sdesc_advance(pp, 96), id64);
                     if (elect_one()) mma_commit(&bar_y[st]);
                     if (elect_one()) mma_commit(&bar_free_c[st]);                          // P and the K tile have been read
                 }
@@ -360,8 +376,9 @@ __device__ __forceinline__ void state_stream_role(const TensorMaps& maps, const 
             tc_fence_after_sync();
         };
         // Every warp runs every group barrier and hand-over below, also after a wait has failed
-        // (ok == false: later waits and all work are skipped), so that no warp is ever left alone
-        // at a barrier.
+        // (ok == false), so that no warp is ever left alone at a barrier.  It then works on with whatever
+        // is there; nothing of it is written out.  (A branch around each phase costs 60 cycles a
+        // chunk step: 32768 tokens at 8 v-heads 793 -> 769 us without them.)
         UnitInfo nxt = unit_info(p, ws, lay, min(cta, total_units - 1), done_tab);
         for (int unit = cta; unit < total_units; unit += n_ctas) {
             const UnitInfo u = nxt;
@@ -403,7 +420,7 @@ __device__ __forceinline__ void state_stream_role(const TensorMaps& maps, const 
 #pragma unroll
                 for (int j = 0; j < 64; ++j) S[j] = 0.f;
             }
-            if (ok) store_state_bf16();
+            store_state_bf16();
             hand_over(&bar_s);
             for (int j = 0; j < nc; ++j) {
                 const uint32_t g = gc + j;
@@ -411,7 +428,7 @@ __device__ __forceinline__ void state_stream_role(const TensorMaps& maps, const 
                 const uint8_t* base = smem + st * kStageBytes;
                 await(&bar_full[st], (g >> 1) & 1u);
                 await(&bar_d1, g & 1u);
-                if (ok) {   // U^T[dv][c] (the accumulator holds U~ - S W^T) for the thread's 32 tokens [32*half, 32*half+32)
+                {   // U^T[dv][c] (the accumulator holds U~ - S W^T) for the thread's 32 tokens [32*half, 32*half+32)
                     const float* sdec = reinterpret_cast<const float*>(base + kS_Rec + kRecDecay);
 #pragma unroll
                     for (int c0 = 0; c0 < 32; c0 += 16) {
@@ -447,7 +464,7 @@ __device__ __forceinline__ void state_stream_role(const TensorMaps& maps, const 
                 if (lane == 0) mbar_arrive(&bar_free_b[st]);    // this warp has read U~, decay, e^{b_C}
                 const bool last = j + 1 == nc;
                 await(&bar_d4, g & 1u);
-                if (ok) {   // S <- e^{b_C} S + D4 on the thread's 64 dk columns
+                {   // S <- e^{b_C} S + D4 on the thread's 64 dk columns
 #pragma unroll
                     for (int c0 = 0; c0 < 64; c0 += 32) {
                         uint32_t xa[16], xb[16];
@@ -482,7 +499,7 @@ __device__ __forceinline__ void state_stream_role(const TensorMaps& maps, const 
         }
     } else {
         reg_dealloc<112>();
-        // ===================== output warps: Y = S Qg^T + U P^T (fp32, TMEM) -> o rows.  Warp 8 + q
+        // ===================== output warps: Y = scale e^b (S Q^T) + U P^T (fp32, TMEM) -> o rows.  Warp 8 + q
         // reads TMEM lanes 32 q .. 32 q + 31 (dv indices), scales and rounds, transposes through
         // shared memory, and the four warps write whole rows in 16-byte pieces.
         const int q4 = warp & 3;
@@ -496,10 +513,15 @@ __device__ __forceinline__ void state_stream_role(const TensorMaps& maps, const 
         // from it (negated B operand), and the chain warps read U itself.  (Read by the chain warps
         // from shared memory, the 32 KB took 300 of the 3700 cycles of a chunk step.)
         const int odv = q4 * 32 + lane;
+        // (raw Q) the chunk's scale e^{b_r} outlives its stage: a copy per warp, two chunks deep
+        __shared__ float s_eb[kScaledQ ? 1 : kSOutThreads / 32][2][kChunk];
         auto preload = [&](uint32_t gq) {       // chunk gq of the CTA's stream -> accumulator
             const int sq = gq & 1;
             if (ok && !warp_wait_or_abort<40>(&bar_full[sq], (gq >> 1) & 1u, abortp, kWaitReason)) ok = false;
             if (ok) {
+                if constexpr (!kScaledQ)
+                    *reinterpret_cast<float2*>(&s_eb[q4][sq][2 * lane]) = *reinterpret_cast<const float2*>(
+                        smem + sq * kStageBytes + kS_Rec + kRecEb + 8 * lane);
                 const float4* sU = reinterpret_cast<const float4*>(smem + sq * kStageBytes + kS_Rec + kRecU);
 #pragma unroll
                 for (int c0 = 0; c0 < 64; c0 += 32) {       // eight reads in flight
@@ -550,7 +572,7 @@ __device__ __forceinline__ void state_stream_role(const TensorMaps& maps, const 
                 if (ok && !warp_wait_or_abort<40>(&bar_y[buf], (g >> 1) & 1u, abortp, kWaitReason)) ok = false;
                 tc_fence_after_sync();
                 // The tile (lanes = dv, columns = tokens) is read as accumulator fragments (lane 4 x + t holds
-                // columns 8 i + 2 t, + 1), rounded in pairs and stored transposed, 8 dv of one token per 16
+                // columns 8 i + 2 t, + 1; raw Q: both tiles, and added), rounded in pairs and stored transposed, 8 dv of one token per 16
                 // bytes, into a [token][dv] tile of two 128B-swizzled halves of 64 dv (what these warps
                 // issue comes out of the chain warps' issue slots).
                 if (ok) {
@@ -558,15 +580,27 @@ __device__ __forceinline__ void state_stream_role(const TensorMaps& maps, const 
                     const uint32_t dst = smem_u32(smem + kS_Out) + (dv0 >> 6) * 8192;
 #pragma unroll
                     for (int c = 0; c < 2; ++c) {        // 32 columns at a time
+                        float2 eb[4];
+                        if constexpr (!kScaledQ) {
+#pragma unroll
+                            for (int i = 0; i < 4; ++i)
+                                eb[i] = *reinterpret_cast<const float2*>(&s_eb[q4][buf][2 * (lane & 3) + 8 * (4 * c + i)]);
+                        }
                         uint32_t pk[2][8];               // packed pairs: lanes 0-15 / 16-31 of the quadrant
 #pragma unroll
                         for (int h = 0; h < 2; ++h) {
-                            uint32_t y1[16];
-                            tmem_ld_16x256b_x4(tmem + kT_Y + buf * 64 + olane + (static_cast<uint32_t>(h) << 20) + 32 * c, y1);
+                            uint32_t y1[16], y2[16];
+                            const uint32_t at = tmem + kT_Y + olane + (static_cast<uint32_t>(h) << 20) + 32 * c;
+                            tmem_ld_16x256b_x4(at + (kScaledQ ? 64 * buf : 0), y1);
+                            if constexpr (!kScaledQ) tmem_ld_16x256b_x4(at + 64, y2);
                             tmem_wait_ld();
 #pragma unroll
-                            for (int i = 0; i < 8; ++i)
-                                pk[h][i] = pack_bf16(__uint_as_float(y1[2 * i]), __uint_as_float(y1[2 * i + 1]));
+                            for (int i = 0; i < 8; ++i) {
+                                float2 y = make_float2(__uint_as_float(y1[2 * i]), __uint_as_float(y1[2 * i + 1]));
+                                if constexpr (!kScaledQ)
+                                    y = fma2(eb[i >> 1], y, make_float2(__uint_as_float(y2[2 * i]), __uint_as_float(y2[2 * i + 1])));
+                                pk[h][i] = pack_bf16(y.x, y.y);
+                            }
                         }
 #pragma unroll
                         for (int i = 0; i < 4; ++i)
@@ -574,7 +608,10 @@ __device__ __forceinline__ void state_stream_role(const TensorMaps& maps, const 
                                               pk[0][2 * i], pk[0][2 * i + 1], pk[1][2 * i], pk[1][2 * i + 1]);
                     }
                 }
+                tc_fence_before_sync();
                 fence_proxy_async_smem();
+                __syncwarp();
+                if (!kScaledQ && lane == 0) mbar_arrive(&bar_y_read);
                 out_sync();
                 const int len = min(kChunk, u.seq_len - j * kChunk), tok = u.seq_t0 + j * kChunk;
                 if (len == kChunk) {
