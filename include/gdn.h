@@ -203,8 +203,10 @@ int gdn_prefill(const void* q, const void* k, const void* v,
 /*
  * gdn_prefill routes by shape: a batch whose longest sequence has at most
  * GDN_RECURRENT_MAX_SEQLEN tokens (by max_seqlen_hint if given, else by the
- * bound T) goes to the token-by-token kernel; anything longer to one of the
- * chunked variants (gdn_prefill_fused for a few long sequence-heads,
+ * bound T) goes to gdn_prefill_recurrent's kernel (GDN_ROUTE_RECURRENT), and
+ * so do a few sequence-heads of up to GDN_BLOCKS_MAX_SEQLEN tokens
+ * (GDN_ROUTE_BLOCKS: the same kernel with the next block's tokens staged beside
+ * the current block); anything longer to one of the chunked variants (gdn_prefill_fused for a few long sequence-heads,
  * gdn_prefill_overlap when max_seqlen_hint tells of chains of at least 40
  * chunks and the sequence-heads number between a third and half of the SMs,
  * gdn_prefill_stream for everything else).  Each route can also be called
@@ -216,12 +218,14 @@ int gdn_prefill(const void* q, const void* k, const void* v,
  * GDN_ROUTE_CHUNKED any more), or GDN_ROUTE_NONE for an empty batch.
  */
 #define GDN_RECURRENT_MAX_SEQLEN 16
+#define GDN_BLOCKS_MAX_SEQLEN 64
 #define GDN_ROUTE_NONE      0
 #define GDN_ROUTE_RECURRENT 1
 #define GDN_ROUTE_CHUNKED   2
 #define GDN_ROUTE_FUSED     3
 #define GDN_ROUTE_STREAM    4
 #define GDN_ROUTE_OVERLAP   5
+#define GDN_ROUTE_BLOCKS    6
 int gdn_prefill_route(int32_t T, int32_t N, int32_t max_seqlen_hint, int32_t Hv,
                       int32_t sm_count, int32_t cooperative_launch);
 int gdn_prefill_chunked(const void* q, const void* k, const void* v,
@@ -307,10 +311,10 @@ int gdn_prefill_overlap(const void* q, const void* k, const void* v,
 
 /*
  * gdn_prefill_recurrent - the same operator and arguments as gdn_prefill,
- * evaluated token by token on the CUDA cores (no chunking, no workspace).  The
- * rows of a state tile evolve independently under the gated delta rule, so the
- * dv rows are spread over warps.  It is the route for very short batches and
- * an independent GPU cross-check of the chunked path.
+ * evaluated in blocks of up to 16 tokens on a state tile in registers (no chunk
+ * records, no workspace).  The rows of a state tile evolve independently under
+ * the gated delta rule, so the dv rows are spread over warps.  It is the route
+ * for short prompts and an independent GPU cross-check of the chunked path.
  */
 int gdn_prefill_recurrent(const void* q, const void* k, const void* v,
                           const float* g, const float* beta, const int32_t* cu_seqlens,

@@ -139,7 +139,7 @@ def gdn_state_transpose(state_pool, slot_idx=None, n=None, dev_status=None):
         raise GdnError(rc, "gdn_state_transpose")
 
 
-ROUTES = {0: "none", 1: "recurrent", 2: "chunked", 3: "fused", 4: "stream", 5: "overlap"}
+ROUTES = {0: "none", 1: "recurrent", 2: "chunked", 3: "fused", 4: "stream", 5: "overlap", 6: "blocks"}
 _ROUTE_CODES = {"auto": 0, "chunked": 2, "fused": 3, "stream": 4, "overlap": 5}
 
 
@@ -170,7 +170,7 @@ def gdn_prefill(q, k, v, g, beta, cu_seqlens, init_state, final_state, slot_idx,
 
 def gdn_prefill_recurrent(q, k, v, g, beta, cu_seqlens, init_state, final_state, slot_idx, o,
                           scale, dev_status=None):
-    """Token-by-token prefill on the CUDA cores; same arguments as gdn_prefill, no workspace."""
+    """Prefill in blocks of up to 16 tokens; same arguments as gdn_prefill, no workspace."""
     T, Hqk, dk = q.shape
     _, Hv, dv = v.shape
     N = cu_seqlens.shape[0] - 1

@@ -261,9 +261,14 @@ int gdn_prefill_route(int32_t T, int32_t N, int32_t max_seqlen_hint, int32_t Hv,
     if (T <= 0 || N <= 0 || Hv <= 0 || sm_count <= 0) return GDN_ROUTE_NONE;
     // the length is known on the host only through the caller's hint or the bound T
     const int32_t longest = (max_seqlen_hint > 0 && max_seqlen_hint < T) ? max_seqlen_hint : T;
-    // very short sequences: the token-by-token kernel (one launch, no workspace traffic)
+    // very short sequences: one block of tokens each (one launch, no workspace traffic)
     if (longest <= GDN_RECURRENT_MAX_SEQLEN) return GDN_ROUTE_RECURRENT;
     const long long units = static_cast<long long>(N) * Hv;
+    // Up to four blocks of few units: 3.3 us a block against the 16-17 us of the chunked kernels' start-up
+    // (one sequence at 32 v-heads: 17 tokens 16.0 -> 8.8 us, 32 16.0 -> 9.7, 48 16.8 -> 13.0, 64 17.2 ->
+    // 16.3; five blocks are level).  With more units than half the SMs a block takes longer: 4 x 30
+    // tokens (128 units) 18.7 against 18.5.
+    if (units <= sm_count / 2 && longest <= GDN_BLOCKS_MAX_SEQLEN) return GDN_ROUTE_BLOCKS;
     // Few (sequence, v-head) units and long sequences: the serial state pass would occupy only a
     // few SMs while the rest idle, so run it next to the record producers in one cooperative launch.
     if (cooperative_launch && units <= sm_count / 3 && longest > 16 * gdn::kChunk) return GDN_ROUTE_FUSED;
@@ -298,7 +303,7 @@ int gdn_prefill(const void* q, const void* k, const void* v, const float* g, con
         coop = di.cooperative;
     }
     const int route_id = gdn_prefill_route(T, N, max_seqlen_hint, Hv, sms, coop);
-    if (chunk == gdn::kChunk && route_id == GDN_ROUTE_RECURRENT) {
+    if (chunk == gdn::kChunk && (route_id == GDN_ROUTE_RECURRENT || route_id == GDN_ROUTE_BLOCKS)) {
         // same validation of the workspace arguments as the chunked route, so that a call does
         // not start failing when its batch grows
         if (!workspace) {

@@ -52,10 +52,12 @@ decode_multi_kernel(const DecodeMultiParams mp) {
     }
     float* tile = p.pool + (static_cast<size_t>(slot) * p.Hv + hv) * (kD * kD);
     TokenLoads<kTransposed, kWarps, kMax> ld;
-    load_tokens(ld, t, row_base);
+    load_tokens(ld, t, row_base, threadIdx.x);
     State<kTransposed> s;
     load_state<kTransposed>(s, tile, row_base);
-    stage_block(t, st, ld);
+    // (both barriers are passed while the tile's loads are in flight)
+    stage_block(t, st, ld, threadIdx.x, [] { __syncthreads(); });
+    __syncthreads();
     apply_block(t, st, s, row_base);
     store_state<kTransposed>(s, tile, row_base);
 }

@@ -68,10 +68,11 @@ __device__ __forceinline__ void mma_m16n8k8_tf32(float (&c)[4], const uint32_t (
         : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
         : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b[0]), "r"(b[1]));
 }
-template <int kSteps>
+// kN tiles side by side: columns 8 nb .. of B and of the output.
+template <int kSteps, int kN>
 __device__ __forceinline__ void mma_tile_tf32(const float* A, int lda, const float* B, int ldb,
-                                              float (&c)[4], int g, int t) {
-    uint32_t a[kSteps][4], b[kSteps][2];
+                                              float (&c)[kN][4], int g, int t) {
+    uint32_t a[kSteps][4], b[kSteps][kN][2];
 #pragma unroll
     for (int ks = 0; ks < kSteps; ++ks) {          // every load first, then the products
         const float* a_ = A + 8 * ks;
@@ -80,11 +81,16 @@ __device__ __forceinline__ void mma_tile_tf32(const float* A, int lda, const flo
         a[ks][1] = to_tf32(a_[(g + 8) * lda + t]);
         a[ks][2] = to_tf32(a_[g * lda + t + 4]);
         a[ks][3] = to_tf32(a_[(g + 8) * lda + t + 4]);
-        b[ks][0] = to_tf32(b_[t * ldb + g]);
-        b[ks][1] = to_tf32(b_[(t + 4) * ldb + g]);
+#pragma unroll
+        for (int nb = 0; nb < kN; ++nb) {
+            b[ks][nb][0] = to_tf32(b_[t * ldb + 8 * nb + g]);
+            b[ks][nb][1] = to_tf32(b_[(t + 4) * ldb + 8 * nb + g]);
+        }
     }
 #pragma unroll
-    for (int ks = 0; ks < kSteps; ++ks) mma_m16n8k8_tf32(c, a[ks], b[ks]);
+    for (int ks = 0; ks < kSteps; ++ks)
+#pragma unroll
+        for (int nb = 0; nb < kN; ++nb) mma_m16n8k8_tf32(c[nb], a[ks], b[ks][nb]);
 }
 
 __device__ __forceinline__ uint32_t scale_bf16x2(uint32_t packed, float f) {
@@ -102,15 +108,15 @@ struct IntraStatics {
 };
 
 // T = (I + A)^{-1} for the strictly lower-triangular 64x64 A in sA (fp32, row-major, stride kLdA),
-// in place, in two warp-local stages that need no barrier wider than a warp:
+// in place, in two stages:
 //   solve_blocks_16_32: a warp inverts two neighbouring diagonal 16x16 blocks by forward
-//     substitution (thread (I, j) computes column j of (I + A_II)^{-1}, right-looking) and joins
-//     them into the inverse of their 32x32 block,
-//   solve_merge_64: a warp computes an 8-column block of the last off-diagonal 32x32 block,
+//     substitution (thread (I, j) computes column j of (I + A_II)^{-1}, right-looking, four columns of A
+//     at a time so that a row's are one 16-byte read) and joins them into the inverse of their 32x32 block,
+//   solve_merge_64: four warps compute the last off-diagonal 32x32 block, a 16x16 quarter each,
 // both by block elimination  [[Ta, 0], [X, Tb]],  X = -Tb (A_ba Ta),  whose small products run on
 // the legacy mma.sync path (tcgen05 needs M >= 64).  The intermediate product A_ba Ta changes
-// from accumulator to operand layout through the block of sA that mirrors X above the diagonal
-// (zero in A and in T), which the warp clears again.
+// from accumulator to operand layout through the block of sA that mirrors X above the diagonal.
+// What is left there is not cleared: readers of T take every 16x16 block above the diagonal as zero.
 // Warp `pr` (0 or 1) of the group: diagonal blocks 2 pr, 2 pr + 1 and block (2 pr + 1, 2 pr).
 __device__ __forceinline__ void solve_blocks_16_32(float* sA, const int pr, const int lane,
                                                    const int len) {
@@ -121,10 +127,15 @@ __device__ __forceinline__ void solve_blocks_16_32(float* sA, const int pr, cons
 #pragma unroll
         for (int r = 0; r < 16; ++r) t[r] = (r == j) ? 1.f : 0.f;
 #pragma unroll
-        for (int i = 0; i < 15; ++i) {
-            const float ti = t[i];
+        for (int c = 0; c < 16; c += 4) {
 #pragma unroll
-            for (int r = i + 1; r < 16; ++r) t[r] = fmaf(-blk[r * kLdA + i], ti, t[r]);
+            for (int r = c + 1; r < 16; ++r) {
+                const float4 a = *reinterpret_cast<const float4*>(blk + r * kLdA + c);
+                t[r] = fmaf(-a.x, t[c], t[r]);
+                if (r > c + 1) t[r] = fmaf(-a.y, t[c + 1], t[r]);
+                if (r > c + 2) t[r] = fmaf(-a.z, t[c + 2], t[r]);
+                if (r > c + 3) t[r] = fmaf(-a.w, t[c + 3], t[r]);
+            }
         }
         __syncwarp();                      // every column of the block has read A_II
 #pragma unroll
@@ -135,26 +146,18 @@ __device__ __forceinline__ void solve_blocks_16_32(float* sA, const int pr, cons
     const int g = lane >> 2, t = lane & 3;
     const int I = 2 * pr + 1, J = 2 * pr;
     float* A_IJ = sA + (16 * I) * kLdA + 16 * J;
-    float* X = sA + (16 * J) * kLdA + 16 * I;          // the mirror block, zero on entry
+    float* X = sA + (16 * J) * kLdA + 16 * I;          // the mirror block
+    float c[2][4] = {{0.f, 0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}};
+    mma_tile_tf32<2, 2>(A_IJ, kLdA, sA + (16 * J) * kLdA + 16 * J, kLdA, c, g, t);      // X = A_IJ T_JJ
 #pragma unroll
-    for (int nb = 0; nb < 2; ++nb) {                   // X = A_IJ T_JJ
-        float c[4] = {0.f, 0.f, 0.f, 0.f};
-        mma_tile_tf32<2>(A_IJ, kLdA, sA + (16 * J) * kLdA + 16 * J + 8 * nb, kLdA, c, g, t);
-        *reinterpret_cast<float2*>(X + g * kLdA + 8 * nb + 2 * t) = make_float2(c[0], c[1]);
-        *reinterpret_cast<float2*>(X + (g + 8) * kLdA + 8 * nb + 2 * t) = make_float2(c[2], c[3]);
+    for (int nb = 0; nb < 2; ++nb) {
+        *reinterpret_cast<float2*>(X + g * kLdA + 8 * nb + 2 * t) = make_float2(c[nb][0], c[nb][1]);
+        *reinterpret_cast<float2*>(X + (g + 8) * kLdA + 8 * nb + 2 * t) = make_float2(c[nb][2], c[nb][3]);
+        c[nb][0] = c[nb][1] = c[nb][2] = c[nb][3] = 0.f;
     }
     __syncwarp();
-    float c[2][4] = {{0.f, 0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}};
-#pragma unroll
-    for (int nb = 0; nb < 2; ++nb)                     // T_IJ = -T_II X
-        mma_tile_tf32<2>(sA + (16 * I) * kLdA + 16 * I, kLdA, X + 8 * nb, kLdA, c[nb], g, t);
-    __syncwarp();                                      // every lane has read X and A_IJ
-    {
-        const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
-        float* xr = X + (lane >> 1) * kLdA + 8 * (lane & 1);
-        *reinterpret_cast<float4*>(xr) = zero;
-        *reinterpret_cast<float4*>(xr + 4) = zero;
-    }
+    mma_tile_tf32<2, 2>(sA + (16 * I) * kLdA + 16 * I, kLdA, X, kLdA, c, g, t);         // T_IJ = -T_II X
+    __syncwarp();                                      // every lane has read A_IJ (above)
 #pragma unroll
     for (int nb = 0; nb < 2; ++nb) {
         float* dst = A_IJ + 8 * nb;
@@ -163,37 +166,38 @@ __device__ __forceinline__ void solve_blocks_16_32(float* sA, const int pr, cons
     }
 }
 
-// Columns 8 nb .. 8 nb + 7 (nb = 0..3) of the 32x32 block (1, 0), by one warp, given the inverses
-// of the two diagonal 32x32 blocks.  Called by four consecutive warps together: each reads all
-// of A_ba for its first product and writes its columns of the result over A_ba afterwards, so
-// the four meet at a barrier of their own (`bar_id`, 128 threads) in between.
-__device__ __forceinline__ void solve_merge_64(float* sA, const int nb, const int lane,
+// Quarter w (0..3: rows 16 (w & 1), columns 16 (w >> 1)) of the 32x32 block (1, 0), given the inverses of
+// the two diagonal 32x32 blocks.  Called by four consecutive warps together, which meet at a
+// barrier of their own (`bar_id`, 128 threads) between the products: the second reads what two warps
+// wrote and overwrites what all four have read.
+__device__ __forceinline__ void solve_merge_64(float* sA, const int w, const int lane,
                                                const int bar_id) {
     const int g = lane >> 2, t = lane & 3;
-    float* Y = sA + 32 + 8 * nb;                       // rows 0-31 of the mirror block, zero on entry
-#pragma unroll
-    for (int mr = 0; mr < 2; ++mr) {                   // Y = A_ba Ta
-        float c[4] = {0.f, 0.f, 0.f, 0.f};
-        mma_tile_tf32<4>(sA + (32 + 16 * mr) * kLdA, kLdA, sA + 8 * nb, kLdA, c, g, t);
-        *reinterpret_cast<float2*>(Y + (16 * mr + g) * kLdA + 2 * t) = make_float2(c[0], c[1]);
-        *reinterpret_cast<float2*>(Y + (16 * mr + g + 8) * kLdA + 2 * t) = make_float2(c[2], c[3]);
-    }
-    asm volatile("bar.sync %0, 128;" ::"r"(bar_id) : "memory");      // A_ba has been read by all four warps
+    const int r0 = 16 * (w & 1), c0 = 16 * (w >> 1);
+    float* Y = sA + 32 + c0;                           // rows 0-31 of the mirror block
     float c[2][4] = {{0.f, 0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}};
+    // Y = A_ba Ta; Ta is lower triangular: its columns 16-31 have rows 16-31 only
+    if (c0 == 0)
+        mma_tile_tf32<4, 2>(sA + (32 + r0) * kLdA, kLdA, sA, kLdA, c, g, t);
+    else
+        mma_tile_tf32<2, 2>(sA + (32 + r0) * kLdA + 16, kLdA, sA + 16 * kLdA + 16, kLdA, c, g, t);
 #pragma unroll
-    for (int mr = 0; mr < 2; ++mr)                     // X = -Tb Y
-        mma_tile_tf32<4>(sA + (32 + 16 * mr) * kLdA + 32, kLdA, Y, kLdA, c[mr], g, t);
-    __syncwarp();                                      // every lane has read Y and A_ba
-    {
-        const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
-        *reinterpret_cast<float4*>(Y + lane * kLdA) = zero;
-        *reinterpret_cast<float4*>(Y + lane * kLdA + 4) = zero;
+    for (int nb = 0; nb < 2; ++nb) {
+        *reinterpret_cast<float2*>(Y + (r0 + g) * kLdA + 8 * nb + 2 * t) = make_float2(c[nb][0], c[nb][1]);
+        *reinterpret_cast<float2*>(Y + (r0 + g + 8) * kLdA + 8 * nb + 2 * t) = make_float2(c[nb][2], c[nb][3]);
+        c[nb][0] = c[nb][1] = c[nb][2] = c[nb][3] = 0.f;
     }
+    asm volatile("bar.sync %0, 128;" ::"r"(bar_id) : "memory");
+    // X = -Tb Y; the rows 0-15 of Tb have columns 0-15 only
+    if (r0 == 0)
+        mma_tile_tf32<2, 2>(sA + 32 * kLdA + 32, kLdA, Y, kLdA, c, g, t);
+    else
+        mma_tile_tf32<4, 2>(sA + 48 * kLdA + 32, kLdA, Y, kLdA, c, g, t);
 #pragma unroll
-    for (int mr = 0; mr < 2; ++mr) {
-        float* dst = sA + (32 + 16 * mr) * kLdA + 8 * nb;
-        *reinterpret_cast<float2*>(dst + g * kLdA + 2 * t) = make_float2(-c[mr][0], -c[mr][1]);
-        *reinterpret_cast<float2*>(dst + (g + 8) * kLdA + 2 * t) = make_float2(-c[mr][2], -c[mr][3]);
+    for (int nb = 0; nb < 2; ++nb) {
+        float* dst = sA + (32 + r0) * kLdA + c0 + 8 * nb;
+        *reinterpret_cast<float2*>(dst + g * kLdA + 2 * t) = make_float2(-c[nb][0], -c[nb][1]);
+        *reinterpret_cast<float2*>(dst + (g + 8) * kLdA + 2 * t) = make_float2(-c[nb][2], -c[nb][3]);
     }
 }
 
@@ -450,7 +454,9 @@ __device__ __forceinline__ bool intra_item(const TensorMaps& maps, const Prefill
         uint32_t tw[4][2], tu[4][2];
 #pragma unroll
         for (int it = 0; it < 4; ++it) {
-            const float4 t = *reinterpret_cast<const float4*>(sA + (irow + 16 * it) * kLdA + 4 * icol);
+            // (a 16x16 block above the diagonal is zero whatever the solve has left there)
+            float4 t = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (icol >> 2 <= it) t = *reinterpret_cast<const float4*>(sA + (irow + 16 * it) * kLdA + 4 * icol);
             const float u0 = t.x * fb.x, u1 = t.y * fb.y, u2 = t.z * fb.z, u3 = t.w * fb.w;
             const uint32_t h0 = pack_bf16(u0, u1), h1 = pack_bf16(u2, u3);
             tu_lo[it][0] = pack_bf16(u0 - __uint_as_float(h0 << 16), u1 - __uint_as_float(h0 & 0xffff0000u));

@@ -2,22 +2,25 @@
 // records and no workspace (gdn_token_block.cuh describes a block's algebra and its layout).
 //
 // The rows of a state tile evolve independently under the gated delta rule, so a (sequence,
-// v-head) tile is spread over four CTAs of two warps; a CTA carries its 32 rows through all
-// blocks of its sequence.  Bound by latency: the token-by-token loop this replaces took 0.43 us a
-// token (one L2 round trip each), a block of 16 takes about 3.7 us.  One sequence, device time per
-// call: 6 tokens 4.9 -> 4.1 us, 12 tokens 7.8 -> 6.1 us, 128 tokens 57 -> 38 us.
+// v-head) tile is spread over four CTAs of 32 rows, which two warps carry through the blocks of the
+// sequence.  kPipelined: two more warps load and stage the next block (tokens, decays, coefficients)
+// meanwhile, in the other half of a double buffer.  Without (prompts of one block, where there may be
+// thousands of them and occupancy counts) the two warps do both.  Bound by latency: the token-by-token loop this
+// replaces took 0.43 us a token (one L2 round trip each).  One sequence, device time per call: 6 tokens
+// 4.9 -> 4.1 us, 12 tokens 7.8 -> 6.1 us; longer prompts: see the routing rule.
 #include "gdn_token_block.cuh"
 #include "gdn_sm100.cuh"
 
 namespace gdn {
 
-constexpr int kRecWarps = 2;
+constexpr int kRecWarps = 2;                  // that apply blocks
 
-template <int kMax>
-__global__ void __launch_bounds__(kRecWarps * 32, kMax == 16 ? 6 : 8)
+template <int kMax, bool kPipelined>
+__global__ void __launch_bounds__(kRecWarps * (kPipelined ? 64 : 32), kPipelined ? 2 : kMax == 16 ? 6 : 8)
 prefill_recurrent_kernel(const PrefillParams p) {
     using Block = TokenBlock<false, kRecWarps, kMax>;
-    __shared__ __align__(16) Block st;
+    __shared__ __align__(16) Block st[kPipelined ? 2 : 1];
+    constexpr int kThreads = kRecWarps * (kPipelined ? 64 : 32);
     constexpr int kSplit = kD / Block::kRows;
     const int unit = blockIdx.x / kSplit;
     const int row_base = (blockIdx.x - unit * kSplit) * Block::kRows;
@@ -39,7 +42,7 @@ prefill_recurrent_kernel(const PrefillParams p) {
     }
     if (slot < 0 || slot >= p.num_slots) {
         if (slot >= p.num_slots && tid == 0) report(p.dev_status, kDevBadSlot);
-        for (int idx = tid; idx < (t1 - t0) * (Block::kRows / 8); idx += kRecWarps * 32) {
+        for (int idx = tid; idx < (t1 - t0) * (Block::kRows / 8); idx += kThreads) {
             const int t = t0 + idx / (Block::kRows / 8), c = (idx % (Block::kRows / 8)) * 8;
             *reinterpret_cast<uint4*>(p.o + (static_cast<size_t>(t) * p.Hv + hv) * kD + row_base + c) =
                 make_uint4(0u, 0u, 0u, 0u);
@@ -62,11 +65,28 @@ prefill_recurrent_kernel(const PrefillParams p) {
         t.beta = p.beta + tv;
         t.count = min(kMax, t1 - tok);
     };
-
     const size_t tile = (static_cast<size_t>(slot) * p.Hv + hv) * (kD * kD);
+    const int blocks = (t1 - t0 + kMax - 1) / kMax;
+
+    if (kPipelined && tid >= kRecWarps * 32) {           // staging warps: block i + 1 while block i is applied
+        const int stid = tid - kRecWarps * 32;
+        auto stage_sync = [] { asm volatile("bar.sync 1, %0;" ::"n"(kRecWarps * 32) : "memory"); };
+        TokenLoads<false, kRecWarps, kMax> ld;
+        block_at(t0);
+        if (blocks > 0) load_tokens(ld, t, row_base, stid);
+        for (int i = 0; i < blocks; ++i) {
+            stage_block(t, st[kPipelined ? i & 1 : 0], ld, stid, stage_sync);
+            if (i + 1 < blocks) {          // on their way while the others apply this block
+                block_at(t0 + (i + 1) * kMax);
+                load_tokens(ld, t, row_base, stid);
+            }
+            __syncthreads();               // block i is staged, block i - 1 has been applied
+        }
+        return;
+    }
     TokenLoads<false, kRecWarps, kMax> ld;
     block_at(t0);
-    load_tokens(ld, t, row_base);
+    if (!kPipelined && blocks > 0) load_tokens(ld, t, row_base, tid);
     State<false> s;
     if (p.init_state) {
         load_state<false>(s, p.init_state + tile, row_base);
@@ -74,15 +94,17 @@ prefill_recurrent_kernel(const PrefillParams p) {
 #pragma unroll
         for (auto& c : s[0]) c[0] = c[1] = c[2] = c[3] = 0.f;
     }
-    for (int tok = t0; tok < t1;) {
-        stage_block(t, st, ld);
-        apply_block(t, st, s, row_base);
-        tok += kMax;
-        if (tok < t1) {
-            block_at(tok);
-            load_tokens(ld, t, row_base);
-            __syncthreads();               // the staged block has been read
+    for (int i = 0; i < blocks; ++i) {
+        block_at(t0 + i * kMax);
+        if constexpr (!kPipelined) {
+            if (i > 0) {
+                load_tokens(ld, t, row_base, tid);
+                __syncthreads();           // the staged block has been read
+            }
+            stage_block(t, st[0], ld, tid, [] { __syncthreads(); });
         }
+        __syncthreads();
+        apply_block(t, st[kPipelined ? i & 1 : 0], s, row_base);
     }
     store_state<false>(s, p.final_state + tile, row_base);
 }
@@ -90,11 +112,13 @@ prefill_recurrent_kernel(const PrefillParams p) {
 cudaError_t launch_prefill_recurrent(const PrefillParams& p, int longest, cudaStream_t stream) {
     const long long ctas = static_cast<long long>(p.N) * p.Hv * (8 / kRecWarps);
     if (ctas == 0 || p.T == 0) return cudaSuccess;
-    // a bound on the longest sequence picks the block size; longer sequences take more blocks
-    auto kernel = longest <= 4   ? prefill_recurrent_kernel<4>
-                  : longest <= 8 ? prefill_recurrent_kernel<8>
-                                 : prefill_recurrent_kernel<16>;
-    return launch_dependent(kernel, dim3(static_cast<unsigned>(ctas)), dim3(kRecWarps * 32), 0, stream, p);
+    // a bound on the longest sequence picks the variant; longer sequences take more blocks
+    auto kernel = longest <= 4    ? prefill_recurrent_kernel<4, false>
+                  : longest <= 8  ? prefill_recurrent_kernel<8, false>
+                  : longest <= 16 ? prefill_recurrent_kernel<16, false>
+                                  : prefill_recurrent_kernel<16, true>;
+    return launch_dependent(kernel, dim3(static_cast<unsigned>(ctas)),
+                            dim3(kRecWarps * (longest <= 16 ? 32 : 64)), 0, stream, p);
 }
 
 }  // namespace gdn

@@ -205,9 +205,9 @@ __device__ __forceinline__ float ld_scalar(const float* p) {
     return r;
 }
 template <bool kTransposed, int kWarps, int kMax>
-__device__ __forceinline__ void load_tokens(TokenLoads<kTransposed, kWarps, kMax>& ld, const TokenRows& t, const int row_base) {
+__device__ __forceinline__ void load_tokens(TokenLoads<kTransposed, kWarps, kMax>& ld, const TokenRows& t,
+                                            const int row_base, const int tid) {
     using L = TokenLoads<kTransposed, kWarps, kMax>;
-    const int tid = threadIdx.x;
     ld.g = ld.beta = 0.f;
     if (tid < t.count) {
         ld.g = ld_scalar(t.g + tid * t.g_stride);
@@ -230,13 +230,13 @@ __device__ __forceinline__ void load_tokens(TokenLoads<kTransposed, kWarps, kMax
     }
 }
 
-// Tokens -> shared memory, decays; then the solve's coefficients.  Two CTA barriers, both passed
-// while the tile's loads are in flight.
-template <bool kTransposed, int kWarps, int kMax>
+// Tokens -> shared memory, decays; then the solve's coefficients.  Run by kWarps warps (tid counts them
+// from 0), which meet at `sync` in between; the caller's next barrier makes the block ready.
+template <bool kTransposed, int kWarps, int kMax, class Sync>
 __device__ __forceinline__ void stage_block(const TokenRows& t, TokenBlock<kTransposed, kWarps, kMax>& st,
-                                            const TokenLoads<kTransposed, kWarps, kMax>& ld) {
+                                            const TokenLoads<kTransposed, kWarps, kMax>& ld, const int tid, Sync sync) {
     using L = TokenLoads<kTransposed, kWarps, kMax>;
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int lane = tid & 31, warp = tid >> 5;
     if (warp == 0) {       // decays: lane j < kMax walks D_ij down i, lane kMax walks D_i
         float alpha = 1.f;
         if (lane < t.count) {
@@ -270,7 +270,7 @@ __device__ __forceinline__ void stage_block(const TokenRows& t, TokenBlock<kTran
         if (L::kV % L::kThreads != 0 && idx >= L::kV) break;
         *reinterpret_cast<uint4*>(&st.v[0][0] + idx * 8) = ld.v[it];
     }
-    __syncthreads();
+    sync();
 
     // k.k and q.k of the block's tokens: 16 fragment rows are 16 k or q rows (kMax = 16: one warp each),
     // k then q (8), or k, q and nothing (4)
@@ -303,7 +303,6 @@ __device__ __forceinline__ void stage_block(const TokenRows& t, TokenBlock<kTran
                 }
             }
     }
-    __syncthreads();
 }
 
 // The staged block on the state in registers.  Barriers of the warp only (tiles [dk][dv]: of the pair).

@@ -28,12 +28,15 @@ def test_decode_block_edges(layout, B, Hv, L):
     assert np.array_equal(pool[untouched], d["state"][untouched])
 
 
-@pytest.mark.parametrize("lens", [[1], [4, 3], [5], [8, 1, 0], [9], [16, 7], [17], [32, 33, 0, 15], [70]])
+@pytest.mark.parametrize("lens", [[1], [4, 3], [5], [8, 1, 0], [9], [16, 7], [17], [32, 33, 0, 15], [64], [48, 16, 1]])
 @pytest.mark.parametrize("init", ["zero", "normal"])
-def test_short_prompt_block_edges(lens, init):
+@pytest.mark.parametrize("route", ["recurrent", "auto"])
+def test_short_prompt_block_edges(lens, init, route):
     p = I.prefill_inputs(lens, 2, 4, seed=9500 + sum(lens), alpha_lo=0.5, init=init)
-    o, S, status = run_prefill(p, "recurrent")
+    o, S, status = run_prefill(p, route)
     o_ref, S_ref, _ = oracle_prefill(p)
     assert status == 0
     U.check_o(o, o_ref, U.O_REL_L2_DECODE)
-    assert U.rel_l2(S.astype(np.float64), S_ref) < 1e-5
+    # (gdn_prefill sends more than 64 tokens, whose lengths it is not told, to the chunked kernels)
+    blocks = route == "recurrent" or sum(lens) <= 64
+    assert U.rel_l2(S.astype(np.float64), S_ref) < (1e-5 if blocks else U.STATE_REL_L2_PREFILL)
