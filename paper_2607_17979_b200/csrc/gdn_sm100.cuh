@@ -100,11 +100,6 @@ __device__ __forceinline__ void bulk_wait_all() {
 __device__ __forceinline__ void bulk_wait_read_all() {
     asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
 }
-// Hint: bring one box of a tiled tensor into L2 (no shared memory, no completion to wait for).
-__device__ __forceinline__ void tma_prefetch_2d(const CUtensorMap* map, int x, int y) {
-    asm volatile("cp.async.bulk.prefetch.tensor.2d.L2.global [%0, {%1, %2}];" ::"l"(map), "r"(x), "r"(y)
-                 : "memory");
-}
 __device__ __forceinline__ void prefetch_tensormap(const CUtensorMap* map) {
     asm volatile("prefetch.tensormap [%0];" ::"l"(map) : "memory");
 }
@@ -162,29 +157,12 @@ __device__ __forceinline__ void mma_ss(uint32_t d_tmem, uint64_t a_desc, uint64_
         "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(static_cast<uint32_t>(accumulate))
         : "memory");
 }
-// D[tmem] (+)= A[tmem] * B[smem]; A is K-major, two bf16 per 32-bit column.
-__device__ __forceinline__ void mma_ts(uint32_t d_tmem, uint32_t a_tmem, uint64_t b_desc,
-                                       uint32_t idesc, bool accumulate) {
-    asm volatile(
-        "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}" ::"r"(d_tmem),
-        "r"(a_tmem), "l"(b_desc), "r"(idesc), "r"(static_cast<uint32_t>(accumulate))
-        : "memory");
-}
-// Same with the accumulate flag fixed at compile time, and a descriptor helper that moves the
-// start address of an existing descriptor by a byte offset (one 64-bit add): together they keep
-// the issuing thread's work per instruction to a handful of ALU operations.
+// D[tmem] (+)= A[tmem] * B[smem] (A is K-major, two bf16 per 32-bit column) with the accumulate flag
+// fixed at compile time, and a descriptor helper that moves the start address of an existing
+// descriptor by a byte offset (one 64-bit add): together they keep the issuing thread's work per
+// instruction to a handful of ALU operations.
 __device__ __forceinline__ uint64_t sdesc_advance(uint64_t desc, uint32_t byte_off) {
     return desc + static_cast<uint64_t>(byte_off >> 4);
-}
-template <bool kAccumulate>
-__device__ __forceinline__ void mma_ss_c(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc,
-                                         uint32_t idesc) {
-    asm volatile(
-        "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(d_tmem),
-        "l"(a_desc), "l"(b_desc), "r"(idesc), "n"(kAccumulate ? 1 : 0)
-        : "memory");
 }
 template <bool kAccumulate>
 __device__ __forceinline__ void mma_ts_c(uint32_t d_tmem, uint32_t a_tmem, uint64_t b_desc,
@@ -261,12 +239,6 @@ __device__ __forceinline__ void stmatrix_x4_trans(uint32_t saddr, uint32_t m0, u
                                                   uint32_t m3) {
     asm volatile("stmatrix.sync.aligned.m8n8.x4.trans.shared.b16 [%0], {%1, %2, %3, %4};" ::"r"(saddr),
                  "r"(m0), "r"(m1), "r"(m2), "r"(m3)
-                 : "memory");
-}
-// Two matrices; lanes 0-15 supply the addresses.
-__device__ __forceinline__ void stmatrix_x2_trans(uint32_t saddr, uint32_t m0, uint32_t m1) {
-    asm volatile("stmatrix.sync.aligned.m8n8.x2.trans.shared.b16 [%0], {%1, %2};" ::"r"(saddr), "r"(m0),
-                 "r"(m1)
                  : "memory");
 }
 __device__ __forceinline__ void tmem_wait_ld() {
