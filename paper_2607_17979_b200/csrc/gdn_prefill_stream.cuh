@@ -370,6 +370,39 @@ __device__ __forceinline__ void state_stream_role(const TensorMaps& maps, const 
             }
         };
         bool ok = true;
+        // Whole states move between global memory and the chain threads through TMEM, whose fragment
+        // shape gives a warp access 8 rows of 32 bytes.  Straight from the threads' own rows it touched
+        // 32 rows of 16 bytes, 4100 load/store cycles per state, in front of the next unit (8192 tokens
+        // in 57 sequences 246 -> 225 us, with initial states 306 -> 250 us; 100 tokens 18.5 -> 16.9 us).
+        // Fragment piece i (0..3): rows 16 (i & 1) .., columns 64 half + 32 (i >> 1) ..
+        auto frag_off = [&] { return ((warp & 3) * 32 + (lane >> 2)) * kD + half * 64 + 2 * (lane & 3); };
+        auto piece_off = [&](int i, int b, int r) { return ((i & 1) * 16 + 8 * r) * kD + 32 * (i >> 1) + 8 * b; };
+        // The final state of the unit before, still in the D4 tile: written once the next unit's first
+        // product is on its way (which does not touch that tile; the next state product waits for
+        // these warps).
+        int pending = -1, pending_unit = 0;
+        auto flush = [&] {
+            if (pending < 0) return;
+            float* out = p.final_state + static_cast<size_t>(pending) * (kD * kD) + frag_off();
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                uint32_t y[16];
+                tmem_ld_16x256b_x4(tmem + kT_D4 + lane_base + half * 64 + (static_cast<uint32_t>(i & 1) << 20) +
+                                       32 * (i >> 1),
+                                   y);
+                tmem_wait_ld();
+#pragma unroll
+                for (int b = 0; b < 4; ++b)
+#pragma unroll
+                    for (int r = 0; r < 2; ++r)
+                        *reinterpret_cast<uint2*>(out + piece_off(i, b, r)) =
+                            make_uint2(y[4 * b + 2 * r], y[4 * b + 2 * r + 1]);
+            }
+            if constexpr (kGated == 2) {
+                if (tid == 0) done_w[pending_unit] = 1;
+            }
+            pending = -1;
+        };
         // Bounded wait + tcgen05 fence
         auto await = [&](uint64_t* bar, uint32_t parity) {
             if (ok && !warp_wait_or_abort(bar, parity, abortp, kWaitReason)) ok = false;
@@ -379,14 +412,21 @@ __device__ __forceinline__ void state_stream_role(const TensorMaps& maps, const 
         // (ok == false), so that no warp is ever left alone at a barrier.  It then works on with whatever
         // is there; nothing of it is written out.  (A branch around each phase costs 60 cycles a
         // chunk step: 32768 tokens at 8 v-heads 793 -> 769 us without them.)
-        UnitInfo nxt = unit_info(p, ws, lay, min(cta, total_units - 1), done_tab);
+        // A unit's chunks (0: nothing for the chain) and state tile; the rest of its entry is read again
+        // where a unit is left out (registers).
+        auto brief = [&](int unit) {
+            const UnitInfo u = unit_info(p, ws, lay, min(unit, total_units - 1), done_tab);
+            return make_int2(u.done || u.skip ? 0 : u.nc, u.slot * p.Hv + u.hv);
+        };
+        int2 nxt = brief(cta);
         for (int unit = cta; unit < total_units; unit += n_ctas) {
-            const UnitInfo u = nxt;
-            nxt = unit_info(p, ws, lay, min(unit + n_ctas, total_units - 1), done_tab);
-            const size_t tile_off = (static_cast<size_t>(u.bad_slot ? 0 : u.slot) * p.Hv + u.hv) * (kD * kD) +
-                                    static_cast<size_t>(dv) * kD + half * 64;
-            if (u.done) continue;
-            if (u.skip) {
+            const int nc = nxt.x, tile = nxt.y;
+            nxt = brief(unit + n_ctas);
+            if (nc == 0) {
+                const UnitInfo u = unit_info(p, ws, lay, unit, done_tab);
+                if (u.done) continue;
+                const size_t tile_off = (static_cast<size_t>(u.bad_slot ? 0 : u.slot) * p.Hv + u.hv) * (kD * kD) +
+                                        static_cast<size_t>(dv) * kD + half * 64;
                 if constexpr (kGated == 2) {
                     if (tid == 0) done_w[unit] = 1;
                 }
@@ -408,13 +448,38 @@ __device__ __forceinline__ void state_stream_role(const TensorMaps& maps, const 
                 }
                 continue;
             }
-            const int nc = u.nc;
             // the unit's initial state
             if (p.init_state) {
+                const float* in = p.init_state + static_cast<size_t>(tile) * (kD * kD) + frag_off();
+                uint32_t x[4][16];
 #pragma unroll
-                for (int j = 0; j < 64; j += 4) {
-                    const float4 x = *reinterpret_cast<const float4*>(p.init_state + tile_off + j);
-                    S[j] = x.x; S[j + 1] = x.y; S[j + 2] = x.z; S[j + 3] = x.w;
+                for (int i = 0; i < 4; ++i)
+#pragma unroll
+                    for (int b = 0; b < 4; ++b)
+#pragma unroll
+                        for (int r = 0; r < 2; ++r) {
+                            const uint2 v = *reinterpret_cast<const uint2*>(in + piece_off(i, b, r));
+                            x[i][4 * b + 2 * r] = v.x;
+                            x[i][4 * b + 2 * r + 1] = v.y;
+                        }
+                // (through the columns of the decayed U, which the last state product has read)
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    const uint32_t t = tmem + kT_Us + lane_base + half * 32;
+                    tmem_st_16x256b_x4(t, x[2 * h]);
+                    tmem_st_16x256b_x4(t + (16u << 16), x[2 * h + 1]);
+                    tmem_wait_st();
+                    __syncwarp();
+                    uint32_t y0[16], y1[16];
+                    tmem_ld16(t, y0);
+                    tmem_ld16(t + 16, y1);
+                    tmem_wait_ld();
+                    __syncwarp();
+#pragma unroll
+                    for (int q = 0; q < 16; ++q) {
+                        S[32 * h + q] = __uint_as_float(y0[q]);
+                        S[32 * h + 16 + q] = __uint_as_float(y1[q]);
+                    }
                 }
             } else {
 #pragma unroll
@@ -422,6 +487,10 @@ __device__ __forceinline__ void state_stream_role(const TensorMaps& maps, const 
             }
             store_state_bf16();
             hand_over(&bar_s);
+            // the next unit's initial state, towards L2
+            if (p.init_state && tid == 0 && nxt.x > 0 && unit + n_ctas < total_units)
+                bulk_prefetch_l2(p.init_state + static_cast<size_t>(nxt.y) * (kD * kD), kD * kD * 4);
+            flush();
             for (int j = 0; j < nc; ++j) {
                 const uint32_t g = gc + j;
                 const int st = g & 1;
@@ -477,26 +546,32 @@ __device__ __forceinline__ void state_stream_role(const TensorMaps& maps, const 
                             S[c0 + 16 + jj] = fmaf(gC, S[c0 + 16 + jj], __uint_as_float(xb[jj]));
                         }
                     }
-                    if (!last) store_state_bf16();   // the next chunk's A operand
                 }
                 if (last) {
-                    ok = group_all<2, kSEpiThreads>(ok);     // nothing of a unit is written after a failed wait
+                    // nothing of a unit is written after a failed wait (every record of the unit has been loaded by
+                    // now: no flag wait of it can fail any more)
+                    ok = group_all<2, kSEpiThreads>(ok);
                     if (ok) {
 #pragma unroll
-                        for (int j4 = 0; j4 < 64; j4 += 4)
-                            *reinterpret_cast<float4*>(p.final_state + tile_off + j4) =
-                                make_float4(S[j4], S[j4 + 1], S[j4 + 2], S[j4 + 3]);
-                        // (every record of the unit has been loaded by now: no flag wait can
-                        // fail after this point, and any other failure is reported as an error)
-                        if constexpr (kGated == 2) {
-                            if (tid == 0) done_w[unit] = 1;
+                        for (int c0 = 0; c0 < 64; c0 += 8) {
+                            uint32_t y[8];
+#pragma unroll
+                            for (int q = 0; q < 8; ++q) y[q] = __float_as_uint(S[c0 + q]);
+                            tmem_st8(tmem + kT_D4 + lane_base + half * 64 + c0, y);
                         }
+                        tmem_wait_st();
+                        __syncwarp();
+                        pending = tile;
+                        pending_unit = unit;
                     }
+                } else {
+                    store_state_bf16();          // the next chunk's A operand
+                    hand_over(&bar_s);
                 }
-                if (!last) hand_over(&bar_s);
             }
             gc += nc;
         }
+        flush();
     } else {
         reg_dealloc<112>();
         // ===================== output warps: Y = scale e^b (S Q^T) + U P^T (fp32, TMEM) -> o rows.  Warp 8 + q

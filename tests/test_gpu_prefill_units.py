@@ -1,0 +1,29 @@
+"""Chunked prefill with more (sequence, v-head) units than SMs, so that a CTA goes from one unit's final state
+to the next one's initial state: unequal lengths, empty sequences and padding slots in between, states in place."""
+import numpy as np
+import pytest
+
+import gpu_util as U
+from paper_2607_17979_b200 import inputs as I
+from test_gpu_prefill import oracle_prefill, run_prefill
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("route", ["stream", "fused", "overlap"])
+@pytest.mark.parametrize("alias", [False, True])
+@pytest.mark.parametrize("lens", [[1] * 20, [64, 65, 0, 129, 7] * 8, [200] + [1, 63, 0] * 12])
+def test_unit_changes(lens, alias, route):
+    n = len(lens)
+    p = I.prefill_inputs(lens, 4, 16, seed=9700 + n, alpha_lo=0.5, init="normal")
+    slots = np.arange(n, dtype=np.int32)[::-1].copy()
+    slots[3::7] = -1
+    o, S, status = run_prefill(p, route, slot_idx=slots, num_slots=n, alias=alias, pool_fill=7.0)
+    o_ref, S_ref, _ = oracle_prefill(p, slot_idx=slots, num_slots=n)
+    assert status == 0
+    U.check_o(o, o_ref, U.O_REL_L2_PREFILL)
+    used = np.sort(slots[slots >= 0])
+    unused = np.setdiff1d(np.arange(n), used)
+    for s in used:
+        U.check_state(S[s:s + 1].astype(np.float64), S_ref[s:s + 1], U.STATE_REL_L2_PREFILL)
+    assert np.array_equal(S[unused], p["init_state"][unused] if alias else np.full_like(S[unused], 7.0))
