@@ -1,4 +1,5 @@
 // C-ABI entry points: argument validation and launch.  See include/gdn.h.
+#include <algorithm>
 #include "gdn_common.cuh"
 #include "gdn_prefill_chunk.cuh"
 #include "../../include/gdn.h"
@@ -271,7 +272,20 @@ int gdn_prefill_route(int32_t T, int32_t N, int32_t max_seqlen_hint, int32_t Hv,
     if (units <= sm_count / 2 && longest <= GDN_BLOCKS_MAX_SEQLEN) return GDN_ROUTE_BLOCKS;
     // Few (sequence, v-head) units and long sequences: the serial state pass would occupy only a
     // few SMs while the rest idle, so run it next to the record producers in one cooperative launch.
-    if (cooperative_launch && units <= sm_count / 3 && longest > 16 * gdn::kChunk) return GDN_ROUTE_FUSED;
+    // That launch starts ~10 us later (two table launches, one CTA per SM) and gains what the
+    // intra-chunk kernel would have taken alone, which grows with the units, until at about a
+    // quarter of the SMs the producing CTAs no longer keep up with the chains.  The lengths at which three
+    // launches are level with it on 148 SMs: 38 chunks at 8 units, 29 at 16, 24 at 32, 27 at 36, 31 at
+    // 40, 55 at 44, none at 48 (8 units, 1536 tokens 53.3 us in three launches, 56.8 in one; 48 units,
+    // 2048 tokens 98.8 and 110).  With the longest length known, the two-part route below is ahead from 40
+    // units on (48 units, 3400 tokens 132 us against 165); from 64 chunks on the answer of
+    // gdn_prefill_route is kept as it has been.
+    const int32_t u = static_cast<int32_t>(std::min<long long>(units, sm_count));
+    const int32_t level = std::max({16, 3 * sm_count / 10 - u, 16 + 2 * (u - sm_count * 9 / 40)});
+    const bool two_part = max_seqlen_hint > 0 && units <= sm_count / 2 && longest >= 40 * gdn::kChunk;
+    if (cooperative_launch && units <= sm_count / 3 && longest > level * gdn::kChunk &&
+        !(two_part && units > sm_count / 4 && longest < 64 * gdn::kChunk))
+        return GDN_ROUTE_FUSED;
     // More units than the cooperative launch takes but at most half as many as SMs, with long
     // chains (known only through the caller's hint): the state pass leaves half the machine free
     // from the start, so part of the records is produced beside it (two sequences of 4096 tokens
@@ -283,8 +297,7 @@ int gdn_prefill_route(int32_t T, int32_t N, int32_t max_seqlen_hint, int32_t Hv,
     // first and free it as their short chains end would gain 5-12 %, but the records produced late
     // are still dirty in L2 when the call ends and their write-back falls into whatever runs
     // next, and batches of equal chains lose up to 7 %: those stay with the persistent pass.
-    if (max_seqlen_hint > 0 && units <= sm_count / 2 && longest >= 40 * gdn::kChunk)
-        return GDN_ROUTE_OVERLAP;
+    if (two_part) return GDN_ROUTE_OVERLAP;
     // Everything else: the three launches (table kernel, or none for small batches; the intra-chunk
     // kernel over all items; the persistent state pass).
     return GDN_ROUTE_STREAM;
