@@ -38,7 +38,7 @@ bool make_prefill_tensor_maps(TensorMaps* maps, const PrefillParams& p);
 // one CTA writes the per-sequence tables (first chunk, validity, rank) for the state pass.  Only
 // for batches of few sequences: see prefill_tables_inline().
 cudaError_t launch_prefill_intra(const TensorMaps& maps, const ChunkedParams& cp, cudaStream_t stream,
-                                 bool inline_tables);
+                                 bool inline_tables, bool scaled_q);
 bool prefill_tables_inline(const ChunkedParams& cp);
 
 __device__ __forceinline__ float ex2_approx(float x) {

@@ -27,3 +27,17 @@ def test_unit_changes(lens, alias, route):
     for s in used:
         U.check_state(S[s:s + 1].astype(np.float64), S_ref[s:s + 1], U.STATE_REL_L2_PREFILL)
     assert np.array_equal(S[unused], p["init_state"][unused] if alias else np.full_like(S[unused], 7.0))
+
+
+@pytest.mark.parametrize("n, hv", [(37, 2), (75, 1), (37, 4), (149, 1)])
+def test_record_forms(n, hv):
+    """Half as many units as SMs and one more, as many and one more (148 SMs): the records change form there, in
+    the three launches and in the two-part route alike."""
+    p = I.prefill_inputs([130 - i % 67 for i in range(n)], 1, hv, seed=9800 + n + hv, alpha_lo=0.5, init="normal")
+    o, S, status = run_prefill(p, "stream")
+    o2, S2, status2 = run_prefill(p, "overlap", split_permille=300)
+    o_ref, S_ref, _ = oracle_prefill(p)
+    assert status == 0 and status2 == 0
+    assert np.array_equal(o, o2) and np.array_equal(S, S2)
+    U.check_o(o, o_ref, U.O_REL_L2_PREFILL)
+    U.check_state(S.astype(np.float64), S_ref, U.STATE_REL_L2_PREFILL)
