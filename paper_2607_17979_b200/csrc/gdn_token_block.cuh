@@ -15,10 +15,12 @@
 // (shared-memory reads of k and q and the cross-lane sums as much as the multiply-adds), against
 // 5900 cycles for the tile's HBM traffic, and the two did not overlap well: 52 / 73 / 121 us at L =
 // 4 / 8 / 16 (B = 64, 32 v-heads, floor 42).  Both state GEMMs here are mma.sync with M = 16 rows
-// per warp; the state in fp32 is the accumulator fragment of the update, and the same registers,
+// per warp; the state in fp32 lies in registers as an accumulator fragment, and the same registers,
 // split EXACTLY into three bf16 terms (8 + 8 + 8 bits), are the A operand of the products with k and
-// q, which are bf16 in memory: no operand is rounded and every sum is fp32.  (w is split the same
-// way.)  tcgen05 would need the split terms in TMEM and a 128-row tile per instruction: a detour
+// q, which are bf16 in memory: no operand is rounded.  (w is split the same way.)  The tensor cores sum in
+// fp32 but cut off where an fp32 addition rounds to nearest, so the state itself is never their
+// accumulator: the update's sum starts from zero and one fma per element joins it to the decayed
+// state.  tcgen05 would need the split terms in TMEM and a 128-row tile per instruction: a detour
 // through two more memories for a kernel whose floor is the tile's HBM traffic.
 //
 // Fragment map (m16n8k16): lane = 4 g + t; a warp holds 64 state values per lane, s[m][n][c], c = {fragment
@@ -459,26 +461,40 @@ __device__ __forceinline__ void apply_block(const TokenRows& t, TokenBlock<kTran
         } else {
             ldmatrix_x4<true>(bn[0], &st.kq[lane & (kMax - 1)][col0 + 8 * (n0 + (lane >> 3))]);
         }
+        // The sum starts from zero: with the decayed state as the first addend every call cut part of an ulp off
+        // each element, always towards zero (400 calls of 4 tokens, no decay, beta < 0.001: state error
+        // 1.3e-5, all of it one-sided; under 2e-6 with the state joined by fma).
+        constexpr int kGroup = 4 / kTiles;        // 8-column blocks at a time, 16 accumulators
 #pragma unroll
-        for (int n = 0; n < 4; ++n)
+        for (int q = 0; q < 4; q += kGroup) {
+            float d[kTiles][kGroup][4];
 #pragma unroll
-            for (int m = 0; m < kTiles; ++m)
+            for (auto& m : d)
 #pragma unroll
-                for (float& y : s[m][n0 + n]) y *= last;
+                for (auto& n : m) n[0] = n[1] = n[2] = n[3] = 0.f;
 #pragma unroll
-        for (int i = kA - 1; i >= 0; --i)         // small terms first
+            for (int i = kA - 1; i >= 0; --i)     // small terms first
 #pragma unroll
-            for (int n = 0; n < 4; ++n)
+                for (int n = 0; n < kGroup; ++n)
 #pragma unroll
-                for (int m = 0; m < kTiles; ++m) {
-                    float(&d)[4] = s[m][n0 + n];
-                    if constexpr (kMax == 16)
-                        mma_k16(d, a[m][i], bn[n >> 1][2 * (n & 1)], bn[n >> 1][2 * (n & 1) + 1]);
-                    else if (kMax == 8 && i == 1)
-                        mma_k8(d, a[m][1][0], a[m][1][1], bn[0][n]);
-                    else
-                        mma_k16(d, a[m][0], bn[0][n], bn[0][n]);
-                }
+                    for (int m = 0; m < kTiles; ++m) {
+                        if constexpr (kMax == 16)
+                            mma_k16(d[m][n], a[m][i], bn[(q + n) >> 1][2 * (n & 1)], bn[(q + n) >> 1][2 * (n & 1) + 1]);
+                        else if (kMax == 8 && i == 1)
+                            mma_k8(d[m][n], a[m][1][0], a[m][1][1], bn[0][q + n]);
+                        else
+                            mma_k16(d[m][n], a[m][0], bn[0][q + n], bn[0][q + n]);
+                    }
+#pragma unroll
+            for (int n = 0; n < kGroup; ++n)
+#pragma unroll
+                for (int m = 0; m < kTiles; ++m)
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) {
+                        float& y = s[m][n0 + q + n][e];
+                        y = fmaf(last, y, d[m][n][e]);
+                    }
+        }
     }
     if constexpr (kTransposed) exchange_state(s, 4 * (lane & 7) + (lane >> 3));      // and back
 }
