@@ -596,7 +596,7 @@ __device__ __forceinline__ void state_stream_role(const TensorMaps& maps, const 
         // from shared memory, the 32 KB took 300 of the 3700 cycles of a chunk step.)
         const int odv = q4 * 32 + lane;
         // (raw Q) the chunk's scale e^{b_r} outlives its stage: a copy per warp, two chunks deep
-        __shared__ float s_eb[kScaledQ ? 1 : kSOutThreads / 32][2][kChunk];
+        __shared__ __align__(8) float s_eb[kScaledQ ? 1 : kSOutThreads / 32][2][kChunk];
         auto preload = [&](uint32_t gq) {       // chunk gq of the CTA's stream -> accumulator
             const int sq = gq & 1;
             if (ok && !warp_wait_or_abort<40>(&bar_full[sq], (gq >> 1) & 1u, abortp, kWaitReason)) ok = false;
