@@ -297,7 +297,7 @@ __device__ __forceinline__ void state_stream_role(const TensorMaps& maps, const 
                     // Y.  Scaled Q: both terms in one of two tiles.  Raw Q: a tile for each term.
                     const uint32_t tY1 = tmem + kT_Y + (kScaledQ ? 64 * st : 0);
                     const uint32_t tY2 = tmem + kT_Y + (kScaledQ ? 64 * st : 64);
-                    if (!wait_or_abort(&bar_s, g & 1u, abortp, kWaitReason)) {      // record landed, bf16 S and U~ in TMEM
+                    if (!warp_wait_or_abort(&bar_s, g & 1u, abortp, kWaitReason)) {      // record landed, bf16 S and U~ in TMEM
                         live = false;
                         break;
                     }
@@ -315,7 +315,7 @@ __device__ __forceinline__ void state_stream_role(const TensorMaps& maps, const 
                     if (elect_one()) mma_commit(&bar_d1);
                     // S Q^T  (off the chain) overwrites the tile the output warps read two chunks ago (raw Q: one
                     // chunk ago)
-                    if (!kScaledQ && g > 0 && !wait_or_abort(&bar_y_read, (g - 1) & 1u, abortp, kWaitReason)) {
+                    if (!kScaledQ && g > 0 && !warp_wait_or_abort(&bar_y_read, (g - 1) & 1u, abortp, kWaitReason)) {
                         live = false;
                         break;
                     }
@@ -329,7 +329,7 @@ __device__ __forceinline__ void state_stream_role(const TensorMaps& maps, const 
                     if (elect_one()) mma_ts_c<true>(tY1, tS + 48, sdesc_advance(qg, 8192 + 64), id64);
                     if (elect_one()) mma_ts_c<true>(tY1, tS + 56, sdesc_advance(qg, 8192 + 96), id64);
                     if (elect_one()) mma_commit(&bar_free_a[st]);                          // W and Q have been read
-                    if (!wait_or_abort(&bar_u, g & 1u, abortp, kWaitReason)) {         // U operands in TMEM
+                    if (!warp_wait_or_abort(&bar_u, g & 1u, abortp, kWaitReason)) {         // U operands in TMEM
                         live = false;
                         break;
                     }
@@ -410,9 +410,11 @@ __device__ __forceinline__ void state_stream_role(const TensorMaps& maps, const 
             }
             pending = -1;
         };
-        // Bounded wait + tcgen05 fence
+        // Bounded wait + tcgen05 fence.  `ok` is each lane's own until the unit's last chunk, where the group
+        // agrees on it; no warp-wide instruction before that depends on it.
         auto await = [&](uint64_t* bar, uint32_t parity) {
-            if (ok && !warp_wait_or_abort(bar, parity, abortp, kWaitReason)) ok = false;
+            if (ok) ok = wait_or_abort(bar, parity, abortp, kWaitReason);
+            __syncwarp();
             tc_fence_after_sync();
         };
         // Every warp runs every group barrier and hand-over below, also after a wait has failed
@@ -589,7 +591,13 @@ __device__ __forceinline__ void state_stream_role(const TensorMaps& maps, const 
         const int ot = tid - kSOutWarp0 * 32;
         const size_t tok_stride = static_cast<size_t>(p.Hv) * kD;
         auto out_sync = [] { asm volatile("bar.sync 1, %0;" ::"n"(kSOutThreads) : "memory"); };
+        // As in the chain warps: each lane's own, and after a failed wait the work goes on with whatever is there; only
+        // the stores of rows depend on it.
         bool ok = true;
+        auto await = [&](uint64_t* bar, uint32_t parity) {
+            if (ok) ok = wait_or_abort<40>(bar, parity, abortp, kWaitReason);
+            __syncwarp();
+        };
         // U~ (fp32, 32 KB per chunk) reaches the chain through the accumulator of S W^T: this group
         // copies it from the record into TMEM one chunk ahead, the product then subtracts S W^T
         // from it (negated B operand), and the chain warps read U itself.  (Read by the chain warps
@@ -599,25 +607,23 @@ __device__ __forceinline__ void state_stream_role(const TensorMaps& maps, const 
         __shared__ __align__(8) float s_eb[kScaledQ ? 1 : kSOutThreads / 32][2][kChunk];
         auto preload = [&](uint32_t gq) {       // chunk gq of the CTA's stream -> accumulator
             const int sq = gq & 1;
-            if (ok && !warp_wait_or_abort<40>(&bar_full[sq], (gq >> 1) & 1u, abortp, kWaitReason)) ok = false;
-            if (ok) {
-                if constexpr (!kScaledQ)
-                    *reinterpret_cast<float2*>(&s_eb[q4][sq][2 * lane]) = *reinterpret_cast<const float2*>(
-                        smem + sq * kStageBytes + kS_Rec + kRecEb + 8 * lane);
-                const float4* sU = reinterpret_cast<const float4*>(smem + sq * kStageBytes + kS_Rec + kRecU);
+            await(&bar_full[sq], (gq >> 1) & 1u);
+            if constexpr (!kScaledQ)
+                *reinterpret_cast<float2*>(&s_eb[q4][sq][2 * lane]) = *reinterpret_cast<const float2*>(
+                    smem + sq * kStageBytes + kS_Rec + kRecEb + 8 * lane);
+            const float4* sU = reinterpret_cast<const float4*>(smem + sq * kStageBytes + kS_Rec + kRecU);
 #pragma unroll
-                for (int c0 = 0; c0 < 64; c0 += 32) {       // eight reads in flight
-                    uint32_t r[2][16];
+            for (int c0 = 0; c0 < 64; c0 += 32) {       // eight reads in flight
+                uint32_t r[2][16];
 #pragma unroll
-                    for (int q = 0; q < 8; ++q) {
-                        const float4 v = sU[((c0 >> 2) + q) * kD + odv];
-                        uint32_t(&x)[16] = r[q >> 2];
-                        x[4 * (q & 3)] = __float_as_uint(v.x); x[4 * (q & 3) + 1] = __float_as_uint(v.y);
-                        x[4 * (q & 3) + 2] = __float_as_uint(v.z); x[4 * (q & 3) + 3] = __float_as_uint(v.w);
-                    }
-                    tmem_st16(tmem + kT_D1 + olane + c0, r[0]);
-                    tmem_st16(tmem + kT_D1 + olane + c0 + 16, r[1]);
+                for (int q = 0; q < 8; ++q) {
+                    const float4 v = sU[((c0 >> 2) + q) * kD + odv];
+                    uint32_t(&x)[16] = r[q >> 2];
+                    x[4 * (q & 3)] = __float_as_uint(v.x); x[4 * (q & 3) + 1] = __float_as_uint(v.y);
+                    x[4 * (q & 3) + 2] = __float_as_uint(v.z); x[4 * (q & 3) + 3] = __float_as_uint(v.w);
                 }
+                tmem_st16(tmem + kT_D1 + olane + c0, r[0]);
+                tmem_st16(tmem + kT_D1 + olane + c0 + 16, r[1]);
             }
             tmem_wait_st();
             tc_fence_before_sync();
@@ -641,7 +647,7 @@ __device__ __forceinline__ void state_stream_role(const TensorMaps& maps, const 
 #pragma unroll 1
                 for (int k = preloaded ? 1 : 0; k < 2; ++k) {
                     if (k == 1) {
-                        if (ok && !warp_wait_or_abort<40>(&bar_u, g & 1u, abortp, kWaitReason)) ok = false;
+                        await(&bar_u, g & 1u);
                         tc_fence_after_sync();
                         if (!ahead) break;
                     }
@@ -651,13 +657,13 @@ __device__ __forceinline__ void state_stream_role(const TensorMaps& maps, const 
                 // every warp runs both group barriers of every chunk, also after a failed wait
                 if (ot == 0) bulk_wait_read_all();       // the last chunk's rows have left the staging tile
                 out_sync();
-                if (ok && !warp_wait_or_abort<40>(&bar_y[buf], (g >> 1) & 1u, abortp, kWaitReason)) ok = false;
+                await(&bar_y[buf], (g >> 1) & 1u);
                 tc_fence_after_sync();
                 // The tile (lanes = dv, columns = tokens) is read as accumulator fragments (lane 4 x + t holds
                 // columns 8 i + 2 t, + 1; raw Q: both tiles, and added), rounded in pairs and stored transposed, 8 dv of one token per 16
                 // bytes, into a [token][dv] tile of two 128B-swizzled halves of 64 dv (what these warps
                 // issue comes out of the chain warps' issue slots).
-                if (ok) {
+                {
                     const int dv0 = q4 * 32 + 8 * (lane >> 3);         // the 8 dv this lane's address covers
                     const uint32_t dst = smem_u32(smem + kS_Out) + (dv0 >> 6) * 8192;
 #pragma unroll
