@@ -11,7 +11,7 @@ namespace gdn {
 // kInlineTable: a batch of at most kInlineTableSeqs sequences needs no table-building launch in
 // front: every CTA finds its own chunk by walking cu_seqlens, and CTA (0, 0) writes the two small
 // per-sequence tables the state pass reads after this kernel (2.5 us less on a 100-token prompt).
-template <bool kInlineTable, bool kScaledQ>
+template <bool kInlineTable>
 __global__ void __launch_bounds__(kIntraThreads, 4)
 prefill_intra_kernel(const __grid_constant__ TensorMaps maps, const PrefillParams p, uint8_t* ws,
                      const WorkspaceLayout lay) {
@@ -94,7 +94,7 @@ prefill_intra_kernel(const __grid_constant__ TensorMaps maps, const PrefillParam
     __syncthreads();
     tc_fence_after_sync();
     const uint32_t tmem = tmem_base_s;
-    intra_item<kScaledQ>(maps, p, rec, ci, hqk, hv, smem, st, tmem, tid, [] { __syncthreads(); });
+    intra_item<false>(maps, p, rec, ci, hqk, hv, smem, st, tmem, tid, [] { __syncthreads(); });
     tc_fence_before_sync();
     __syncthreads();
     if (warp == 0) tmem_dealloc(tmem, kIntraTmemCols);
@@ -153,9 +153,8 @@ bool prefill_tables_inline(const ChunkedParams& cp) {
 }
 
 cudaError_t launch_prefill_intra(const TensorMaps& maps, const ChunkedParams& cp, cudaStream_t stream,
-                                 bool inline_tables, bool scaled_q) {
-    auto kernel = inline_tables ? (scaled_q ? prefill_intra_kernel<true, true> : prefill_intra_kernel<true, false>)
-                                : (scaled_q ? prefill_intra_kernel<false, true> : prefill_intra_kernel<false, false>);
+                                 bool inline_tables) {
+    auto kernel = inline_tables ? prefill_intra_kernel<true> : prefill_intra_kernel<false>;
     cudaError_t e = ensure_dynamic_smem(kernel, kIntraSmem);
     if (e != cudaSuccess) return e;
     dim3 grid(cp.lay.max_chunks, cp.p.Hv);

@@ -27,16 +27,18 @@ namespace gdn {
 // byte image the state-pass kernel wants in shared memory (linear bulk copies):
 //   [0, 16384)      W   as one MN-major 128B-swizzled tile [128 dk][64 tokens] bf16 (a row per dk)
 //   [16384, 32768)  Qg  = diag(scale e^b) Q as two K-major 128B-swizzled halves [64 tokens][64 dk] bf16:
-//                   only where kScaledQ
+//                   in the cooperative launch only
 //   [32768, 40960)  P   as one K-major 128B-swizzled tile   [64 r][64 i]      bf16, scale folded in
 //   [40960, 73728)  U~  as [16 token-groups][128 dv][4 tokens] fp32
 //   [73728, 73984)  e^{b_C - b_c} for c = 0..63, fp32 (rows past the chunk's length hold 1)
 //   [73984, 74240)  scale e^{b_r} for r = 0..63, fp32
 //   [74240, 74496)  e^{b_C} in the first float, rest unused
-// The output's first term is diag(scale e^b) Q S0^T.  kScaledQ: the record carries Qg, both terms meet in
-// one accumulator.  Otherwise the state pass loads the raw Q tile and scales the rows of the product:
-// the intra-chunk kernel saves a pass over Q and a fifth of its writes and can load V early (4
-// sequences, 7680 tokens: 98 -> 89 us), the state pass pays with a second accumulator to read.
+// The output's first term is diag(scale e^b) Q S0^T.  Cooperative launch (kScaledQ): the record carries Qg and
+// both terms meet in one accumulator, since whatever the output warps do there comes out of the chain's issue
+// slots (32768 tokens 792 us, with raw Q 854).  Elsewhere the state pass loads the raw Q tile and scales the
+// rows of the product: the intra-chunk kernel saves a pass over Q and a fifth of its writes and can load V
+// early, the state pass pays with a second accumulator to read (4 x 2048 tokens at 32 heads 163 us, with the
+// scaled Q 172; 512 + 1024 + 2048 + 4096 200.7 and 203.3, 57 sequences 223 and 240).
 constexpr uint32_t kRecW = 0;
 constexpr uint32_t kRecQg = 16384;
 constexpr uint32_t kRecP = 32768;

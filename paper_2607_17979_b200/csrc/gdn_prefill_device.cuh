@@ -38,7 +38,7 @@ bool make_prefill_tensor_maps(TensorMaps* maps, const PrefillParams& p);
 // one CTA writes the per-sequence tables (first chunk, validity, rank) for the state pass.  Only
 // for batches of few sequences: see prefill_tables_inline().
 cudaError_t launch_prefill_intra(const TensorMaps& maps, const ChunkedParams& cp, cudaStream_t stream,
-                                 bool inline_tables, bool scaled_q);
+                                 bool inline_tables);
 bool prefill_tables_inline(const ChunkedParams& cp);
 
 __device__ __forceinline__ float ex2_approx(float x) {
@@ -234,7 +234,7 @@ template <int kId, int kThreads> __device__ __forceinline__ bool group_all(const
 // loop is a vote, so the verdict is the same on every lane whatever each lane's poll answers: callers
 // issue warp-wide instructions on the strength of it.  (Polling by lane 0 and broadcasting the verdict costs a
 // divergent branch and a shuffle: a wait on a completed barrier took 140 cycles instead of 4, and a waiting
-// warp saw an arrival after 183 instead of 62.  The vote: 7680 tokens in 4 sequences 200 -> 203 us.)
+// warp saw an arrival after 183 instead of 62.)
 __device__ __forceinline__ bool warp_wait_or_abort(uint64_t* bar, uint32_t parity, volatile int* abort_flag,
                                                    const int reason = 1) {
     for (uint32_t i = 0; i < kSpinLimit; ++i) {

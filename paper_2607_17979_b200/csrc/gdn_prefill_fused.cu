@@ -365,7 +365,7 @@ prefill_fused_kernel(const __grid_constant__ TensorMaps maps, const PrefillParam
     tc_fence_after_sync();
     const uint32_t tmem = tmem_base_s;
     if (static_cast<int>(blockIdx.x) < n_state) {
-        state_stream_role<1, true>(maps, p, ws, lay, smem, tmem, blockIdx.x, n_state);
+        state_stream_role<1>(maps, p, ws, lay, smem, tmem, blockIdx.x, n_state);
     } else {
         fused_intra_role(maps, p, ws, lay, smem, intra_statics, tmem);
         tc_fence_before_sync();

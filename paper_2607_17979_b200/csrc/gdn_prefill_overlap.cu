@@ -35,7 +35,6 @@ namespace gdn {
 constexpr int kOverlapSpareSms = 8;
 
 // First part: one CTA per item [0, cut) of the processing order (surplus CTAs exit).
-template <bool kScaledQ>
 __global__ void __launch_bounds__(kIntraThreads, 4)
 prefill_intra_first_kernel(const __grid_constant__ TensorMaps maps, const PrefillParams p,
                            uint8_t* ws, const WorkspaceLayout lay) {
@@ -64,7 +63,7 @@ prefill_intra_first_kernel(const __grid_constant__ TensorMaps maps, const Prefil
     __syncthreads();
     tc_fence_after_sync();
     const uint32_t tmem = tmem_base_s;
-    intra_item<kScaledQ>(maps, p, rec, ci, hv / (p.Hv / p.Hqk), hv, smem, st, tmem, tid, [] { __syncthreads(); });
+    intra_item<false>(maps, p, rec, ci, hv / (p.Hv / p.Hqk), hv, smem, st, tmem, tid, [] { __syncthreads(); });
     tc_fence_before_sync();
     __syncthreads();
     if (warp == 0) tmem_dealloc(tmem, kIntraTmemCols);
@@ -74,7 +73,6 @@ prefill_intra_first_kernel(const __grid_constant__ TensorMaps maps, const Prefil
 // consume them, and publish each record through its flag.  No wait for the state pass (this kernel
 // feeds it): every state-pass CTA has passed its own wait for the first part, hence for prep,
 // before this kernel's CTAs are scheduled.
-template <bool kScaledQ>
 __global__ void __launch_bounds__(kIntraThreads, 4)
 prefill_intra_second_kernel(const __grid_constant__ TensorMaps maps, const PrefillParams p,
                             uint8_t* ws, const WorkspaceLayout lay) {
@@ -112,7 +110,7 @@ prefill_intra_second_kernel(const __grid_constant__ TensorMaps maps, const Prefi
             const ChunkInfo ci = chunks[c];
             const size_t slot = static_cast<size_t>(c) * p.Hv + hv;
             uint8_t* rec = ws + lay.records + slot * kRecBytes;
-            const bool ok = intra_item<kScaledQ>(maps, p, rec, ci, hv / G, hv, smem, st, tmem, tid,
+            const bool ok = intra_item<false>(maps, p, rec, ci, hv / G, hv, smem, st, tmem, tid,
                                        [] { __syncthreads(); }, n_done);
             ++n_done;
             // publish: every thread's own stores first, then the bulk stores, then the flag
@@ -134,7 +132,6 @@ prefill_intra_second_kernel(const __grid_constant__ TensorMaps maps, const Prefi
     if (blockIdx.x == 0) pdl_wait();        // the call is complete when this launch is
 }
 
-template <bool kScaledQ>
 __global__ void __launch_bounds__(kStreamThreads, 1)
 prefill_state_stream_gated_kernel(const __grid_constant__ TensorMaps maps, const PrefillParams p,
                                   uint8_t* ws, const WorkspaceLayout lay) {
@@ -153,14 +150,13 @@ prefill_state_stream_gated_kernel(const __grid_constant__ TensorMaps maps, const
     const uint32_t tmem = tmem_base_s;
     pdl_wait();                     // tables, cleared flags and the first part's records
     pdl_launch_dependents();        // now the second part may take the SMs that are left
-    state_stream_role<2, kScaledQ>(maps, p, ws, lay, smem, tmem, blockIdx.x, gridDim.x);
+    state_stream_role<2>(maps, p, ws, lay, smem, tmem, blockIdx.x, gridDim.x);
     __syncwarp();
     if (warp == kSIssueWarp) tmem_dealloc(tmem, kStateTmemCols);
 }
 
 // Last launch: the plain persistent pass over the units the gated pass did not finish (none, when
 // the producers ran beside it as intended: then every CTA finds its units done and returns).
-template <bool kScaledQ>
 __global__ void __launch_bounds__(kStreamThreads, 1)
 prefill_state_stream_rest_kernel(const __grid_constant__ TensorMaps maps, const PrefillParams p,
                                  uint8_t* ws, const WorkspaceLayout lay) {
@@ -185,22 +181,24 @@ prefill_state_stream_rest_kernel(const __grid_constant__ TensorMaps maps, const 
     __syncthreads();
     tc_fence_after_sync();
     const uint32_t tmem = tmem_base_s;
-    state_stream_role<3, kScaledQ>(maps, p, ws, lay, smem, tmem, blockIdx.x, gridDim.x);
+    state_stream_role<3>(maps, p, ws, lay, smem, tmem, blockIdx.x, gridDim.x);
     __syncwarp();
     if (warp == kSIssueWarp) tmem_dealloc(tmem, kStateTmemCols);
 }
 
-namespace {
-template <bool kScaledQ>
-cudaError_t launch_parts(const ChunkedParams& cp, cudaStream_t stream, int split_permille, int sms) {
+cudaError_t launch_prefill_overlap(const ChunkedParams& cp, cudaStream_t stream, int split_permille) {
+    DeviceInfo di;
+    cudaError_t e = device_info(&di);
+    if (e != cudaSuccess) return e;
+    const int sms = di.sms;
     const PrefillParams& p = cp.p;
-    cudaError_t e = ensure_dynamic_smem(prefill_state_stream_gated_kernel<kScaledQ>, kStreamSmem);
+    e = ensure_dynamic_smem(prefill_state_stream_gated_kernel, kStreamSmem);
     if (e != cudaSuccess) return e;
-    e = ensure_dynamic_smem(prefill_state_stream_rest_kernel<kScaledQ>, kStreamSmem);
+    e = ensure_dynamic_smem(prefill_state_stream_rest_kernel, kStreamSmem);
     if (e != cudaSuccess) return e;
-    e = ensure_dynamic_smem(prefill_intra_first_kernel<kScaledQ>, kIntraSmem);
+    e = ensure_dynamic_smem(prefill_intra_first_kernel, kIntraSmem);
     if (e != cudaSuccess) return e;
-    e = ensure_dynamic_smem(prefill_intra_second_kernel<kScaledQ>, kIntraSmem);
+    e = ensure_dynamic_smem(prefill_intra_second_kernel, kIntraSmem);
     if (e != cudaSuccess) return e;
     TensorMaps maps;
     if (!make_prefill_tensor_maps(&maps, p)) return cudaErrorInvalidValue;
@@ -224,11 +222,11 @@ cudaError_t launch_parts(const ChunkedParams& cp, cudaStream_t stream, int split
     e = launch_prefill_ranked_prep(cp, stream, 2, split_permille, sms);
     if (e != cudaSuccess) return e;
     const dim3 items(static_cast<unsigned>(cp.lay.max_chunks) * static_cast<unsigned>(p.Hv));
-    e = launch_dependent(prefill_intra_first_kernel<kScaledQ>, items, dim3(kIntraThreads), kIntraSmem,
+    e = launch_dependent(prefill_intra_first_kernel, items, dim3(kIntraThreads), kIntraSmem,
                          stream, maps, p, cp.ws, cp.lay);
     if (e != cudaSuccess) return e;
     const int grid = static_cast<int>(units < sms ? units : sms);
-    e = launch_dependent(prefill_state_stream_gated_kernel<kScaledQ>, dim3(grid), dim3(kStreamThreads),
+    e = launch_dependent(prefill_state_stream_gated_kernel, dim3(grid), dim3(kStreamThreads),
                          kStreamSmem, stream, maps, p, cp.ws, cp.lay);
     if (e != cudaSuccess) return e;
     // Producers beyond what the chains consume only add memory traffic beside them (one sequence
@@ -240,27 +238,17 @@ cudaError_t launch_parts(const ChunkedParams& cp, cudaStream_t stream, int split
     if (resident > 4u * static_cast<unsigned>(sms)) resident = 4u * static_cast<unsigned>(sms);
     const dim3 producers(items.x < resident ? items.x : resident);
     if (serialised) {
-        prefill_intra_second_kernel<kScaledQ><<<producers, kIntraThreads, kIntraSmem, stream>>>(maps, p, cp.ws, cp.lay);
+        prefill_intra_second_kernel<<<producers, kIntraThreads, kIntraSmem, stream>>>(maps, p, cp.ws, cp.lay);
         e = cudaGetLastError();
     } else {
-        e = launch_dependent(prefill_intra_second_kernel<kScaledQ>, producers, dim3(kIntraThreads), kIntraSmem,
+        e = launch_dependent(prefill_intra_second_kernel, producers, dim3(kIntraThreads), kIntraSmem,
                              stream, maps, p, cp.ws, cp.lay);
     }
     if (e != cudaSuccess) return e;
     // an ordinary launch: it starts when the second part has ended, and the second part's first
     // CTA ends only after the state pass
-    prefill_state_stream_rest_kernel<kScaledQ><<<grid, kStreamThreads, kStreamSmem, stream>>>(maps, p, cp.ws, cp.lay);
+    prefill_state_stream_rest_kernel<<<grid, kStreamThreads, kStreamSmem, stream>>>(maps, p, cp.ws, cp.lay);
     return cudaGetLastError();
-}
-}  // namespace
-
-cudaError_t launch_prefill_overlap(const ChunkedParams& cp, cudaStream_t stream, int split_permille) {
-    DeviceInfo di;
-    cudaError_t e = device_info(&di);
-    if (e != cudaSuccess) return e;
-    return records_carry_q(static_cast<long long>(cp.p.N) * cp.p.Hv, di.sms)
-               ? launch_parts<true>(cp, stream, split_permille, di.sms)
-               : launch_parts<false>(cp, stream, split_permille, di.sms);
 }
 
 }  // namespace gdn

@@ -4,7 +4,6 @@
 
 namespace gdn {
 
-template <bool kScaledQ>
 __global__ void __launch_bounds__(kStreamThreads, 1)
 prefill_state_stream_kernel(const __grid_constant__ TensorMaps maps, const PrefillParams p,
                             uint8_t* ws, const WorkspaceLayout lay) {
@@ -21,7 +20,7 @@ prefill_state_stream_kernel(const __grid_constant__ TensorMaps maps, const Prefi
     __syncthreads();
     tc_fence_after_sync();
     const uint32_t tmem = tmem_base_s;
-    state_stream_role<0, kScaledQ>(maps, p, ws, lay, smem, tmem, blockIdx.x, gridDim.x);
+    state_stream_role<0>(maps, p, ws, lay, smem, tmem, blockIdx.x, gridDim.x);
     __syncwarp();
     if (warp == kSIssueWarp) tmem_dealloc(tmem, kStateTmemCols);
 }
@@ -35,9 +34,7 @@ cudaError_t launch_prefill_stream(const ChunkedParams& cp, cudaStream_t stream) 
     if (e != cudaSuccess) return e;
     const int sms = di.sms;
     const long long units = static_cast<long long>(p.N) * p.Hv;
-    const bool scaled_q = records_carry_q(units, sms);
-    auto kernel = scaled_q ? prefill_state_stream_kernel<true> : prefill_state_stream_kernel<false>;
-    e = ensure_dynamic_smem(kernel, kStreamSmem);
+    e = ensure_dynamic_smem(prefill_state_stream_kernel, kStreamSmem);
     if (e != cudaSuccess) return e;
     TensorMaps maps;
     if (!make_prefill_tensor_maps(&maps, p)) return cudaErrorInvalidValue;
@@ -47,11 +44,11 @@ cudaError_t launch_prefill_stream(const ChunkedParams& cp, cudaStream_t stream) 
         if (e != cudaSuccess) return e;
     }
     if (cp.lay.max_chunks > 0) {
-        e = launch_prefill_intra(maps, cp, stream, inline_tables, scaled_q);
+        e = launch_prefill_intra(maps, cp, stream, inline_tables);
         if (e != cudaSuccess) return e;
     }
     const int grid = static_cast<int>(units < sms ? units : sms);
-    return launch_dependent(kernel, dim3(grid), dim3(kStreamThreads), kStreamSmem,
+    return launch_dependent(prefill_state_stream_kernel, dim3(grid), dim3(kStreamThreads), kStreamSmem,
                             stream, maps, p, cp.ws, cp.lay);
 }
 

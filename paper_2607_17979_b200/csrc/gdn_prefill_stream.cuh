@@ -93,14 +93,6 @@ __device__ __forceinline__ void fence_proxy_async_all() {
     asm volatile("fence.proxy.async;" ::: "memory");
 }
 
-// Whether the records of the three launches and of the two-part route carry the scaled Q (both by one
-// rule: their results agree bit for bit).  It shortens the chunk step (the output warps read one
-// accumulator instead of two) and adds a fifth to the records' writes, so it pays where the chains
-// bound the call: every SM has at most one unit (7680 tokens in 4 sequences at 32 heads 202 -> 200 us, 2048
-// in 3 70.2 -> 68.3; 57 sequences 223 -> 240, 8 x 1024 174 -> 180).  With half the SMs without a unit the
-// two-part route produces records beside the chains and wants the smaller ones (2 x 4096 183 -> 192).
-inline bool records_carry_q(long long units, int sms) { return units <= sms && 2 * units > sms; }
-
 // The state pass of one CTA of 512 threads over the units cta, cta + n_ctas, ... of the rank-sorted
 // list.  kGated = 0: every record exists (the intra-chunk kernel ran before).  kGated = 1:
 // records are being produced by other CTAs of the same cooperative launch and the loading warp
@@ -110,7 +102,7 @@ inline bool records_carry_q(long long units, int sms) { return units <= sms && 2
 // marked in the done table, the others are left to a later launch).  kGated = 3: that later launch:
 // every record exists, the units marked done are left out.  `tmem` = 512 allocated columns; ends
 // with a CTA barrier.
-template <int kGated, bool kScaledQ>
+template <int kGated>
 __device__ __forceinline__ void state_stream_role(const TensorMaps& maps, const PrefillParams& p,
                                                   uint8_t* ws, const WorkspaceLayout& lay,
                                                   uint8_t* smem, const uint32_t tmem, const int cta,
@@ -124,6 +116,8 @@ __device__ __forceinline__ void state_stream_role(const TensorMaps& maps, const 
     // flag is the shortest, but the limits are counted in polls, not in time): the units this CTA
     // has not finished are left to the last launch, which reports real failures.
     constexpr int kWaitReason = kGated == 2 ? 2 : 1;
+    // Only the cooperative launch's records carry the scaled Q (gdn_prefill_chunk.cuh).
+    constexpr bool kScaledQ = kGated == 1;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int half = (warp >> 2) & 1;                 // which half of the columns this thread owns
     const int dv = (warp & 3) * 32 + lane;            // TMEM lane = state row
