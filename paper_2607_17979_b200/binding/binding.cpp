@@ -7,6 +7,8 @@
 // Errors are the same types and texts the Python marshalling raises (api.py).
 #include <Python.h>
 
+#include <array>
+
 #include <c10/cuda/CUDAStream.h>
 #include <torch/csrc/autograd/python_variable.h>
 
@@ -42,8 +44,9 @@ void* bf16(PyObject* o, const char* name) { return dev<void>(o, at::kBFloat16, n
 float* f32(PyObject* o, const char* name, bool opt = false) { return dev<float>(o, at::kFloat, name, opt); }
 int32_t* i32(PyObject* o, const char* name, bool opt = false) { return dev<int32_t>(o, at::kInt, name, opt); }
 
-// `obj.shape` of a tensor that must have n dimensions (as unpacking it into n names would check).
-at::IntArrayRef shape(PyObject* obj, int n) {
+// `obj.shape` of a tensor that must have N dimensions (as unpacking it into N names would check).  A copy:
+// the tensor's own array may be changed by another thread while the call runs without the interpreter lock.
+template <int N> std::array<int32_t, N> shape(PyObject* obj) {
     const at::Tensor* t = tensor(obj);
     if (!t) {
         PyObject* s = PyObject_GetAttrString(obj, "shape");       // AttributeError for what has none
@@ -54,15 +57,18 @@ at::IntArrayRef shape(PyObject* obj, int n) {
         throw Failed();
     }
     const int64_t d = t->dim();
-    if (d < n)
-        PyErr_Format(PyExc_ValueError, "not enough values to unpack (expected %d, got %lld)", n, (long long)d);
-    if (d > n) PyErr_Format(PyExc_ValueError, "too many values to unpack (expected %d)", n);
-    if (d != n) throw Failed();
-    return t->sizes();
+    if (d < N)
+        PyErr_Format(PyExc_ValueError, "not enough values to unpack (expected %d, got %lld)", N, (long long)d);
+    if (d > N) PyErr_Format(PyExc_ValueError, "too many values to unpack (expected %d)", N);
+    if (d != N) throw Failed();
+    const at::IntArrayRef now = t->sizes();
+    std::array<int32_t, N> sizes;
+    for (int i = 0; i < N; ++i) sizes[i] = static_cast<int32_t>(now[i]);
+    return sizes;
 }
 int64_t rows(PyObject* obj) {
     const at::Tensor* t = tensor(obj);
-    if (!t) shape(obj, 1);
+    if (!t) shape<1>(obj);
     if (t->dim() == 0) {
         PyErr_SetString(PyExc_IndexError, "tuple index out of range");
         throw Failed();
@@ -115,7 +121,7 @@ template <class F> int unlocked(F call) {
 // decode(q, k, v, g, beta, state_pool, slot_idx, o, scale, dev_status)
 PyObject* decode(PyObject*, PyObject* const* a, Py_ssize_t n) {
     return guarded(n, 10, [&] {
-        const auto qs = shape(a[0], 3), vs = shape(a[2], 3);
+        const auto qs = shape<3>(a[0]), vs = shape<3>(a[2]);
         const void *q = bf16(a[0], "q"), *k = bf16(a[1], "k"), *v = bf16(a[2], "v");
         const float *g = f32(a[3], "g"), *beta = f32(a[4], "beta");
         float* pool = f32(a[5], "state_pool");
@@ -135,7 +141,7 @@ PyObject* decode(PyObject*, PyObject* const* a, Py_ssize_t n) {
 // decode_multi(q, k, v, g, beta, state_pool, slot_idx, o, scale, state_layout, dev_status)
 PyObject* decode_multi(PyObject*, PyObject* const* a, Py_ssize_t n) {
     return guarded(n, 11, [&] {
-        const auto qs = shape(a[0], 4), vs = shape(a[2], 4);
+        const auto qs = shape<4>(a[0]), vs = shape<4>(a[2]);
         const void *q = bf16(a[0], "q"), *k = bf16(a[1], "k"), *v = bf16(a[2], "v");
         const float *g = f32(a[3], "g"), *beta = f32(a[4], "beta");
         float* pool = f32(a[5], "state_pool");
@@ -156,7 +162,7 @@ PyObject* decode_multi(PyObject*, PyObject* const* a, Py_ssize_t n) {
 // gate(a, b, A_log, dt_bias, g, beta)
 PyObject* gate(PyObject*, PyObject* const* x, Py_ssize_t n) {
     return guarded(n, 6, [&] {
-        const auto s = shape(x[0], 2);
+        const auto s = shape<2>(x[0]);
         const void *a = bf16(x[0], "a"), *b = bf16(x[1], "b");
         const float *A_log = f32(x[2], "A_log"), *dt_bias = f32(x[3], "dt_bias");
         float *g = f32(x[4], "g"), *beta = f32(x[5], "beta");
@@ -171,7 +177,7 @@ PyObject* prefill(PyObject*, PyObject* const* args, Py_ssize_t n) {
     return guarded(n, 17, [&] {
         const int32_t route = as_int(args[0]);
         PyObject* const* a = args + 1;
-        const auto qs = shape(a[0], 3), vs = shape(a[2], 3);
+        const auto qs = shape<3>(a[0]), vs = shape<3>(a[2]);
         const int32_t N = static_cast<int32_t>(rows(a[5])) - 1;
         const int32_t split = route == GDN_ROUTE_OVERLAP ? as_int(a[15]) : 0;
         const void *q = bf16(a[0], "q"), *k = bf16(a[1], "k"), *v = bf16(a[2], "v");
