@@ -37,7 +37,12 @@ if not os.path.exists(LIB_PATH):
         "(nvcc, sm_100a). There is no CPU or PyTorch fallback for the gated delta rule kernels.")
 
 _lib = ctypes.CDLL(LIB_PATH)
-from . import _binding  # noqa: E402  (after torch and the library it links against)
+try:
+    from . import _binding  # noqa: E402  (after torch and the library it links against)
+except ImportError as e:
+    raise ImportError(
+        f"the binding's native module cannot be loaded ({e}): build it with "
+        "`python -m paper_2607_17979_b200.build`, for the torch that is installed now.") from e
 _P, _I, _F, _Z = ctypes.c_void_p, ctypes.c_int32, ctypes.c_float, ctypes.c_size_t
 _lib.gdn_prefill_workspace_bytes.restype = _Z
 _lib.gdn_state_transpose.restype = ctypes.c_int

@@ -216,8 +216,19 @@ PyMethodDef methods[] = {
     {"prefill", GDN_FASTCALL(prefill), "gdn_prefill and its routes"},
     {nullptr, nullptr, 0, nullptr},
 };
+#ifndef GDN_BINDING_KEY
+#define GDN_BINDING_KEY ""
+#endif
 PyModuleDef module = {PyModuleDef_HEAD_INIT, "_binding", nullptr, -1, methods, nullptr, nullptr, nullptr, nullptr};
 
 }  // namespace
 
-PyMODINIT_FUNC PyInit__binding(void) { return PyModule_Create(&module); }
+PyMODINIT_FUNC PyInit__binding(void) {
+    PyObject* m = PyModule_Create(&module);
+    // what it was built for, which build.py also looks for in the file
+    if (m && PyModule_AddStringConstant(m, "built_for", GDN_BINDING_KEY) < 0) {
+        Py_DECREF(m);
+        return nullptr;
+    }
+    return m;
+}

@@ -34,6 +34,20 @@ def is_stale() -> bool:
     return _newer(LIB, sources() + glob.glob(os.path.join(CSRC, "*.cuh")) + _headers())
 
 
+def binding_key() -> str:
+    """What the binding is compiled against besides its sources.  It goes into the module as a string, so that one
+    built for another torch is found stale however old or new its file is."""
+    import torch
+    return f"gdn-binding-key:torch-{torch.__version__}-{torch.version.git_version}:abi-{int(torch._C._GLIBCXX_USE_CXX11_ABI)};"
+
+
+def binding_is_stale() -> bool:
+    if _newer(BINDING, [BINDING_SRC, *_headers()]):
+        return True
+    with open(BINDING, "rb") as f:
+        return binding_key().encode() not in f.read()
+
+
 def _build_binding() -> None:
     """The extension module links against the library next to it and against the torch libraries
     that `import torch` has loaded."""
@@ -41,7 +55,8 @@ def _build_binding() -> None:
     root = os.path.dirname(torch.__file__)
     cuda = os.environ.get("CUDA_HOME", "/usr/local/cuda")
     tmp = BINDING + f".tmp{os.getpid()}"
-    cmd = [os.environ.get("CXX", "g++")] + CXX_FLAGS + [f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}"]
+    cmd = [os.environ.get("CXX", "g++")] + CXX_FLAGS + [f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}",
+                                                              f'-DGDN_BINDING_KEY="{binding_key()}"']
     for inc in (os.path.join(root, "include"), os.path.join(root, "include", "torch", "csrc", "api", "include"),
                 sysconfig.get_paths()["include"], os.path.join(cuda, "include")):
         cmd += ["-isystem", inc]
@@ -58,7 +73,7 @@ def build(force: bool = False, verbose: bool = False) -> str:
         cmd = [nvcc] + NVCC_FLAGS + (["-Xptxas", "-v"] if verbose else []) + sources() + ["-o", tmp]
         subprocess.check_call(cmd)
         os.replace(tmp, LIB)
-    if force or _newer(BINDING, [BINDING_SRC, *_headers()]):
+    if force or binding_is_stale():
         _build_binding()
     return LIB
 
