@@ -270,34 +270,41 @@ int gdn_prefill_route(int32_t T, int32_t N, int32_t max_seqlen_hint, int32_t Hv,
     // 16.3; five blocks are level).  With more units than half the SMs a block takes longer: 4 x 30
     // tokens (128 units) 18.7 against 18.5.
     if (units <= sm_count / 2 && longest <= GDN_BLOCKS_MAX_SEQLEN) return GDN_ROUTE_BLOCKS;
-    // Few (sequence, v-head) units and long sequences: the serial state pass would occupy only a
-    // few SMs while the rest idle, so run it next to the record producers in one cooperative launch.
-    // That launch starts ~10 us later (two table launches, one CTA per SM) and gains what the
-    // intra-chunk kernel would have taken alone, which grows with the units, until at about a
-    // quarter of the SMs the producing CTAs no longer keep up with the chains.  The lengths at which three
-    // launches are level with it on 148 SMs: 38 chunks at 8 units, 29 at 16, 24 at 32, 27 at 36, 31 at
-    // 40, 55 at 44, none at 48 (8 units, 1536 tokens 53.3 us in three launches, 56.8 in one; 48 units,
-    // 2048 tokens 98.8 and 110).  With the longest length known, the two-part route below is ahead from 40
-    // units on (48 units, 3400 tokens 132 us against 165); from 64 chunks on the answer of
-    // gdn_prefill_route is kept as it has been.
-    const int32_t u = static_cast<int32_t>(std::min<long long>(units, sm_count));
-    const int32_t level = std::max({16, 3 * sm_count / 10 - u, 16 + 2 * (u - sm_count * 9 / 40)});
+    // Few (sequence, v-head) units and long sequences: the serial state pass would occupy only a few SMs
+    // while the rest idle, so run it next to the record producers: in one cooperative launch, or
+    // in two parts.  What decides is the longest chain and how many chains are alive beside it on average
+    // (equal sequences: all units).  Without a hint the longest of several sequences is taken to hold
+    // half of the tokens.
+    const bool known = max_seqlen_hint > 0 || N == 1;
+    const int32_t chain = known ? longest : std::max(T / 2, 1);
+    const int32_t live =
+        static_cast<int32_t>(std::min(std::min(units, static_cast<long long>(T) * Hv / chain), static_cast<long long>(sm_count)));
+    // The cooperative launch starts ~10 us later (two table launches, one CTA per SM) and gains what the
+    // intra-chunk kernel would have taken alone, which grows with the chains, until at a quarter
+    // of the SMs the producing CTAs no longer keep up with them.  Chunks at which three launches are level
+    // with it on 148 SMs, measured / by the rule: 4 chains 45 / 41, 8 38 / 38, 12 33 / 35, 16 30 / 32, 20
+    // 28 / 29, 24 26 / 26, 28 22 / 23, 32 23 / 23, 36 26 / 25, 40 29 / 30, 44 49 / 50, 48 none / none.  Either
+    // side of a line: 32 chains of 18 chunks 51.8 us in three launches, 56.7 in one; 30 chunks 80.0 and
+    // 74.6.
+    const int32_t level = std::max({23, 3 * sm_count / 10 - 3 * live / 4, 23 + 6 * (live - sm_count * 9 / 40) / 7,
+                                    30 + 5 * (live - sm_count * 11 / 40)});
+    // Two parts: long chains that leave at least half of the SMs free from the start, the length known
+    // through the caller's hint (two chains of 32 chunks at 32 heads were 4 % slower than three launches,
+    // hence 40).  That route wants two launches to run side by side, which the device does but CUDA
+    // does not promise; if they do not, its last launch finishes the work (same results,
+    // milliseconds lost), so choosing it is safe.  Batches that fill the machine at first and free it as their short
+    // chains end would gain 5-12 %, but the records produced late are still dirty in L2 when the call
+    // ends and their write-back falls into whatever runs next, and batches of equal chains lose up
+    // to 7 %: those stay with the persistent pass.
     const bool two_part = max_seqlen_hint > 0 && units <= sm_count / 2 && longest >= 40 * gdn::kChunk;
-    if (cooperative_launch && units <= sm_count / 3 && longest > level * gdn::kChunk &&
-        !(two_part && units > sm_count / 4 && longest < 64 * gdn::kChunk))
+    // Between the two: up to a quarter of the SMs alive the cooperative launch is ahead (36 chains of 90 chunks 185
+    // us, in two parts 188; 6 sequences of 60 chunks and less at 8 heads, 19 alive, 121 and 131), beyond it
+    // the two parts are (40 chains of 70 chunks 167 and 155, 48 of 64 192 and 151).
+    const bool few = cooperative_launch && units <= sm_count / 3;
+    if (few && chain > level * gdn::kChunk &&
+        (live <= sm_count / 4 || (units <= 3 * sm_count / 10 && !two_part)))
         return GDN_ROUTE_FUSED;
-    // More units than the cooperative launch takes but at most half as many as SMs, with long
-    // chains (known only through the caller's hint): the state pass leaves half the machine free
-    // from the start, so part of the records is produced beside it (two sequences of 4096 tokens
-    // at 32 heads 261 -> 238 us, 4096 + 2048 230 -> 198 us, 8192 + 1024 382 -> 303 us; two chains of
-    // 32 chunks were 4 % slower, hence 40).  That route wants two launches to run side by side,
-    // which the device does but CUDA does not promise; if they do not, its last launch finishes
-    // the work (same results, milliseconds lost), so choosing it is safe.  Below a third of the
-    // SMs the cooperative launch is level with it or ahead; batches that fill the machine at
-    // first and free it as their short chains end would gain 5-12 %, but the records produced late
-    // are still dirty in L2 when the call ends and their write-back falls into whatever runs
-    // next, and batches of equal chains lose up to 7 %: those stay with the persistent pass.
-    if (two_part) return GDN_ROUTE_OVERLAP;
+    if (two_part && !(few && live <= sm_count / 4)) return GDN_ROUTE_OVERLAP;
     // Everything else: the three launches (table kernel, or none for small batches; the intra-chunk
     // kernel over all items; the persistent state pass).
     return GDN_ROUTE_STREAM;

@@ -116,11 +116,11 @@ def f32(*shape):
 @pytest.mark.parametrize("name", ["decode", "decode_multi", "gate", "prefill", "prefill_overlap"])
 def test_sizes_are_those_at_the_time_of_the_call(recorder, name):
     if name == "decode":
-        args = (bf16(3, 2, 128), bf16(3, 2, 128), bf16(3, 4, 128), f32(3, 4), f32(3, 4), f32(5, 4, 128, 128), None,
+        args = (bf16(3, 2, 128), bf16(3, 2, 128), bf16(3, 4, 128), f32(3, 4), f32(3, 4), f32(5, 4, 1, 1), None,
                 bf16(3, 4, 128), 1.0, None)
         want = [3, 2, 4, 128, 128, 5]
     elif name == "decode_multi":
-        args = (bf16(3, 7, 2, 128), bf16(3, 7, 2, 128), bf16(3, 7, 4, 128), f32(3, 7, 4), f32(3, 7, 4), f32(5, 4, 128, 128), None,
+        args = (bf16(3, 7, 2, 128), bf16(3, 7, 2, 128), bf16(3, 7, 4, 128), f32(3, 7, 4), f32(3, 7, 4), f32(5, 4, 1, 1), None,
                 bf16(3, 7, 4, 128), 1.0, 0, None)
         want = [3, 7, 2, 4, 128, 128, 5]
     elif name == "gate":
@@ -128,7 +128,7 @@ def test_sizes_are_those_at_the_time_of_the_call(recorder, name):
         want = [9, 4]
     else:
         args = (5 if name == "prefill_overlap" else 0, bf16(9, 2, 128), bf16(9, 2, 128), bf16(9, 4, 128), f32(9, 4), f32(9, 4),
-                torch.zeros(3, dtype=torch.int32), None, f32(2, 4, 128, 128), None, bf16(9, 4, 128), 1.0,
+                torch.zeros(3, dtype=torch.int32), None, f32(2, 4, 1, 1), None, bf16(9, 4, 128), 1.0,
                 torch.zeros(64, dtype=torch.uint8), 0, 64, None, -1)
         want, name = [9, 2, 2, 4, 128, 128, 2], "prefill"
     assert recorder(name, args, want) == want

@@ -111,8 +111,8 @@ def test_prefill_routing_rules_are_pure_host_arithmetic():
     assert r(10, 1, 5000, 32) == "recurrent"
     # few long units: one cooperative launch, if the device can
     assert r(32768, 1, 0, 32) == "fused" and r(32768, 1, 0, 32, 148, False) == "stream"
-    assert r(1025, 1, 0, 32) == "fused" and r(1024, 1, 0, 32) == "stream"
-    assert r(32768, 1, 0, 49) == "fused" and r(32768, 1, 0, 50) == "stream"       # 148 // 3 = 49 units
+    assert r(1473, 1, 0, 32) == "fused" and r(1472, 1, 0, 32) == "stream"
+    assert r(32768, 1, 0, 44) == "fused" and r(32768, 1, 0, 45) == "stream"       # 3 * 148 // 10 = 44 units
     # everything else that is chunked: the three launches with the persistent state pass
     assert r(7680, 4, 0, 32) == "stream" and r(129, 1, 0, 32) == "stream"
     assert r(128, 1, 0, 32) == "stream" and r(400, 4, 100, 32) == "stream"
@@ -124,7 +124,8 @@ def test_prefill_routing_rules_are_pure_host_arithmetic():
     assert r(8192, 2, 4096, 32) == "overlap" and r(4000, 2, 3000, 32) == "overlap"
     assert r(8192, 2, 0, 32) == "stream" and r(5118, 2, 2559, 32) == "stream"
     assert r(8192, 2, 4096, 37) == "overlap" and r(8192, 2, 4096, 38) == "stream"   # 74 / 76 units
-    assert r(8192, 2, 4096, 24) == "fused" and r(8192, 2, 4096, 25) == "overlap"    # 48 / 50 units
+    assert r(8192, 2, 4096, 18) == "fused" and r(8192, 2, 4096, 19) == "overlap"    # 36 / 38 units
+    assert r(8192, 2, 6144, 24) == "fused" and r(8192, 2, 6144, 25) == "overlap"    # 32 chains alive of 48 / 50
     assert r(7680, 4, 4096, 32) == "stream" and r(6144, 3, 2048, 32) == "stream"
     # the thresholds follow the SM count given
     assert r(1184, 37, 32, 4, 100) == "stream"
