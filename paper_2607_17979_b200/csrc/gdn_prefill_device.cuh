@@ -320,6 +320,7 @@ __device__ __forceinline__ bool intra_item(const TensorMaps& maps, const Prefill
     auto bail = [&](bool stores_pending) {
         if (tid == 0) {
             report(p.dev_status, kDevTimeout);
+            mbar_wait(&st.bar_tma, par1, 1u << 12);
             if (v_started) mbar_wait(&st.bar_v, par1, 1u << 12);
             if (stores_pending) bulk_wait_read_all();
         }

@@ -91,3 +91,13 @@ def test_issuing_warps_wait_as_one():
     item = item[item.index("bool intra_item("):]
     for section in (issuer, item):
         assert not re.search(r"(?<!warp_)wait_or_abort[<(]", section)
+
+
+def test_an_item_that_gives_up_waits_for_all_its_copies():
+    """Every barrier on which the intra-chunk item's copies land is waited for (bounded) on the way out."""
+    item = open(os.path.join(CSRC, "gdn_prefill_device.cuh")).read()
+    item = item[item.index("bool intra_item("):]
+    armed = set(re.findall(r"mbar_expect_tx\(&st\.(\w+)", item))
+    bail = item[item.index("auto bail ="):]
+    bail = bail[:bail.index("};")]
+    assert armed == {"bar_tma", "bar_v"} and armed == set(re.findall(r"mbar_wait\(&st\.(\w+)", bail))
