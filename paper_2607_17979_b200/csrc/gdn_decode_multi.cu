@@ -82,10 +82,10 @@ cudaError_t launch_decode_multi(const DecodeMultiParams& mp, cudaStream_t stream
     const int sms = device_info(&di) == cudaSuccess ? di.sms : 148;
     // Four CTAs of two warps per tile, or two of four, with 16 warps an SM either way.  Up to four tokens
     // a CTA lives little longer than its tile's loads and more, smaller CTAs overlap better; beyond,
-    // what every CTA does for its tokens counts.  B = 64, 32 v-heads, two / four warps, us: L = 2 42.3 /
-    // 43.3, L = 4 43.6 / 44.7, L = 8 55.1 / 52.5, L = 16 87.0 / 74.3; tiles [dk][dv] L = 2 45.4 / 47.2,
-    // L = 8 56.8 / 57.6, L = 16 98.9 / 84.3.  With too few tiles to fill the SMs, two: B = 1, L = 8, 8
-    // v-heads 3.7 / 4.0.
+    // what every CTA does for its tokens counts.  B = 64, 32 v-heads, two / four warps, us: L = 2 43.0 /
+    // 43.8, L = 4 44.8 / 45.5, L = 8 55.7 / 53.8, L = 16 86.5 / 74.0; tiles [dk][dv] L = 2 46.3 / 47.9,
+    // L = 8 58.7 / 59.0, L = 16 99.2 / 82.1.  With too few tiles to fill the SMs, two: B = 1, L = 8, 8
+    // v-heads 4.0 / 4.3.
     const bool two = mp.L <= 4 || (mp.L <= 8 && (mp.layout != 0 || units * 4 <= 2LL * sms));
     if (mp.layout == 0) return two ? launch_shape<false, 2>(mp, stream) : launch_shape<false, 4>(mp, stream);
     return two ? launch_shape<true, 2>(mp, stream) : launch_shape<true, 4>(mp, stream);

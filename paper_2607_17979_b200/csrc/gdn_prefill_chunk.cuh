@@ -13,10 +13,10 @@
 // Three launches: a prep kernel builds the chunk table from cu_seqlens; the
 // intra-chunk kernel (one CTA per chunk and v-head, all chunks in parallel)
 // computes W, U~, P and b with tcgen05 GEMMs and an fp32 triangular solve and
-// writes them as a record; the state-pass kernel (one CTA per sequence and
-// v-head, or one persistent CTA per SM walking a list of them) walks the chunks
-// in order carrying S in fp32 registers.  A fused variant runs the last two as
-// one cooperative launch.
+// writes them as a record; the state pass (one persistent CTA per SM that takes
+// sequence after sequence of a v-head from a list) walks the chunks in order
+// carrying S in fp32 registers.  A fused variant runs the last two as one
+// cooperative launch, another produces part of the records beside the state pass.
 #pragma once
 #include "gdn_common.cuh"
 #include <cuda.h>
@@ -68,8 +68,8 @@ struct ChunkInfo {      // 16 bytes
 //                                sequence has zero chunks and seq_bad[n] = 1
 //   seq_bad[N]                   int32
 //   chunks[max_chunks]           ChunkInfo
-//   -- used by the fused single-launch path only --
 //   seq_by_rank[N]               int32: sequences sorted by chunk count, longest first
+//   -- used by the cooperative launch and the two-part route only --
 //   rank_of[N]                   int32: the inverse (rank of each sequence)
 //   order[max_chunks]            int32: chunk ids in processing order: by position inside the
 //                                sequence first, by sequence rank second (so that the records
@@ -78,7 +78,7 @@ struct ChunkInfo {      // 16 bytes
 //   flags[max_chunks][Hv]        uint32: 1 once the record is complete and visible
 //   done[N][Hv]                  int32: 1 once the two-part route's state pass has finished the unit
 //                                (rank-major, like the unit list); the rest is left to a last launch
-//   -- both paths --
+//   -- every route --
 //   records[max_chunks][Hv]      kRecBytes each
 struct WorkspaceLayout {
     size_t seq_first, seq_bad, chunks, seq_by_rank, rank_of, order, hist, fill, cnt, pos, flags,
@@ -123,8 +123,8 @@ struct ChunkedParams {
 cudaError_t launch_prefill_chunked(const ChunkedParams& cp, cudaStream_t stream);
 // One cooperative launch: some CTAs produce the records, the others run the state pass behind them.
 cudaError_t launch_prefill_fused(const ChunkedParams& cp, cudaStream_t stream);
-// Three launches with a persistent state pass: CTAs walk lists of (sequence, v-head) units and
-// stream their records without draining between units (for batches with many more units than SMs).
+// Three launches (for small batches two: no table-building one): CTAs of the state pass walk lists of
+// (sequence, v-head) units and stream their records without draining between units.
 cudaError_t launch_prefill_stream(const ChunkedParams& cp, cudaStream_t stream);
 // Pieces shared by the launchers: the prep kernel that also ranks the sequences by chunk count
 // (longest first) and, for the fused launch, orders the chunks and clears the queues and flags;

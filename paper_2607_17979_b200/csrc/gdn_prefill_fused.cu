@@ -2,7 +2,7 @@
 //
 // The grid has one CTA of 512 threads per SM.  The first `n_state` CTAs run the serial state pass
 // (the role of the persistent state pass, gdn_prefill_stream.cuh: 8 chain warps, 4 output warps, an
-// issuing warp and a loading warp), CTA b over the units b, b + n_state, ... of the list that has
+// issuing warp and 3 loading warps), CTA b over the units b, b + n_state, ... of the list that has
 // the longest sequences first.  The other CTAs run two independent groups of 256 threads that pull
 // (chunk, v-head) items from a queue and write their records (the intra-chunk routine of
 // gdn_prefill_device.cuh), in the order the state pass consumes them: by position inside the
@@ -344,8 +344,8 @@ __device__ __forceinline__ void fused_intra_role(const TensorMaps& maps, const P
 
 // ---------------------------------------------------------------------------------------------
 // The kernel: 512 threads per CTA (128 registers).  State CTA b runs the persistent state pass's
-// role over the units b, b + n_state, ... of the rank-sorted list, its loading warp waiting for
-// each record's flag; the other CTAs run two producer groups.
+// role over the units b, b + n_state, ... of the rank-sorted list, its loading warps waiting
+// for each record's flag; the other CTAs run two producer groups.
 // ---------------------------------------------------------------------------------------------
 __global__ void __launch_bounds__(kFusedThreads, 1)
 prefill_fused_kernel(const __grid_constant__ TensorMaps maps, const PrefillParams p, uint8_t* ws,

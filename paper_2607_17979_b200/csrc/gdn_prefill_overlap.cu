@@ -6,7 +6,7 @@
 // which the chains consume the records (by position inside the sequence first): the first part
 // runs alone, then the state pass starts, one CTA per unit, and the second part runs beside it on
 // the SMs that have no live chain, each record published through a flag (release) that the state
-// pass's loading warp waits for (acquire, bounded).
+// pass's loading warps wait for (acquire, bounded).
 //
 // Five launches in one stream, the first four each a programmatic dependent of the one before:
 //   prep          chunk table, ranking, processing order, cleared flags and done table, the cut
@@ -213,8 +213,8 @@ cudaError_t launch_prefill_overlap(const ChunkedParams& cp, cudaStream_t stream,
     // The state pass waits for a launch that comes after it in the stream: the two must be able to
     // run at the same time.  Where launches are known to be serialised, produce everything first
     // (then no record is waited for).  A profiler that replays kernels one at a time cannot be
-    // seen from here: under it the waits run out (GDN_DEV_TIMEOUT, no hang); profile
-    // gdn_prefill_stream instead, which runs the same kernels' arithmetic.
+    // seen from here: under it the waits run out after milliseconds and the last launch does the work;
+    // profile gdn_prefill_stream instead, which runs the same kernels' arithmetic.
     const char* blocking = std::getenv("CUDA_LAUNCH_BLOCKING");
     if (blocking && blocking[0] != '\0' && blocking[0] != '0') split_permille = 1000;
     if (split_permille > 1000) split_permille = 1000;

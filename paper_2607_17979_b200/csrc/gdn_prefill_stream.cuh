@@ -4,9 +4,9 @@
 // intra-chunk kernel (one CTA per SM), and the state CTAs of the fused cooperative launch, whose
 // records are produced by other CTAs while the pass runs.
 //
-// The one-CTA-per-unit state kernel pays, for every unit, a launch slot, barrier and TMEM set-up,
-// the first record's memory latency and the tail of its last chunk; with thousands of short
-// units (many short sequences) that overhead is longer than the chunk steps themselves.  Here
+// One CTA per unit would pay, for every unit, a launch slot, barrier and TMEM set-up, the first
+// record's memory latency and the tail of its last chunk; with thousands of short units (many
+// short sequences) that overhead is longer than the chunk steps themselves.  Here
 //   * warps 13-15 (loaders) copy records and K tiles in unit order, running up to two chunks ahead
 //     of the consumers and straight across unit boundaries (in the fused launch they first wait for
 //     each record's flag); a stage is released in three parts and each warp refills one, so that no
@@ -29,7 +29,7 @@
 // left unconsumed.
 //
 // The fp32 master state lives in the chain threads' registers (64 per thread; TMEM lane = state
-// row, two column halves), as in the one-CTA-per-unit state kernel.
+// row, two column halves).
 #pragma once
 #include "gdn_prefill_device.cuh"
 
@@ -95,8 +95,8 @@ __device__ __forceinline__ void fence_proxy_async_all() {
 
 // The state pass of one CTA of 512 threads over the units cta, cta + n_ctas, ... of the rank-sorted
 // list.  kGated = 0: every record exists (the intra-chunk kernel ran before).  kGated = 1:
-// records are being produced by other CTAs of the same cooperative launch and the loading warp
-// waits for each record's flag first.  kGated = 2: the records of the first hdr[kHdrSplit] items of
+// records are being produced by other CTAs of the same cooperative launch and the loading warps
+// wait for each record's flag first.  kGated = 2: the records of the first hdr[kHdrSplit] items of
 // the processing order exist, the others are being produced by a concurrent kernel and are waited
 // for; a wait that runs out ends the CTA's work without an error (the units it has finished are
 // marked in the done table, the others are left to a later launch).  kGated = 3: that later launch:
