@@ -208,8 +208,9 @@ int gdn_prefill(const void* q, const void* k, const void* v,
  * (GDN_ROUTE_BLOCKS: the same kernel with the next block's tokens staged beside
  * the current block); anything longer to one of the chunked variants (gdn_prefill_fused for a few long sequence-heads,
  * gdn_prefill_overlap when max_seqlen_hint tells of chains of at least 40
- * chunks, the sequence-heads number at most half of the SMs and more than a
- * quarter of the SMs' worth of them is alive beside the longest on average,
+ * chunks and the sequence-heads number at most half of the SMs, unless they
+ * are at most a third and at most a quarter of the SMs' worth of them is alive
+ * beside the longest on average,
  * gdn_prefill_stream for everything else).  Each route can also be called
  * directly; arguments are gdn_prefill's.  gdn_prefill_chunked is the three
  * launches under their older name: it runs gdn_prefill_stream.
