@@ -206,15 +206,20 @@ int gdn_prefill(const void* q, const void* k, const void* v,
  * bound T) goes to gdn_prefill_recurrent's kernel (GDN_ROUTE_RECURRENT), and
  * so do a few sequence-heads of up to GDN_BLOCKS_MAX_SEQLEN tokens
  * (GDN_ROUTE_BLOCKS: the same kernel with the next block's tokens staged beside
- * the current block); anything longer to one of the chunked variants (gdn_prefill_fused for a few long sequence-heads,
- * gdn_prefill_overlap when max_seqlen_hint tells of chains of at least 40
- * chunks and the sequence-heads number at most half of the SMs, unless they
- * are at most a third and at most a quarter of the SMs' worth of them is alive
- * beside the longest on average,
- * gdn_prefill_stream for everything else).  Each route can also be called
+ * the current block).  Anything longer is a matter of chunks.  GDN_ROUTE_FUSED
+ * (a few long sequence-heads) and GDN_ROUTE_OVERLAP (max_seqlen_hint tells of
+ * chains of at least 40 chunks and the sequence-heads number at most half of
+ * the SMs, unless they are at most a third and at most a quarter of the SMs'
+ * worth of them is alive beside the longest on average) name batches whose
+ * serial chains leave most of the machine idle: gdn_prefill runs those as
+ * gdn_prefill_overlap does where producing the records beside the chains pays
+ * for its two launches more, else as gdn_prefill_stream does;
+ * gdn_prefill_fused's cooperative launch is slower on every shape and
+ * runs where it is called by name.  GDN_ROUTE_STREAM, everything else, is
+ * gdn_prefill_stream.  Each entry point can also be called
  * directly; arguments are gdn_prefill's.  gdn_prefill_chunked is the three
  * launches under their older name: it runs gdn_prefill_stream.
- * gdn_prefill_route answers which one gdn_prefill would take (host-only
+ * gdn_prefill_route answers which of these a batch is (host-only
  * arithmetic on the shapes; sm_count and cooperative_launch describe the
  * device, gdn_prefill itself queries them): one of GDN_ROUTE_* (never
  * GDN_ROUTE_CHUNKED any more), or GDN_ROUTE_NONE for an empty batch.
@@ -260,7 +265,10 @@ int gdn_prefill_fused(const void* q, const void* k, const void* v,
  * gdn_prefill_stream - the chunked algorithm in three launches whose state
  * pass is a persistent kernel: one CTA per SM walks a list of (sequence,
  * v-head) units and streams their chunks without draining its pipeline
- * between units.  Arguments, workspace and results are gdn_prefill_chunked's.
+ * between units.  Where the longest chain decides the time a unit is
+ * shared by two CTAs, half of the state's rows each: with at most half as many
+ * units as SMs, or when max_seqlen_hint tells of a chain that long (the two
+ * forms agree to the rounding of fp32 sums).  Arguments, workspace and results are gdn_prefill_chunked's.
  */
 int gdn_prefill_stream(const void* q, const void* k, const void* v,
                        const float* g, const float* beta, const int32_t* cu_seqlens,
@@ -285,8 +293,8 @@ int gdn_prefill_stream(const void* q, const void* k, const void* v,
  *   split_permille  share of the (chunk, v-head) items, in the order the
  *                   chains consume them, produced before the state pass
  *                   starts: 0..1000, or negative = chosen on the device from
- *                   the sequence lengths.  With more units than the GPU has
- *                   SMs to spare everything is produced first (1000).
+ *                   the sequence lengths.  With more half units than the
+ *                   GPU has SMs to spare this is gdn_prefill_stream.
  *                   -2 = as negative, but the producers of the second part
  *                   are launched as an ordinary successor of the state pass
  *                   (serialised on purpose: the recovery path, for tests).
@@ -295,11 +303,11 @@ int gdn_prefill_stream(const void* q, const void* k, const void* v,
  * at the same time, which programmatic dependent launch makes the device do
  * but which CUDA does not promise (and a tool that replays kernels one at a
  * time prevents).  If it does not happen the waits for records run out after
- * a few milliseconds, the state pass marks the (sequence, v-head) units it
+ * a few milliseconds, the state pass marks the half (sequence, v-head) units it
  * has finished and the last launch runs the others once the records exist:
  * the results are the same, only time is lost (so profile gdn_prefill_stream
- * instead under such a tool).  With CUDA_LAUNCH_BLOCKING set everything is
- * produced first.
+ * instead under such a tool).  With CUDA_LAUNCH_BLOCKING set this is
+ * gdn_prefill_stream.
  */
 int gdn_prefill_overlap(const void* q, const void* k, const void* v,
                         const float* g, const float* beta, const int32_t* cu_seqlens,

@@ -177,7 +177,7 @@ enum PrefillRoute { kRouteChunked, kRouteFused, kRouteStream, kRouteOverlap };
 int prefill_chunked_impl(PrefillRoute route, const void* q, const void* k, const void* v, const float* g,
                          const float* beta, const int32_t* cu_seqlens, const float* init_state,
                          float* final_state, const int32_t* slot_idx, void* o, int32_t T, int32_t N,
-                         int32_t Hqk, int32_t Hv, int32_t dk, int32_t dv, int32_t chunk,
+                         int32_t max_seqlen_hint, int32_t Hqk, int32_t Hv, int32_t dk, int32_t dv, int32_t chunk,
                          int32_t num_slots, float scale, void* workspace, size_t workspace_bytes,
                          int32_t* dev_status, void* stream, int32_t split_permille = -1) {
     if (chunk != gdn::kChunk) return GDN_ERR_SHAPE;
@@ -200,6 +200,7 @@ int prefill_chunked_impl(PrefillRoute route, const void* q, const void* k, const
     p.dev_status = dev_status;
     cp.ws = static_cast<uint8_t*>(workspace);
     cp.lay = gdn::workspace_layout(T, N, Hv);
+    cp.longest = max_seqlen_hint > 0 ? std::min(max_seqlen_hint, T) : N == 1 ? T : 0;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     return cuda_status(route == kRouteFused     ? gdn::launch_prefill_fused(cp, st)
                        : route == kRouteStream  ? gdn::launch_prefill_stream(cp, st)
@@ -214,9 +215,8 @@ int gdn_prefill_chunked(const void* q, const void* k, const void* v, const float
                         int32_t max_seqlen_hint, int32_t Hqk, int32_t Hv, int32_t dk, int32_t dv,
                         int32_t chunk, int32_t num_slots, float scale, void* workspace,
                         size_t workspace_bytes, int32_t* dev_status, void* stream) {
-    (void)max_seqlen_hint;
     return prefill_chunked_impl(kRouteChunked, q, k, v, g, beta, cu_seqlens, init_state, final_state,
-                                slot_idx, o, T, N, Hqk, Hv, dk, dv, chunk, num_slots, scale,
+                                slot_idx, o, T, N, max_seqlen_hint, Hqk, Hv, dk, dv, chunk, num_slots, scale,
                                 workspace, workspace_bytes, dev_status, stream);
 }
 
@@ -226,9 +226,8 @@ int gdn_prefill_fused(const void* q, const void* k, const void* v, const float* 
                       int32_t max_seqlen_hint, int32_t Hqk, int32_t Hv, int32_t dk, int32_t dv,
                       int32_t chunk, int32_t num_slots, float scale, void* workspace,
                       size_t workspace_bytes, int32_t* dev_status, void* stream) {
-    (void)max_seqlen_hint;
     return prefill_chunked_impl(kRouteFused, q, k, v, g, beta, cu_seqlens, init_state, final_state,
-                                slot_idx, o, T, N, Hqk, Hv, dk, dv, chunk, num_slots, scale,
+                                slot_idx, o, T, N, max_seqlen_hint, Hqk, Hv, dk, dv, chunk, num_slots, scale,
                                 workspace, workspace_bytes, dev_status, stream);
 }
 
@@ -238,9 +237,8 @@ int gdn_prefill_stream(const void* q, const void* k, const void* v, const float*
                        int32_t max_seqlen_hint, int32_t Hqk, int32_t Hv, int32_t dk, int32_t dv,
                        int32_t chunk, int32_t num_slots, float scale, void* workspace,
                        size_t workspace_bytes, int32_t* dev_status, void* stream) {
-    (void)max_seqlen_hint;
     return prefill_chunked_impl(kRouteStream, q, k, v, g, beta, cu_seqlens, init_state, final_state,
-                                slot_idx, o, T, N, Hqk, Hv, dk, dv, chunk, num_slots, scale,
+                                slot_idx, o, T, N, max_seqlen_hint, Hqk, Hv, dk, dv, chunk, num_slots, scale,
                                 workspace, workspace_bytes, dev_status, stream);
 }
 
@@ -251,9 +249,8 @@ int gdn_prefill_overlap(const void* q, const void* k, const void* v, const float
                         int32_t chunk, int32_t num_slots, float scale, void* workspace,
                         size_t workspace_bytes, int32_t* dev_status, void* stream,
                         int32_t split_permille) {
-    (void)max_seqlen_hint;
     return prefill_chunked_impl(kRouteOverlap, q, k, v, g, beta, cu_seqlens, init_state, final_state,
-                                slot_idx, o, T, N, Hqk, Hv, dk, dv, chunk, num_slots, scale,
+                                slot_idx, o, T, N, max_seqlen_hint, Hqk, Hv, dk, dv, chunk, num_slots, scale,
                                 workspace, workspace_bytes, dev_status, stream, split_permille);
 }
 
@@ -310,6 +307,24 @@ int gdn_prefill_route(int32_t T, int32_t N, int32_t max_seqlen_hint, int32_t Hv,
     return GDN_ROUTE_STREAM;
 }
 
+namespace {
+// Few long chains (GDN_ROUTE_FUSED, GDN_ROUTE_OVERLAP): whether their records are produced in two parts, the second beside the
+// chains, or all of them first.  The two parts cost 13 us (the tables with the processing order, two more launches)
+// and hide the intra-chunk kernel's time, which grows with the items, as far as the SMs that the chains leave free keep up:
+// two for each live chain are taken.  us in three launches / in two parts, equal chains on 148 SMs: 4 chains of 128
+// chunks 165 / 176; 8 of 80 115 / 121, of 128 176 / 177; 16 of 56 92 / 95, of 80 131 / 121; 24 of 40 76 / 76, of 56 107 / 95; 32 of 32
+// 68 / 70, of 40 86 / 80, of 512 923 / 640; 40 of 32 76 / 77, of 56 123 / 116; 48 of 56 132 / 132, of 128 280 / 261; 64 of 128 324 / 384.  (The
+// cooperative launch: 4 of 56 99 against 77, 8 of 128 204 against 176, 32 of 128 211 against 189.)
+bool two_parts_pay(int32_t T, int32_t N, int32_t max_seqlen_hint, int32_t Hv, int32_t sms) {
+    const long long units = static_cast<long long>(N) * Hv;
+    const int32_t longest = (max_seqlen_hint > 0 && max_seqlen_hint < T) ? max_seqlen_hint : T;
+    const long long chain = max_seqlen_hint > 0 || N == 1 ? longest : std::max(T / 2, 1);      // as in gdn_prefill_route
+    const long long live = std::min(units, static_cast<long long>(T) * Hv / chain);
+    const long long level = 1050 + 150 * std::max(0ll, live - sms / 4);
+    return live <= sms * 7 / 20 && live * chain >= level * gdn::kChunk;
+}
+}  // namespace
+
 int gdn_prefill(const void* q, const void* k, const void* v, const float* g, const float* beta,
                 const int32_t* cu_seqlens, const float* init_state, float* final_state,
                 const int32_t* slot_idx, void* o, int32_t T, int32_t N, int32_t max_seqlen_hint,
@@ -340,12 +355,12 @@ int gdn_prefill(const void* q, const void* k, const void* v, const float* g, con
                                       slot_idx, o, T, N, Hqk, Hv, dk, dv, num_slots, scale, longest,
                                       dev_status, stream);
     }
-    const PrefillRoute route = route_id == GDN_ROUTE_FUSED     ? kRouteFused
-                               : route_id == GDN_ROUTE_STREAM  ? kRouteStream
-                               : route_id == GDN_ROUTE_OVERLAP ? kRouteOverlap
-                                                               : kRouteChunked;
+    const PrefillRoute route = (route_id == GDN_ROUTE_FUSED || route_id == GDN_ROUTE_OVERLAP) &&
+                                       two_parts_pay(T, N, max_seqlen_hint, Hv, sms)
+                                   ? kRouteOverlap
+                                   : kRouteStream;
     return prefill_chunked_impl(route, q, k, v, g, beta, cu_seqlens, init_state,
-                                final_state, slot_idx, o, T, N, Hqk, Hv, dk, dv, chunk, num_slots,
+                                final_state, slot_idx, o, T, N, max_seqlen_hint, Hqk, Hv, dk, dv, chunk, num_slots,
                                 scale, workspace, workspace_bytes, dev_status, stream);
 }
 

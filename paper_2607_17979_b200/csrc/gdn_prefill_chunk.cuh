@@ -29,7 +29,7 @@ namespace gdn {
 //   [16384, 32768)  Qg  = diag(scale e^b) Q as two K-major 128B-swizzled halves [64 tokens][64 dk] bf16:
 //                   in the cooperative launch only
 //   [32768, 40960)  P   as one K-major 128B-swizzled tile   [64 r][64 i]      bf16, scale folded in
-//   [40960, 73728)  U~  as [16 token-groups][128 dv][4 tokens] fp32
+//   [40960, 73728)  U~  as [2 halves of dv][16 token-groups][64 dv][4 tokens] fp32, dv swizzled (rec_u_index)
 //   [73728, 73984)  e^{b_C - b_c} for c = 0..63, fp32 (rows past the chunk's length hold 1)
 //   [73984, 74240)  scale e^{b_r} for r = 0..63, fp32
 //   [74240, 74496)  e^{b_C} in the first float, rest unused
@@ -47,6 +47,10 @@ constexpr uint32_t kRecDecay = 73728;
 constexpr uint32_t kRecEb = 73984;
 constexpr uint32_t kRecGammaC = 74240;
 constexpr uint32_t kRecBytes = 74496;
+constexpr uint32_t kRecUHalf = (kRecDecay - kRecU) / 2;
+// Place (in 16-byte units) of a token group and dv within one half of U~.  Odd groups have their dv swapped in fours, so
+// that a fragment read (four dv of two neighbouring groups per half warp) touches every bank once.
+__device__ __forceinline__ int rec_u_index(int group, int dv) { return group * 64 + (dv ^ ((group & 1) << 2)); }
 
 // Small batches of at most this many sequences need no table-building launch: the intra-chunk
 // kernel finds its chunks from cu_seqlens itself and writes the per-sequence tables for the state pass.
@@ -76,7 +80,7 @@ struct ChunkInfo {      // 16 bytes
 //                                every state-pass unit needs next are produced first)
 //   hist, fill, cnt, pos[max_nc+2]  int32 scratch of the counting sort (max_nc = T/64 + 1)
 //   flags[max_chunks][Hv]        uint32: 1 once the record is complete and visible
-//   done[N][Hv]                  int32: 1 once the two-part route's state pass has finished the unit
+//   done[N][Hv][2]               uint16: 1 once the two-part route's state pass has finished the half unit
 //                                (rank-major, like the unit list); the rest is left to a last launch
 //   -- every route --
 //   records[max_chunks][Hv]      kRecBytes each
@@ -118,6 +122,7 @@ struct ChunkedParams {
     PrefillParams p;
     uint8_t* ws;
     WorkspaceLayout lay;
+    int32_t longest = 0;      // tokens of the longest sequence as far as the caller has told, 0: not known (picks kernels only)
 };
 
 cudaError_t launch_prefill_chunked(const ChunkedParams& cp, cudaStream_t stream);
@@ -133,8 +138,9 @@ cudaError_t launch_prefill_stream(const ChunkedParams& cp, cudaStream_t stream);
 // launch); 2: + the cut of the two-part production (split_permille < 0: the kernel's own model).
 cudaError_t launch_prefill_ranked_prep(const ChunkedParams& cp, cudaStream_t stream, int mode,
                                        int split_permille = -1, int sms = 0);
-// The intra-chunk kernel in two parts around a flag-gated persistent state pass: the second part
-// of the records is produced beside the chains, on the SMs the state pass leaves free.
+// The intra-chunk kernel in two parts around a flag-gated state pass of two CTAs per unit: the second part
+// of the records is produced beside the chains, on the SMs the state pass leaves free.  (The three launches where it
+// leaves too few.)
 cudaError_t launch_prefill_overlap(const ChunkedParams& cp, cudaStream_t stream, int split_permille);
 
 }  // namespace gdn

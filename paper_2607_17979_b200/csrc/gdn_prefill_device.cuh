@@ -245,6 +245,17 @@ __device__ __forceinline__ bool warp_wait_or_abort(uint64_t* bar, uint32_t parit
     return false;
 }
 
+// The same with the first poll in one piece with its vote (it blocks for a while by itself and so is nearly always the last)
+// and the rest out of line.  The roles of a warp-specialised kernel share 32 KB of instruction cache, and past it each
+// runs at the pace of its instruction misses: eight roles of 3 KB a round take 573 cycles, of 4 KB 929; the half-unit state pass
+// had 128 misses a chunk step with its waits in line and unrolled, and has 2.
+static __device__ __noinline__ bool warp_wait_more(uint64_t* bar, uint32_t parity, volatile int* abort_flag, const int reason) {
+    return warp_wait_or_abort(bar, parity, abort_flag, reason);
+}
+__device__ __forceinline__ bool warp_wait(uint64_t* bar, uint32_t parity, volatile int* abort_flag, const int reason = 1) {
+    return mbar_try_wait_all(bar, parity) || warp_wait_more(bar, parity, abort_flag, reason);
+}
+
 // kScaledQ: whether the record carries the scaled Q (gdn_prefill_chunk.cuh).
 // The intra-chunk quantities of one (chunk, v-head) item, computed by a group of 256 threads
 // (tid = 0..255 within the group; its warps must be CTA warps 0-3 mod 4 aligned, because a warp
@@ -548,8 +559,8 @@ __device__ __forceinline__ bool intra_item(const TensorMaps& maps, const Prefill
     warp_wait_or_abort(&st.bar_mma, par3, abortp);
     tc_fence_after_sync();
 
-    {   // U~^T[d][32 tokens] -> record, [token group][dv][4 tokens] fp32
-        float4* urec = reinterpret_cast<float4*>(rec + kRecU);
+    {   // U~^T[d][32 tokens] -> record, [half of dv][token group][dv][4 tokens] fp32
+        float4* urec = reinterpret_cast<float4*>(rec + kRecU + (d >> 6) * kRecUHalf);
 #pragma unroll
         for (int step = 0; step < 2; ++step) {
             const int cbase = colhalf * 32 + step * 16;
@@ -558,7 +569,7 @@ __device__ __forceinline__ bool intra_item(const TensorMaps& maps, const Prefill
             tmem_wait_ld();
 #pragma unroll
             for (int q4 = 0; q4 < 4; ++q4)
-                urec[((cbase >> 2) + q4) * kD + d] =
+                urec[rec_u_index((cbase >> 2) + q4, d & 63)] =
                     make_float4(__uint_as_float(y[4 * q4]), __uint_as_float(y[4 * q4 + 1]),
                                 __uint_as_float(y[4 * q4 + 2]), __uint_as_float(y[4 * q4 + 3]));
         }

@@ -20,7 +20,7 @@ namespace gdn {
 constexpr int kFPrepThreads = 256;
 // model of the two-part production (see the kernel): items per SM and chunk step, start-up lag of
 // the second part in chunk steps, and a safety margin in items
-constexpr int kSplitProdPermille = 600;
+constexpr int kSplitProdPermille = 330;
 constexpr int kSplitLeadSteps = 6;
 constexpr int kSplitMarginItems = 128;
 
@@ -156,11 +156,11 @@ prefill_fused_prep_kernel(const int32_t* __restrict__ cu, int32_t T, int32_t N, 
     // produced before the state pass starts, the others beside it, on the SMs it leaves free.
     // The cut is the smallest head start with which the chains never catch up with the
     // producers, by a simple model: every live (sequence, v-head) unit consumes one item per
-    // chunk step, the SMs without a live unit produce kProdPermille / 1000 items per chunk step
+    // chunk step and holds two SMs, the others produce kProdPermille / 1000 items per chunk step
     // each, and an item started when the state pass starts is ready kLeadSteps chunk steps
     // later.  In step j the chains need the Hv * pos[j + 1] first items of the order; by then the
-    // second part has produced r * sum_{i < j - lead} (sms - Hv * cnt[i]), and that sum is
-    // m * sms - Hv * pos[m] with m = j - lead.
+    // second part has produced r * sum_{i < j - lead} (sms - 2 Hv * cnt[i]), and that sum is
+    // m * sms - 2 Hv * pos[m] with m = j - lead.
     if (for_fused == 2) {
         __shared__ int32_t need_max;
         if (tid == 0) need_max = 0;
@@ -171,7 +171,7 @@ prefill_fused_prep_kernel(const int32_t* __restrict__ cu, int32_t T, int32_t N, 
         for (int j = tid; j < lay.max_nc; j += kFPrepThreads) {
             const int m = j > lead ? j - lead : 0;
             long long produced =
-                (static_cast<long long>(m) * sms - static_cast<long long>(Hv) * pos[m]) * prod / 1000;
+                (static_cast<long long>(m) * sms - 2ll * Hv * pos[m]) * prod / 1000;
             if (produced < 0) produced = 0;
             const long long need = static_cast<long long>(Hv) * pos[j + 1] - produced;
             local = need > local ? need : local;
@@ -365,7 +365,7 @@ prefill_fused_kernel(const __grid_constant__ TensorMaps maps, const PrefillParam
     tc_fence_after_sync();
     const uint32_t tmem = tmem_base_s;
     if (static_cast<int>(blockIdx.x) < n_state) {
-        state_stream_role<1>(maps, p, ws, lay, smem, tmem, blockIdx.x, n_state);
+        state_stream_role<true>(maps, p, ws, lay, smem, tmem, blockIdx.x, n_state);
     } else {
         fused_intra_role(maps, p, ws, lay, smem, intra_statics, tmem);
         tc_fence_before_sync();

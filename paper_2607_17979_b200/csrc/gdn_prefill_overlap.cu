@@ -4,9 +4,9 @@
 // chains: most SMs hold a short chain that ends early, or none, while the intra-chunk kernel
 // before it needs the whole machine.  Here the intra-chunk work is cut in two along the order in
 // which the chains consume the records (by position inside the sequence first): the first part
-// runs alone, then the state pass starts, one CTA per unit, and the second part runs beside it on
+// runs alone, then the state pass starts, two CTAs per unit (gdn_prefill_half.cuh), and the second part runs beside it on
 // the SMs that have no live chain, each record published through a flag (release) that the state
-// pass's loading warps wait for (acquire, bounded).
+// pass's loading warp waits for (acquire, bounded).
 //
 // Five launches in one stream, the first four each a programmatic dependent of the one before:
 //   prep          chunk table, ranking, processing order, cleared flags and done table, the cut
@@ -15,39 +15,36 @@
 //                 CTAs are scheduled only once every state-pass CTA is resident: they can never
 //                 take the SMs the chains need, and every chain that waits for a record is
 //                 resident while the producers still have SMs of their own (the launcher keeps
-//                 units <= SMs - kOverlapSpareSms, so every CTA has one unit)
+//                 2 units <= SMs - kOverlapSpareSms, so every CTA has one half unit)
 //   second part   does not wait for the state pass (it only feeds it); items [cut, total), pulled
-//                 from a queue by seven CTAs per unit (at most four per SM).  Its CTA 0 waits
+//                 from a queue by twelve CTAs per unit (at most four per SM).  Its CTA 0 waits
 //                 for the state pass at its very end, so that the completion of this launch
 //                 implies the state pass's.
 //   rest          an ordinary launch.  CUDA lets a programmatic dependent start early, it does not
 //                 promise to; if the second part did not run beside the state pass, the state
-//                 pass's waits for records ran out (soon, and without an error: a unit's final
+//                 pass's waits for records ran out (soon, and without an error: a half unit's final
 //                 state is written only after its last record has been loaded, so an unfinished
-//                 unit has left its initial state alone), it marked the units it finished, and
-//                 this launch runs the persistent pass over the others now that every record
-//                 exists.  Normally every CTA finds its unit done and returns at once.
-#include "gdn_prefill_stream.cuh"
+//                 one has left its initial state alone), it marked the half units it finished, and
+//                 this launch runs the others now that every record exists.  Normally every CTA finds
+//                 its half unit done and returns at once.
+#include "gdn_prefill_half.cuh"
+#include <algorithm>
 #include <cstdlib>
 
 namespace gdn {
 
 constexpr int kOverlapSpareSms = 8;
 
-// First part: one CTA per item [0, cut) of the processing order (surplus CTAs exit).
+// First part: resident CTAs over the items [0, cut) of the processing order.  (With one CTA per item the grid has to be
+// sized for all of them, the cut being known on the device only, and the CTAs that find nothing to do leave at 4 ns each:
+// 32768 tokens at 32 heads, a fifth of the items first, 52 us of nothing else.)
 __global__ void __launch_bounds__(kIntraThreads, 4)
 prefill_intra_first_kernel(const __grid_constant__ TensorMaps maps, const PrefillParams p,
                            uint8_t* ws, const WorkspaceLayout lay) {
     pdl_launch_dependents();
     pdl_wait();                     // the tables are the prep kernel's
-    const int32_t* hdr = reinterpret_cast<const int32_t*>(ws);
-    const int item = blockIdx.x;
-    if (item >= hdr[kHdrSplit]) return;
-    const int k = item / p.Hv;
-    const int hv = item - k * p.Hv;
-    const int c = reinterpret_cast<const int32_t*>(ws + lay.order)[k];
-    const ChunkInfo ci = reinterpret_cast<const ChunkInfo*>(ws + lay.chunks)[c];
-    uint8_t* rec = ws + lay.records + (static_cast<size_t>(c) * p.Hv + hv) * kRecBytes;
+    const int cut = reinterpret_cast<const int32_t*>(ws)[kHdrSplit];
+    if (static_cast<int>(blockIdx.x) >= cut) return;
 
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
@@ -63,9 +60,22 @@ prefill_intra_first_kernel(const __grid_constant__ TensorMaps maps, const Prefil
     __syncthreads();
     tc_fence_after_sync();
     const uint32_t tmem = tmem_base_s;
-    intra_item<false>(maps, p, rec, ci, hv / (p.Hv / p.Hqk), hv, smem, st, tmem, tid, [] { __syncthreads(); });
-    tc_fence_before_sync();
-    __syncthreads();
+    uint32_t n_done = 0;
+#pragma unroll 1
+    for (int item = blockIdx.x; item < cut; item += gridDim.x) {
+        const int k = item / p.Hv;
+        const int hv = item - k * p.Hv;
+        const int c = reinterpret_cast<const int32_t*>(ws + lay.order)[k];
+        const ChunkInfo ci = reinterpret_cast<const ChunkInfo*>(ws + lay.chunks)[c];
+        uint8_t* rec = ws + lay.records + (static_cast<size_t>(c) * p.Hv + hv) * kRecBytes;
+        const bool ok = intra_item<false>(maps, p, rec, ci, hv / (p.Hv / p.Hqk), hv, smem, st, tmem, tid,
+                                          [] { __syncthreads(); }, n_done);
+        ++n_done;
+        tc_fence_before_sync();
+        __syncthreads();
+        tc_fence_after_sync();
+        if (!ok) break;
+    }
     if (warp == 0) tmem_dealloc(tmem, kIntraTmemCols);
 }
 
@@ -133,7 +143,7 @@ prefill_intra_second_kernel(const __grid_constant__ TensorMaps maps, const Prefi
 }
 
 __global__ void __launch_bounds__(kStreamThreads, 1)
-prefill_state_stream_gated_kernel(const __grid_constant__ TensorMaps maps, const PrefillParams p,
+prefill_state_half_gated_kernel(const __grid_constant__ TensorMaps maps, const PrefillParams p,
                                   uint8_t* ws, const WorkspaceLayout lay) {
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
@@ -150,7 +160,7 @@ prefill_state_stream_gated_kernel(const __grid_constant__ TensorMaps maps, const
     const uint32_t tmem = tmem_base_s;
     pdl_wait();                     // tables, cleared flags and the first part's records
     pdl_launch_dependents();        // now the second part may take the SMs that are left
-    state_stream_role<2>(maps, p, ws, lay, smem, tmem, blockIdx.x, gridDim.x);
+    state_half_role<kHalfGated>(maps, p, ws, lay, smem, tmem, blockIdx.x, gridDim.x);
     __syncwarp();
     if (warp == kSIssueWarp) tmem_dealloc(tmem, kStateTmemCols);
 }
@@ -158,15 +168,12 @@ prefill_state_stream_gated_kernel(const __grid_constant__ TensorMaps maps, const
 // Last launch: the plain persistent pass over the units the gated pass did not finish (none, when
 // the producers ran beside it as intended: then every CTA finds its units done and returns).
 __global__ void __launch_bounds__(kStreamThreads, 1)
-prefill_state_stream_rest_kernel(const __grid_constant__ TensorMaps maps, const PrefillParams p,
+prefill_state_half_rest_kernel(const __grid_constant__ TensorMaps maps, const PrefillParams p,
                                  uint8_t* ws, const WorkspaceLayout lay) {
     // nothing left for this CTA: leave before any set-up
     {
-        const int32_t* done = reinterpret_cast<const int32_t*>(ws + lay.done);
-        const int total_units = p.N * p.Hv;
-        bool any = false;
-        for (int unit = blockIdx.x; unit < total_units; unit += gridDim.x) any = any || done[unit] == 0;
-        if (!any) return;
+        // (one half unit per CTA)
+        if (reinterpret_cast<const uint16_t*>(ws + lay.done)[blockIdx.x] != 0) return;
     }
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
@@ -181,7 +188,7 @@ prefill_state_stream_rest_kernel(const __grid_constant__ TensorMaps maps, const 
     __syncthreads();
     tc_fence_after_sync();
     const uint32_t tmem = tmem_base_s;
-    state_stream_role<3>(maps, p, ws, lay, smem, tmem, blockIdx.x, gridDim.x);
+    state_half_role<kHalfRest>(maps, p, ws, lay, smem, tmem, blockIdx.x, gridDim.x);
     __syncwarp();
     if (warp == kSIssueWarp) tmem_dealloc(tmem, kStateTmemCols);
 }
@@ -192,9 +199,9 @@ cudaError_t launch_prefill_overlap(const ChunkedParams& cp, cudaStream_t stream,
     if (e != cudaSuccess) return e;
     const int sms = di.sms;
     const PrefillParams& p = cp.p;
-    e = ensure_dynamic_smem(prefill_state_stream_gated_kernel, kStreamSmem);
+    e = ensure_dynamic_smem(prefill_state_half_gated_kernel, kHalfSmem);
     if (e != cudaSuccess) return e;
-    e = ensure_dynamic_smem(prefill_state_stream_rest_kernel, kStreamSmem);
+    e = ensure_dynamic_smem(prefill_state_half_rest_kernel, kHalfSmem);
     if (e != cudaSuccess) return e;
     e = ensure_dynamic_smem(prefill_intra_first_kernel, kIntraSmem);
     if (e != cudaSuccess) return e;
@@ -203,37 +210,35 @@ cudaError_t launch_prefill_overlap(const ChunkedParams& cp, cudaStream_t stream,
     TensorMaps maps;
     if (!make_prefill_tensor_maps(&maps, p)) return cudaErrorInvalidValue;
 
-    // The second part needs SMs of its own for as long as a chain may wait for it: with (nearly)
-    // as many units as SMs everything is produced before the state pass starts.
+    // The second part needs SMs of its own for as long as a chain may wait for it: with (nearly) as many half units as
+    // SMs everything is produced before the state pass starts.  So it is where launches are known to be serialised: the state
+    // pass waits for a launch that comes after it in the stream, the two must be able to run at the same time.  A
+    // profiler that replays kernels one at a time cannot be seen from here: under it the waits run out after
+    // milliseconds and the last launch does the work; profile gdn_prefill_stream instead, which runs the same kernels'
+    // arithmetic.
+    const long long units = static_cast<long long>(p.N) * p.Hv;
+    const char* blocking = std::getenv("CUDA_LAUNCH_BLOCKING");
+    if (2 * units > sms - kOverlapSpareSms || (blocking && blocking[0] != '\0' && blocking[0] != '0'))
+        return launch_prefill_stream(cp, stream);
     // split_permille == -2 (for tests): the second part is launched as an ordinary successor of
     // the state pass, i.e. the launches are serialised on purpose
     const bool serialised = split_permille == -2;
-    const long long units = static_cast<long long>(p.N) * p.Hv;
-    if (units > sms - kOverlapSpareSms) split_permille = 1000;
-    // The state pass waits for a launch that comes after it in the stream: the two must be able to
-    // run at the same time.  Where launches are known to be serialised, produce everything first
-    // (then no record is waited for).  A profiler that replays kernels one at a time cannot be
-    // seen from here: under it the waits run out after milliseconds and the last launch does the work;
-    // profile gdn_prefill_stream instead, which runs the same kernels' arithmetic.
-    const char* blocking = std::getenv("CUDA_LAUNCH_BLOCKING");
-    if (blocking && blocking[0] != '\0' && blocking[0] != '0') split_permille = 1000;
     if (split_permille > 1000) split_permille = 1000;
 
     e = launch_prefill_ranked_prep(cp, stream, 2, split_permille, sms);
     if (e != cudaSuccess) return e;
     const dim3 items(static_cast<unsigned>(cp.lay.max_chunks) * static_cast<unsigned>(p.Hv));
-    e = launch_dependent(prefill_intra_first_kernel, items, dim3(kIntraThreads), kIntraSmem,
+    const dim3 resident_first(std::min(items.x, 4u * static_cast<unsigned>(sms)));
+    e = launch_dependent(prefill_intra_first_kernel, resident_first, dim3(kIntraThreads), kIntraSmem,
                          stream, maps, p, cp.ws, cp.lay);
     if (e != cudaSuccess) return e;
-    const int grid = static_cast<int>(units < sms ? units : sms);
-    e = launch_dependent(prefill_state_stream_gated_kernel, dim3(grid), dim3(kStreamThreads),
-                         kStreamSmem, stream, maps, p, cp.ws, cp.lay);
+    const int grid = static_cast<int>(2 * units);
+    e = launch_dependent(prefill_state_half_gated_kernel, dim3(grid), dim3(kStreamThreads),
+                         kHalfSmem, stream, maps, p, cp.ws, cp.lay);
     if (e != cudaSuccess) return e;
-    // Producers beyond what the chains consume only add memory traffic beside them (one sequence
-    // of 32768 tokens at 32 heads: 1024 us with 592 producer CTAs, 986 us with 222, 1203 us with
-    // 148): a unit takes a record per chunk step and a producer CTA needs about seven chunk steps
-    // per item, so seven CTAs per unit keep up.
-    unsigned resident = 7u * static_cast<unsigned>(units);
+    // Producers beyond what the chains consume only add memory traffic beside them: a unit takes a record per chunk step
+    // and a producer CTA needs about twelve chunk steps per item (four on an SM), so twelve CTAs per unit keep up.
+    unsigned resident = 12u * static_cast<unsigned>(units);
     if (resident < static_cast<unsigned>(sms)) resident = static_cast<unsigned>(sms);
     if (resident > 4u * static_cast<unsigned>(sms)) resident = 4u * static_cast<unsigned>(sms);
     const dim3 producers(items.x < resident ? items.x : resident);
@@ -247,7 +252,7 @@ cudaError_t launch_prefill_overlap(const ChunkedParams& cp, cudaStream_t stream,
     if (e != cudaSuccess) return e;
     // an ordinary launch: it starts when the second part has ended, and the second part's first
     // CTA ends only after the state pass
-    prefill_state_stream_rest_kernel<<<grid, kStreamThreads, kStreamSmem, stream>>>(maps, p, cp.ws, cp.lay);
+    prefill_state_half_rest_kernel<<<grid, kStreamThreads, kHalfSmem, stream>>>(maps, p, cp.ws, cp.lay);
     return cudaGetLastError();
 }
 

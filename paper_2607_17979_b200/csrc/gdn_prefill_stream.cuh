@@ -50,12 +50,10 @@ struct UnitInfo {
     int n, hv, hqk, c_first, nc, seq_t0, seq_len, slot;
     bool skip;          // invalid sequence, padding / out-of-range slot, or no chunks
     bool bad_seq, bad_slot;
-    bool done;          // finished by an earlier launch (the two-part route's last launch only)
 };
 
 __device__ __forceinline__ UnitInfo unit_info(const PrefillParams& p, const uint8_t* ws,
-                                              const WorkspaceLayout& lay, int unit,
-                                              const int32_t* done = nullptr) {   // units to leave out
+                                              const WorkspaceLayout& lay, int unit) {
     const int32_t* seq_first = reinterpret_cast<const int32_t*>(ws + lay.seq_first);
     const int32_t* seq_bad = reinterpret_cast<const int32_t*>(ws + lay.seq_bad);
     const int32_t* seq_by_rank = reinterpret_cast<const int32_t*>(ws + lay.seq_by_rank);
@@ -72,14 +70,10 @@ __device__ __forceinline__ UnitInfo unit_info(const PrefillParams& p, const uint
     u.bad_seq = seq_bad[u.n] != 0;
     u.bad_slot = u.slot < 0 || u.slot >= p.num_slots;
     u.skip = u.bad_seq || u.bad_slot || u.nc == 0;
-    u.done = done != nullptr && done[unit] != 0;
     return u;
 }
 
 constexpr uint32_t kSpinFlagLimit = 1u << 22;
-// a few milliseconds: far longer than the producers ever lag when they do run beside the state
-// pass, far shorter than the other roles' mbarrier waits (which would report an error)
-constexpr uint32_t kSpinFlagLimitSoft = 1u << 13;
 
 __device__ __forceinline__ uint32_t ld_acquire_u32(const uint32_t* p) {
     uint32_t v;
@@ -94,15 +88,10 @@ __device__ __forceinline__ void fence_proxy_async_all() {
 }
 
 // The state pass of one CTA of 512 threads over the units cta, cta + n_ctas, ... of the rank-sorted
-// list.  kGated = 0: every record exists (the intra-chunk kernel ran before).  kGated = 1:
-// records are being produced by other CTAs of the same cooperative launch and the loading warps
-// wait for each record's flag first.  kGated = 2: the records of the first hdr[kHdrSplit] items of
-// the processing order exist, the others are being produced by a concurrent kernel and are waited
-// for; a wait that runs out ends the CTA's work without an error (the units it has finished are
-// marked in the done table, the others are left to a later launch).  kGated = 3: that later launch:
-// every record exists, the units marked done are left out.  `tmem` = 512 allocated columns; ends
-// with a CTA barrier.
-template <int kGated>
+// list.  kGated = false: every record exists (the intra-chunk kernel ran before).  true: records are being produced by
+// other CTAs of the same cooperative launch and the loading warps wait for each record's flag first.  `tmem` = 512 allocated
+// columns; ends with a CTA barrier.
+template <bool kGated>
 __device__ __forceinline__ void state_stream_role(const TensorMaps& maps, const PrefillParams& p,
                                                   uint8_t* ws, const WorkspaceLayout& lay,
                                                   uint8_t* smem, const uint32_t tmem, const int cta,
@@ -111,21 +100,13 @@ __device__ __forceinline__ void state_stream_role(const TensorMaps& maps, const 
         bar_y_read, bar_d1, bar_d4, bar_s, bar_u;
     __shared__ int abort_flag;
     __shared__ uint32_t armed_chunks;     // chunks of the CTA's stream whose copies a loader has started
-    // kGated == 2 waits for records of a launch that may not be running beside this one: there no
-    // wait that runs out is an error, whichever role it happens in (the loader's own wait for a
-    // flag is the shortest, but the limits are counted in polls, not in time): the units this CTA
-    // has not finished are left to the last launch, which reports real failures.
-    constexpr int kWaitReason = kGated == 2 ? 2 : 1;
     // Only the cooperative launch's records carry the scaled Q (gdn_prefill_chunk.cuh).
-    constexpr bool kScaledQ = kGated == 1;
+    constexpr bool kScaledQ = kGated;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int half = (warp >> 2) & 1;                 // which half of the columns this thread owns
     const int dv = (warp & 3) * 32 + lane;            // TMEM lane = state row
     const uint32_t lane_base = static_cast<uint32_t>((warp & 3) * 32) << 16;
     const int total_units = p.N * p.Hv;
-    int32_t* done_w = reinterpret_cast<int32_t*>(ws + lay.done);      // written by kGated == 2
-    const int32_t* done_tab = kGated == 3 ? done_w : nullptr;         // read by kGated == 3
-    (void)done_w;
 
     if (tid == 0) {
         mbar_init(&bar_full[0], 3);      // one arrival (and its bytes) per loading warp
@@ -160,7 +141,7 @@ __device__ __forceinline__ void state_stream_role(const TensorMaps& maps, const 
     __syncthreads();
     tc_fence_after_sync();
     volatile int* abortp = &abort_flag;
-    if constexpr (kGated == 0) pdl_wait();     // tables and records are the previous kernels'
+    if constexpr (!kGated) pdl_wait();     // tables and records are the previous kernels'
 
     // gc = chunks of earlier units of this CTA; chunk j of the current unit is chunk g = gc + j of
     // the CTA's stream: stage g & 1, phase g >> 1 of bar_full / bar_free_* of that stage, phase g of
@@ -183,22 +164,14 @@ __device__ __forceinline__ void state_stream_role(const TensorMaps& maps, const 
             const uint32_t* flags = reinterpret_cast<const uint32_t*>(ws + lay.flags);
             (void)flags;
             bool live = true;
-            // kGated == 2: chunk j of the sequence of rank r is item (pos[j] + r) * Hv + hv of
-            // the processing order; items from `cut` on are waited for
-            const int32_t* pos = reinterpret_cast<const int32_t*>(ws + lay.pos);
-            const int32_t cut = kGated == 2 ? reinterpret_cast<const int32_t*>(ws)[kHdrSplit] : 0;
-            (void)pos;
-            (void)cut;
             // the next unit's table entries are fetched while the current unit is processed
-            UnitInfo nxt = unit_info(p, ws, lay, min(cta, total_units - 1), done_tab);
+            UnitInfo nxt = unit_info(p, ws, lay, min(cta, total_units - 1));
             for (int unit = cta; unit < total_units && live; unit += n_ctas) {
                 const UnitInfo u = nxt;
-                nxt = unit_info(p, ws, lay, min(unit + n_ctas, total_units - 1), done_tab);
-                if (u.skip || u.done) continue;
+                nxt = unit_info(p, ws, lay, min(unit + n_ctas, total_units - 1));
+                if (u.skip) continue;
                 const uint8_t* records =
                     ws + lay.records + (static_cast<size_t>(u.c_first) * p.Hv + u.hv) * kRecBytes;
-                const int32_t rank = unit / p.Hv;
-                int32_t pos_j = kGated == 2 ? pos[0] : 0;       // fetched one chunk ahead
                 for (int j = 0; j < u.nc; ++j) {
                     const uint32_t g = gc + j;
                     const int st = g & 1;
@@ -206,26 +179,17 @@ __device__ __forceinline__ void state_stream_role(const TensorMaps& maps, const 
                     const uint32_t par_free = ((g - 2) >> 1) & 1u;
                     uint8_t* base = smem + st * kStageBytes;
                     const uint8_t* rec = records + j * rec_stride;
-                    bool gated = kGated == 1;
-                    if constexpr (kGated == 2) {
-                        gated = (pos_j + rank) * p.Hv + u.hv >= cut;
-                        pos_j = pos[j + 1];                     // pos has an entry past the longest chain
-                    }
-                    if (gated) {
+                    if constexpr (kGated) {
                         // the record must have been published by its producer CTA
                         const uint32_t* f = flags + (static_cast<size_t>(u.c_first + j) * p.Hv + u.hv);
                         uint32_t v = 0;
-                        // kGated == 2: a wait that runs out is no error (the producers' launch may
-                        // not be running beside this one): give up soon, well before any of the
-                        // other roles' waits, and leave the unit to the last launch
-                        const uint32_t limit = kGated == 2 ? kSpinFlagLimitSoft : kSpinFlagLimit;
-                        for (uint32_t i = 0; i < limit; ++i) {
+                        for (uint32_t i = 0; i < kSpinFlagLimit; ++i) {
                             v = ld_acquire_u32(f);
                             if (v != 0 || *abortp) break;
                             __nanosleep(64);
                         }
                         if (v != 1) {
-                            if (*abortp == 0) *abortp = (kGated == 2 && v == 0) ? 2 : 1;
+                            if (*abortp == 0) *abortp = 1;
                             live = false;
                             break;
                         }
@@ -234,7 +198,7 @@ __device__ __forceinline__ void state_stream_role(const TensorMaps& maps, const 
                         // below; one here would also wait for this thread's copies in flight (3 %
                         // of a long sequence's run time).
                     }
-                    if (g >= 2 && !wait_or_abort<40>(&bar_free[st], par_free, abortp, kWaitReason)) { live = false; break; }
+                    if (g >= 2 && !wait_or_abort<40>(&bar_free[st], par_free, abortp)) { live = false; break; }
                     atomicMax(&armed_chunks, g + 1);
                     const int tok = u.seq_t0 + j * kChunk;
                     if (part == 0) {
@@ -278,11 +242,11 @@ __device__ __forceinline__ void state_stream_role(const TensorMaps& maps, const 
             const uint32_t tS = tmem + kT_S, tD1 = tmem + kT_D1, tD4 = tmem + kT_D4;
             bool live = true;
             // the next unit's table entries are fetched while the current unit is processed
-            UnitInfo nxt = unit_info(p, ws, lay, min(cta, total_units - 1), done_tab);
+            UnitInfo nxt = unit_info(p, ws, lay, min(cta, total_units - 1));
             for (int unit = cta; unit < total_units && live; unit += n_ctas) {
                 const UnitInfo u = nxt;
-                nxt = unit_info(p, ws, lay, min(unit + n_ctas, total_units - 1), done_tab);
-                if (u.skip || u.done) continue;
+                nxt = unit_info(p, ws, lay, min(unit + n_ctas, total_units - 1));
+                if (u.skip) continue;
                 for (int j = 0; j < u.nc; ++j) {
                     const uint32_t g = gc + j;
                     const int st = g & 1;
@@ -291,7 +255,7 @@ __device__ __forceinline__ void state_stream_role(const TensorMaps& maps, const 
                     // Y.  Scaled Q: both terms in one of two tiles.  Raw Q: a tile for each term.
                     const uint32_t tY1 = tmem + kT_Y + (kScaledQ ? 64 * st : 0);
                     const uint32_t tY2 = tmem + kT_Y + (kScaledQ ? 64 * st : 64);
-                    if (!warp_wait_or_abort(&bar_s, g & 1u, abortp, kWaitReason)) {      // record landed, bf16 S and U~ in TMEM
+                    if (!warp_wait_or_abort(&bar_s, g & 1u, abortp)) {      // record landed, bf16 S and U~ in TMEM
                         live = false;
                         break;
                     }
@@ -309,7 +273,7 @@ __device__ __forceinline__ void state_stream_role(const TensorMaps& maps, const 
                     if (elect_one()) mma_commit(&bar_d1);
                     // S Q^T  (off the chain) overwrites the tile the output warps read two chunks ago (raw Q: one
                     // chunk ago)
-                    if (!kScaledQ && g > 0 && !warp_wait_or_abort(&bar_y_read, (g - 1) & 1u, abortp, kWaitReason)) {
+                    if (!kScaledQ && g > 0 && !warp_wait_or_abort(&bar_y_read, (g - 1) & 1u, abortp)) {
                         live = false;
                         break;
                     }
@@ -323,7 +287,7 @@ __device__ __forceinline__ void state_stream_role(const TensorMaps& maps, const 
                     if (elect_one()) mma_ts_c<true>(tY1, tS + 48, sdesc_advance(qg, 8192 + 64), id64);
                     if (elect_one()) mma_ts_c<true>(tY1, tS + 56, sdesc_advance(qg, 8192 + 96), id64);
                     if (elect_one()) mma_commit(&bar_free_a[st]);                          // W and Q have been read
-                    if (!warp_wait_or_abort(&bar_u, g & 1u, abortp, kWaitReason)) {         // U operands in TMEM
+                    if (!warp_wait_or_abort(&bar_u, g & 1u, abortp)) {         // U operands in TMEM
                         live = false;
                         break;
                     }
@@ -381,7 +345,7 @@ __device__ __forceinline__ void state_stream_role(const TensorMaps& maps, const 
         // The final state of the unit before, still in the D4 tile: written once the next unit's first
         // product is on its way (which does not touch that tile; the next state product waits for
         // these warps).
-        int pending = -1, pending_unit = 0;
+        int pending = -1;
         auto flush = [&] {
             if (pending < 0) return;
             float* out = p.final_state + static_cast<size_t>(pending) * (kD * kD) + frag_off();
@@ -399,15 +363,12 @@ __device__ __forceinline__ void state_stream_role(const TensorMaps& maps, const 
                         *reinterpret_cast<uint2*>(out + piece_off(i, b, r)) =
                             make_uint2(y[4 * b + 2 * r], y[4 * b + 2 * r + 1]);
             }
-            if constexpr (kGated == 2) {
-                if (tid == 0) done_w[pending_unit] = 1;
-            }
             pending = -1;
         };
         // Bounded wait + tcgen05 fence.  `ok` is each lane's own until the unit's last chunk, where the group
         // agrees on it; no warp-wide instruction before that depends on it.
         auto await = [&](uint64_t* bar, uint32_t parity) {
-            if (ok) ok = wait_or_abort(bar, parity, abortp, kWaitReason);
+            if (ok) ok = wait_or_abort(bar, parity, abortp);
             __syncwarp();
             tc_fence_after_sync();
         };
@@ -418,21 +379,17 @@ __device__ __forceinline__ void state_stream_role(const TensorMaps& maps, const 
         // A unit's chunks (0: nothing for the chain) and state tile; the rest of its entry is read again
         // where a unit is left out (registers).
         auto brief = [&](int unit) {
-            const UnitInfo u = unit_info(p, ws, lay, min(unit, total_units - 1), done_tab);
-            return make_int2(u.done || u.skip ? 0 : u.nc, u.slot * p.Hv + u.hv);
+            const UnitInfo u = unit_info(p, ws, lay, min(unit, total_units - 1));
+            return make_int2(u.skip ? 0 : u.nc, u.slot * p.Hv + u.hv);
         };
         int2 nxt = brief(cta);
         for (int unit = cta; unit < total_units; unit += n_ctas) {
             const int nc = nxt.x, tile = nxt.y;
             nxt = brief(unit + n_ctas);
             if (nc == 0) {
-                const UnitInfo u = unit_info(p, ws, lay, unit, done_tab);
-                if (u.done) continue;
+                const UnitInfo u = unit_info(p, ws, lay, unit);
                 const size_t tile_off = (static_cast<size_t>(u.bad_slot ? 0 : u.slot) * p.Hv + u.hv) * (kD * kD) +
                                         static_cast<size_t>(dv) * kD + half * 64;
-                if constexpr (kGated == 2) {
-                    if (tid == 0) done_w[unit] = 1;
-                }
                 if (u.bad_seq) continue;
                 if (u.bad_slot) {          // padding / out-of-range slot: zero rows, no state
                     if (u.slot >= p.num_slots && tid == 0) report(p.dev_status, kDevBadSlot);
@@ -551,8 +508,7 @@ __device__ __forceinline__ void state_stream_role(const TensorMaps& maps, const 
                     }
                 }
                 if (last) {
-                    // nothing of a unit is written after a failed wait (every record of the unit has been loaded by
-                    // now: no flag wait of it can fail any more)
+                    // nothing of a unit is written after a failed wait
                     ok = group_all<2, kSEpiThreads>(ok);
                     if (ok) {
 #pragma unroll
@@ -565,7 +521,6 @@ __device__ __forceinline__ void state_stream_role(const TensorMaps& maps, const 
                         tmem_wait_st();
                         __syncwarp();
                         pending = tile;
-                        pending_unit = unit;
                     }
                 } else {
                     store_state_bf16();          // the next chunk's A operand
@@ -589,7 +544,7 @@ __device__ __forceinline__ void state_stream_role(const TensorMaps& maps, const 
         // the stores of rows depend on it.
         bool ok = true;
         auto await = [&](uint64_t* bar, uint32_t parity) {
-            if (ok) ok = wait_or_abort<40>(bar, parity, abortp, kWaitReason);
+            if (ok) ok = wait_or_abort<40>(bar, parity, abortp);
             __syncwarp();
         };
         // U~ (fp32, 32 KB per chunk) reaches the chain through the accumulator of S W^T: this group
@@ -605,13 +560,14 @@ __device__ __forceinline__ void state_stream_role(const TensorMaps& maps, const 
             if constexpr (!kScaledQ)
                 *reinterpret_cast<float2*>(&s_eb[q4][sq][2 * lane]) = *reinterpret_cast<const float2*>(
                     smem + sq * kStageBytes + kS_Rec + kRecEb + 8 * lane);
-            const float4* sU = reinterpret_cast<const float4*>(smem + sq * kStageBytes + kS_Rec + kRecU);
+            const float4* sU = reinterpret_cast<const float4*>(smem + sq * kStageBytes + kS_Rec + kRecU +
+                                                                   (odv >> 6) * kRecUHalf);
 #pragma unroll
             for (int c0 = 0; c0 < 64; c0 += 32) {       // eight reads in flight
                 uint32_t r[2][16];
 #pragma unroll
                 for (int q = 0; q < 8; ++q) {
-                    const float4 v = sU[((c0 >> 2) + q) * kD + odv];
+                    const float4 v = sU[rec_u_index((c0 >> 2) + q, odv & 63)];
                     uint32_t(&x)[16] = r[q >> 2];
                     x[4 * (q & 3)] = __float_as_uint(v.x); x[4 * (q & 3) + 1] = __float_as_uint(v.y);
                     x[4 * (q & 3) + 2] = __float_as_uint(v.z); x[4 * (q & 3) + 3] = __float_as_uint(v.w);
@@ -625,11 +581,11 @@ __device__ __forceinline__ void state_stream_role(const TensorMaps& maps, const 
             if (lane == 0) mbar_arrive(&bar_s);
         };
         bool preloaded = false;     // U~ of the chunk about to be processed is already in place
-        UnitInfo nxt = unit_info(p, ws, lay, min(cta, total_units - 1), done_tab);
+        UnitInfo nxt = unit_info(p, ws, lay, min(cta, total_units - 1));
         for (int unit = cta; unit < total_units; unit += n_ctas) {
             const UnitInfo u = nxt;
-            nxt = unit_info(p, ws, lay, min(unit + n_ctas, total_units - 1), done_tab);
-            if (u.skip || u.done) continue;
+            nxt = unit_info(p, ws, lay, min(unit + n_ctas, total_units - 1));
+            if (u.skip) continue;
             for (int j = 0; j < u.nc; ++j) {
                 const uint32_t g = gc + j;
                 const int buf = g & 1;
@@ -637,7 +593,7 @@ __device__ __forceinline__ void state_stream_role(const TensorMaps& maps, const 
                 // k = 1: once the chain warps have read U of this chunk the accumulator is free for
                 // the next chunk's U~ (when the next chunk is known without looking past a skipped
                 // unit), which is then in place long before the chain warps hand the state over.
-                const bool ahead = j + 1 < u.nc || (unit + n_ctas < total_units && !nxt.skip && !nxt.done);
+                const bool ahead = j + 1 < u.nc || (unit + n_ctas < total_units && !nxt.skip);
 #pragma unroll 1
                 for (int k = preloaded ? 1 : 0; k < 2; ++k) {
                     if (k == 1) {
@@ -719,7 +675,7 @@ __device__ __forceinline__ void state_stream_role(const TensorMaps& maps, const 
     tc_fence_before_sync();
     __syncthreads();
     if (abort_flag != 0 && warp == kSIssueWarp && lane == 0) {
-        if (abort_flag == 1) report(p.dev_status, kDevTimeout);     // 2: a record not produced yet, no error
+        report(p.dev_status, kDevTimeout);
         // let copies already in flight land before the CTA's shared memory goes away: the last two
         // chunks a loader started, each on its stage's barrier at that chunk's own parity
         const uint32_t armed = *reinterpret_cast<volatile uint32_t*>(&armed_chunks);
