@@ -209,6 +209,7 @@ __device__ __forceinline__ void solve_merge_64(float* sA, const int w, const int
 template <int kSleepNs = 0>
 __device__ __forceinline__ bool wait_or_abort(uint64_t* bar, uint32_t parity, volatile int* abort_flag,
                                               const int reason = 1) {
+#pragma unroll 1
     for (uint32_t i = 0; i < kSpinLimit; ++i) {
         if (mbar_try_wait(bar, parity)) return true;
         if (kSleepNs) __nanosleep(kSleepNs);
@@ -237,9 +238,10 @@ template <int kId, int kThreads> __device__ __forceinline__ bool group_all(const
 // warp saw an arrival after 183 instead of 62.)
 __device__ __forceinline__ bool warp_wait_or_abort(uint64_t* bar, uint32_t parity, volatile int* abort_flag,
                                                    const int reason = 1) {
+#pragma unroll 1
     for (uint32_t i = 0; i < kSpinLimit; ++i) {
         if (__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) return true;
-        if ((i & 255u) == 255u && __any_sync(0xffffffffu, *abort_flag)) return false;
+        if ((i & 255u) == 0u && __any_sync(0xffffffffu, *abort_flag)) return false;
     }
     if (*abort_flag == 0) *abort_flag = reason;      // keep an earlier, different reason
     return false;
@@ -327,6 +329,11 @@ __device__ __forceinline__ bool intra_item(const TensorMaps& maps, const Prefill
     // goes on to its next barrier, behind which everyone leaves together; thread 0 drains what it has
     // in flight and the caller unwinds.
     volatile int* abortp = &st.abort_flag;
+    // (the cooperative launch re-allocates registers, which functions out of line do not go with)
+    auto wait_bar = [](uint64_t* bar, uint32_t parity, volatile int* abort_flag) {
+        if constexpr (kScaledQ) return warp_wait_or_abort(bar, parity, abort_flag);
+        else return warp_wait(bar, parity, abort_flag);
+    };
     bool v_started = false;         // (thread 0's)
     auto bail = [&](bool stores_pending) {
         if (tid == 0) {
@@ -339,21 +346,22 @@ __device__ __forceinline__ bool intra_item(const TensorMaps& maps, const Prefill
 
     const uint32_t tG = tmem, tW = tmem, tU = tmem + 64;     // W reuses the Gram columns
     const uint32_t sQK = smem_u32(smem + kI_QK);
-    // Tensor-core instructions are issued by warp 0, converged, one elected lane each (issuing eight
-    // from a single-lane branch takes 500 cycles instead of 180).
-    if (warp == 0 && warp_wait_or_abort(&st.bar_tma, par1, abortp)) {
+    // Tensor-core instructions are issued by warp 0, converged, a product by one elected lane (elect_one).
+    if (warp == 0 && wait_bar(&st.bar_tma, par1, abortp)) {
         tc_fence_after_sync();
         // [Q;K] (128 x 128, K-major) times K^T: lanes 0-63 = q.k, lanes 64-127 = k.k
         const uint32_t idesc = make_idesc_bf16(128, 64, false, false);
         const uint64_t dA = make_sdesc_sw128(sQK, 16, 1024), dB = make_sdesc_sw128(sQK + 8192, 16, 1024);
+        if (elect_one()) {
 #pragma unroll
-        for (int ks = 0; ks < 8; ++ks) {
-            const uint32_t off = (ks >> 2) * 16384 + (ks & 3) * 32;
-            if (elect_one()) mma_ss(tG, sdesc_advance(dA, off), sdesc_advance(dB, off), idesc, ks > 0);
+            for (int ks = 0; ks < 8; ++ks) {
+                const uint32_t off = (ks >> 2) * 16384 + (ks & 3) * 32;
+                mma_ss(tG, sdesc_advance(dA, off), sdesc_advance(dB, off), idesc, ks > 0);
+            }
+            mma_commit(&st.bar_mma);
         }
-        if (elect_one()) mma_commit(&st.bar_mma);
     }
-    const bool gram_ok = warp_wait_or_abort(&st.bar_mma, par3, abortp);
+    const bool gram_ok = wait_bar(&st.bar_mma, par3, abortp);
     tc_fence_after_sync();
     auto load_v = [&] {             // thread 0, once Q is dead
         v_started = true;
@@ -496,13 +504,15 @@ __device__ __forceinline__ bool intra_item(const TensorMaps& maps, const Prefill
     if (warp == 0) {     // W^T (dk x r) = K^T T_w^T with the raw K tile read MN-major
         const uint64_t dK = make_sdesc_sw128(sQK + 8192, 16384, 1024), dT = make_sdesc_sw128(smem_u32(smem + kI_Tw), 16, 1024);
         // columns of T_w and T_u past the chunk's length are zero: their k-steps are left out
+        if (elect_one()) {
 #pragma unroll
-        for (int ks = 0; ks < 4; ++ks)
-            if (ks * 16 < ci.len && elect_one())
-                mma_ss(tW, sdesc_advance(dK, ks * 2048), sdesc_advance(dT, ks * 32), idesc_t, ks > 0);
-        if (elect_one()) mma_commit(&st.bar_mma);
+            for (int ks = 0; ks < 4; ++ks)
+                if (ks * 16 < ci.len)
+                    mma_ss(tW, sdesc_advance(dK, ks * 2048), sdesc_advance(dT, ks * 32), idesc_t, ks > 0);
+            mma_commit(&st.bar_mma);
+        }
     }
-    warp_wait_or_abort(&st.bar_mma, par3 ^ 1u, abortp);
+    wait_bar(&st.bar_mma, par3 ^ 1u, abortp);
     tc_fence_after_sync();
 
     const int d = (warp & 3) * 32 + (tid & 31);   // TMEM lane of this thread: a dk / dv index
@@ -541,22 +551,24 @@ __device__ __forceinline__ bool intra_item(const TensorMaps& maps, const Prefill
         bulk_commit();
     }
     __syncwarp();
-    if (warp == 0 && warp_wait_or_abort(&st.bar_v, par1, abortp)) {        // V has landed
+    if (warp == 0 && wait_bar(&st.bar_v, par1, abortp)) {        // V has landed
         tc_fence_after_sync();
         // U~^T (dv x r) = V^T T_u^T with T_u = hi + lo
         const uint64_t dV = make_sdesc_sw128(sV, 16384, 1024);
         const uint64_t dH = make_sdesc_sw128(smem_u32(smem + kI_Tu), 16, 1024), dL = make_sdesc_sw128(smem_u32(smem + kI_TuLo), 16, 1024);
+        if (elect_one()) {
 #pragma unroll
-        for (int ks = 0; ks < 4; ++ks)
-            if (ks * 16 < ci.len && elect_one())
-                mma_ss(tU, sdesc_advance(dV, ks * 2048), sdesc_advance(dH, ks * 32), idesc_t, ks > 0);
+            for (int ks = 0; ks < 4; ++ks)
+                if (ks * 16 < ci.len)
+                    mma_ss(tU, sdesc_advance(dV, ks * 2048), sdesc_advance(dH, ks * 32), idesc_t, ks > 0);
 #pragma unroll
-        for (int ks = 0; ks < 4; ++ks)
-            if (ks * 16 < ci.len && elect_one())
-                mma_ss(tU, sdesc_advance(dV, ks * 2048), sdesc_advance(dL, ks * 32), idesc_t, true);
-        if (elect_one()) mma_commit(&st.bar_mma);
+            for (int ks = 0; ks < 4; ++ks)
+                if (ks * 16 < ci.len)
+                    mma_ss(tU, sdesc_advance(dV, ks * 2048), sdesc_advance(dL, ks * 32), idesc_t, true);
+            mma_commit(&st.bar_mma);
+        }
     }
-    warp_wait_or_abort(&st.bar_mma, par3, abortp);
+    wait_bar(&st.bar_mma, par3, abortp);
     tc_fence_after_sync();
 
     {   // U~^T[d][32 tokens] -> record, [half of dv][token group][dv][4 tokens] fp32

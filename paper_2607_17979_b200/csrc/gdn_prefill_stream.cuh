@@ -166,12 +166,14 @@ __device__ __forceinline__ void state_stream_role(const TensorMaps& maps, const 
             bool live = true;
             // the next unit's table entries are fetched while the current unit is processed
             UnitInfo nxt = unit_info(p, ws, lay, min(cta, total_units - 1));
+#pragma unroll 1
             for (int unit = cta; unit < total_units && live; unit += n_ctas) {
                 const UnitInfo u = nxt;
                 nxt = unit_info(p, ws, lay, min(unit + n_ctas, total_units - 1));
                 if (u.skip) continue;
                 const uint8_t* records =
                     ws + lay.records + (static_cast<size_t>(u.c_first) * p.Hv + u.hv) * kRecBytes;
+#pragma unroll 1
                 for (int j = 0; j < u.nc; ++j) {
                     const uint32_t g = gc + j;
                     const int st = g & 1;
@@ -226,7 +228,7 @@ __device__ __forceinline__ void state_stream_role(const TensorMaps& maps, const 
         __syncwarp();
     } else {
         // ===================== issuer: tensor-core instructions
-        {   // the whole warp runs this warp-uniform code; one elected lane executes each tcgen05 instruction
+        {   // the whole warp waits, one elected lane issues a product and its commit
             const uint32_t id64 = make_idesc_bf16(128, 64, false, false);
             const uint32_t id128mn = make_idesc_bf16(128, 128, false, true);
             const uint32_t id64mn = make_idesc_bf16(128, 64, false, true) | kIdescNegateB;
@@ -243,10 +245,12 @@ __device__ __forceinline__ void state_stream_role(const TensorMaps& maps, const 
             bool live = true;
             // the next unit's table entries are fetched while the current unit is processed
             UnitInfo nxt = unit_info(p, ws, lay, min(cta, total_units - 1));
+#pragma unroll 1
             for (int unit = cta; unit < total_units && live; unit += n_ctas) {
                 const UnitInfo u = nxt;
                 nxt = unit_info(p, ws, lay, min(unit + n_ctas, total_units - 1));
                 if (u.skip) continue;
+#pragma unroll 1
                 for (int j = 0; j < u.nc; ++j) {
                     const uint32_t g = gc + j;
                     const int st = g & 1;
@@ -262,15 +266,17 @@ __device__ __forceinline__ void state_stream_role(const TensorMaps& maps, const 
                     tc_fence_after_sync();
                     // U = U~ - S W^T  (on the chain): the accumulator holds U~, the B operand is negated;
                     // W is MN-major: k-step ks reads 16 dk rows = 2048 bytes
-                    if (elect_one()) mma_ts_c<true>(tD1, tS, w, id64mn);
-                    if (elect_one()) mma_ts_c<true>(tD1, tS + 8, sdesc_advance(w, 2048), id64mn);
-                    if (elect_one()) mma_ts_c<true>(tD1, tS + 16, sdesc_advance(w, 4096), id64mn);
-                    if (elect_one()) mma_ts_c<true>(tD1, tS + 24, sdesc_advance(w, 6144), id64mn);
-                    if (elect_one()) mma_ts_c<true>(tD1, tS + 32, sdesc_advance(w, 8192), id64mn);
-                    if (elect_one()) mma_ts_c<true>(tD1, tS + 40, sdesc_advance(w, 10240), id64mn);
-                    if (elect_one()) mma_ts_c<true>(tD1, tS + 48, sdesc_advance(w, 12288), id64mn);
-                    if (elect_one()) mma_ts_c<true>(tD1, tS + 56, sdesc_advance(w, 14336), id64mn);
-                    if (elect_one()) mma_commit(&bar_d1);
+                    if (elect_one()) {
+                        mma_ts_c<true>(tD1, tS, w, id64mn);
+                        mma_ts_c<true>(tD1, tS + 8, sdesc_advance(w, 2048), id64mn);
+                        mma_ts_c<true>(tD1, tS + 16, sdesc_advance(w, 4096), id64mn);
+                        mma_ts_c<true>(tD1, tS + 24, sdesc_advance(w, 6144), id64mn);
+                        mma_ts_c<true>(tD1, tS + 32, sdesc_advance(w, 8192), id64mn);
+                        mma_ts_c<true>(tD1, tS + 40, sdesc_advance(w, 10240), id64mn);
+                        mma_ts_c<true>(tD1, tS + 48, sdesc_advance(w, 12288), id64mn);
+                        mma_ts_c<true>(tD1, tS + 56, sdesc_advance(w, 14336), id64mn);
+                        mma_commit(&bar_d1);
+                    }
                     // S Q^T  (off the chain) overwrites the tile the output warps read two chunks ago (raw Q: one
                     // chunk ago)
                     if (!kScaledQ && g > 0 && !warp_wait_or_abort(&bar_y_read, (g - 1) & 1u, abortp)) {
@@ -278,37 +284,43 @@ __device__ __forceinline__ void state_stream_role(const TensorMaps& maps, const 
                         break;
                     }
                     if (!kScaledQ) tc_fence_after_sync();
-                    if (elect_one()) mma_ts_c<false>(tY1, tS, qg, id64);
-                    if (elect_one()) mma_ts_c<true>(tY1, tS + 8, sdesc_advance(qg, 32), id64);
-                    if (elect_one()) mma_ts_c<true>(tY1, tS + 16, sdesc_advance(qg, 64), id64);
-                    if (elect_one()) mma_ts_c<true>(tY1, tS + 24, sdesc_advance(qg, 96), id64);
-                    if (elect_one()) mma_ts_c<true>(tY1, tS + 32, sdesc_advance(qg, 8192), id64);
-                    if (elect_one()) mma_ts_c<true>(tY1, tS + 40, sdesc_advance(qg, 8192 + 32), id64);
-                    if (elect_one()) mma_ts_c<true>(tY1, tS + 48, sdesc_advance(qg, 8192 + 64), id64);
-                    if (elect_one()) mma_ts_c<true>(tY1, tS + 56, sdesc_advance(qg, 8192 + 96), id64);
-                    if (elect_one()) mma_commit(&bar_free_a[st]);                          // W and Q have been read
+                    if (elect_one()) {
+                        mma_ts_c<false>(tY1, tS, qg, id64);
+                        mma_ts_c<true>(tY1, tS + 8, sdesc_advance(qg, 32), id64);
+                        mma_ts_c<true>(tY1, tS + 16, sdesc_advance(qg, 64), id64);
+                        mma_ts_c<true>(tY1, tS + 24, sdesc_advance(qg, 96), id64);
+                        mma_ts_c<true>(tY1, tS + 32, sdesc_advance(qg, 8192), id64);
+                        mma_ts_c<true>(tY1, tS + 40, sdesc_advance(qg, 8192 + 32), id64);
+                        mma_ts_c<true>(tY1, tS + 48, sdesc_advance(qg, 8192 + 64), id64);
+                        mma_ts_c<true>(tY1, tS + 56, sdesc_advance(qg, 8192 + 96), id64);
+                        mma_commit(&bar_free_a[st]);                          // W and Q have been read
+                    }
                     if (!warp_wait_or_abort(&bar_u, g & 1u, abortp)) {         // U operands in TMEM
                         live = false;
                         break;
                     }
                     tc_fence_after_sync();
                     // D4 = (U decayed, hi + lo) K   (K tile MN-major: 16 tokens = 2048 bytes)
-                    if (elect_one()) mma_ts_c<false>(tD4, tmem + kT_Us, kk, id128mn);
-                    if (elect_one()) mma_ts_c<true>(tD4, tmem + kT_Us + 8, sdesc_advance(kk, 2048), id128mn);
-                    if (elect_one()) mma_ts_c<true>(tD4, tmem + kT_Us + 16, sdesc_advance(kk, 4096), id128mn);
-                    if (elect_one()) mma_ts_c<true>(tD4, tmem + kT_Us + 24, sdesc_advance(kk, 6144), id128mn);
-                    if (elect_one()) mma_ts_c<true>(tD4, tmem + kT_UsLo, kk, id128mn);
-                    if (elect_one()) mma_ts_c<true>(tD4, tmem + kT_UsLo + 8, sdesc_advance(kk, 2048), id128mn);
-                    if (elect_one()) mma_ts_c<true>(tD4, tmem + kT_UsLo + 16, sdesc_advance(kk, 4096), id128mn);
-                    if (elect_one()) mma_ts_c<true>(tD4, tmem + kT_UsLo + 24, sdesc_advance(kk, 6144), id128mn);
-                    if (elect_one()) mma_commit(&bar_d4);
+                    if (elect_one()) {
+                        mma_ts_c<false>(tD4, tmem + kT_Us, kk, id128mn);
+                        mma_ts_c<true>(tD4, tmem + kT_Us + 8, sdesc_advance(kk, 2048), id128mn);
+                        mma_ts_c<true>(tD4, tmem + kT_Us + 16, sdesc_advance(kk, 4096), id128mn);
+                        mma_ts_c<true>(tD4, tmem + kT_Us + 24, sdesc_advance(kk, 6144), id128mn);
+                        mma_ts_c<true>(tD4, tmem + kT_UsLo, kk, id128mn);
+                        mma_ts_c<true>(tD4, tmem + kT_UsLo + 8, sdesc_advance(kk, 2048), id128mn);
+                        mma_ts_c<true>(tD4, tmem + kT_UsLo + 16, sdesc_advance(kk, 4096), id128mn);
+                        mma_ts_c<true>(tD4, tmem + kT_UsLo + 24, sdesc_advance(kk, 6144), id128mn);
+                        mma_commit(&bar_d4);
+                    }
                     // U P^T
-                    if (elect_one()) mma_ts_c<kScaledQ>(tY2, tmem + kT_U, pp, id64);
-                    if (elect_one()) mma_ts_c<true>(tY2, tmem + kT_U + 8, sdesc_advance(pp, 32), id64);
-                    if (elect_one()) mma_ts_c<true>(tY2, tmem + kT_U + 16, sdesc_advance(pp, 64), id64);
-                    if (elect_one()) mma_ts_c<true>(tY2, tmem + kT_U + 24, sdesc_advance(pp, 96), id64);
-                    if (elect_one()) mma_commit(&bar_y[st]);
-                    if (elect_one()) mma_commit(&bar_free_c[st]);                          // P and the K tile have been read
+                    if (elect_one()) {
+                        mma_ts_c<kScaledQ>(tY2, tmem + kT_U, pp, id64);
+                        mma_ts_c<true>(tY2, tmem + kT_U + 8, sdesc_advance(pp, 32), id64);
+                        mma_ts_c<true>(tY2, tmem + kT_U + 16, sdesc_advance(pp, 64), id64);
+                        mma_ts_c<true>(tY2, tmem + kT_U + 24, sdesc_advance(pp, 96), id64);
+                        mma_commit(&bar_y[st]);
+                        mma_commit(&bar_free_c[st]);                          // P and the K tile have been read
+                    }
                 }
                 gc += u.nc;
             }
@@ -365,11 +377,10 @@ __device__ __forceinline__ void state_stream_role(const TensorMaps& maps, const 
             }
             pending = -1;
         };
-        // Bounded wait + tcgen05 fence.  `ok` is each lane's own until the unit's last chunk, where the group
-        // agrees on it; no warp-wide instruction before that depends on it.
+        // Bounded wait + tcgen05 fence.  `ok` is each warp's own until the unit's last chunk, where the group
+        // agrees on it.
         auto await = [&](uint64_t* bar, uint32_t parity) {
-            if (ok) ok = wait_or_abort(bar, parity, abortp);
-            __syncwarp();
+            if (!warp_wait_or_abort(bar, parity, abortp)) ok = false;
             tc_fence_after_sync();
         };
         // Every warp runs every group barrier and hand-over below, also after a wait has failed
@@ -383,6 +394,7 @@ __device__ __forceinline__ void state_stream_role(const TensorMaps& maps, const 
             return make_int2(u.skip ? 0 : u.nc, u.slot * p.Hv + u.hv);
         };
         int2 nxt = brief(cta);
+#pragma unroll 1
         for (int unit = cta; unit < total_units; unit += n_ctas) {
             const int nc = nxt.x, tile = nxt.y;
             nxt = brief(unit + n_ctas);
@@ -451,6 +463,7 @@ __device__ __forceinline__ void state_stream_role(const TensorMaps& maps, const 
             if (p.init_state && tid == 0 && nxt.x > 0 && unit + n_ctas < total_units)
                 bulk_prefetch_l2(p.init_state + static_cast<size_t>(nxt.y) * (kD * kD), kD * kD * 4);
             flush();
+#pragma unroll 1
             for (int j = 0; j < nc; ++j) {
                 const uint32_t g = gc + j;
                 const int st = g & 1;
@@ -540,7 +553,7 @@ __device__ __forceinline__ void state_stream_role(const TensorMaps& maps, const 
         const int ot = tid - kSOutWarp0 * 32;
         const size_t tok_stride = static_cast<size_t>(p.Hv) * kD;
         auto out_sync = [] { asm volatile("bar.sync 1, %0;" ::"n"(kSOutThreads) : "memory"); };
-        // As in the chain warps: each lane's own, and after a failed wait the work goes on with whatever is there; only
+        // As in the chain warps: each warp's own, and after a failed wait the work goes on with whatever is there; only
         // the stores of rows depend on it.
         bool ok = true;
         auto await = [&](uint64_t* bar, uint32_t parity) {
@@ -582,10 +595,12 @@ __device__ __forceinline__ void state_stream_role(const TensorMaps& maps, const 
         };
         bool preloaded = false;     // U~ of the chunk about to be processed is already in place
         UnitInfo nxt = unit_info(p, ws, lay, min(cta, total_units - 1));
+#pragma unroll 1
         for (int unit = cta; unit < total_units; unit += n_ctas) {
             const UnitInfo u = nxt;
             nxt = unit_info(p, ws, lay, min(unit + n_ctas, total_units - 1));
             if (u.skip) continue;
+#pragma unroll 1
             for (int j = 0; j < u.nc; ++j) {
                 const uint32_t g = gc + j;
                 const int buf = g & 1;

@@ -60,6 +60,7 @@ __device__ __forceinline__ bool mbar_try_wait_all(uint64_t* bar, uint32_t parity
 constexpr uint32_t kSpinLimit = 1u << 20;
 __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity,
                                           uint32_t limit = kSpinLimit) {
+#pragma unroll 1
     for (uint32_t i = 0; i < limit; ++i)
         if (mbar_try_wait(bar, parity)) return true;
     return false;
