@@ -19,10 +19,12 @@ namespace gdn {
 // =============================================================================================
 constexpr int kFPrepThreads = 256;
 // model of the two-part production (see the kernel): items per SM and chunk step, start-up lag of
-// the second part in chunk steps, and a safety margin in items
-constexpr int kSplitProdPermille = 330;
-constexpr int kSplitLeadSteps = 6;
-constexpr int kSplitMarginItems = 128;
+// the second part in chunk steps, and a safety margin in items.  (0.3 would be what the producers do, 0.385 leaves 32 chains
+// the small cut although their chains then wait a little: records are read while still in L2, and the machine is at its
+// power limit.  32 chains of 512 chunks 805 -> 696 us, of 188 296 -> 271; 40 chains, which need the larger cut, 233 -> 227.)
+constexpr int kSplitProdPermille = 385;
+constexpr int kSplitLeadSteps = 4;
+constexpr int kSplitMarginItems = 64;
 
 __global__ void __launch_bounds__(kFPrepThreads)
 prefill_fused_prep_kernel(const int32_t* __restrict__ cu, int32_t T, int32_t N, int32_t Hv,
