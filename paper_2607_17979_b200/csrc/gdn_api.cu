@@ -66,9 +66,10 @@ int gdn_decode(const void* q, const void* k, const void* v, const float* g, cons
     p.v = static_cast<const __nv_bfloat16*>(v);
     p.g = g; p.beta = beta; p.pool = state_pool; p.slot_idx = slot_idx;
     p.o = static_cast<__nv_bfloat16*>(o);
-    p.B = B; p.Hqk = Hqk; p.Hv = Hv; p.num_slots = num_slots; p.scale = scale;
+    p.set_heads(Hqk, Hv);
+    p.num_slots = num_slots; p.scale = scale;
     p.dev_status = dev_status;
-    return cuda_status(gdn::launch_decode(p, static_cast<cudaStream_t>(stream)));
+    return cuda_status(gdn::launch_decode(p, B, static_cast<cudaStream_t>(stream)));
 }
 
 int gdn_decode_multi(const void* q, const void* k, const void* v, const float* g,
@@ -95,11 +96,13 @@ int gdn_decode_multi(const void* q, const void* k, const void* v, const float* g
     p.v = static_cast<const __nv_bfloat16*>(v);
     p.g = g; p.beta = beta; p.pool = state_pool; p.slot_idx = slot_idx;
     p.o = static_cast<__nv_bfloat16*>(o);
-    p.B = B; p.Hqk = Hqk; p.Hv = Hv; p.num_slots = num_slots; p.scale = scale;
+    p.set_heads(Hqk, Hv);
+    p.num_slots = num_slots; p.scale = scale;
     p.dev_status = dev_status;
+    mp.Hqk = Hqk;
     mp.L = L;
     mp.layout = state_layout;
-    return cuda_status(gdn::launch_decode_multi(mp, static_cast<cudaStream_t>(stream)));
+    return cuda_status(gdn::launch_decode_multi(mp, B, static_cast<cudaStream_t>(stream)));
 }
 
 int gdn_gate(const void* a, const void* b, const float* A_log, const float* dt_bias,
@@ -154,7 +157,9 @@ int prefill_recurrent_impl(const void* q, const void* k, const void* v, const fl
     p.g = g; p.beta = beta; p.cu_seqlens = cu_seqlens; p.init_state = init_state;
     p.final_state = final_state; p.slot_idx = slot_idx;
     p.o = static_cast<__nv_bfloat16*>(o);
-    p.T = T; p.N = N; p.Hqk = Hqk; p.Hv = Hv; p.num_slots = num_slots; p.scale = scale;
+    p.T = T; p.N = N; p.Hqk = Hqk; p.Hv = Hv; p.num_slots = num_slots;
+    p.by_hv = gdn::fast_div(Hv); p.by_group = gdn::fast_div(Hv / Hqk);
+    p.scale = scale;
     p.dev_status = dev_status;
     return cuda_status(gdn::launch_prefill_recurrent(p, longest, static_cast<cudaStream_t>(stream)));
 }
@@ -196,7 +201,9 @@ int prefill_chunked_impl(PrefillRoute route, const void* q, const void* k, const
     p.g = g; p.beta = beta; p.cu_seqlens = cu_seqlens; p.init_state = init_state;
     p.final_state = final_state; p.slot_idx = slot_idx;
     p.o = static_cast<__nv_bfloat16*>(o);
-    p.T = T; p.N = N; p.Hqk = Hqk; p.Hv = Hv; p.num_slots = num_slots; p.scale = scale;
+    p.T = T; p.N = N; p.Hqk = Hqk; p.Hv = Hv; p.num_slots = num_slots;
+    p.by_hv = gdn::fast_div(Hv); p.by_group = gdn::fast_div(Hv / Hqk);
+    p.scale = scale;
     p.dev_status = dev_status;
     cp.ws = static_cast<uint8_t*>(workspace);
     cp.lay = gdn::workspace_layout(T, N, Hv);

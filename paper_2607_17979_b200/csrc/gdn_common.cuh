@@ -16,6 +16,22 @@ constexpr int kDevBadSlot = 1;
 constexpr int kDevBadCuSeqlens = 2;
 constexpr int kDevTimeout = 4;
 
+// Division of 0 <= x < 2^31 by a number known on the host: x * ceil(2^(31 + s) / d) >> 31 + s with 2^s >= d, exact because the
+// product's error is below x / 2^31 of a unit.  In line a division by a kernel argument takes about 150 cycles, and the three
+// that map a CTA to its sequence and heads stand in front of its first load.
+struct FastDiv {
+    uint32_t mul;
+    uint16_t shift;
+};
+inline FastDiv fast_div(uint32_t d) {
+    uint32_t s = 0;
+    while ((1ull << s) < d) ++s;
+    return FastDiv{static_cast<uint32_t>(((1ull << (31 + s)) + d - 1) / d), static_cast<uint16_t>(31 + s)};
+}
+__host__ __device__ inline int32_t operator/(int32_t x, const FastDiv& d) {
+    return static_cast<int32_t>(static_cast<uint64_t>(static_cast<uint32_t>(x)) * d.mul >> d.shift);
+}
+
 struct DecodeParams {
     const __nv_bfloat16* q;
     const __nv_bfloat16* k;
@@ -25,13 +41,27 @@ struct DecodeParams {
     float* pool;
     const int32_t* slot_idx;
     __nv_bfloat16* o;
-    int32_t B, Hqk, Hv, num_slots;
-    float scale;
     int32_t* dev_status;
+    int32_t Hv, num_slots;
+    // 96 bytes in all: a launch with 88 or 96 bytes of arguments takes 2.03 us of host time, with 80 or less and 104 or more
+    // 2.4-2.5, and the smallest calls are bound by it
+    uint32_t mul_hv, mul_group;          // by_hv(), by_group(): division by Hv, by Hv / Hqk
+    uint16_t shift_hv, shift_group;
+    float scale;
+    void set_heads(int32_t Hqk, int32_t Hv_) {
+        Hv = Hv_;
+        const FastDiv a = fast_div(Hv), b = fast_div(Hv / Hqk);
+        mul_hv = a.mul; shift_hv = a.shift;
+        mul_group = b.mul; shift_group = b.shift;
+    }
+    __device__ FastDiv by_hv() const { return FastDiv{mul_hv, shift_hv}; }
+    __device__ FastDiv by_group() const { return FastDiv{mul_group, shift_group}; }
 };
+static_assert(sizeof(DecodeParams) == 96, "see above");
 
 struct DecodeMultiParams {
     DecodeParams d;      // q,k [B][L][Hqk][128]; v,o [B][L][Hv][128]; g,beta [B][L][Hv]
+    int32_t Hqk;
     int32_t L;           // new tokens per sequence, 1..kDecodeMaxTokens
     int32_t layout;      // 0: tile [dv][dk];  1: tile [dk][dv]
 };
@@ -48,6 +78,7 @@ struct PrefillParams {
     const int32_t* slot_idx;
     __nv_bfloat16* o;
     int32_t T, N, Hqk, Hv, num_slots;
+    FastDiv by_hv, by_group;      // division by Hv, by Hv / Hqk
     float scale;
     int32_t* dev_status;
 };
@@ -63,8 +94,8 @@ template <class K> inline cudaError_t ensure_dynamic_smem(K* kernel, int bytes) 
     return ensure_dynamic_smem(reinterpret_cast<const void*>(kernel), bytes);
 }
 
-cudaError_t launch_decode(const DecodeParams& p, cudaStream_t stream);
-cudaError_t launch_decode_multi(const DecodeMultiParams& mp, cudaStream_t stream);
+cudaError_t launch_decode(const DecodeParams& p, int32_t B, cudaStream_t stream);
+cudaError_t launch_decode_multi(const DecodeMultiParams& mp, int32_t B, cudaStream_t stream);
 cudaError_t launch_gate(const __nv_bfloat16* a, const __nv_bfloat16* b, const float* A_log,
                         const float* dt_bias, float* g, float* beta, long long n, int Hv,
                         cudaStream_t stream);

@@ -40,9 +40,7 @@ decode_kernel(const DecodeParams p) {
     constexpr int kSplit = 4 / kPasses;
     const int unit = blockIdx.x / kSplit;
     const int part = blockIdx.x - unit * kSplit;
-    const int i = unit / p.Hv;
-    const int hv = unit - i * p.Hv;
-    const int hqk = hv / (p.Hv / p.Hqk);
+    const int i = unit / p.by_hv();
     const int lane = threadIdx.x & 31;
     const int warp = threadIdx.x >> 5;
     const int sub = lane & 7;        // which 16-column share of the row
@@ -50,7 +48,7 @@ decode_kernel(const DecodeParams p) {
     sm100::pdl_launch_dependents();
     sm100::pdl_wait();
 
-    __nv_bfloat16* o_row = p.o + (static_cast<size_t>(i) * p.Hv + hv) * kD;
+    __nv_bfloat16* o_row = p.o + static_cast<size_t>(unit) * kD;
     const int slot = p.slot_idx ? p.slot_idx[i] : i;
     if (slot < 0 || slot >= p.num_slots) {
         if (slot >= p.num_slots && threadIdx.x == 0 && part == 0) report(p.dev_status, kDevBadSlot);
@@ -58,7 +56,7 @@ decode_kernel(const DecodeParams p) {
         return;
     }
 
-    float* tile = p.pool + (static_cast<size_t>(slot) * p.Hv + hv) * (kD * kD);
+    float* tile = p.pool + (static_cast<size_t>(slot) * p.Hv + (unit - i * p.Hv)) * (kD * kD);
     const int row0 = part * (kD / kSplit) + warp * (4 * kPasses) + rsel;
     float4 s[kPasses][4];
 #pragma unroll
@@ -68,9 +66,10 @@ decode_kernel(const DecodeParams p) {
             s[ps][j] = ld_stream(reinterpret_cast<const float4*>(
                 tile + (row0 + ps * 4) * kD + sub * 4 + j * 32));
 
-    const __nv_bfloat16* kp = p.k + (static_cast<size_t>(i) * p.Hqk + hqk) * kD;
-    const __nv_bfloat16* qp = p.q + (static_cast<size_t>(i) * p.Hqk + hqk) * kD;
-    const __nv_bfloat16* vp = p.v + (static_cast<size_t>(i) * p.Hv + hv) * kD;
+    const size_t qk_row = unit / p.by_group();       // i Hqk + hv / (Hv / Hqk)
+    const __nv_bfloat16* kp = p.k + qk_row * kD;
+    const __nv_bfloat16* qp = p.q + qk_row * kD;
+    const __nv_bfloat16* vp = p.v + static_cast<size_t>(unit) * kD;
     float4 kf[4], qf[4];
     float kq = 0.f;
 #pragma unroll
@@ -80,8 +79,8 @@ decode_kernel(const DecodeParams p) {
         kq = dot4(kf[j], qf[j], kq);
     }
     kq = sum8(kq);
-    const float alpha = expf(p.g[static_cast<size_t>(i) * p.Hv + hv]);
-    const float beta = p.beta[static_cast<size_t>(i) * p.Hv + hv];
+    const float alpha = expf(p.g[unit]);
+    const float beta = p.beta[unit];
     float vj[kPasses];
 #pragma unroll
     for (int ps = 0; ps < kPasses; ++ps) vj[ps] = __bfloat162float(vp[row0 + ps * 4]);
@@ -111,8 +110,8 @@ decode_kernel(const DecodeParams p) {
     }
 }
 
-cudaError_t launch_decode(const DecodeParams& p, cudaStream_t stream) {
-    const long long units = static_cast<long long>(p.B) * p.Hv;
+cudaError_t launch_decode(const DecodeParams& p, int32_t B, cudaStream_t stream) {
+    const long long units = static_cast<long long>(B) * p.Hv;
     if (units == 0) return cudaSuccess;
     // below about two CTAs per SM of whole tiles, quarter tiles spread the same bytes over four
     // times as many SMs (the state rows are independent)

@@ -25,19 +25,19 @@ decode_multi_kernel(const DecodeMultiParams mp) {
     const int row_base = (blockIdx.x - unit * kSplit) * Block::kRows;
     const int i = unit / p.Hv;
     const int hv = unit - i * p.Hv;
-    const int hqk = hv / (p.Hv / p.Hqk);
+    const int hqk = hv / (p.Hv / mp.Hqk);
     sm100::pdl_launch_dependents();
     sm100::pdl_wait();
 
     const size_t tok0 = static_cast<size_t>(i) * mp.L;
     TokenRows t;
-    t.q = p.q + (tok0 * p.Hqk + hqk) * kD;
-    t.k = p.k + (tok0 * p.Hqk + hqk) * kD;
+    t.q = p.q + (tok0 * mp.Hqk + hqk) * kD;
+    t.k = p.k + (tok0 * mp.Hqk + hqk) * kD;
     t.v = p.v + (tok0 * p.Hv + hv) * kD;
     t.g = p.g + tok0 * p.Hv + hv;
     t.beta = p.beta + tok0 * p.Hv + hv;
     t.o = p.o + (tok0 * p.Hv + hv) * kD;
-    t.qk_stride = static_cast<size_t>(p.Hqk) * kD;
+    t.qk_stride = static_cast<size_t>(mp.Hqk) * kD;
     t.v_stride = static_cast<size_t>(p.Hv) * kD;
     t.g_stride = p.Hv;
     t.count = mp.L;
@@ -66,8 +66,8 @@ decode_multi_kernel(const DecodeMultiParams mp) {
 
 namespace {
 template <bool kTransposed, int kWarps>
-cudaError_t launch_shape(const DecodeMultiParams& mp, cudaStream_t stream) {
-    const unsigned grid = static_cast<unsigned>(static_cast<long long>(mp.d.B) * mp.d.Hv * (8 / kWarps));
+cudaError_t launch_shape(const DecodeMultiParams& mp, int32_t B, cudaStream_t stream) {
+    const unsigned grid = static_cast<unsigned>(static_cast<long long>(B) * mp.d.Hv * (8 / kWarps));
     auto kernel = mp.L <= 4   ? decode_multi_kernel<kTransposed, kWarps, 4>
                   : mp.L <= 8 ? decode_multi_kernel<kTransposed, kWarps, 8>
                               : decode_multi_kernel<kTransposed, kWarps, 16>;
@@ -75,8 +75,8 @@ cudaError_t launch_shape(const DecodeMultiParams& mp, cudaStream_t stream) {
 }
 }  // namespace
 
-cudaError_t launch_decode_multi(const DecodeMultiParams& mp, cudaStream_t stream) {
-    const long long units = static_cast<long long>(mp.d.B) * mp.d.Hv;
+cudaError_t launch_decode_multi(const DecodeMultiParams& mp, int32_t B, cudaStream_t stream) {
+    const long long units = static_cast<long long>(B) * mp.d.Hv;
     if (units == 0) return cudaSuccess;
     DeviceInfo di;
     const int sms = device_info(&di) == cudaSuccess ? di.sms : 148;
@@ -87,8 +87,8 @@ cudaError_t launch_decode_multi(const DecodeMultiParams& mp, cudaStream_t stream
     // L = 8 58.7 / 59.0, L = 16 99.2 / 82.1.  With too few tiles to fill the SMs, two: B = 1, L = 8, 8
     // v-heads 4.0 / 4.3.
     const bool two = mp.L <= 4 || (mp.L <= 8 && (mp.layout != 0 || units * 4 <= 2LL * sms));
-    if (mp.layout == 0) return two ? launch_shape<false, 2>(mp, stream) : launch_shape<false, 4>(mp, stream);
-    return two ? launch_shape<true, 2>(mp, stream) : launch_shape<true, 4>(mp, stream);
+    if (mp.layout == 0) return two ? launch_shape<false, 2>(mp, B, stream) : launch_shape<false, 4>(mp, B, stream);
+    return two ? launch_shape<true, 2>(mp, B, stream) : launch_shape<true, 4>(mp, B, stream);
 }
 
 }  // namespace gdn

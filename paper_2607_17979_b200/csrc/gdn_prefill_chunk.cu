@@ -8,96 +8,79 @@ namespace gdn {
 // =============================================================================================
 // K1: intra-chunk quantities, one CTA (256 threads) per (chunk, v-head); see intra_item().
 // =============================================================================================
-// kInlineTable: a batch of at most kInlineTableSeqs sequences needs no table-building launch in
-// front: every CTA finds its own chunk by walking cu_seqlens, and CTA (0, 0) writes the two small
-// per-sequence tables the state pass reads after this kernel (2.5 us less on a 100-token prompt).
+// kInlineTable: a batch of at most kSmallSeqs sequences needs no table-building launch in front: every warp finds the CTA's
+// chunk from cu_seqlens, a sequence a lane.
 template <bool kInlineTable>
 __global__ void __launch_bounds__(kIntraThreads, 4)
 prefill_intra_kernel(const __grid_constant__ TensorMaps maps, const PrefillParams p, uint8_t* ws,
                      const WorkspaceLayout lay) {
     const int c = blockIdx.x;
     const int hv = blockIdx.y;
+    __shared__ uint32_t tmem_base_s;
+    const int tid = threadIdx.x, warp = tid >> 5;
     pdl_launch_dependents();
-    if (threadIdx.x == 0) {         // (before the wait: a first use would fetch them in front of the tiles)
-        prefetch_tensormap(&maps.q);
-        prefetch_tensormap(&maps.k);
-        prefetch_tensormap(&maps.v);
+    // what needs nothing of the previous kernel's comes before the wait for it
+    if (warp == 0) {
+        if (tid == 0) {
+            prefetch_tensormap(&maps.q);
+            prefetch_tensormap(&maps.k);
+            prefetch_tensormap(&maps.v);
+        }
+        __syncwarp();
+        tmem_alloc(&tmem_base_s, kIntraTmemCols);
+        tmem_relinquish();
+        tc_fence_before_sync();
     }
     pdl_wait();                     // the chunk table is the previous kernel's
     ChunkInfo ci;
+    bool mine;
     if constexpr (kInlineTable) {
         // same rules as the table-building kernel: a sequence whose bounds are out of order or
         // out of range has no chunks and is flagged
-        const bool writer = blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0;
-        int32_t* seq_first = reinterpret_cast<int32_t*>(ws + lay.seq_first);
-        int32_t* seq_bad = reinterpret_cast<int32_t*>(ws + lay.seq_bad);
-        // one round trip for all bounds (a loop of dependent global loads would cost one each)
-        __shared__ int32_t s_cu[kInlineTableSeqs + 1];
-        if (static_cast<int>(threadIdx.x) <= p.N) s_cu[threadIdx.x] = p.cu_seqlens[threadIdx.x];
-        __syncthreads();
-        if (writer && (s_cu[0] != 0 || s_cu[p.N] != p.T)) report(p.dev_status, kDevBadCuSeqlens);
-        int first = 0;
-        ci.seq = -1;
-        for (int n = 0; n < p.N; ++n) {
-            const int32_t t0 = s_cu[n], t1 = s_cu[n + 1];
-            const bool ok = t0 >= 0 && t1 >= t0 && t1 <= p.T;
-            const int nc = ok ? (t1 - t0 + kChunk - 1) / kChunk : 0;
-            if (writer) {
-                if (!ok) report(p.dev_status, kDevBadCuSeqlens);
-                seq_bad[n] = ok ? 0 : 1;
-                seq_first[n] = first;
-            }
-            if (c >= first && c < first + nc) {
-                ci.seq = n;
-                ci.t0 = t0 + (c - first) * kChunk;
-                ci.len = min(kChunk, t1 - ci.t0);
-                ci.pad = 0;
-            }
-            first += nc;
+        const int lane = tid & 31;
+        int32_t t0 = 0, t1 = 0;
+        if (lane < p.N) {
+            t0 = p.cu_seqlens[lane];
+            t1 = p.cu_seqlens[lane + 1];
         }
-        if (writer) {
-            seq_first[p.N] = first;
-            *reinterpret_cast<int32_t*>(ws) = first;
-            // sequences by chunk count, more chunks first (the persistent state pass walks them in
-            // this order); with so few sequences, by counting
-            int32_t* seq_by_rank = reinterpret_cast<int32_t*>(ws + lay.seq_by_rank);
-            for (int n = 0; n < p.N; ++n) {
-                const int nc_n = seq_first[n + 1] - seq_first[n];
-                int rank = 0;
-                for (int m = 0; m < p.N; ++m) {
-                    const int nc_m = seq_first[m + 1] - seq_first[m];
-                    rank += (nc_m > nc_n || (nc_m == nc_n && m < n)) ? 1 : 0;
-                }
-                seq_by_rank[rank] = n;
-            }
+        const bool ok = t0 >= 0 && t1 >= t0 && t1 <= p.T;
+        const int nc = ok ? (t1 - t0 + kChunk - 1) / kChunk : 0;
+        int incl = nc;
+#pragma unroll
+        for (int d = 1; d < 32; d <<= 1) {
+            const int y = __shfl_up_sync(0xffffffffu, incl, d);
+            if (lane >= d) incl += y;
         }
-        if (ci.seq < 0) return;
+        if (c == 0 && hv == 0 && warp == 0 &&
+            (!ok || (lane == 0 && t0 != 0) || (lane == p.N - 1 && t1 != p.T)))
+            report(p.dev_status, kDevBadCuSeqlens);
+        const unsigned here = __ballot_sync(0xffffffffu, c < incl && c >= incl - nc);
+        mine = here != 0;
+        ci.seq = __ffs(here) - 1;
+        ci.t0 = t0 + (c - (incl - nc)) * kChunk;
+        ci.len = min(kChunk, t1 - ci.t0);
+        ci.t0 = __shfl_sync(0xffffffffu, ci.t0, ci.seq & 31);
+        ci.len = __shfl_sync(0xffffffffu, ci.len, ci.seq & 31);
+        ci.pad = 0;
     } else {
-        const int32_t total = *reinterpret_cast<const int32_t*>(ws);
-        if (c >= total) return;
-        ci = reinterpret_cast<const ChunkInfo*>(ws + lay.chunks)[c];
+        mine = c < *reinterpret_cast<const int32_t*>(ws);
+        if (mine) ci = reinterpret_cast<const ChunkInfo*>(ws + lay.chunks)[c];
     }
-    const int hqk = hv / (p.Hv / p.Hqk);
+    if (!mine) {
+        if (warp == 0) tmem_dealloc(tmem_base_s, kIntraTmemCols);
+        return;
+    }
+    const int hqk = hv / p.by_group;
     uint8_t* rec = ws + lay.records + (static_cast<size_t>(c) * p.Hv + hv) * kRecBytes;
 
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
                                                ~static_cast<uintptr_t>(1023));
     __shared__ IntraStatics st;
-    __shared__ uint32_t tmem_base_s;
-    const int tid = threadIdx.x, warp = tid >> 5;
-    if (warp == 0) {
-        tmem_alloc(&tmem_base_s, kIntraTmemCols);
-        tmem_relinquish();
-    }
+    intra_item<false>(maps, p, rec, ci, hqk, hv, smem, st, &tmem_base_s, 0, tid, [] { __syncthreads(); });
     tc_fence_before_sync();
     __syncthreads();
-    tc_fence_after_sync();
-    const uint32_t tmem = tmem_base_s;
-    intra_item<false>(maps, p, rec, ci, hqk, hv, smem, st, tmem, tid, [] { __syncthreads(); });
-    tc_fence_before_sync();
-    __syncthreads();
-    if (warp == 0) tmem_dealloc(tmem, kIntraTmemCols);
+    if (warp == 0) tmem_dealloc(tmem_base_s, kIntraTmemCols);
 }
 
 // =============================================================================================
@@ -146,11 +129,7 @@ bool make_prefill_tensor_maps(TensorMaps* maps, const PrefillParams& p) {
 }
 
 bool prefill_tables_inline(const ChunkedParams& cp) {
-    // Worth it for small batches only: the walk costs every CTA a barrier and a few hundred cycles,
-    // which over many waves of CTAs adds up to more than the launch it saves (512 + 1024 + 2048 + 4096
-    // tokens at 32 heads: +2 us).
-    return cp.p.N <= kInlineTableSeqs && cp.lay.max_chunks > 0 &&
-           static_cast<long long>(cp.lay.max_chunks) * cp.p.Hv <= kInlineTableItems;
+    return cp.p.N <= kSmallSeqs && cp.lay.max_chunks > 0;
 }
 
 cudaError_t launch_prefill_intra(const TensorMaps& maps, const ChunkedParams& cp, cudaStream_t stream,

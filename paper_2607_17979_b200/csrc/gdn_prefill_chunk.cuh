@@ -52,10 +52,9 @@ constexpr uint32_t kRecUHalf = (kRecDecay - kRecU) / 2;
 // that a fragment read (four dv of two neighbouring groups per half warp) touches every bank once.
 __device__ __forceinline__ int rec_u_index(int group, int dv) { return group * 64 + (dv ^ ((group & 1) << 2)); }
 
-// Small batches of at most this many sequences need no table-building launch: the intra-chunk
-// kernel finds its chunks from cu_seqlens itself and writes the per-sequence tables for the state pass.
-constexpr int kInlineTableSeqs = 16;
-constexpr int kInlineTableItems = 2 * 148 * 4;     // and at most about two waves of (chunk, v-head) CTAs
+// Batches of at most this many sequences need no table-building launch in front of the intra-chunk kernel and the state
+// pass: a warp reads all bounds at once.
+constexpr int kSmallSeqs = 32;
 
 struct ChunkInfo {      // 16 bytes
     int32_t seq;        // sequence the chunk belongs to

@@ -34,9 +34,8 @@ struct TensorMaps {
 // Host side: 2-D maps over the packed q, k, v, o (64 x 64 boxes, 128B swizzle); false on failure.
 bool make_prefill_tensor_maps(TensorMaps* maps, const PrefillParams& p);
 // Launch of the intra-chunk kernel over every (chunk, v-head) item of the batch.
-// inline_tables: no table-building launch went before; every CTA finds its chunk from cu_seqlens and
-// one CTA writes the per-sequence tables (first chunk, validity, rank) for the state pass.  Only
-// for batches of few sequences: see prefill_tables_inline().
+// inline_tables: no table-building launch went before; every CTA finds its chunk from cu_seqlens.  For batches of few
+// sequences: see prefill_tables_inline().
 cudaError_t launch_prefill_intra(const TensorMaps& maps, const ChunkedParams& cp, cudaStream_t stream,
                                  bool inline_tables);
 bool prefill_tables_inline(const ChunkedParams& cp);
@@ -262,13 +261,14 @@ __device__ __forceinline__ bool warp_wait(uint64_t* bar, uint32_t parity, volati
 // The intra-chunk quantities of one (chunk, v-head) item, computed by a group of 256 threads
 // (tid = 0..255 within the group; its warps must be CTA warps 0-3 mod 4 aligned, because a warp
 // reaches TMEM lanes 32 (warp % 4) ...).  `smem` is the group's 1024-aligned slice of kI_End
-// bytes, `tmem` its 128 TMEM columns, `sync` a barrier over exactly the group.  Writes the item's
+// bytes, `tmem_base` + `tmem_off` its 128 TMEM columns (read behind the group's first barrier, which so also covers their
+// allocation), `sync` a barrier over exactly the group.  Writes the item's
 // record; returns false after a bounded wait gave up (status word set, nothing left in flight).
 template <bool kScaledQ, class Sync>
 __device__ __forceinline__ bool intra_item(const TensorMaps& maps, const PrefillParams& p,
                                            uint8_t* rec, const ChunkInfo ci, const int hqk,
                                            const int hv, uint8_t* smem, IntraStatics& st,
-                                           const uint32_t tmem, const int tid, Sync sync,
+                                           const uint32_t* tmem_base, const uint32_t tmem_off, const int tid, Sync sync,
                                            const uint32_t n_done = 0) {
     // `n_done` = items this group has processed before (persistent callers): the mbarriers are
     // initialised once and keep flipping phase, one completion of bar_tma and bar_v and three
@@ -325,6 +325,8 @@ __device__ __forceinline__ bool intra_item(const TensorMaps& maps, const Prefill
         if (lane == 0) *reinterpret_cast<float*>(rec + kRecGammaC) = ex2_approx(bC * kLog2e);
     }
     sync();
+    tc_fence_after_sync();
+    const uint32_t tmem = *tmem_base + tmem_off;
     // Every warp polls the barriers it needs itself.  A wait that runs out flags the item and the group
     // goes on to its next barrier, behind which everyone leaves together; thread 0 drains what it has
     // in flight and the caller unwinds.

@@ -298,18 +298,17 @@ template <int kId, int kCount> __device__ __forceinline__ void named_sync() {
 __device__ __forceinline__ void fused_intra_role(const TensorMaps& maps, const PrefillParams& p,
                                                  uint8_t* ws, const WorkspaceLayout& lay,
                                                  uint8_t* smem, IntraStatics* statics,
-                                                 const uint32_t tmem_base) {
+                                                 const uint32_t* tmem_base) {
     const int group = threadIdx.x >> 8;
     const int gtid = threadIdx.x & 255;
     IntraStatics& st = statics[group];
     uint8_t* gsmem = smem + group * kFGroupSmem;
-    const uint32_t tmem = tmem_base + group * kIntraTmemCols;
+    const uint32_t tmem_off = group * kIntraTmemCols;
     int32_t* hdr = reinterpret_cast<int32_t*>(ws);
     const int32_t total_items = hdr[kHdrTotalItems];
     const int32_t* order = reinterpret_cast<const int32_t*>(ws + lay.order);
     const ChunkInfo* chunks = reinterpret_cast<const ChunkInfo*>(ws + lay.chunks);
     uint32_t* flags = reinterpret_cast<uint32_t*>(ws + lay.flags);
-    const int G = p.Hv / p.Hqk;
 
     auto gsync = [group] {
         if (group == 0) named_sync<1, 256>();
@@ -322,13 +321,13 @@ __device__ __forceinline__ void fused_intra_role(const TensorMaps& maps, const P
         gsync();
         const int item = st.item;
         if (item >= total_items) break;
-        const int k = item / p.Hv;
+        const int k = item / p.by_hv;
         const int hv = item - k * p.Hv;
         const int c = order[k];
         const ChunkInfo ci = chunks[c];
         const size_t slot = static_cast<size_t>(c) * p.Hv + hv;
         uint8_t* rec = ws + lay.records + slot * kRecBytes;
-        const bool ok = intra_item<true>(maps, p, rec, ci, hv / G, hv, gsmem, st, tmem, gtid, gsync, n_done);
+        const bool ok = intra_item<true>(maps, p, rec, ci, hv / p.by_group, hv, gsmem, st, tmem_base, tmem_off, gtid, gsync, n_done);
         ++n_done;
         // publish: every thread's own stores first, then the bulk stores, then the flag
         __threadfence();
@@ -369,7 +368,7 @@ prefill_fused_kernel(const __grid_constant__ TensorMaps maps, const PrefillParam
     if (static_cast<int>(blockIdx.x) < n_state) {
         state_stream_role<true>(maps, p, ws, lay, smem, tmem, blockIdx.x, n_state);
     } else {
-        fused_intra_role(maps, p, ws, lay, smem, intra_statics, tmem);
+        fused_intra_role(maps, p, ws, lay, smem, intra_statics, &tmem_base_s);
         tc_fence_before_sync();
         __syncthreads();
     }

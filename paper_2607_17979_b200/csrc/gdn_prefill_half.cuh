@@ -97,15 +97,19 @@ __device__ __forceinline__ void state_half_role(const TensorMaps& maps, const Pr
         armed[0] = armed[1] = armed[2] = 0;
         fence_barrier_init();
     }
+    // (the two parts go by the order of production in the workspace)
+    __shared__ __align__(16) SeqEntry seq_entries[kMode == kHalfAll ? kSmallSeqs : 1];
+    const SeqEntry* const seq_tab = kMode == kHalfAll && p.N <= kSmallSeqs ? seq_entries : nullptr;
+    if constexpr (kMode == kHalfAll) pdl_wait();     // tables and records are the previous kernels'
+    if (seq_tab && warp > kHLoadWarp) build_seq_table(seq_entries, p, lane);
     tc_fence_before_sync();
     __syncthreads();
     tc_fence_after_sync();
     volatile int* abortp = &abort_flag;
-    if constexpr (kMode == kHalfAll) pdl_wait();     // tables and records are the previous kernels'
 
     // The i-th half unit of this CTA, or one past the end.  Every role walks this list.
     auto at = [&](int i) { return i * n_ctas + ((i & 1) ? n_ctas - 1 - cta : cta); };
-    auto info = [&](int hu) { return unit_info(p, ws, lay, min(hu, total - 1) >> 1); };
+    auto info = [&](int hu) { return unit_info(p, ws, lay, seq_tab, min(hu, total - 1) >> 1); };
     // chunks of earlier units of this CTA; chunk j of the current one is chunk g = gc + j of the CTA's stream: stage
     // g & 1, phase g >> 1 of the barriers that come in pairs, phase g of the others
     uint32_t gc = 0;
@@ -141,7 +145,7 @@ __device__ __forceinline__ void state_half_role(const TensorMaps& maps, const Pr
             if (u.skip || is_done(hu)) continue;
             const uint8_t* rec = ws + lay.records + (static_cast<size_t>(u.c_first) * p.Hv + u.hv) * kRecBytes;
             const uint32_t u_off = kRecU + (hu & 1) * kRecUHalf;
-            const int32_t rank = (hu >> 1) / p.Hv;
+            const int32_t rank = (hu >> 1) / p.by_hv;
             int32_t pos_j = kMode == kHalfGated ? pos[0] : 0;       // fetched one chunk ahead
 #pragma unroll 1
             for (int j = 0; j < u.nc; ++j, rec += rec_stride) {

@@ -59,16 +59,15 @@ prefill_intra_first_kernel(const __grid_constant__ TensorMaps maps, const Prefil
     tc_fence_before_sync();
     __syncthreads();
     tc_fence_after_sync();
-    const uint32_t tmem = tmem_base_s;
     uint32_t n_done = 0;
 #pragma unroll 1
     for (int item = blockIdx.x; item < cut; item += gridDim.x) {
-        const int k = item / p.Hv;
+        const int k = item / p.by_hv;
         const int hv = item - k * p.Hv;
         const int c = reinterpret_cast<const int32_t*>(ws + lay.order)[k];
         const ChunkInfo ci = reinterpret_cast<const ChunkInfo*>(ws + lay.chunks)[c];
         uint8_t* rec = ws + lay.records + (static_cast<size_t>(c) * p.Hv + hv) * kRecBytes;
-        const bool ok = intra_item<false>(maps, p, rec, ci, hv / (p.Hv / p.Hqk), hv, smem, st, tmem, tid,
+        const bool ok = intra_item<false>(maps, p, rec, ci, hv / p.by_group, hv, smem, st, &tmem_base_s, 0, tid,
                                           [] { __syncthreads(); }, n_done);
         ++n_done;
         tc_fence_before_sync();
@@ -76,7 +75,7 @@ prefill_intra_first_kernel(const __grid_constant__ TensorMaps maps, const Prefil
         tc_fence_after_sync();
         if (!ok) break;
     }
-    if (warp == 0) tmem_dealloc(tmem, kIntraTmemCols);
+    if (warp == 0) tmem_dealloc(tmem_base_s, kIntraTmemCols);
 }
 
 // Second part: resident CTAs pull the items [cut, total) from a queue, in the order the chains
@@ -91,7 +90,6 @@ prefill_intra_second_kernel(const __grid_constant__ TensorMaps maps, const Prefi
     const int32_t* order = reinterpret_cast<const int32_t*>(ws + lay.order);
     const ChunkInfo* chunks = reinterpret_cast<const ChunkInfo*>(ws + lay.chunks);
     uint32_t* flags = reinterpret_cast<uint32_t*>(ws + lay.flags);
-    const int G = p.Hv / p.Hqk;
 
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
@@ -107,20 +105,19 @@ prefill_intra_second_kernel(const __grid_constant__ TensorMaps maps, const Prefi
         tc_fence_before_sync();
         __syncthreads();
         tc_fence_after_sync();
-        const uint32_t tmem = tmem_base_s;
         uint32_t n_done = 0;
         for (;;) {
             if (tid == 0) st.item = cut + atomicAdd(&hdr[kHdrItemHead], 1);
             __syncthreads();
             const int item = st.item;
             if (item >= total) break;
-            const int k = item / p.Hv;
+            const int k = item / p.by_hv;
             const int hv = item - k * p.Hv;
             const int c = order[k];
             const ChunkInfo ci = chunks[c];
             const size_t slot = static_cast<size_t>(c) * p.Hv + hv;
             uint8_t* rec = ws + lay.records + slot * kRecBytes;
-            const bool ok = intra_item<false>(maps, p, rec, ci, hv / G, hv, smem, st, tmem, tid,
+            const bool ok = intra_item<false>(maps, p, rec, ci, hv / p.by_group, hv, smem, st, &tmem_base_s, 0, tid,
                                        [] { __syncthreads(); }, n_done);
             ++n_done;
             // publish: every thread's own stores first, then the bulk stores, then the flag
@@ -137,7 +134,7 @@ prefill_intra_second_kernel(const __grid_constant__ TensorMaps maps, const Prefi
         }
         tc_fence_before_sync();
         __syncthreads();
-        if (warp == 0) tmem_dealloc(tmem, kIntraTmemCols);
+        if (warp == 0) tmem_dealloc(tmem_base_s, kIntraTmemCols);
     }
     if (blockIdx.x == 0) pdl_wait();        // the call is complete when this launch is
 }
