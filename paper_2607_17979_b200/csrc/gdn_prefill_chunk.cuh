@@ -32,7 +32,9 @@ namespace gdn {
 //   [40960, 73728)  U~  as [2 halves of dv][16 token-groups][64 dv][4 tokens] fp32, dv swizzled (rec_u_index)
 //   [73728, 73984)  e^{b_C - b_c} for c = 0..63, fp32 (rows past the chunk's length hold 1)
 //   [73984, 74240)  scale e^{b_r} for r = 0..63, fp32
-//   [74240, 74496)  e^{b_C} in the first float, rest unused
+//   [74240, 74496)  e^{b_C}, then (int32) the number of 16-token blocks that hold tokens, rest unused
+// Of a chunk with fewer than 64 tokens only the 16-token blocks that hold tokens (rows of P, token groups of U~) are
+// written, copied and read; W is zero in the others, the state pass puts zeros in U~'s place, and so U is zero there.
 // The output's first term is diag(scale e^b) Q S0^T.  Cooperative launch (kScaledQ): the record carries Qg and
 // both terms meet in one accumulator, since whatever the output warps do there comes out of the chain's issue
 // slots (32768 tokens 792 us, with raw Q 854).  Elsewhere the state pass loads the raw Q tile and scales the
@@ -48,6 +50,8 @@ constexpr uint32_t kRecEb = 73984;
 constexpr uint32_t kRecGammaC = 74240;
 constexpr uint32_t kRecBytes = 74496;
 constexpr uint32_t kRecUHalf = (kRecDecay - kRecU) / 2;
+constexpr uint32_t kRecUBlock = kRecUHalf / 4, kRecPBlock = (kRecU - kRecP) / 4;      // bytes of a 16-token block
+__device__ __forceinline__ int token_blocks(int seq_len, int chunk) { return (min(kChunk, seq_len - chunk * kChunk) + 15) >> 4; }
 // Place (in 16-byte units) of a token group and dv within one half of U~.  Odd groups have their dv swapped in fours, so
 // that a fragment read (four dv of two neighbouring groups per half warp) touches every bank once.
 __device__ __forceinline__ int rec_u_index(int group, int dv) { return group * 64 + (dv ^ ((group & 1) << 2)); }

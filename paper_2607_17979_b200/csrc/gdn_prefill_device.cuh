@@ -277,6 +277,7 @@ __device__ __forceinline__ bool intra_item(const TensorMaps& maps, const Prefill
     const uint32_t par3 = (3u * n_done) & 1u;    // parity of this item's first bar_mma phase
     const int warp = tid >> 5;
     const int colhalf = warp >> 2;                   // which 32 of the 64 accumulator columns
+    const int nb = (ci.len + 15) >> 4;               // 16-token blocks that hold tokens
     if (tid == 0) {
         if (n_done == 0) {
             mbar_init(&st.bar_tma, 1);
@@ -322,7 +323,8 @@ __device__ __forceinline__ bool intra_item(const TensorMaps& maps, const Prefill
         *reinterpret_cast<float2*>(rec + kRecDecay + 8 * lane) =
             make_float2(ex2_approx((bC - b0) * kLog2e), ex2_approx((bC - b1) * kLog2e));
         *reinterpret_cast<float2*>(rec + kRecEb + 8 * lane) = make_float2(p.scale * e0, p.scale * e1);
-        if (lane == 0) *reinterpret_cast<float*>(rec + kRecGammaC) = ex2_approx(bC * kLog2e);
+        if (lane == 0)
+            *reinterpret_cast<float2*>(rec + kRecGammaC) = make_float2(ex2_approx(bC * kLog2e), __int_as_float(nb));
     }
     sync();
     tc_fence_after_sync();
@@ -386,6 +388,8 @@ __device__ __forceinline__ bool intra_item(const TensorMaps& maps, const Prefill
         const float br2 = st.s_b2[r];
         const float rowscale = is_p ? p.scale : st.s_beta[r];      // the output scale rides on P
         const int limit = is_p ? r : r - 1;              // keep columns i <= limit
+        // (rows of a half without tokens are not read)
+        if ((row & 32) < ci.len)
 #pragma unroll
         for (int step = 0; step < 2; ++step) {
             const int cbase = colhalf * 32 + step * 16;
@@ -437,7 +441,7 @@ __device__ __forceinline__ bool intra_item(const TensorMaps& maps, const Prefill
     // Warps 0-1 invert the two diagonal 32x32 blocks of I + A (serial forward substitutions and two
     // small products each, all inside the warp), then warps 4-7 the block below them.
     if (warp < 2) {
-        solve_blocks_16_32(sA, warp, tid & 31, ci.len);
+        if (32 * warp < ci.len) solve_blocks_16_32(sA, warp, tid & 31, ci.len);
     } else if constexpr (kScaledQ) {
         // beside them the others scale the Q rows by scale * e^{b_r} in place: the Qg image
 #pragma unroll 2
@@ -502,14 +506,14 @@ __device__ __forceinline__ bool intra_item(const TensorMaps& maps, const Prefill
     sync();
 
     const uint32_t sV = smem_u32(smem + kI_V);
-    const uint32_t idesc_t = make_idesc_bf16(128, 64, true, false);
+    // the blocks that hold tokens, as columns (N) and as k-steps
+    const uint32_t idesc_t = make_idesc_bf16(128, 16 * nb, true, false);
     if (warp == 0) {     // W^T (dk x r) = K^T T_w^T with the raw K tile read MN-major
         const uint64_t dK = make_sdesc_sw128(sQK + 8192, 16384, 1024), dT = make_sdesc_sw128(smem_u32(smem + kI_Tw), 16, 1024);
-        // columns of T_w and T_u past the chunk's length are zero: their k-steps are left out
         if (elect_one()) {
 #pragma unroll
             for (int ks = 0; ks < 4; ++ks)
-                if (ks * 16 < ci.len)
+                if (ks < nb)
                     mma_ss(tW, sdesc_advance(dK, ks * 2048), sdesc_advance(dT, ks * 32), idesc_t, ks > 0);
             mma_commit(&st.bar_mma);
         }
@@ -525,9 +529,11 @@ __device__ __forceinline__ bool intra_item(const TensorMaps& maps, const Prefill
 #pragma unroll
         for (int step = 0; step < 2; ++step) {
             const int cbase = colhalf * 32 + step * 16;
-            uint32_t x[16];
-            tmem_ld16(tW + lane_base + cbase, x);
-            tmem_wait_ld();
+            uint32_t x[16] = {};            // (no tokens: W is zero there, and so U)
+            if (cbase < ci.len) {
+                tmem_ld16(tW + lane_base + cbase, x);
+                tmem_wait_ld();
+            }
 #pragma unroll
             for (int h = 0; h < 2; ++h) {
                 uint4 w;
@@ -561,11 +567,11 @@ __device__ __forceinline__ bool intra_item(const TensorMaps& maps, const Prefill
         if (elect_one()) {
 #pragma unroll
             for (int ks = 0; ks < 4; ++ks)
-                if (ks * 16 < ci.len)
+                if (ks < nb)
                     mma_ss(tU, sdesc_advance(dV, ks * 2048), sdesc_advance(dH, ks * 32), idesc_t, ks > 0);
 #pragma unroll
             for (int ks = 0; ks < 4; ++ks)
-                if (ks * 16 < ci.len)
+                if (ks < nb)
                     mma_ss(tU, sdesc_advance(dV, ks * 2048), sdesc_advance(dL, ks * 32), idesc_t, true);
             mma_commit(&st.bar_mma);
         }
@@ -578,6 +584,7 @@ __device__ __forceinline__ bool intra_item(const TensorMaps& maps, const Prefill
 #pragma unroll
         for (int step = 0; step < 2; ++step) {
             const int cbase = colhalf * 32 + step * 16;
+            if (cbase >= ci.len) break;     // (neither written nor read)
             uint32_t y[16];
             tmem_ld16(tU + lane_base + cbase, y);
             tmem_wait_ld();

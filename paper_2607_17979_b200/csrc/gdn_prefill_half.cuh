@@ -170,7 +170,7 @@ __device__ __forceinline__ void state_half_role(const TensorMaps& maps, const Pr
                         }
                     }
                 }
-                const int tok = u.seq_t0 + j * kChunk;
+                const int tok = u.seq_t0 + j * kChunk, nb = token_blocks(u.seq_len, j);
                 const int sb = g & 1;
                 uint8_t* const b_at = smem + kHS_B + sb * kHBBytes;
                 uint8_t* const a_at = smem + kHS_A + ring.st * kHABytes;
@@ -179,8 +179,8 @@ __device__ __forceinline__ void state_half_role(const TensorMaps& maps, const Pr
                 if (!(live = warp_wait(&bar_free_b[sb], ~(g >> 1) & 1u, abortp, kWaitReason))) break;
                 if (elect_one()) {
                     armed[1] = g + 1;
-                    mbar_expect_tx(&bar_full_b[sb], kRecUHalf + (kRecBytes - kRecDecay));
-                    bulk_load(b_at + kHB_U, rec + u_off, kRecUHalf, &bar_full_b[sb]);
+                    mbar_expect_tx(&bar_full_b[sb], nb * kRecUBlock + (kRecBytes - kRecDecay));
+                    bulk_load(b_at + kHB_U, rec + u_off, nb * kRecUBlock, &bar_full_b[sb]);
                     bulk_load(b_at + kHB_Vec, rec + kRecDecay, kRecBytes - kRecDecay, &bar_full_b[sb]);
                 }
                 if (!(live = warp_wait(&bar_free_a[ring.st], ring.par ^ 1u, abortp, kWaitReason))) break;
@@ -194,8 +194,8 @@ __device__ __forceinline__ void state_half_role(const TensorMaps& maps, const Pr
                 if (!(live = warp_wait(&bar_free_c[ring.st], ring.par ^ 1u, abortp, kWaitReason))) break;
                 if (elect_one()) {
                     armed[2] = g + 1;
-                    mbar_expect_tx(&bar_full_c[ring.st], kHCBytes);
-                    bulk_load(c_at + kHC_P, rec + kRecP, 8192, &bar_full_c[ring.st]);
+                    mbar_expect_tx(&bar_full_c[ring.st], 16384 + nb * kRecPBlock);
+                    bulk_load(c_at + kHC_P, rec + kRecP, nb * kRecPBlock, &bar_full_c[ring.st]);
                     tma_load_2d(c_at + kHC_K, &maps.k, u.hqk * kD, tok, &bar_full_c[ring.st]);
                     tma_load_2d(c_at + kHC_K + 8192, &maps.k, u.hqk * kD + 64, tok, &bar_full_c[ring.st]);
                 }
@@ -478,6 +478,7 @@ __device__ __forceinline__ void state_half_role(const TensorMaps& maps, const Pr
                 *reinterpret_cast<const float2*>(base + kHB_Vec + (kRecEb - kRecDecay) + 8 * lane);
             // tokens 8 b + 2 t4, + 1 of row 16 q + g8 + 8 r: token group 2 b + (t4 >> 1), see rec_u_index
             const float* sU = reinterpret_cast<const float*>(base + kHB_U) + 2 * (t4 & 1);
+            const int nb = *reinterpret_cast<const int*>(base + kHB_Vec + (kRecGammaC + 4 - kRecDecay));
 #pragma unroll
             for (int c = 0; c < 2; ++c) {
                 uint32_t x[16];
@@ -492,6 +493,9 @@ __device__ __forceinline__ void state_half_role(const TensorMaps& maps, const Pr
                     }
                 tmem_st_16x256b_x4(tmem + kH_D1 + 64 * sq + lane_base + 32 * c, x);
             }
+            // blocks without tokens were not copied: whatever was there is replaced
+#pragma unroll 1
+            for (int b = nb; b < 4; ++b) tmem_zero_16x256b_x2(tmem + kH_D1 + 64 * sq + lane_base + 16 * b);
             tmem_wait_st();
             tc_fence_before_sync();
             __syncwarp();

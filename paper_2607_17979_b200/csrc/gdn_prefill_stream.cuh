@@ -252,7 +252,7 @@ __device__ __forceinline__ void state_stream_role(const TensorMaps& maps, const 
                     }
                     if (g >= 2 && !wait_or_abort<40>(&bar_free[st], par_free, abortp)) { live = false; break; }
                     atomicMax(&armed_chunks, g + 1);
-                    const int tok = u.seq_t0 + j * kChunk;
+                    const int tok = u.seq_t0 + j * kChunk, nb = token_blocks(u.seq_len, j);
                     if (part == 0) {
                         mbar_expect_tx(&bar_full[st], kRecP - kRecW);
                         if constexpr (kScaledQ) {
@@ -263,11 +263,13 @@ __device__ __forceinline__ void state_stream_role(const TensorMaps& maps, const 
                             tma_load_2d(base + kS_Q + 8192, &maps.q, u.hqk * kD + 64, tok, &bar_full[st]);
                         }
                     } else if (part == 1) {
-                        mbar_expect_tx(&bar_full[st], kRecBytes - kRecU);
-                        bulk_load(base + kS_Rec + kRecU, rec + kRecU, kRecBytes - kRecU, &bar_full[st]);
+                        mbar_expect_tx(&bar_full[st], 2 * nb * kRecUBlock + (kRecBytes - kRecDecay));
+                        bulk_load(base + kS_Rec + kRecU, rec + kRecU, nb * kRecUBlock, &bar_full[st]);
+                        bulk_load(base + kS_Rec + kRecU + kRecUHalf, rec + kRecU + kRecUHalf, nb * kRecUBlock, &bar_full[st]);
+                        bulk_load(base + kS_Rec + kRecDecay, rec + kRecDecay, kRecBytes - kRecDecay, &bar_full[st]);
                     } else {
-                        mbar_expect_tx(&bar_full[st], kRecU - kRecP + 16384);
-                        bulk_load(base + kS_Rec + kRecP, rec + kRecP, kRecU - kRecP, &bar_full[st]);
+                        mbar_expect_tx(&bar_full[st], nb * kRecPBlock + 16384);
+                        bulk_load(base + kS_Rec + kRecP, rec + kRecP, nb * kRecPBlock, &bar_full[st]);
                         tma_load_2d(base + kS_K, &maps.k, u.hqk * kD, tok, &bar_full[st]);
                         tma_load_2d(base + kS_K + 8192, &maps.k, u.hqk * kD + 64, tok, &bar_full[st]);
                     }
@@ -625,6 +627,7 @@ __device__ __forceinline__ void state_stream_role(const TensorMaps& maps, const 
                     smem + sq * kStageBytes + kS_Rec + kRecEb + 8 * lane);
             const float4* sU = reinterpret_cast<const float4*>(smem + sq * kStageBytes + kS_Rec + kRecU +
                                                                    (odv >> 6) * kRecUHalf);
+            const int nb = *reinterpret_cast<const int*>(smem + sq * kStageBytes + kS_Rec + kRecGammaC + 4);
 #pragma unroll
             for (int c0 = 0; c0 < 64; c0 += 32) {       // eight reads in flight
                 uint32_t r[2][16];
@@ -637,6 +640,12 @@ __device__ __forceinline__ void state_stream_role(const TensorMaps& maps, const 
                 }
                 tmem_st16(tmem + kT_D1 + olane + c0, r[0]);
                 tmem_st16(tmem + kT_D1 + olane + c0 + 16, r[1]);
+            }
+            // blocks without tokens were not copied: whatever was there is replaced
+#pragma unroll 1
+            for (int b = nb; b < 4; ++b) {
+                const uint32_t zero[16] = {};
+                tmem_st16(tmem + kT_D1 + olane + 16 * b, zero);
             }
             tmem_wait_st();
             tc_fence_before_sync();

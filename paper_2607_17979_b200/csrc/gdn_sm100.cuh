@@ -261,6 +261,10 @@ __device__ __forceinline__ void tmem_st_16x256b_x4(uint32_t taddr, const uint32_
         "r"(r[15])
         : "memory");
 }
+// 16 columns of it, all zero.
+__device__ __forceinline__ void tmem_zero_16x256b_x2(uint32_t taddr) {
+    asm volatile("tcgen05.st.sync.aligned.16x256b.x2.b32 [%0], {%1,%1,%1,%1,%1,%1,%1,%1};" ::"r"(taddr), "r"(0u) : "memory");
+}
 // 16 lanes x 32-bit columns, the packed-pair counterpart: for column block i (4 columns = 8 packed values) thread t
 // gives r[2i] = lane t/4, column 4i + t%4 and r[2i+1] = lane t/4 + 8, same column.
 __device__ __forceinline__ void tmem_st_16x128b_x4(uint32_t taddr, const uint32_t (&r)[8]) {
