@@ -101,14 +101,19 @@ __device__ __forceinline__ void state_half_role(const TensorMaps& maps, const Pr
     __shared__ __align__(16) SeqEntry seq_entries[kMode == kHalfAll ? kSmallSeqs : 1];
     const SeqEntry* const seq_tab = kMode == kHalfAll && p.N <= kSmallSeqs ? seq_entries : nullptr;
     if constexpr (kMode == kHalfAll) pdl_wait();     // tables and records are the previous kernels'
-    if (seq_tab && warp > kHLoadWarp) build_seq_table(seq_entries, p, lane);
+    __shared__ int first_later;
+    if (warp > kHLoadWarp) {
+        const int v = seq_tab ? build_seq_table(seq_entries, p, lane, 2 * p.Hv, n_ctas) : 0;
+        if (lane == 0) first_later = v;
+    }
     tc_fence_before_sync();
     __syncthreads();
     tc_fence_after_sync();
     volatile int* abortp = &abort_flag;
 
-    // The i-th half unit of this CTA, or one past the end.  Every role walks this list.
-    auto at = [&](int i) { return i * n_ctas + ((i & 1) ? n_ctas - 1 - cta : cta); };
+    // Every role walks the CTA's list of half units.
+    const UnitWalk walk = {cta, n_ctas, first_later};
+    auto at = [&](int i) { return walk.at(i); };
     auto info = [&](int hu) { return unit_info(p, ws, lay, seq_tab, min(hu, total - 1) >> 1); };
     // chunks of earlier units of this CTA; chunk j of the current one is chunk g = gc + j of the CTA's stream: stage
     // g & 1, phase g >> 1 of the barriers that come in pairs, phase g of the others

@@ -50,18 +50,18 @@ prefill_state_half_kernel(const __grid_constant__ TensorMaps maps, const Prefill
 
 // Whether the state pass runs two CTAs per unit.  A half unit's chunk step takes 1.06 us against 1.40 of a whole unit's, so
 // half units win where the longest chain decides: always while every one of them has an SM of its own, and for more units
-// if the longest chain (known from the caller) is at least 1.2 times what an SM has to do on average.  On 148 SMs, whole /
-// half, us: 32 units of 64 chunks 144 / 126; 64 of 32 109 / 94; 4 sequences of 8 to 64 chunks at 32 heads (ratio 2.5) 191 / 177;
-// 520 units up to 15 chunks (1.65) 83.6 / 80.1; 320 up to 65 (1.19) 344 / 333; 448 up to 16 (0.76) 140.7 / 140.3; 4 x 32 chunks at 32
-// heads (1.15) 156 / 172; 288 units of 2 chunks (0.5) 35.1 / 38.9.  Chains of a few chunks are mostly set-up, which comes once
-// per half unit: 416 units up to 8 chunks (1.4) 55.3 / 58.3.
+// if the longest chain (known from the caller) is at least twice what an SM has to do on average, set-up of the units
+// included.  On 148 SMs (sustained, us, whole / half; ratio of the longest chain to the average of an SM): 32 units of 64 chunks
+// 144 / 126; 96 units up to 64 chunks (3.1) 171 / 151; 136 up to 37 (8.7) 80 / 66; 128 up to 4 (3.1) 22.8 / 19.7; 336 up to 32 (3.7)
+// 98 / 90.5; 256 up to 53 (2.0) 183 / 179.5; 544 up to 24 (1.75) 106.7 / 106.5; 448 up to 17 (1.4) 87 / 91; 440 up to 17 (1.3)
+// 96 / 99; 480 up to 31 (1.0) 205 / 217; 448 units of which most have one chunk, up to 9 (2.6), 41.9 / 44.6.
 static bool half_units(const ChunkedParams& cp, long long units, int sms) {
     if (2 * units <= sms) return true;
     if (cp.longest <= 0) return false;
     const long long chain = (cp.longest + kChunk - 1) / kChunk;
     // about, half a chunk lost per sequence
     const long long items = std::max((2ll * (cp.p.T / kChunk) + cp.p.N) * cp.p.Hv / 2, units);
-    return 5 * chain * sms >= 6 * items && (chain >= 10 || chain * sms >= 2 * items);
+    return chain * sms >= 2 * items + units;
 }
 
 // Prep (chunk table + sequences ranked by chunk count) is the fused path's; then the intra-chunk

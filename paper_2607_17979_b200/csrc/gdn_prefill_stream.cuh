@@ -59,9 +59,23 @@ struct SeqEntry {       // by rank
     int32_t n, c_first, nc, t0, len, slot, bad, pad;
 };
 
-// By one converged warp, N <= kSmallSeqs.  The rules are the table-building kernels': a sequence whose bounds are out of
+// Which of the rank-sorted units a CTA takes: its first one by its number, then more in passes that turn round, so that a CTA that
+// took a long one of a pass takes a short one of the next.  The CTAs whose first unit is longer than half the longest are
+// left out of the later passes where the others can do the rest in the longest one's time.
+struct UnitWalk {
+    int cta, n_ctas, first_later;       // CTAs first_later .. n_ctas - 1 walk the later passes
+    __device__ __forceinline__ int at(int i) const {       // i-th unit, or one past the end
+        if (i == 0) return cta;
+        if (cta < first_later) return 0x7fffffff;
+        const int n = n_ctas - first_later, c = cta - first_later;
+        return n_ctas + (i - 1) * n + ((i & 1) ? n - 1 - c : c);
+    }
+};
+
+// By one converged warp, N <= kSmallSeqs; returns UnitWalk::first_later for `per_seq` units a sequence.  The rules are the table-building kernels': a sequence whose bounds are out of
 // order or out of range has no chunks and is flagged; more chunks first, ties by index.
-__device__ __forceinline__ void build_seq_table(SeqEntry* tab, const PrefillParams& p, const int lane) {
+__device__ __forceinline__ int build_seq_table(SeqEntry* tab, const PrefillParams& p, const int lane, const int per_seq,
+                                               const int n_ctas) {
     SeqEntry e = {lane, 0, 0, 0, 0, lane, 0, 0};
     if (lane < p.N) {
         e.t0 = p.cu_seqlens[lane];
@@ -85,6 +99,12 @@ __device__ __forceinline__ void build_seq_table(SeqEntry* tab, const PrefillPara
         rank += (nm > e.nc || (nm == e.nc && m < lane)) ? 1 : 0;
     }
     if (lane < p.N) tab[rank] = e;
+    if (p.N * per_seq <= n_ctas) return 0;          // one pass
+    const int longest = __reduce_max_sync(0xffffffffu, e.nc);
+    const bool is_long = 2 * e.nc > longest;
+    const int n_long = __popc(__ballot_sync(0xffffffffu, is_long)) * per_seq;
+    const long long rest = static_cast<long long>(__reduce_add_sync(0xffffffffu, is_long ? 0 : e.nc)) * per_seq;
+    return n_long < n_ctas && rest <= static_cast<long long>(longest) * (n_ctas - n_long) ? n_long : 0;
 }
 
 // `tab`: that table, or null for the one in the workspace.
@@ -134,8 +154,7 @@ __device__ __forceinline__ void fence_proxy_async_all() {
     asm volatile("fence.proxy.async;" ::: "memory");
 }
 
-// The state pass of one CTA of 512 threads over the units cta, cta + n_ctas, ... of the rank-sorted
-// list.  kGated = false: every record exists (the intra-chunk kernel ran before).  true: records are being produced by
+// The state pass of one CTA of 512 threads over its share of the rank-sorted units.  kGated = false: every record exists (the intra-chunk kernel ran before).  true: records are being produced by
 // other CTAs of the same cooperative launch and the loading warps wait for each record's flag first.  `tmem` = 512 allocated
 // columns; ends with a CTA barrier.
 template <bool kGated>
@@ -187,11 +206,17 @@ __device__ __forceinline__ void state_stream_role(const TensorMaps& maps, const 
     __shared__ __align__(16) SeqEntry seq_entries[kGated ? 1 : kSmallSeqs];
     const SeqEntry* const seq_tab = !kGated && p.N <= kSmallSeqs ? seq_entries : nullptr;
     if constexpr (!kGated) pdl_wait();     // tables and records are the previous kernels'
-    if (seq_tab && warp == kStreamThreads / 32 - 1) build_seq_table(seq_entries, p, lane);
+    __shared__ int first_later;
+    if (warp == kStreamThreads / 32 - 1) {
+        const int v = seq_tab ? build_seq_table(seq_entries, p, lane, p.Hv, n_ctas) : 0;
+        if (lane == 0) first_later = v;
+    }
     tc_fence_before_sync();
     __syncthreads();
     tc_fence_after_sync();
     volatile int* abortp = &abort_flag;
+    const UnitWalk walk = {cta, n_ctas, first_later};
+    auto at = [&](int i) { return walk.at(i); };
 
     // gc = chunks of earlier units of this CTA; chunk j of the current unit is chunk g = gc + j of
     // the CTA's stream: stage g & 1, phase g >> 1 of bar_full / bar_free_* of that stage, phase g of
@@ -217,9 +242,9 @@ __device__ __forceinline__ void state_stream_role(const TensorMaps& maps, const 
             // the next unit's table entries are fetched while the current unit is processed
             UnitInfo nxt = unit_info(p, ws, lay, seq_tab, min(cta, total_units - 1));
 #pragma unroll 1
-            for (int unit = cta; unit < total_units && live; unit += n_ctas) {
+            for (int i = 0, unit = cta; unit < total_units && live; unit = at(++i)) {
                 const UnitInfo u = nxt;
-                nxt = unit_info(p, ws, lay, seq_tab, min(unit + n_ctas, total_units - 1));
+                nxt = unit_info(p, ws, lay, seq_tab, min(at(i + 1), total_units - 1));
                 if (u.skip) continue;
                 const uint8_t* records =
                     ws + lay.records + (static_cast<size_t>(u.c_first) * p.Hv + u.hv) * kRecBytes;
@@ -235,7 +260,7 @@ __device__ __forceinline__ void state_stream_role(const TensorMaps& maps, const 
                         // the record must have been published by its producer CTA
                         const uint32_t* f = flags + (static_cast<size_t>(u.c_first + j) * p.Hv + u.hv);
                         uint32_t v = 0;
-                        for (uint32_t i = 0; i < kSpinFlagLimit; ++i) {
+                        for (uint32_t k = 0; k < kSpinFlagLimit; ++k) {
                             v = ld_acquire_u32(f);
                             if (v != 0 || *abortp) break;
                             __nanosleep(64);
@@ -298,9 +323,9 @@ __device__ __forceinline__ void state_stream_role(const TensorMaps& maps, const 
             // the next unit's table entries are fetched while the current unit is processed
             UnitInfo nxt = unit_info(p, ws, lay, seq_tab, min(cta, total_units - 1));
 #pragma unroll 1
-            for (int unit = cta; unit < total_units && live; unit += n_ctas) {
+            for (int i = 0, unit = cta; unit < total_units && live; unit = at(++i)) {
                 const UnitInfo u = nxt;
-                nxt = unit_info(p, ws, lay, seq_tab, min(unit + n_ctas, total_units - 1));
+                nxt = unit_info(p, ws, lay, seq_tab, min(at(i + 1), total_units - 1));
                 if (u.skip) continue;
 #pragma unroll 1
                 for (int j = 0; j < u.nc; ++j) {
@@ -447,9 +472,9 @@ __device__ __forceinline__ void state_stream_role(const TensorMaps& maps, const 
         };
         int2 nxt = brief(cta);
 #pragma unroll 1
-        for (int unit = cta; unit < total_units; unit += n_ctas) {
+        for (int i = 0, unit = cta; unit < total_units; unit = at(++i)) {
             const int nc = nxt.x, tile = nxt.y;
-            nxt = brief(unit + n_ctas);
+            nxt = brief(at(i + 1));
             if (nc == 0) {
                 const UnitInfo u = unit_info(p, ws, lay, seq_tab, unit);
                 const size_t tile_off = (static_cast<size_t>(u.bad_slot ? 0 : u.slot) * p.Hv + u.hv) * (kD * kD) +
@@ -512,7 +537,7 @@ __device__ __forceinline__ void state_stream_role(const TensorMaps& maps, const 
             store_state_bf16();
             hand_over(&bar_s);
             // the next unit's initial state, towards L2
-            if (p.init_state && tid == 0 && nxt.x > 0 && unit + n_ctas < total_units)
+            if (p.init_state && tid == 0 && nxt.x > 0 && at(i + 1) < total_units)
                 bulk_prefetch_l2(p.init_state + static_cast<size_t>(nxt.y) * (kD * kD), kD * kD * 4);
             flush();
 #pragma unroll 1
@@ -655,9 +680,9 @@ __device__ __forceinline__ void state_stream_role(const TensorMaps& maps, const 
         bool preloaded = false;     // U~ of the chunk about to be processed is already in place
         UnitInfo nxt = unit_info(p, ws, lay, seq_tab, min(cta, total_units - 1));
 #pragma unroll 1
-        for (int unit = cta; unit < total_units; unit += n_ctas) {
+        for (int i = 0, unit = cta; unit < total_units; unit = at(++i)) {
             const UnitInfo u = nxt;
-            nxt = unit_info(p, ws, lay, seq_tab, min(unit + n_ctas, total_units - 1));
+            nxt = unit_info(p, ws, lay, seq_tab, min(at(i + 1), total_units - 1));
             if (u.skip) continue;
 #pragma unroll 1
             for (int j = 0; j < u.nc; ++j) {
@@ -667,7 +692,7 @@ __device__ __forceinline__ void state_stream_role(const TensorMaps& maps, const 
                 // k = 1: once the chain warps have read U of this chunk the accumulator is free for
                 // the next chunk's U~ (when the next chunk is known without looking past a skipped
                 // unit), which is then in place long before the chain warps hand the state over.
-                const bool ahead = j + 1 < u.nc || (unit + n_ctas < total_units && !nxt.skip);
+                const bool ahead = j + 1 < u.nc || (at(i + 1) < total_units && !nxt.skip);
 #pragma unroll 1
                 for (int k = preloaded ? 1 : 0; k < 2; ++k) {
                     if (k == 1) {
