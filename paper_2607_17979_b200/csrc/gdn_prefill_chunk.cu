@@ -10,12 +10,26 @@ namespace gdn {
 // =============================================================================================
 // kInlineTable: a batch of at most kSmallSeqs sequences needs no table-building launch in front: every warp finds the CTA's
 // chunk from cu_seqlens, a sequence a lane.
-template <bool kInlineTable>
+// Order of the CTAs. In a row (kRow) the heads of a chunk stand next to one another, so that the heads that share Q
+// and K find them in L2, and the last chunks come first, so that what the state pass opens with (the first chunks of the first
+// sequences) was written last and is still there. Against all chunks of one head after the other a call of 1337 + 512 + 199
+// tokens takes 54.3 us instead of 55.7, 57 x 144 214.5 instead of 219, 20 sequences of 1684 tokens with 16 heads 37.1 instead of 38.3. Few items run all at
+// once, find nothing that an earlier one fetched, and only ask for the same lines at the same time: there 200 tokens take 16.5
+// instead of 16.3 and 10 sequences of 376 tokens with 8 heads 15.8 instead of 15.5, so those have a grid of chunks x heads (two kernels: testing for the form inside one costs 0.1 us a call).
+template <bool kInlineTable, bool kRow>
 __global__ void __launch_bounds__(kIntraThreads, 4)
 prefill_intra_kernel(const __grid_constant__ TensorMaps maps, const PrefillParams p, uint8_t* ws,
                      const WorkspaceLayout lay) {
-    const int c = blockIdx.x;
-    const int hv = blockIdx.y;
+    const int at = static_cast<int>(blockIdx.x);
+    int c = at, hv = blockIdx.y;
+    // this CTA's item; false beyond the batch's chunks, which the host can only bound
+    const auto place = [&](int chunks) {
+        if constexpr (!kRow) return c < chunks;
+        const int item = chunks * p.Hv - 1 - at;
+        c = item / p.by_hv;
+        hv = item - c * p.Hv;
+        return item >= 0;
+    };
     __shared__ uint32_t tmem_base_s;
     const int tid = threadIdx.x, warp = tid >> 5;
     pdl_launch_dependents();
@@ -51,11 +65,11 @@ prefill_intra_kernel(const __grid_constant__ TensorMaps maps, const PrefillParam
             const int y = __shfl_up_sync(0xffffffffu, incl, d);
             if (lane >= d) incl += y;
         }
-        if (c == 0 && hv == 0 && warp == 0 &&
+        mine = place(__shfl_sync(0xffffffffu, incl, 31));
+        if (at == 0 && blockIdx.y == 0 && warp == 0 &&
             (!ok || (lane == 0 && t0 != 0) || (lane == p.N - 1 && t1 != p.T)))
             report(p.dev_status, kDevBadCuSeqlens);
         const unsigned here = __ballot_sync(0xffffffffu, c < incl && c >= incl - nc);
-        mine = here != 0;
         ci.seq = __ffs(here) - 1;
         ci.t0 = t0 + (c - (incl - nc)) * kChunk;
         ci.len = min(kChunk, t1 - ci.t0);
@@ -63,7 +77,7 @@ prefill_intra_kernel(const __grid_constant__ TensorMaps maps, const PrefillParam
         ci.len = __shfl_sync(0xffffffffu, ci.len, ci.seq & 31);
         ci.pad = 0;
     } else {
-        mine = c < *reinterpret_cast<const int32_t*>(ws);
+        mine = place(*reinterpret_cast<const int32_t*>(ws));
         if (mine) ci = reinterpret_cast<const ChunkInfo*>(ws + lay.chunks)[c];
     }
     if (!mine) {
@@ -134,10 +148,17 @@ bool prefill_tables_inline(const ChunkedParams& cp) {
 
 cudaError_t launch_prefill_intra(const TensorMaps& maps, const ChunkedParams& cp, cudaStream_t stream,
                                  bool inline_tables) {
-    auto kernel = inline_tables ? prefill_intra_kernel<true> : prefill_intra_kernel<false>;
-    cudaError_t e = ensure_dynamic_smem(kernel, kIntraSmem);
+    DeviceInfo di;
+    cudaError_t e = device_info(&di);
     if (e != cudaSuccess) return e;
-    dim3 grid(cp.lay.max_chunks, cp.p.Hv);
+    // from about two items an SM on the row of items is no slower (13 chunks x 16 heads, 22 x 16, 39 x 8: level)
+    const int64_t items = static_cast<int64_t>(cp.lay.max_chunks) * cp.p.Hv;
+    const bool row = items > 2 * di.sms;
+    auto kernel = row ? inline_tables ? prefill_intra_kernel<true, true> : prefill_intra_kernel<false, true>
+                      : inline_tables ? prefill_intra_kernel<true, false> : prefill_intra_kernel<false, false>;
+    e = ensure_dynamic_smem(kernel, kIntraSmem);
+    if (e != cudaSuccess) return e;
+    const dim3 grid = row ? dim3(static_cast<unsigned>(items)) : dim3(cp.lay.max_chunks, cp.p.Hv);
     return launch_dependent(kernel, grid, dim3(kIntraThreads), kIntraSmem, stream, maps, cp.p, cp.ws,
                             cp.lay);
 }
