@@ -93,8 +93,7 @@ struct WorkspaceLayout {
     int32_t max_chunks, max_nc;
 };
 
-constexpr int kHdrTotalChunks = 0, kHdrTotalItems = 1, kHdrItemHead = 2, kHdrUnitHead = 3,
-              kHdrSplit = 4;
+constexpr int kHdrTotalChunks = 0, kHdrTotalItems = 1, kHdrItemHead = 2, kHdrSplit = 4;
 
 inline size_t round256(size_t x) { return (x + 255) & ~static_cast<size_t>(255); }
 

@@ -232,9 +232,9 @@ template <int kId, int kThreads> __device__ __forceinline__ bool group_all(const
 
 // Same, for a whole converged warp: every lane polls, so the instruction stays warp-wide, and what ends the
 // loop is a vote, so the verdict is the same on every lane whatever each lane's poll answers: callers
-// issue warp-wide instructions on the strength of it.  (Polling by lane 0 and broadcasting the verdict costs a
-// divergent branch and a shuffle: a wait on a completed barrier took 140 cycles instead of 4, and a waiting
-// warp saw an arrival after 183 instead of 62.)
+// issue warp-wide instructions on the strength of it.  (Polling by one lane and broadcasting the verdict costs a
+// divergent branch and a shuffle, and that lane alone wakes later: a waiting warp saw an arrival after 200 cycles instead
+// of 89.)
 __device__ __forceinline__ bool warp_wait_or_abort(uint64_t* bar, uint32_t parity, volatile int* abort_flag,
                                                    const int reason = 1) {
 #pragma unroll 1

@@ -60,7 +60,6 @@ prefill_fused_prep_kernel(const int32_t* __restrict__ cu, int32_t T, int32_t N, 
     if (tid == 0) {
         running = 0;
         hdr[kHdrItemHead] = 0;
-        hdr[kHdrUnitHead] = 0;
         if (cu[0] != 0 || cu[N] != T) report(dev_status, kDevBadCuSeqlens);
     }
     __syncthreads();
@@ -277,7 +276,6 @@ prefill_small_prep_kernel(const int32_t* __restrict__ cu, int32_t T, int32_t N, 
         hdr[kHdrTotalChunks] = total;
         hdr[kHdrTotalItems] = 0;       // (the queues of the other modes are not used)
         hdr[kHdrItemHead] = 0;
-        hdr[kHdrUnitHead] = 0;
     }
 }
 

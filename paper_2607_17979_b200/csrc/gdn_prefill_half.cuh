@@ -213,7 +213,7 @@ __device__ __forceinline__ void state_half_role(const TensorMaps& maps, const Pr
         // one warp to spare
     } else if (warp >= kSIssueWarp) {
         // ===================== issuers: the whole warp waits, one elected lane issues.  An instruction takes
-        // 45-55 cycles to issue here, so the chain's products (S W^T, the state product) have a warp of their own; the other
+        // 29 cycles to issue at best, so the chain's products (S W^T, the state product) have a warp of their own; the other
         // issues the outputs' (S Q^T, U P^T), each behind a chain product's completion, so that it never runs in front of
         // the next or beside it.
         const bool outputs = warp > kSIssueWarp;
