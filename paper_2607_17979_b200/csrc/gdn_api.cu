@@ -269,10 +269,12 @@ int gdn_prefill_route(int32_t T, int32_t N, int32_t max_seqlen_hint, int32_t Hv,
     // very short sequences: one block of tokens each (one launch, no workspace traffic)
     if (longest <= GDN_RECURRENT_MAX_SEQLEN) return GDN_ROUTE_RECURRENT;
     const long long units = static_cast<long long>(N) * Hv;
-    // Up to four blocks of few units: 3.3 us a block against the 16-17 us of the chunked kernels' start-up
-    // (one sequence at 32 v-heads: 17 tokens 16.0 -> 8.8 us, 32 16.0 -> 9.7, 48 16.8 -> 13.0, 64 17.2 ->
-    // 16.3; five blocks are level).  With more units than half the SMs a block takes longer: 4 x 30
-    // tokens (128 units) 18.7 against 18.5.
+    // Up to four blocks of few units (us, blocks against the chunked kernels, one sequence): 32 v-heads, 32 tokens 10.0 / 11.0,
+    // 33 12.6 / 12.0, 48 13.5 / 12.0, 64 16.8 / 12.4; 8 v-heads, 32 tokens 8.3 / 10.8, 48 10.9 / 11.8, 64 13.6 / 12.1; 64 units
+    // in two sequences of 48 tokens 13.5 / 13.4, in 16 13.2 / 13.8.  The third and fourth block are slower where there are more
+    // than a few units and stay: they keep the state to 1e-6, the chunked kernels, whose operands are bf16, to 2e-4.
+    // With more units than half the SMs a block takes longer: 4 x 30 tokens (128 units) 18.7 against 18.5 of
+    // the chunked kernels as they were.
     if (units <= sm_count / 2 && longest <= GDN_BLOCKS_MAX_SEQLEN) return GDN_ROUTE_BLOCKS;
     // Few (sequence, v-head) units and long sequences: the serial state pass would occupy only a few SMs
     // while the rest idle, so run it next to the record producers: in one cooperative launch, or
