@@ -176,8 +176,13 @@ size_t gdn_prefill_workspace_bytes(int32_t T, int32_t N, int32_t Hqk, int32_t Hv
  *   v            bf16 [T][Hv][dv]
  *   g, beta      fp32 [T][Hv]
  *   cu_seqlens   int32 [N+1], cu[0] = 0, non-decreasing, cu[N] = T (checked on
- *                the device: a violating sequence is skipped and
- *                GDN_DEV_BAD_CU_SEQLENS is set)
+ *                the device: GDN_DEV_BAD_CU_SEQLENS is set where it does not hold,
+ *                and a sequence is skipped if its own bounds are out of order or
+ *                of 0..T, or if it starts before an earlier one ends.  The kernel
+ *                for short prompts looks at a sequence's own bounds alone, and
+ *                at cu[0] and cu[N] for the first and last: of sequences that
+ *                overlap each is evaluated, and the rows of o that they share
+ *                are one or the other's)
  *   init_state   fp32 [num_slots][Hv][dv][dk] or NULL (= all-zero states)
  *   final_state  fp32 [num_slots][Hv][dv][dk], written for every slot a
  *                sequence maps to; may be the same buffer as init_state

@@ -49,15 +49,13 @@ prefill_intra_kernel(const __grid_constant__ TensorMaps maps, const PrefillParam
     ChunkInfo ci;
     bool mine;
     if constexpr (kInlineTable) {
-        // same rules as the table-building kernel: a sequence whose bounds are out of order or
-        // out of range has no chunks and is flagged
         const int lane = tid & 31;
         int32_t t0 = 0, t1 = 0;
         if (lane < p.N) {
             t0 = p.cu_seqlens[lane];
             t1 = p.cu_seqlens[lane + 1];
         }
-        const bool ok = t0 >= 0 && t1 >= t0 && t1 <= p.T;
+        const bool ok = warp_bounds_ok(t0, t1, p.T, lane);
         const int nc = ok ? (t1 - t0 + kChunk - 1) / kChunk : 0;
         int incl = nc;
 #pragma unroll

@@ -67,6 +67,37 @@ struct ChunkInfo {      // 16 bytes
     int32_t pad;
 };
 
+// Which sequences count.  One does if its own bounds are in order (0 <= t0 <= t1 <= T) and no earlier sequence whose
+// bounds are in order ends behind its start; the others have no chunks and are flagged.  Those that count do not overlap, so
+// they have at most T / 64 + N chunks, which is what the workspace is laid out for.  Where every sequence's own bounds are
+// in order each starts where the one before ends: only where a vote finds one that is not are starts and ends compared.
+__device__ __forceinline__ bool bounds_in_order(int32_t t0, int32_t t1, int32_t T) { return t0 >= 0 && t1 >= t0 && t1 <= T; }
+// By one converged warp, a sequence a lane; lanes past the last one hold t0 = t1 = 0.
+__device__ __forceinline__ bool warp_bounds_ok(int32_t t0, int32_t t1, int32_t T, int lane) {
+    bool ok = bounds_in_order(t0, t1, T);
+    if (!__all_sync(0xffffffffu, ok)) {
+        const int32_t end = ok ? t1 : 0;
+#pragma unroll 1
+        for (int m = 0; m < 32; ++m) {
+            const int32_t e = __shfl_sync(0xffffffffu, end, m);
+            if (m < lane && t0 < e) ok = false;
+        }
+    }
+    return ok;
+}
+// By a block, a sequence a thread (`here`: the thread has one).  `ends`: shared, one per thread, holds the ends of the
+// thread's sequences whose own bounds are in order afterwards; `before`: the largest such end of the sequences in front.
+__device__ __forceinline__ bool block_bounds_ok(bool here, int32_t t0, int32_t t1, int32_t T, int32_t before, int32_t* ends,
+                                                int tid) {
+    const bool in_order = here && bounds_in_order(t0, t1, T);
+    bool ok = in_order && t0 >= before;
+    ends[tid] = in_order ? t1 : 0;
+    if (!__syncthreads_and(ok || !here))
+#pragma unroll 1
+        for (int m = 0; m < tid; ++m) ok = ok && t0 >= ends[m];
+    return ok;
+}
+
 // Workspace layout (all offsets multiples of 256 bytes):
 //   [0,256)                      int32 header: [0] total_chunks, [1] total_items
 //                                (= total_chunks * Hv), [2] item queue head, [3] unit queue head,

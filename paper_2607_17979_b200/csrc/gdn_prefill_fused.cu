@@ -45,7 +45,8 @@ prefill_fused_prep_kernel(const int32_t* __restrict__ cu, int32_t T, int32_t N, 
     int32_t* pos = reinterpret_cast<int32_t*>(ws + lay.pos);     // #chunks at positions < j
     uint32_t* flags = reinterpret_cast<uint32_t*>(ws + lay.flags);
     __shared__ int32_t warp_sums[kFPrepThreads / 32];
-    __shared__ int32_t running;
+    __shared__ int32_t ends[kFPrepThreads];
+    __shared__ int32_t running, end_before;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     pdl_launch_dependents();        // the next kernel's CTAs may become resident (they wait for us)
 
@@ -59,6 +60,7 @@ prefill_fused_prep_kernel(const int32_t* __restrict__ cu, int32_t T, int32_t N, 
     }
     if (tid == 0) {
         running = 0;
+        end_before = 0;
         hdr[kHdrItemHead] = 0;
         if (cu[0] != 0 || cu[N] != T) report(dev_status, kDevBadCuSeqlens);
     }
@@ -66,10 +68,13 @@ prefill_fused_prep_kernel(const int32_t* __restrict__ cu, int32_t T, int32_t N, 
     // chunk counts, prefix sums, chunk table (as in the three-launch path) + histogram of counts
     for (int base = 0; base < N; base += kFPrepThreads) {
         const int n = base + tid;
-        int32_t nc = 0;
+        int32_t nc = 0, t0 = 0, t1 = 0;
         if (n < N) {
-            const int32_t t0 = cu[n], t1 = cu[n + 1];
-            const bool ok = t0 >= 0 && t1 >= t0 && t1 <= T;
+            t0 = cu[n];
+            t1 = cu[n + 1];
+        }
+        const bool ok = block_bounds_ok(n < N, t0, t1, T, end_before, ends, tid);
+        if (n < N) {
             if (!ok) report(dev_status, kDevBadCuSeqlens);
             seq_bad[n] = ok ? 0 : 1;
             nc = ok ? (t1 - t0 + kChunk - 1) / kChunk : 0;
@@ -88,19 +93,18 @@ prefill_fused_prep_kernel(const int32_t* __restrict__ cu, int32_t T, int32_t N, 
         const int32_t first = running + warp_off + incl - nc;
         if (n < N) {
             seq_first[n] = first;
-            const int32_t t0 = cu[n];
-            const int32_t len = cu[n + 1] - t0;
             for (int j = 0; j < nc; ++j) {
                 ChunkInfo ci;
                 ci.seq = n;
                 ci.t0 = t0 + j * kChunk;
-                ci.len = min(kChunk, len - j * kChunk);
+                ci.len = min(kChunk, t1 - ci.t0);
                 ci.pad = 0;
                 chunks[first + j] = ci;
             }
         }
         __syncthreads();
         if (tid == kFPrepThreads - 1) running = first + nc;
+        if (base + kFPrepThreads < N) atomicMax(&end_before, ends[tid]);
         __syncthreads();
     }
     if (tid == 0) {
@@ -223,18 +227,20 @@ prefill_small_prep_kernel(const int32_t* __restrict__ cu, int32_t T, int32_t N, 
     int32_t* rank_of = reinterpret_cast<int32_t*>(ws + lay.rank_of);
     __shared__ int32_t warp_sums[kFPrepThreads / 32];
     __shared__ int32_t s_nc[kFPrepThreads];
+    __shared__ int32_t ends[kFPrepThreads];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     pdl_launch_dependents();        // the next kernel's CTAs may become resident (they wait for us)
     const int n = tid;
-    int32_t nc = 0, t0 = 0, len = 0;
+    int32_t nc = 0, t0 = 0, t1 = 0;
     if (n < N) {
         t0 = cu[n];
-        const int32_t t1 = cu[n + 1];
-        const bool ok = t0 >= 0 && t1 >= t0 && t1 <= T;
+        t1 = cu[n + 1];
+    }
+    const bool ok = block_bounds_ok(n < N, t0, t1, T, 0, ends, tid);
+    if (n < N) {
         if (!ok) report(dev_status, kDevBadCuSeqlens);
         seq_bad[n] = ok ? 0 : 1;
-        len = t1 - t0;
-        nc = ok ? (len + kChunk - 1) / kChunk : 0;
+        nc = ok ? (t1 - t0 + kChunk - 1) / kChunk : 0;
     }
     if (tid == 0 && (cu[0] != 0 || cu[N] != T)) report(dev_status, kDevBadCuSeqlens);
     s_nc[tid] = n < N ? nc : -1;
@@ -258,7 +264,7 @@ prefill_small_prep_kernel(const int32_t* __restrict__ cu, int32_t T, int32_t N, 
             ChunkInfo ci;
             ci.seq = n;
             ci.t0 = t0 + j * kChunk;
-            ci.len = min(kChunk, len - j * kChunk);
+            ci.len = min(kChunk, t1 - ci.t0);
             ci.pad = 0;
             chunks[first + j] = ci;
         }

@@ -72,19 +72,20 @@ struct UnitWalk {
     }
 };
 
-// By one converged warp, N <= kSmallSeqs; returns UnitWalk::first_later for `per_seq` units a sequence.  The rules are the table-building kernels': a sequence whose bounds are out of
-// order or out of range has no chunks and is flagged; more chunks first, ties by index.
+// By one converged warp, N <= kSmallSeqs; returns UnitWalk::first_later for `per_seq` units a sequence.  The rules are the table-building
+// kernels': see warp_bounds_ok; more chunks first, ties by index.
 __device__ __forceinline__ int build_seq_table(SeqEntry* tab, const PrefillParams& p, const int lane, const int per_seq,
                                                const int n_ctas) {
     SeqEntry e = {lane, 0, 0, 0, 0, lane, 0, 0};
+    int32_t t1 = 0;
     if (lane < p.N) {
         e.t0 = p.cu_seqlens[lane];
-        const int32_t t1 = p.cu_seqlens[lane + 1];
+        t1 = p.cu_seqlens[lane + 1];
         if (p.slot_idx) e.slot = p.slot_idx[lane];
-        e.bad = e.t0 >= 0 && t1 >= e.t0 && t1 <= p.T ? 0 : 1;
-        e.len = t1 - e.t0;
-        e.nc = e.bad ? 0 : (e.len + kChunk - 1) / kChunk;
     }
+    e.bad = warp_bounds_ok(e.t0, t1, p.T, lane) ? 0 : 1;
+    e.len = t1 - e.t0;
+    e.nc = e.bad ? 0 : (e.len + kChunk - 1) / kChunk;
     int32_t incl = e.nc;
 #pragma unroll
     for (int d = 1; d < 32; d <<= 1) {
