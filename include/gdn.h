@@ -190,7 +190,11 @@ size_t gdn_prefill_workspace_bytes(int32_t T, int32_t N, int32_t Hqk, int32_t Hv
  *                no state written); >= num_slots the same + GDN_DEV_BAD_SLOT
  *   o            bf16 [T][Hv][dv], written
  *   max_seqlen_hint  an upper bound on the longest sequence if the caller
- *                knows one, else 0; only steers launch geometry, never results
+ *                knows one, else 0.  It picks kernels (routes below, and the form
+ *                of the state pass), whose results differ by rounding; with a
+ *                wrong one they are as right, only slower: give a tight one (a
+ *                bound that T tokens in N sequences cannot reach counts as 0; one
+ *                several times too large has cost up to 11 %)
  *   workspace    device scratch of at least gdn_prefill_workspace_bytes(...)
  *                bytes, 256-byte aligned; contents are scratch before and after
  * T == 0 or N == 0 is a no-op that returns 0.
@@ -272,8 +276,9 @@ int gdn_prefill_fused(const void* q, const void* k, const void* v,
  * v-head) units and streams their chunks without draining its pipeline
  * between units.  Where the longest chain decides the time a unit is
  * shared by two CTAs, half of the state's rows each: with at most half as many
- * units as SMs, or when max_seqlen_hint tells of a chain that long (the two
- * forms agree to the rounding of fp32 sums).  Arguments, workspace and results are gdn_prefill_chunked's.
+ * units as SMs, or when max_seqlen_hint tells of a chain at least twice as long
+ * as what an SM has to do on average (the two forms agree to the rounding of
+ * fp32 sums).  Arguments, workspace and results are gdn_prefill_chunked's.
  */
 int gdn_prefill_stream(const void* q, const void* k, const void* v,
                        const float* g, const float* beta, const int32_t* cu_seqlens,

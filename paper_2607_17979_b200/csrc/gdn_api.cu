@@ -207,7 +207,7 @@ int prefill_chunked_impl(PrefillRoute route, const void* q, const void* k, const
     p.dev_status = dev_status;
     cp.ws = static_cast<uint8_t*>(workspace);
     cp.lay = gdn::workspace_layout(T, N, Hv);
-    cp.longest = max_seqlen_hint > 0 ? std::min(max_seqlen_hint, T) : N == 1 ? T : 0;
+    cp.longest = gdn::known_longest(T, N, max_seqlen_hint);
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     return cuda_status(route == kRouteFused     ? gdn::launch_prefill_fused(cp, st)
                        : route == kRouteStream  ? gdn::launch_prefill_stream(cp, st)

@@ -155,8 +155,15 @@ struct ChunkedParams {
     PrefillParams p;
     uint8_t* ws;
     WorkspaceLayout lay;
-    int32_t longest = 0;      // tokens of the longest sequence as far as the caller has told, 0: not known (picks kernels only)
+    int32_t longest = 0;      // known_longest(): picks kernels only
 };
+
+// Tokens of the longest sequence as far as the host can know them, 0: not at all.  The caller's bound counts only if T tokens
+// in N sequences can reach it (empty ones aside): one beyond, a model's context length for example, tells nothing.
+inline int32_t known_longest(int32_t T, int32_t N, int32_t max_seqlen_hint) {
+    if (N == 1) return T;
+    return max_seqlen_hint > 0 && max_seqlen_hint <= T - (N - 1) ? max_seqlen_hint : 0;
+}
 
 cudaError_t launch_prefill_chunked(const ChunkedParams& cp, cudaStream_t stream);
 // One cooperative launch: some CTAs produce the records, the others run the state pass behind them.

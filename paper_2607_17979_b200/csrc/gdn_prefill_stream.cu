@@ -49,18 +49,21 @@ prefill_state_half_kernel(const __grid_constant__ TensorMaps maps, const Prefill
 }
 
 // Whether the state pass runs two CTAs per unit.  A half unit's chunk step takes 1.06 us against 1.40 of a whole unit's, so
-// half units win where the longest chain decides: always while every one of them has an SM of its own, and for more units
-// if the longest chain (known from the caller) is at least twice what an SM has to do on average, set-up of the units
-// included.  On 148 SMs (sustained, us, whole / half; ratio of the longest chain to the average of an SM): 32 units of 64 chunks
-// 144 / 126; 96 units up to 64 chunks (3.1) 171 / 151; 136 up to 37 (8.7) 80 / 66; 128 up to 4 (3.1) 22.8 / 19.7; 336 up to 32 (3.7)
-// 98 / 90.5; 256 up to 53 (2.0) 183 / 179.5; 544 up to 24 (1.75) 106.7 / 106.5; 448 up to 17 (1.4) 87 / 91; 440 up to 17 (1.3)
-// 96 / 99; 480 up to 31 (1.0) 205 / 217; 448 units of which most have one chunk, up to 9 (2.6), 41.9 / 44.6.
-static bool half_units(const ChunkedParams& cp, long long units, int sms) {
+// half units win where the longest chain decides: always while every one of them has an SM of its own (32 units of 64
+// chunks 144 us whole, 126 half), and for more units if the longest chain is at least twice what an SM has to do on
+// average, set-up of the units included (128 units, longest chain 3.1 times the average 22.8 / 19.7; 2.0 times 183 / 179.5,
+// 1.75 times 106.7 / 106.5, once 205 / 217).
+// The longest chain is the caller's word.  If that bound is far too large, whole units would have been faster by 5 to 11 %
+// (57 x 144 tokens at 32 heads 216 us, half 240; 15 x 546 185 / 197; 30 x 300 at 8 heads 55.7 / 61.4).  The device knows
+// better, but a kernel that holds both forms and chooses costs every call of more units 2 us (1337 + 512 + 199 tokens
+// 57.4 -> 59.8).
+static bool half_units(int32_t T, int32_t N, int32_t Hv, int32_t longest, int sms) {
+    const long long units = static_cast<long long>(N) * Hv;
     if (2 * units <= sms) return true;
-    if (cp.longest <= 0) return false;
-    const long long chain = (cp.longest + kChunk - 1) / kChunk;
+    if (longest <= 0) return false;
+    const long long chain = (longest + kChunk - 1) / kChunk;
     // about, half a chunk lost per sequence
-    const long long items = std::max((2ll * (cp.p.T / kChunk) + cp.p.N) * cp.p.Hv / 2, units);
+    const long long items = std::max((2ll * (T / kChunk) + N) * Hv / 2, units);
     return chain * sms >= 2 * items + units;
 }
 
@@ -88,7 +91,7 @@ cudaError_t launch_prefill_stream(const ChunkedParams& cp, cudaStream_t stream) 
         e = launch_prefill_intra(maps, cp, stream, inline_tables);
         if (e != cudaSuccess) return e;
     }
-    if (half_units(cp, units, sms)) {
+    if (half_units(p.T, p.N, p.Hv, cp.longest, sms)) {
         const int grid = static_cast<int>(2 * units < sms ? 2 * units : sms);
         return launch_dependent(prefill_state_half_kernel, dim3(grid), dim3(kStreamThreads), kHalfSmem, stream, maps, p,
                                 cp.ws, cp.lay);
