@@ -210,28 +210,26 @@ int gdn_prefill(const void* q, const void* k, const void* v,
                 int32_t* dev_status, void* stream);
 
 /*
- * gdn_prefill routes by shape: a batch whose longest sequence has at most
+ * gdn_prefill routes by shape.  A batch whose longest sequence has at most
  * GDN_RECURRENT_MAX_SEQLEN tokens (by max_seqlen_hint if given, else by the
  * bound T) goes to gdn_prefill_recurrent's kernel (GDN_ROUTE_RECURRENT), and
  * so do a few sequence-heads of up to GDN_BLOCKS_MAX_SEQLEN tokens
  * (GDN_ROUTE_BLOCKS: the same kernel with the next block's tokens staged beside
- * the current block).  Anything longer is a matter of chunks.  GDN_ROUTE_FUSED
- * (a few long sequence-heads) and GDN_ROUTE_OVERLAP (max_seqlen_hint tells of
- * chains of at least 40 chunks and the sequence-heads number at most half of
- * the SMs, unless they are at most a third and at most a quarter of the SMs'
- * worth of them is alive beside the longest on average) name batches whose
- * serial chains leave most of the machine idle: gdn_prefill runs those as
- * gdn_prefill_overlap does where producing the records beside the chains pays
- * for its two launches more, else as gdn_prefill_stream does;
- * gdn_prefill_fused's cooperative launch is slower on every shape and
- * runs where it is called by name.  GDN_ROUTE_STREAM, everything else, is
- * gdn_prefill_stream.  Each entry point can also be called
- * directly; arguments are gdn_prefill's.  gdn_prefill_chunked is the three
- * launches under their older name: it runs gdn_prefill_stream.
- * gdn_prefill_route answers which of these a batch is (host-only
- * arithmetic on the shapes; sm_count and cooperative_launch describe the
- * device, gdn_prefill itself queries them): one of GDN_ROUTE_* (never
- * GDN_ROUTE_CHUNKED any more), or GDN_ROUTE_NONE for an empty batch.
+ * the current block).  Anything longer is a matter of chunks: GDN_ROUTE_OVERLAP
+ * is gdn_prefill_overlap, taken where a few long chains leave SMs free and the
+ * work hidden beside them outweighs that route's two more launches;
+ * GDN_ROUTE_STREAM, everything else, is gdn_prefill_stream.  Each entry point
+ * can also be called directly; arguments are gdn_prefill's.  By name only:
+ * gdn_prefill_chunked, the three launches under their older name, which runs
+ * gdn_prefill_stream, and gdn_prefill_fused, whose cooperative launch was slower
+ * than the route taken on every shape tried but has nothing wait for a later
+ * launch.
+ * gdn_prefill_route answers which route gdn_prefill takes (host-only
+ * arithmetic on the shapes; sm_count describes the device, gdn_prefill itself
+ * queries it; cooperative_launch is no longer looked at): one of GDN_ROUTE_*
+ * (never GDN_ROUTE_CHUNKED or GDN_ROUTE_FUSED any more), or GDN_ROUTE_NONE for
+ * an empty batch.  (With CUDA_LAUNCH_BLOCKING set GDN_ROUTE_OVERLAP runs as
+ * GDN_ROUTE_STREAM does.)
  */
 #define GDN_RECURRENT_MAX_SEQLEN 16
 #define GDN_BLOCKS_MAX_SEQLEN 64

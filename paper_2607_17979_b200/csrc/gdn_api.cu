@@ -261,8 +261,30 @@ int gdn_prefill_overlap(const void* q, const void* k, const void* v, const float
                                 workspace, workspace_bytes, dev_status, stream, split_permille);
 }
 
+namespace {
+// Whether the records are produced in two parts, the second beside the chains, or all of them first.  Two parts cost about 13 us
+// (the tables with the processing order, two more launches) and hide the intra-chunk kernel's time, which grows with the items,
+// as far as the SMs that hold no half unit keep up.  So what decides is the number of (chunk, v-head) items against the
+// units, and where their lengths differ, half of the units that have ended on average count as gone (`live`; all count
+// without a bound on the longest).  The line was fitted to 1351 drawn batches of 2 to 70 units, 20 to 320 chunks and up to
+// 12000 items, equal and unequal, each timed in both forms: the rule takes 0.12 % more time than the faster form each time,
+// three launches always 5.3 %.  Us in three launches / in two parts on 148 SMs, one sequence: 8 units of 60 chunks 83.7 / 92.2,
+// of 120 158.2 / 159.6, of 240 305.8 / 293.7; 32 of 38 76.3 / 76.8, of 50 96.0 / 91.2, of 320 564 / 428; 48 of 50 115.2 / 119.2, of
+// 100 225.6 / 220.4; 64 of 40 115.0 / 123.1.  64 units in two sequences, 64 chunks both 182 / 185.5, 86 and 28 180.8 / 174.7;
+// 70 units, 60 chunks and six times 30 126.9 / 138.0.
+bool two_parts_pay(int32_t T, int32_t N, int32_t max_seqlen_hint, int32_t Hv, int32_t sms) {
+    const long long units = static_cast<long long>(N) * Hv;
+    if (2 * units > sms - gdn::kOverlapSpareSms) return false;      // (gdn_prefill_overlap would run the three launches)
+    const long long items = (2ll * (T / gdn::kChunk) + N) * Hv / 2;     // about, half a chunk lost per sequence
+    const long long chain = (gdn::known_longest(T, N, max_seqlen_hint) + gdn::kChunk - 1) / gdn::kChunk;
+    const long long live = chain > 0 ? std::min(units, (items + chain - 1) / chain) : units;
+    return items >= 17 * sms / 2 + 55 * std::max(0ll, units + live - 46 * sms / 100);
+}
+}  // namespace
+
 int gdn_prefill_route(int32_t T, int32_t N, int32_t max_seqlen_hint, int32_t Hv, int32_t sm_count,
                       int32_t cooperative_launch) {
+    (void)cooperative_launch;       // no route launches cooperatively
     if (T <= 0 || N <= 0 || Hv <= 0 || sm_count <= 0) return GDN_ROUTE_NONE;
     // the length is known on the host only through the caller's hint or the bound T
     const int32_t longest = (max_seqlen_hint > 0 && max_seqlen_hint < T) ? max_seqlen_hint : T;
@@ -276,63 +298,8 @@ int gdn_prefill_route(int32_t T, int32_t N, int32_t max_seqlen_hint, int32_t Hv,
     // With more units than half the SMs a block takes longer: 4 x 30 tokens (128 units) 18.7 against 18.5 of
     // the chunked kernels as they were.
     if (units <= sm_count / 2 && longest <= GDN_BLOCKS_MAX_SEQLEN) return GDN_ROUTE_BLOCKS;
-    // Few (sequence, v-head) units and long sequences: the serial state pass would occupy only a few SMs
-    // while the rest idle, so run it next to the record producers: in one cooperative launch, or
-    // in two parts.  What decides is the longest chain and how many chains are alive beside it on average
-    // (equal sequences: all units).  Without a hint the longest of several sequences is taken to hold
-    // half of the tokens.
-    const bool known = max_seqlen_hint > 0 || N == 1;
-    const int32_t chain = known ? longest : std::max(T / 2, 1);
-    const int32_t live =
-        static_cast<int32_t>(std::min(std::min(units, static_cast<long long>(T) * Hv / chain), static_cast<long long>(sm_count)));
-    // The cooperative launch starts ~10 us later (two table launches, one CTA per SM) and gains what the
-    // intra-chunk kernel would have taken alone, which grows with the chains, until at a quarter
-    // of the SMs the producing CTAs no longer keep up with them.  Chunks at which three launches are level
-    // with it on 148 SMs, measured / by the rule: 4 chains 45 / 41, 8 38 / 38, 12 33 / 35, 16 30 / 32, 20
-    // 28 / 29, 24 26 / 26, 28 22 / 23, 32 23 / 23, 36 26 / 25, 40 29 / 30, 44 49 / 50, 48 none / none.  Either
-    // side of a line: 32 chains of 18 chunks 51.8 us in three launches, 56.7 in one; 30 chunks 80.0 and
-    // 74.6.
-    const int32_t level = std::max({23, 3 * sm_count / 10 - 3 * live / 4, 23 + 6 * (live - sm_count * 9 / 40) / 7,
-                                    30 + 5 * (live - sm_count * 11 / 40)});
-    // Two parts: long chains that leave at least half of the SMs free from the start, the length known
-    // through the caller's hint (two chains of 32 chunks at 32 heads were 4 % slower than three launches,
-    // hence 40).  That route wants two launches to run side by side, which the device does but CUDA
-    // does not promise; if they do not, its last launch finishes the work (same results,
-    // milliseconds lost), so choosing it is safe.  Batches that fill the machine at first and free it as their short
-    // chains end would gain 5-12 %, but the records produced late are still dirty in L2 when the call
-    // ends and their write-back falls into whatever runs next, and batches of equal chains lose up
-    // to 7 %: those stay with the persistent pass.
-    const bool two_part = max_seqlen_hint > 0 && units <= sm_count / 2 && longest >= 40 * gdn::kChunk;
-    // Between the two: up to a quarter of the SMs alive the cooperative launch is ahead (36 chains of 90 chunks 185
-    // us, in two parts 188; 6 sequences of 60 chunks and less at 8 heads, 19 alive, 121 and 131), beyond it
-    // the two parts are (40 chains of 70 chunks 167 and 155, 48 of 64 192 and 151).
-    const bool few = cooperative_launch && units <= sm_count / 3;
-    if (few && chain > level * gdn::kChunk &&
-        (live <= sm_count / 4 || (units <= 3 * sm_count / 10 && !two_part)))
-        return GDN_ROUTE_FUSED;
-    if (two_part && !(few && live <= sm_count / 4)) return GDN_ROUTE_OVERLAP;
-    // Everything else: the three launches (table kernel, or none for small batches; the intra-chunk
-    // kernel over all items; the persistent state pass).
-    return GDN_ROUTE_STREAM;
+    return two_parts_pay(T, N, max_seqlen_hint, Hv, sm_count) ? GDN_ROUTE_OVERLAP : GDN_ROUTE_STREAM;
 }
-
-namespace {
-// Few long chains (GDN_ROUTE_FUSED, GDN_ROUTE_OVERLAP): whether their records are produced in two parts, the second beside the
-// chains, or all of them first.  The two parts cost 13 us (the tables with the processing order, two more launches)
-// and hide the intra-chunk kernel's time, which grows with the items, as far as the SMs that the chains leave free keep up:
-// two for each live chain are taken.  us in three launches / in two parts, equal chains on 148 SMs: 4 chains of 128
-// chunks 165 / 176; 8 of 80 115 / 121, of 128 176 / 177; 16 of 56 92 / 95, of 80 131 / 121; 24 of 40 76 / 76, of 56 107 / 95; 32 of 32
-// 68 / 70, of 40 86 / 80, of 512 923 / 640; 40 of 32 76 / 77, of 56 123 / 116; 48 of 56 132 / 132, of 128 280 / 261; 64 of 128 324 / 384.  (The
-// cooperative launch: 4 of 56 99 against 77, 8 of 128 204 against 176, 32 of 128 211 against 189.)
-bool two_parts_pay(int32_t T, int32_t N, int32_t max_seqlen_hint, int32_t Hv, int32_t sms) {
-    const long long units = static_cast<long long>(N) * Hv;
-    const int32_t longest = (max_seqlen_hint > 0 && max_seqlen_hint < T) ? max_seqlen_hint : T;
-    const long long chain = max_seqlen_hint > 0 || N == 1 ? longest : std::max(T / 2, 1);      // as in gdn_prefill_route
-    const long long live = std::min(units, static_cast<long long>(T) * Hv / chain);
-    const long long level = 1050 + 150 * std::max(0ll, live - sms / 4);
-    return live <= sms * 7 / 20 && live * chain >= level * gdn::kChunk;
-}
-}  // namespace
 
 int gdn_prefill(const void* q, const void* k, const void* v, const float* g, const float* beta,
                 const int32_t* cu_seqlens, const float* init_state, float* final_state,
@@ -340,13 +307,9 @@ int gdn_prefill(const void* q, const void* k, const void* v, const float* g, con
                 int32_t Hqk, int32_t Hv, int32_t dk, int32_t dv, int32_t chunk,
                 int32_t num_slots, float scale, void* workspace, size_t workspace_bytes,
                 int32_t* dev_status, void* stream) {
-    int sms = 148, coop = 0;
     gdn::DeviceInfo di;
-    if (gdn::device_info(&di) == cudaSuccess) {
-        sms = di.sms;
-        coop = di.cooperative;
-    }
-    const int route_id = gdn_prefill_route(T, N, max_seqlen_hint, Hv, sms, coop);
+    const int sms = gdn::device_info(&di) == cudaSuccess ? di.sms : 148;
+    const int route_id = gdn_prefill_route(T, N, max_seqlen_hint, Hv, sms, 0);
     if (chunk == gdn::kChunk && (route_id == GDN_ROUTE_RECURRENT || route_id == GDN_ROUTE_BLOCKS)) {
         // same validation of the workspace arguments as the chunked route, so that a call does
         // not start failing when its batch grows
@@ -364,10 +327,7 @@ int gdn_prefill(const void* q, const void* k, const void* v, const float* g, con
                                       slot_idx, o, T, N, Hqk, Hv, dk, dv, num_slots, scale, longest,
                                       dev_status, stream);
     }
-    const PrefillRoute route = (route_id == GDN_ROUTE_FUSED || route_id == GDN_ROUTE_OVERLAP) &&
-                                       two_parts_pay(T, N, max_seqlen_hint, Hv, sms)
-                                   ? kRouteOverlap
-                                   : kRouteStream;
+    const PrefillRoute route = route_id == GDN_ROUTE_OVERLAP ? kRouteOverlap : kRouteStream;
     return prefill_chunked_impl(route, q, k, v, g, beta, cu_seqlens, init_state,
                                 final_state, slot_idx, o, T, N, max_seqlen_hint, Hqk, Hv, dk, dv, chunk, num_slots,
                                 scale, workspace, workspace_bytes, dev_status, stream);

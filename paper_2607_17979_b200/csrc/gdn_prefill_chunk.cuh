@@ -178,6 +178,8 @@ cudaError_t launch_prefill_stream(const ChunkedParams& cp, cudaStream_t stream);
 // launch); 2: + the cut of the two-part production (split_permille < 0: the kernel's own model).
 cudaError_t launch_prefill_ranked_prep(const ChunkedParams& cp, cudaStream_t stream, int mode,
                                        int split_permille = -1, int sms = 0);
+// SMs that a batch in two parts must leave to the producers of the second part, one half unit an SM.
+constexpr int kOverlapSpareSms = 8;
 // The intra-chunk kernel in two parts around a flag-gated state pass of two CTAs per unit: the second part
 // of the records is produced beside the chains, on the SMs the state pass leaves free.  (The three launches where it
 // leaves too few.)

@@ -33,8 +33,6 @@
 
 namespace gdn {
 
-constexpr int kOverlapSpareSms = 8;
-
 // First part: resident CTAs over the items [0, cut) of the processing order.  (With one CTA per item the grid has to be
 // sized for all of them, the cut being known on the device only, and the CTAs that find nothing to do leave at 4 ns each:
 // 32768 tokens at 32 heads, a fifth of the items first, 52 us of nothing else.)

@@ -109,23 +109,20 @@ def test_prefill_routing_rules_are_pure_host_arithmetic():
     assert r(17, 1, 0, 32) != "recurrent" and r(4000, 400, 17, 8) != "recurrent"
     # a hint larger than T is ignored
     assert r(10, 1, 5000, 32) == "recurrent"
-    # few long units: one cooperative launch, if the device can
-    assert r(32768, 1, 0, 32) == "fused" and r(32768, 1, 0, 32, 148, False) == "stream"
-    assert r(1473, 1, 0, 32) == "fused" and r(1472, 1, 0, 32) == "stream"
-    assert r(32768, 1, 0, 44) == "fused" and r(32768, 1, 0, 45) == "stream"       # 3 * 148 // 10 = 44 units
+    # few long chains: the two-part production from a number of (chunk, v-head) items on, whether the
+    # length is told or (one sequence) known, and whatever is said about cooperative launches
+    assert r(32768, 1, 0, 32) == "overlap" and r(32768, 1, 0, 32, 148, False) == "overlap"
+    assert r(2496, 1, 0, 32) == "overlap" and r(2495, 1, 0, 32) == "stream"
+    assert r(32768, 1, 0, 70) == "overlap" and r(32768, 1, 0, 71) == "stream"     # (148 - 8) / 2 = 70 units
     # everything else that is chunked: the three launches with the persistent state pass
     assert r(7680, 4, 0, 32) == "stream" and r(129, 1, 0, 32) == "stream"
     assert r(128, 1, 0, 32) == "stream" and r(400, 4, 100, 32) == "stream"
     assert r(1600, 16, 100, 4) == "stream" and r(1700, 17, 100, 4) == "stream"
     assert r(8192, 128, 64, 32) == "stream" and r(296, 37, 8, 4) == "recurrent"
     assert r(1184, 37, 32, 4) == "stream" and r(1216, 38, 32, 4) == "stream"
-    # the caller says how long the longest sequence is, chains of at least 40 chunks, more units
-    # than the cooperative launch takes and at most half as many as SMs: the two-part production
-    assert r(8192, 2, 4096, 32) == "overlap" and r(4000, 2, 3000, 32) == "overlap"
-    assert r(8192, 2, 0, 32) == "stream" and r(5118, 2, 2559, 32) == "stream"
-    assert r(8192, 2, 4096, 37) == "overlap" and r(8192, 2, 4096, 38) == "stream"   # 74 / 76 units
-    assert r(8192, 2, 4096, 18) == "fused" and r(8192, 2, 4096, 19) == "overlap"    # 36 / 38 units
-    assert r(8192, 2, 6144, 24) == "fused" and r(8192, 2, 6144, 25) == "overlap"    # 32 chains alive of 48 / 50
     assert r(7680, 4, 4096, 32) == "stream" and r(6144, 3, 2048, 32) == "stream"
+    # two sequences of 32 heads: equal ones stay, unequal ones go if their length is told
+    assert r(8192, 2, 4096, 32) == "stream" and r(8192, 2, 6144, 32) == "overlap"
+    assert r(8192, 2, 0, 32) == "stream" and r(8192, 2, 8192, 32) == "stream" and r(4000, 2, 3000, 32) == "stream"
     # the thresholds follow the SM count given
     assert r(1184, 37, 32, 4, 100) == "stream"

@@ -181,7 +181,7 @@ def test_host_buffer_prefill_behind_the_two_part_route():
     back to the host follows the last launch.  Five calls in a row, each compared bit for bit with
     the device entry point."""
     from paper_2607_17979_b200 import api
-    lens = [2700, 2600]
+    lens = [5200, 2600]
     p = I.prefill_inputs(lens, 16, 32, seed=21, init="zero")
     T, N = p["T"], p["N"]
     assert api.gdn_prefill_route(T, N, max(lens), 32) == "overlap"
