@@ -240,7 +240,8 @@ __device__ __forceinline__ bool warp_wait_or_abort(uint64_t* bar, uint32_t parit
 #pragma unroll 1
     for (uint32_t i = 0; i < kSpinLimit; ++i) {
         if (__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) return true;
-        if ((i & 255u) == 0u && __any_sync(0xffffffffu, *abort_flag)) return false;
+        // (a poll that fails has blocked for some microseconds)
+        if ((i & 7u) == 0u && __any_sync(0xffffffffu, *abort_flag)) return false;
     }
     if (*abort_flag == 0) *abort_flag = reason;      // keep an earlier, different reason
     return false;

@@ -62,6 +62,7 @@ prefill_fused_prep_kernel(const int32_t* __restrict__ cu, int32_t T, int32_t N, 
         running = 0;
         end_before = 0;
         hdr[kHdrItemHead] = 0;
+        hdr[kHdrStarted] = 0;
         if (cu[0] != 0 || cu[N] != T) report(dev_status, kDevBadCuSeqlens);
     }
     __syncthreads();

@@ -39,9 +39,11 @@ constexpr uint32_t kHalfSmem = kHS_Out + 8192 + 1024;
 // TMEM columns: S W^T (two tiles), S Q^T, U P^T, the state product, bf16 S, decayed U (hi / lo lanes), U
 constexpr uint32_t kH_D1 = 0, kH_Y1 = 128, kH_Y2 = 192, kH_D4 = 256, kH_S = 384, kH_Us = 448, kH_U = 480;
 
-// a few milliseconds: far longer than the producers ever lag when they do run beside the state
-// pass, far shorter than the other roles' mbarrier waits (which would report an error)
-constexpr uint32_t kSpinFlagLimitSoft = 1u << 13;
+// Polls of a record's flag, about half a microsecond each.  A few milliseconds: far longer than the producers ever lag when
+// they do run beside the state pass, far shorter than the other roles' mbarrier waits (which would report an error).  And
+// how long to wait if they have not even started: two launches in a row start within some ten microseconds of each other, and
+// what is lost by giving up too early is no more than the chain has done so far.
+constexpr uint32_t kSpinFlagLimitSoft = 1u << 13, kSpinStartLimit = 1u << 8;
 
 // Which records exist when the state pass starts.
 enum HalfMode {
@@ -141,6 +143,8 @@ __device__ __forceinline__ void state_half_role(const TensorMaps& maps, const Pr
         (void)flags;
         (void)pos;
         (void)cut;
+        uint32_t started = 0;           // (kHalfGated) the producers have been seen to run
+        (void)started;
         bool live = true;
         UnitInfo nxt = info(at(0));
 #pragma unroll 1
@@ -166,6 +170,10 @@ __device__ __forceinline__ void state_half_role(const TensorMaps& maps, const Pr
                         for (uint32_t k = 0; k < kSpinFlagLimitSoft; ++k) {
                             v = __shfl_sync(0xffffffffu, ld_acquire_u32(f), 0);
                             if (v != 0 || __any_sync(0xffffffffu, *abortp)) break;
+                            if (k >= kSpinStartLimit && !started) {
+                                started = __shfl_sync(0xffffffffu, ld_acquire_u32(reinterpret_cast<const uint32_t*>(ws) + kHdrStarted), 0);
+                                if (!started) break;
+                            }
                             __nanosleep(64);
                         }
                         if (v != 1) {
@@ -392,6 +400,8 @@ __device__ __forceinline__ void state_half_role(const TensorMaps& maps, const Pr
                 bulk_prefetch_l2(p.init_state + static_cast<size_t>(nxt.y) * (kHalfRows * kD), kHalfRows * kD * 4);
 #pragma unroll 1
             for (int j = 0; j < nc; ++j) {
+                // (left to the last launch: the rest of the half unit would be a failing wait after another)
+                if (kMode == kHalfGated && !ok) break;
                 const uint32_t g = gc + j;
                 const int st = g & 1;
                 const uint8_t* vec = smem + kHS_B + st * kHBBytes + kHB_Vec;
@@ -530,9 +540,15 @@ __device__ __forceinline__ void state_half_role(const TensorMaps& maps, const Pr
                     preload(g + k);
                 }
                 preloaded = ahead;
-                // every warp runs both group barriers of every chunk, also after a failed wait
+                // Every warp runs both group barriers of every chunk, also after a failed wait; where that is no error they
+                // leave together at the first.
                 if (ot == 0) bulk_wait_read_all();       // the last chunk's rows have left the staging tile
-                out_sync();
+                if constexpr (kMode == kHalfGated) {
+                    ok = group_all<1, kSOutThreads>(ok);
+                    if (!ok) break;
+                } else {
+                    out_sync();
+                }
                 await(&bar_y[buf], (g >> 1) & 1u);
                 // The rows are made once the chain warps have handed the next state over and wait behind the next product: beside
                 // the refresh they take its issue slots (4096 tokens at 8 v-heads 91.5 us, 88.3 this way).

@@ -21,12 +21,12 @@
 //                 for the state pass at its very end, so that the completion of this launch
 //                 implies the state pass's.
 //   rest          an ordinary launch.  CUDA lets a programmatic dependent start early, it does not
-//                 promise to; if the second part did not run beside the state pass, the state
-//                 pass's waits for records ran out (soon, and without an error: a half unit's final
-//                 state is written only after its last record has been loaded, so an unfinished
-//                 one has left its initial state alone), it marked the half units it finished, and
-//                 this launch runs the others now that every record exists.  Normally every CTA finds
-//                 its half unit done and returns at once.
+//                 promise to; if the second part has not started when a chain has waited for a record for 0.1 ms or so,
+//                 the chain gives up (without an error: a half unit's final state is written only after
+//                 its last record has been loaded, so an unfinished one has left its initial state
+//                 alone), the half units that were finished are marked, and this launch runs the others now that
+//                 every record exists.  Normally every CTA finds its half unit done and returns at
+//                 once.
 #include "gdn_prefill_half.cuh"
 #include <algorithm>
 #include <cstdlib>
@@ -84,6 +84,7 @@ __global__ void __launch_bounds__(kIntraThreads, 4)
 prefill_intra_second_kernel(const __grid_constant__ TensorMaps maps, const PrefillParams p,
                             uint8_t* ws, const WorkspaceLayout lay) {
     int32_t* hdr = reinterpret_cast<int32_t*>(ws);
+    if (blockIdx.x == 0 && threadIdx.x == 0) st_release_u32(reinterpret_cast<uint32_t*>(hdr + kHdrStarted), 1u);
     const int32_t cut = hdr[kHdrSplit], total = hdr[kHdrTotalItems];
     const int32_t* order = reinterpret_cast<const int32_t*>(ws + lay.order);
     const ChunkInfo* chunks = reinterpret_cast<const ChunkInfo*>(ws + lay.chunks);
@@ -208,8 +209,9 @@ cudaError_t launch_prefill_overlap(const ChunkedParams& cp, cudaStream_t stream,
     // The second part needs SMs of its own for as long as a chain may wait for it: with (nearly) as many half units as
     // SMs everything is produced before the state pass starts.  So it is where launches are known to be serialised: the state
     // pass waits for a launch that comes after it in the stream, the two must be able to run at the same time.  A
-    // profiler that replays kernels one at a time cannot be seen from here: under it the waits run out after
-    // milliseconds and the last launch does the work; profile gdn_prefill_stream instead, which runs the same kernels'
+    // profiler that replays kernels one at a time cannot be seen from here: under it the state pass gives
+    // up after 0.15 ms and the last launch does the work (2560 tokens at 32 heads 78 us, serialised 249; with waits that
+    // ran out by themselves only, 4800); profile gdn_prefill_stream instead, which runs the same kernels'
     // arithmetic.
     const long long units = static_cast<long long>(p.N) * p.Hv;
     const char* blocking = std::getenv("CUDA_LAUNCH_BLOCKING");
