@@ -61,7 +61,8 @@ __device__ __forceinline__ void state_half_role(const TensorMaps& maps, const Pr
                                                 const WorkspaceLayout& lay, uint8_t* smem, const uint32_t tmem,
                                                 const int cta, const int n_ctas) {
     __shared__ uint64_t bar_full_a[kHStages], bar_full_b[2], bar_full_c[kHStages], bar_free_a[kHStages], bar_free_b[2],
-        bar_free_c[kHStages], bar_y[2], bar_p[2], bar_y_read, bar_y1, bar_d1, bar_d4, bar_s, bar_u;
+        bar_free_c[kHStages], bar_y[2], bar_p[2], bar_y_read, bar_y1, bar_d1, bar_d4, bar_s, bar_u,
+        bar_drain[2];
     __shared__ int abort_flag;
     __shared__ uint32_t armed[3];         // chunks of the CTA's stream whose copies the loader has started, per ring
     // kHalfGated waits for records of a launch that may not be running beside this one: there no
@@ -82,6 +83,7 @@ __device__ __forceinline__ void state_half_role(const TensorMaps& maps, const Pr
             mbar_init(&bar_free_b[st], kSEpiWarps);
             mbar_init(&bar_y[st], 1);
             mbar_init(&bar_p[st], kSOutThreads / 32); // U~ in the accumulator
+            mbar_init(&bar_drain[st], 1);             // an issuer that gave up: its products
         }
         for (int st = 0; st < kHStages; ++st) {
             mbar_init(&bar_full_a[st], 1);
@@ -318,6 +320,11 @@ __device__ __forceinline__ void state_half_role(const TensorMaps& maps, const Pr
             gc += u.nc;
         }
         __syncwarp();
+        if (!live) {        // products still running read shared memory and TMEM that the CTA is about to give back
+            if (elect_one()) mma_commit(&bar_drain[outputs]);
+            mbar_wait(&bar_drain[outputs], 0u, 1u << 12);
+            __syncwarp();
+        }
     } else if (warp < kSEpiWarps) {
         // ===================== chain warps: U and the state refresh (the dependent chain)
         // Warp (q, h): rows 16 q .. + 15 of the half (TMEM lanes 32 q .. + 15), tokens 32 h .. of U, dk 64 h .. of S.
