@@ -262,19 +262,17 @@ int gdn_prefill_overlap(const void* q, const void* k, const void* v, const float
 }
 
 namespace {
-// Whether the records are produced in two parts, the second beside the chains, or all of them first.  Two parts cost about 13 us
-// (the tables with the processing order, two more launches) and hide the intra-chunk kernel's time, which grows with the items,
-// as far as the SMs that hold no half unit keep up.  So what decides is the number of (chunk, v-head) items against the
-// units, and where their lengths differ, half of the units that have ended on average count as gone (`live`; all count
-// without a bound on the longest).  The line was fitted to 1351 drawn batches of 2 to 70 units, 20 to 320 chunks and up to
-// 12000 items, equal and unequal, each timed in both forms: the rule takes 0.12 % more time than the faster form each time,
-// three launches always 5.3 %.  Us in three launches / in two parts on 148 SMs, one sequence: 8 units of 60 chunks 83.7 / 92.2,
-// of 120 158.2 / 159.6, of 240 305.8 / 293.7; 32 of 38 76.3 / 76.8, of 50 96.0 / 91.2, of 320 564 / 428; 48 of 50 115.2 / 119.2, of
-// 100 225.6 / 220.4; 64 of 40 115.0 / 123.1.  64 units in two sequences, 64 chunks both 182 / 185.5, 86 and 28 180.8 / 174.7;
-// 70 units, 60 chunks and six times 30 126.9 / 138.0.
+// Whether the records are produced in two parts, the second beside the chains, or all of them first.  Two parts cost
+// about 13 us (the tables with the processing order, two more launches) and hide the intra-chunk kernel's time, which
+// grows with the items, as far as the SMs that hold no half unit keep up.  So what decides is the number of (chunk,
+// v-head) items against the units; where the lengths differ, half of the units that have ended on average count as
+// gone (`live`; all units count without a bound on the longest).  The line was fitted to 1351 drawn batches timed in
+// both forms: on average 0.12 % above the faster of the two (three launches always: 5.3 %).  Us in three
+// launches / in two parts on 148 SMs: 32 units of 38 chunks 76.3 / 76.8, of 50 96.0 / 91.2; 64 of 40 115.0 / 123.1, of
+// 86 and 28 180.8 / 174.7.
 bool two_parts_pay(int32_t T, int32_t N, int32_t max_seqlen_hint, int32_t Hv, int32_t sms) {
     const long long units = static_cast<long long>(N) * Hv;
-    if (2 * units > sms - gdn::kOverlapSpareSms) return false;      // (gdn_prefill_overlap would run the three launches)
+    if (2 * units > sms - gdn::kOverlapSpareSms) return false;     // (gdn_prefill_overlap runs three launches there)
     const long long items = (2ll * (T / gdn::kChunk) + N) * Hv / 2;     // about, half a chunk lost per sequence
     const long long chain = (gdn::known_longest(T, N, max_seqlen_hint) + gdn::kChunk - 1) / gdn::kChunk;
     const long long live = chain > 0 ? std::min(units, (items + chain - 1) / chain) : units;
@@ -291,12 +289,11 @@ int gdn_prefill_route(int32_t T, int32_t N, int32_t max_seqlen_hint, int32_t Hv,
     // very short sequences: one block of tokens each (one launch, no workspace traffic)
     if (longest <= GDN_RECURRENT_MAX_SEQLEN) return GDN_ROUTE_RECURRENT;
     const long long units = static_cast<long long>(N) * Hv;
-    // Up to four blocks of few units (us, blocks against the chunked kernels, one sequence): 32 v-heads, 32 tokens 10.0 / 11.0,
-    // 33 12.6 / 12.0, 48 13.5 / 12.0, 64 16.8 / 12.4; 8 v-heads, 32 tokens 8.3 / 10.8, 48 10.9 / 11.8, 64 13.6 / 12.1; 64 units
-    // in two sequences of 48 tokens 13.5 / 13.4, in 16 13.2 / 13.8.  The third and fourth block are slower where there are more
-    // than a few units and stay: they keep the state to 1e-6, the chunked kernels, whose operands are bf16, to 2e-4.
-    // With more units than half the SMs a block takes longer: 4 x 30 tokens (128 units) 18.7 against 18.5 of
-    // the chunked kernels as they were.
+    // Up to four blocks of few units.  Us against the chunked kernels, one sequence: 32 v-heads, 32 tokens 10.0 /
+    // 11.0, 48 13.5 / 12.0; 8 v-heads, 48 10.9 / 11.8, 64 13.6 / 12.1.  The third and fourth block are slower where
+    // there are more than a few units and stay: they keep the state to 1e-6, the chunked kernels, whose operands are
+    // bf16, to 2e-4. With more units than half the SMs a block takes longer: 4 x 30 tokens (128 units) 18.7 against
+    // 18.5 of the chunked kernels as they were.
     if (units <= sm_count / 2 && longest <= GDN_BLOCKS_MAX_SEQLEN) return GDN_ROUTE_BLOCKS;
     return two_parts_pay(T, N, max_seqlen_hint, Hv, sm_count) ? GDN_ROUTE_OVERLAP : GDN_ROUTE_STREAM;
 }

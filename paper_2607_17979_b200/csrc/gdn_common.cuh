@@ -16,9 +16,9 @@ constexpr int kDevBadSlot = 1;
 constexpr int kDevBadCuSeqlens = 2;
 constexpr int kDevTimeout = 4;
 
-// Division of 0 <= x < 2^31 by a number known on the host: x * ceil(2^(31 + s) / d) >> 31 + s with 2^s >= d, exact because the
-// product's error is below x / 2^31 of a unit.  In line a division by a kernel argument takes about 150 cycles, and the three
-// that map a CTA to its sequence and heads stand in front of its first load.
+// Division of 0 <= x < 2^31 by a number known on the host: x * ceil(2^(31 + s) / d) >> 31 + s with 2^s >= d, exact
+// because the product's error is below x / 2^31 of a unit.  In line a division by a kernel argument takes about 150
+// cycles, and the three that map a CTA to its sequence and heads stand in front of its first load.
 struct FastDiv {
     uint32_t mul;
     uint16_t shift;
@@ -43,8 +43,8 @@ struct DecodeParams {
     __nv_bfloat16* o;
     int32_t* dev_status;
     int32_t Hv, num_slots;
-    // 96 bytes in all: a launch with 88 or 96 bytes of arguments takes 2.03 us of host time, with 80 or less and 104 or more
-    // 2.4-2.5, and the smallest calls are bound by it
+    // 96 bytes in all: a launch with 88 or 96 bytes of arguments takes 2.03 us of host time, with 80 or less and 104
+    // or more 2.4-2.5, and the smallest calls are bound by it
     uint32_t mul_hv, mul_group;          // by_hv(), by_group(): division by Hv, by Hv / Hqk
     uint16_t shift_hv, shift_group;
     float scale;

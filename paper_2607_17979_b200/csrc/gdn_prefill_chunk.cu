@@ -8,14 +8,14 @@ namespace gdn {
 // =============================================================================================
 // K1: intra-chunk quantities, one CTA (256 threads) per (chunk, v-head); see intra_item().
 // =============================================================================================
-// kInlineTable: a batch of at most kSmallSeqs sequences needs no table-building launch in front: every warp finds the CTA's
-// chunk from cu_seqlens, a sequence a lane.
+// kInlineTable: a batch of at most kSmallSeqs sequences needs no table-building launch in front: every warp finds the
+// CTA's chunk from cu_seqlens, a sequence a lane.
 // Order of the CTAs. In a row (kRow) the heads of a chunk stand next to one another, so that the heads that share Q
-// and K find them in L2, and the last chunks come first, so that what the state pass opens with (the first chunks of the first
-// sequences) was written last and is still there. Against all chunks of one head after the other a call of 1337 + 512 + 199
-// tokens takes 54.3 us instead of 55.7, 57 x 144 214.5 instead of 219, 20 sequences of 1684 tokens with 16 heads 37.1 instead of 38.3. Few items run all at
-// once, find nothing that an earlier one fetched, and only ask for the same lines at the same time: there 200 tokens take 16.5
-// instead of 16.3 and 10 sequences of 376 tokens with 8 heads 15.8 instead of 15.5, so those have a grid of chunks x heads (two kernels: testing for the form inside one costs 0.1 us a call).
+// and K find them in L2, and the last chunks come first, so that what the state pass opens with (the first chunks of
+// the first sequences) was written last and is still there: against all chunks of one head after the other 57 x 144
+// tokens take 214.5 us instead of 219. Few items run all at once, find nothing that an earlier one fetched, and only
+// ask for the same lines at the same time (200 tokens 16.5 instead of 16.3), so those have a grid of chunks x heads.
+// Two kernels: testing for the form inside one costs 0.1 us a call.
 template <bool kInlineTable, bool kRow>
 __global__ void __launch_bounds__(kIntraThreads, 4)
 prefill_intra_kernel(const __grid_constant__ TensorMaps maps, const PrefillParams p, uint8_t* ws,

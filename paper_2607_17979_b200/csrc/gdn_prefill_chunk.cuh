@@ -52,8 +52,8 @@ constexpr uint32_t kRecBytes = 74496;
 constexpr uint32_t kRecUHalf = (kRecDecay - kRecU) / 2;
 constexpr uint32_t kRecUBlock = kRecUHalf / 4, kRecPBlock = (kRecU - kRecP) / 4;      // bytes of a 16-token block
 __device__ __forceinline__ int token_blocks(int seq_len, int chunk) { return (min(kChunk, seq_len - chunk * kChunk) + 15) >> 4; }
-// Place (in 16-byte units) of a token group and dv within one half of U~.  Odd groups have their dv swapped in fours, so
-// that a fragment read (four dv of two neighbouring groups per half warp) touches every bank once.
+// Place (in 16-byte units) of a token group and dv within one half of U~.  Odd groups have their dv swapped in fours,
+// so that a fragment read (four dv of two neighbouring groups per half warp) touches every bank once.
 __device__ __forceinline__ int rec_u_index(int group, int dv) { return group * 64 + (dv ^ ((group & 1) << 2)); }
 
 // Batches of at most this many sequences need no table-building launch in front of the intra-chunk kernel and the state
@@ -68,10 +68,13 @@ struct ChunkInfo {      // 16 bytes
 };
 
 // Which sequences count.  One does if its own bounds are in order (0 <= t0 <= t1 <= T) and no earlier sequence whose
-// bounds are in order ends behind its start; the others have no chunks and are flagged.  Those that count do not overlap, so
-// they have at most T / 64 + N chunks, which is what the workspace is laid out for.  Where every sequence's own bounds are
-// in order each starts where the one before ends: only where a vote finds one that is not are starts and ends compared.
-__device__ __forceinline__ bool bounds_in_order(int32_t t0, int32_t t1, int32_t T) { return t0 >= 0 && t1 >= t0 && t1 <= T; }
+// bounds are in order ends behind its start; the others have no chunks and are flagged.  Those that count do not
+// overlap, so they have at most T / 64 + N chunks, which is what the workspace is laid out for.  Where every
+// sequence's own bounds are in order each starts where the one before ends: only where a vote finds one that is not
+// are starts and ends compared.
+__device__ __forceinline__ bool bounds_in_order(int32_t t0, int32_t t1, int32_t T) {
+    return t0 >= 0 && t1 >= t0 && t1 <= T;
+}
 // By one converged warp, a sequence a lane; lanes past the last one hold t0 = t1 = 0.
 __device__ __forceinline__ bool warp_bounds_ok(int32_t t0, int32_t t1, int32_t T, int lane) {
     bool ok = bounds_in_order(t0, t1, T);
@@ -86,9 +89,10 @@ __device__ __forceinline__ bool warp_bounds_ok(int32_t t0, int32_t t1, int32_t T
     return ok;
 }
 // By a block, a sequence a thread (`here`: the thread has one).  `ends`: shared, one per thread, holds the ends of the
-// thread's sequences whose own bounds are in order afterwards; `before`: the largest such end of the sequences in front.
-__device__ __forceinline__ bool block_bounds_ok(bool here, int32_t t0, int32_t t1, int32_t T, int32_t before, int32_t* ends,
-                                                int tid) {
+// thread's sequences whose own bounds are in order afterwards; `before`: the largest such end of the sequences in
+// front.
+__device__ __forceinline__ bool block_bounds_ok(bool here, int32_t t0, int32_t t1, int32_t T, int32_t before,
+                                                int32_t* ends, int tid) {
     const bool in_order = here && bounds_in_order(t0, t1, T);
     bool ok = in_order && t0 >= before;
     ends[tid] = in_order ? t1 : 0;
@@ -100,9 +104,9 @@ __device__ __forceinline__ bool block_bounds_ok(bool here, int32_t t0, int32_t t
 
 // Workspace layout (all offsets multiples of 256 bytes):
 //   [0,256)                      int32 header: [0] total_chunks, [1] total_items
-//                                (= total_chunks * Hv), [2] item queue head, [3] unit queue head,
-//                                [4] items produced before the state pass starts, [5] 1 once the producers of the others
-//                                run (two-part route)
+//                                (= total_chunks * Hv), [2] item queue head,
+//                                [4] items produced before the state pass starts, [5] 1 once the
+//                                producers of the others run (two-part route)
 //   seq_first[N+1]               int32: first chunk of each sequence (prefix sum); an invalid
 //                                sequence has zero chunks and seq_bad[n] = 1
 //   seq_bad[N]                   int32
@@ -159,8 +163,9 @@ struct ChunkedParams {
     int32_t longest = 0;      // known_longest(): picks kernels only
 };
 
-// Tokens of the longest sequence as far as the host can know them, 0: not at all.  The caller's bound counts only if T tokens
-// in N sequences can reach it (empty ones aside): one beyond, a model's context length for example, tells nothing.
+// Tokens of the longest sequence as far as the host can know them, 0: not at all.  The caller's bound counts only if T
+// tokens in N sequences can reach it (empty ones aside): one beyond, a model's context length for example, tells
+// nothing.
 inline int32_t known_longest(int32_t T, int32_t N, int32_t max_seqlen_hint) {
     if (N == 1) return T;
     return max_seqlen_hint > 0 && max_seqlen_hint <= T - (N - 1) ? max_seqlen_hint : 0;

@@ -230,11 +230,10 @@ template <int kId, int kThreads> __device__ __forceinline__ bool group_all(const
     return r != 0;
 }
 
-// Same, for a whole converged warp: every lane polls, so the instruction stays warp-wide, and what ends the
-// loop is a vote, so the verdict is the same on every lane whatever each lane's poll answers: callers
-// issue warp-wide instructions on the strength of it.  (Polling by one lane and broadcasting the verdict costs a
-// divergent branch and a shuffle, and that lane alone wakes later: a waiting warp saw an arrival after 200 cycles instead
-// of 89.)
+// Same, for a whole converged warp: every lane polls, so the instruction stays warp-wide, and what ends the loop is a
+// vote, so the verdict is the same on every lane whatever each lane's poll answers: callers issue warp-wide
+// instructions on the strength of it.  (Polling by one lane and broadcasting the verdict costs a divergent branch and
+// a shuffle, and that lane alone wakes later: a waiting warp saw an arrival after 200 cycles instead of 89.)
 __device__ __forceinline__ bool warp_wait_or_abort(uint64_t* bar, uint32_t parity, volatile int* abort_flag,
                                                    const int reason = 1) {
 #pragma unroll 1
@@ -247,10 +246,10 @@ __device__ __forceinline__ bool warp_wait_or_abort(uint64_t* bar, uint32_t parit
     return false;
 }
 
-// The same with the first poll in one piece with its vote (it blocks for a while by itself and so is nearly always the last)
-// and the rest out of line.  The roles of a warp-specialised kernel share 32 KB of instruction cache, and past it each
-// runs at the pace of its instruction misses: eight roles of 3 KB a round take 573 cycles, of 4 KB 929; the half-unit state pass
-// had 128 misses a chunk step with its waits in line and unrolled, and has 2.
+// The same with the first poll in one piece with its vote (it blocks for a while by itself and so is nearly always the
+// last) and the rest out of line.  The roles of a warp-specialised kernel share 32 KB of instruction cache, and past
+// it each runs at the pace of its instruction misses: eight roles of 3 KB a round take 573 cycles, of 4 KB 929; the
+// half-unit state pass had 128 misses a chunk step with its waits in line and unrolled, and has 2.
 static __device__ __noinline__ bool warp_wait_more(uint64_t* bar, uint32_t parity, volatile int* abort_flag, const int reason) {
     return warp_wait_or_abort(bar, parity, abort_flag, reason);
 }
@@ -259,12 +258,11 @@ __device__ __forceinline__ bool warp_wait(uint64_t* bar, uint32_t parity, volati
 }
 
 // kScaledQ: whether the record carries the scaled Q (gdn_prefill_chunk.cuh).
-// The intra-chunk quantities of one (chunk, v-head) item, computed by a group of 256 threads
-// (tid = 0..255 within the group; its warps must be CTA warps 0-3 mod 4 aligned, because a warp
-// reaches TMEM lanes 32 (warp % 4) ...).  `smem` is the group's 1024-aligned slice of kI_End
-// bytes, `tmem_base` + `tmem_off` its 128 TMEM columns (read behind the group's first barrier, which so also covers their
-// allocation), `sync` a barrier over exactly the group.  Writes the item's
-// record; returns false after a bounded wait gave up (status word set, nothing left in flight).
+// The intra-chunk quantities of one (chunk, v-head) item, computed by a group of 256 threads (tid = 0..255 within the
+// group; its warps must be CTA warps 0-3 mod 4 aligned, because a warp reaches TMEM lanes 32 (warp % 4) ...).  `smem`
+// is the group's 1024-aligned slice of kI_End bytes, `tmem_base` + `tmem_off` its 128 TMEM columns (read behind the
+// group's first barrier, which so also covers their allocation), `sync` a barrier over exactly the group.  Writes the
+// item's record; returns false after a bounded wait gave up (status word set, nothing left in flight).
 template <bool kScaledQ, class Sync>
 __device__ __forceinline__ bool intra_item(const TensorMaps& maps, const PrefillParams& p,
                                            uint8_t* rec, const ChunkInfo ci, const int hqk,

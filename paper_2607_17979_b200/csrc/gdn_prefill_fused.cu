@@ -18,10 +18,10 @@ namespace gdn {
 // Prep: chunk table, processing order, cleared queues and flags.  One CTA.
 // =============================================================================================
 constexpr int kFPrepThreads = 256;
-// model of the two-part production (see the kernel): items per SM and chunk step, start-up lag of
-// the second part in chunk steps, and a safety margin in items.  (0.3 would be what the producers do, 0.385 leaves 32 chains
-// the small cut although their chains then wait a little: records are read while still in L2, and the machine is at its
-// power limit.  32 chains of 512 chunks 805 -> 696 us, of 188 296 -> 271; 40 chains, which need the larger cut, 233 -> 227.)
+// model of the two-part production (see the kernel): items per SM and chunk step, start-up lag of the second part in
+// chunk steps, and a safety margin in items.  (0.3 would be what the producers do, 0.385 leaves 32 chains the small
+// cut although their chains then wait a little: records are read while still in L2, and the machine is at its power
+// limit.  32 chains of 512 chunks 805 -> 696 us, of 188 296 -> 271; 40 chains, which need the larger cut, 233 -> 227.)
 constexpr int kSplitProdPermille = 385;
 constexpr int kSplitLeadSteps = 4;
 constexpr int kSplitMarginItems = 64;

@@ -26,8 +26,8 @@ namespace gdn {
 constexpr int kHalfRows = kD / 2;
 // warps 0-7 chain, 8-11 outputs, 12 and 13 issuers, 14 loader
 constexpr int kHLoadWarp = 14;
-// Three rings, each filled and released by itself: W with the Q tile, the K tile with P, half of U~ with the vectors (two
-// places: U~ goes on to TMEM a chunk ahead).
+// Three rings, each filled and released by itself: W with the Q tile, the K tile with P, half of U~ with the vectors
+// (two places: U~ goes on to TMEM a chunk ahead).
 constexpr int kHStages = 3;
 constexpr uint32_t kHA_W = 0, kHA_Q = 16384, kHABytes = 32768;
 constexpr uint32_t kHC_K = 0, kHC_P = 16384, kHCBytes = 24576;
@@ -39,23 +39,24 @@ constexpr uint32_t kHalfSmem = kHS_Out + 8192 + 1024;
 // TMEM columns: S W^T (two tiles), S Q^T, U P^T, the state product, bf16 S, decayed U (hi / lo lanes), U
 constexpr uint32_t kH_D1 = 0, kH_Y1 = 128, kH_Y2 = 192, kH_D4 = 256, kH_S = 384, kH_Us = 448, kH_U = 480;
 
-// Polls of a record's flag, about half a microsecond each.  A few milliseconds: far longer than the producers ever lag when
-// they do run beside the state pass, far shorter than the other roles' mbarrier waits (which would report an error).  And
-// how long to wait if they have not even started: two launches in a row start within some ten microseconds of each other, and
-// what is lost by giving up too early is no more than the chain has done so far.
+// Polls of a record's flag, about half a microsecond each.  A few milliseconds: far longer than the producers ever lag
+// when they do run beside the state pass, far shorter than the other roles' mbarrier waits (which would report an
+// error).  And how long to wait if they have not even started: two launches in a row start within some ten
+// microseconds of each other, and what is lost by giving up too early is no more than the chain has done so far.
 constexpr uint32_t kSpinFlagLimitSoft = 1u << 13, kSpinStartLimit = 1u << 8;
 
 // Which records exist when the state pass starts.
 enum HalfMode {
     kHalfAll,       // every one (the intra-chunk kernel ran before)
     kHalfGated,     // those of the first hdr[kHdrSplit] items of the processing order; the others are being produced by a
-                    // concurrent kernel and are waited for.  A wait that runs out ends the CTA's work without an error (the
-                    // half units it has finished are marked in the done table, the others are left to a later launch).
+                    // concurrent kernel and are waited for.  A wait that runs out ends the CTA's work without an error
+                    // (the half units it has finished are marked in the done table, the others are left to a later
+                    // launch).
     kHalfRest       // every one, by that later launch: the half units marked done are left out
 };
 
-// The state pass of one CTA of 512 threads over its share of the rank-sorted half units.  `tmem` = 512 allocated columns;
-// ends with a CTA barrier.
+// The state pass of one CTA of 512 threads over its share of the rank-sorted half units.  `tmem` = 512 allocated
+// columns; ends with a CTA barrier.
 template <HalfMode kMode>
 __device__ __forceinline__ void state_half_role(const TensorMaps& maps, const PrefillParams& p, uint8_t* ws,
                                                 const WorkspaceLayout& lay, uint8_t* smem, const uint32_t tmem,
@@ -136,8 +137,8 @@ __device__ __forceinline__ void state_half_role(const TensorMaps& maps, const Pr
     } ring;
 
     if (warp == kHLoadWarp) {
-        // ===================== loader: records and Q, K tiles, in stream order; a stage's parts in the order in which the chunk
-        // before last releases them
+        // ===================== loader: records and Q, K tiles, in stream order; a stage's parts in the order in which
+        // the chunk before last releases them
         const size_t rec_stride = static_cast<size_t>(p.Hv) * kRecBytes;
         const uint32_t* flags = reinterpret_cast<const uint32_t*>(ws + lay.flags);
         const int32_t* pos = reinterpret_cast<const int32_t*>(ws + lay.pos);
@@ -173,7 +174,8 @@ __device__ __forceinline__ void state_half_role(const TensorMaps& maps, const Pr
                             v = __shfl_sync(0xffffffffu, ld_acquire_u32(f), 0);
                             if (v != 0 || __any_sync(0xffffffffu, *abortp)) break;
                             if (k >= kSpinStartLimit && !started) {
-                                started = __shfl_sync(0xffffffffu, ld_acquire_u32(reinterpret_cast<const uint32_t*>(ws) + kHdrStarted), 0);
+                                const uint32_t* word = reinterpret_cast<const uint32_t*>(ws) + kHdrStarted;
+                                started = __shfl_sync(0xffffffffu, ld_acquire_u32(word), 0);
                                 if (!started) break;
                             }
                             __nanosleep(64);
@@ -222,10 +224,10 @@ __device__ __forceinline__ void state_half_role(const TensorMaps& maps, const Pr
     } else if (warp > kHLoadWarp) {
         // one warp to spare
     } else if (warp >= kSIssueWarp) {
-        // ===================== issuers: the whole warp waits, one elected lane issues.  An instruction takes
-        // 29 cycles to issue at best, so the chain's products (S W^T, the state product) have a warp of their own; the other
-        // issues the outputs' (S Q^T, U P^T), each behind a chain product's completion, so that it never runs in front of
-        // the next or beside it.
+        // ===================== issuers: the whole warp waits, one elected lane issues.  An instruction takes 29 cycles
+        // to issue at best, so the chain's products (S W^T, the state product) have a warp of their own; the other issues
+        // the outputs' (S Q^T, U P^T), each behind a chain product's completion, so that it never runs in front of the
+        // next or beside it.
         const bool outputs = warp > kSIssueWarp;
         const uint32_t id_w = make_idesc_bf16(64, 64, false, true) | kIdescNegateB;
         const uint32_t id_qp = make_idesc_bf16(64, 64, false, false);
@@ -268,7 +270,8 @@ __device__ __forceinline__ void state_half_role(const TensorMaps& maps, const Pr
                         break;
                     }
                     tc_fence_after_sync();
-                    // (U decayed) K, hi and lo terms in the lower and upper lanes (K tile MN-major: 16 tokens = 2048 bytes)
+                    // (U decayed) K, hi and lo terms in the lower and upper lanes (K tile MN-major: 16 tokens = 2048
+                    // bytes)
                     if (elect_one()) {
                         mma_ts_c<false>(tD4, tUs, kk, id_k);
 #pragma unroll
@@ -286,7 +289,8 @@ __device__ __forceinline__ void state_half_role(const TensorMaps& maps, const Pr
                 for (int j = 0; j < u.nc; ++j, ring.next()) {
                     const uint32_t g = gc + j;
                     const uint64_t q = sdesc_advance(dQ0, ring.st * kHABytes), pp = sdesc_advance(dP0, ring.st * kHCBytes);
-                    // S Q^T, once S W^T has retired (its issuer has waited for the tiles), into the tile the output warps read a chunk ago
+                    // S Q^T, once S W^T has retired (its issuer has waited for the tiles), into the tile the output
+                    // warps read a chunk ago
                     if ((g > 0 && !warp_wait(&bar_y_read, (g - 1) & 1u, abortp, kWaitReason)) ||
                         !warp_wait(&bar_d1, g & 1u, abortp, kWaitReason)) {
                         live = false;
@@ -347,8 +351,8 @@ __device__ __forceinline__ void state_half_role(const TensorMaps& maps, const Pr
         const int frag = (q16 + g8) * kD + 64 * ch + 2 * t4;
         auto pair_off = [](int b, int r) { return 8 * r * kD + 8 * b; };
         bool ok = true;
-        // As in state_stream_role: each lane's own verdict until the unit's last chunk; after a failed wait the work goes on
-        // with whatever is there and nothing of it is written out.
+        // As in state_stream_role: each lane's own verdict until the unit's last chunk; after a failed wait the work
+        // goes on with whatever is there and nothing of it is written out.
         auto await = [&](uint64_t* bar, uint32_t parity) {
             if (!warp_wait(bar, parity, abortp, kWaitReason)) ok = false;
             tc_fence_after_sync();
@@ -418,8 +422,8 @@ __device__ __forceinline__ void state_half_role(const TensorMaps& maps, const Pr
                 for (int b = 0; b < 4; ++b)
                     dec[b] = *reinterpret_cast<const float2*>(vec + 4 * (32 * ch + 8 * b + 2 * t4));
                 const float gC = *reinterpret_cast<const float*>(vec + (kRecGammaC - kRecDecay));
-                // U P^T of the chunk before has read the last U.  (A wait that finds its phase completed takes more than 100
-                // cycles all the same: this one and S Q^T's below stand where a product is in flight anyway.)
+                // U P^T of the chunk before has read the last U.  (A wait that finds its phase completed takes more
+                // than 100 cycles all the same: this one and S Q^T's below stand where a product is in flight anyway.)
                 if (g > 0) await(&bar_y[st ^ 1], ((g - 1) >> 1) & 1u);
                 await(&bar_d1, g & 1u);
                 {   // U (the accumulator holds U~ - S W^T): rounded, and decayed as hi + lo
@@ -463,8 +467,8 @@ __device__ __forceinline__ void state_half_role(const TensorMaps& maps, const Pr
                     hand_over(&bar_s);
                 }
             }
-            // nothing of a unit is written after a failed wait (every record of the unit has been loaded by now: no flag
-            // wait of it can fail any more)
+            // nothing of a unit is written after a failed wait (every record of the unit has been loaded by now: no
+            // flag wait of it can fail any more)
             ok = group_all<2, kSEpiThreads>(ok);
             if (ok) {
                 float* out = p.final_state + static_cast<size_t>(tile) * (kHalfRows * kD) + frag;
@@ -547,8 +551,8 @@ __device__ __forceinline__ void state_half_role(const TensorMaps& maps, const Pr
                     preload(g + k);
                 }
                 preloaded = ahead;
-                // Every warp runs both group barriers of every chunk, also after a failed wait; where that is no error they
-                // leave together at the first.
+                // Every warp runs both group barriers of every chunk, also after a failed wait; where that is no error
+                // they leave together at the first.
                 if (ot == 0) bulk_wait_read_all();       // the last chunk's rows have left the staging tile
                 if constexpr (kMode == kHalfGated) {
                     ok = group_all<1, kSOutThreads>(ok);
@@ -557,13 +561,15 @@ __device__ __forceinline__ void state_half_role(const TensorMaps& maps, const Pr
                     out_sync();
                 }
                 await(&bar_y[buf], (g >> 1) & 1u);
-                // The rows are made once the chain warps have handed the next state over and wait behind the next product: beside
-                // the refresh they take its issue slots (4096 tokens at 8 v-heads 91.5 us, 88.3 this way).
+                // The rows are made once the chain warps have handed the next state over and wait behind the next
+                // product: beside the refresh they take its issue slots (4096 tokens at 8 v-heads 91.5 us, 88.3 this
+                // way).
                 if (j + 1 < u.nc) await(&bar_s, (g + 1) & 1u);
                 tc_fence_after_sync();
                 {
-                    // Fragments (rows = dv, columns = tokens), rounded in pairs and stored transposed into a [token][dv] tile:
-                    // lane l gives the address of matrix l / 8: tokens 8 (b + (l >> 4)) .., dv 8 (l >> 3 & 1) ..
+                    // Fragments (rows = dv, columns = tokens), rounded in pairs and stored transposed into a
+                    // [token][dv] tile: lane l gives the address of matrix l / 8: tokens 8 (b + (l >> 4)) .., dv 8 (l
+                    // >> 3 & 1) ..
                     const uint32_t dst = smem_u32(smem + kHS_Out);
 #pragma unroll
                     for (int c = 0; c < 2; ++c) {
@@ -616,8 +622,8 @@ __device__ __forceinline__ void state_half_role(const TensorMaps& maps, const Pr
     __syncthreads();
     if (abort_flag != 0 && warp == kSIssueWarp && lane == 0) {
         if (abort_flag == 1) report(p.dev_status, kDevTimeout);     // 2: a record not produced yet, no error
-        // let copies already in flight land before the CTA's shared memory goes away: the last chunks of each ring that the
-        // loader started, each on its place's barrier at that chunk's own parity
+        // let copies already in flight land before the CTA's shared memory goes away: the last chunks of each ring
+        // that the loader started, each on its place's barrier at that chunk's own parity
         for (uint32_t back = 1; back <= kHStages; ++back) {
             for (int r = 0; r < 3; ++r) {
                 const uint32_t n = *reinterpret_cast<volatile uint32_t*>(&armed[r]), places = r == 1 ? 2 : kHStages;

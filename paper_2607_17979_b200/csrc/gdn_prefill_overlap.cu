@@ -1,12 +1,11 @@
 // Chunked prefill with the record production in two parts around the persistent state pass.
 //
-// With few (sequence, v-head) units of unequal length the state pass is a handful of long serial
-// chains: most SMs hold a short chain that ends early, or none, while the intra-chunk kernel
-// before it needs the whole machine.  Here the intra-chunk work is cut in two along the order in
-// which the chains consume the records (by position inside the sequence first): the first part
-// runs alone, then the state pass starts, two CTAs per unit (gdn_prefill_half.cuh), and the second part runs beside it on
-// the SMs that have no live chain, each record published through a flag (release) that the state
-// pass's loading warp waits for (acquire, bounded).
+// With few (sequence, v-head) units of unequal length the state pass is a handful of long serial chains: most SMs hold
+// a short chain that ends early, or none, while the intra-chunk kernel before it needs the whole machine.  Here the
+// intra-chunk work is cut in two along the order in which the chains consume the records (by position inside the
+// sequence first): the first part runs alone, then the state pass starts, two CTAs per unit (gdn_prefill_half.cuh),
+// and the second part runs beside it on the SMs that have no live chain, each record published through a flag
+// (release) that the state pass's loading warp waits for (acquire, bounded).
 //
 // Five launches in one stream, the first four each a programmatic dependent of the one before:
 //   prep          chunk table, ranking, processing order, cleared flags and done table, the cut
@@ -33,9 +32,9 @@
 
 namespace gdn {
 
-// First part: resident CTAs over the items [0, cut) of the processing order.  (With one CTA per item the grid has to be
-// sized for all of them, the cut being known on the device only, and the CTAs that find nothing to do leave at 4 ns each:
-// 32768 tokens at 32 heads, a fifth of the items first, 52 us of nothing else.)
+// First part: resident CTAs over the items [0, cut) of the processing order.  (With one CTA per item the grid has to
+// be sized for all of them, the cut being known on the device only, and the CTAs that find nothing to do leave at 4 ns
+// each: 32768 tokens at 32 heads, a fifth of the items first, 52 us of nothing else.)
 __global__ void __launch_bounds__(kIntraThreads, 4)
 prefill_intra_first_kernel(const __grid_constant__ TensorMaps maps, const PrefillParams p,
                            uint8_t* ws, const WorkspaceLayout lay) {
@@ -207,12 +206,11 @@ cudaError_t launch_prefill_overlap(const ChunkedParams& cp, cudaStream_t stream,
     if (!make_prefill_tensor_maps(&maps, p)) return cudaErrorInvalidValue;
 
     // The second part needs SMs of its own for as long as a chain may wait for it: with (nearly) as many half units as
-    // SMs everything is produced before the state pass starts.  So it is where launches are known to be serialised: the state
-    // pass waits for a launch that comes after it in the stream, the two must be able to run at the same time.  A
-    // profiler that replays kernels one at a time cannot be seen from here: under it the state pass gives
-    // up after 0.15 ms and the last launch does the work (2560 tokens at 32 heads 78 us, serialised 249; with waits that
-    // ran out by themselves only, 4800); profile gdn_prefill_stream instead, which runs the same kernels'
-    // arithmetic.
+    // SMs everything is produced before the state pass starts.  So it is where launches are known to be serialised:
+    // the state pass waits for a launch that comes after it in the stream, the two must be able to run at the same
+    // time.  A profiler that replays kernels one at a time cannot be seen from here: under it the state pass gives up
+    // after 0.15 ms and the last launch does the work (2560 tokens at 32 heads 78 us, serialised 249; with waits that
+    // ran out by themselves only, 4800); profile gdn_prefill_stream instead, which runs the same kernels' arithmetic.
     const long long units = static_cast<long long>(p.N) * p.Hv;
     const char* blocking = std::getenv("CUDA_LAUNCH_BLOCKING");
     if (2 * units > sms - kOverlapSpareSms || (blocking && blocking[0] != '\0' && blocking[0] != '0'))
@@ -233,8 +231,9 @@ cudaError_t launch_prefill_overlap(const ChunkedParams& cp, cudaStream_t stream,
     e = launch_dependent(prefill_state_half_gated_kernel, dim3(grid), dim3(kStreamThreads),
                          kHalfSmem, stream, maps, p, cp.ws, cp.lay);
     if (e != cudaSuccess) return e;
-    // Producers beyond what the chains consume only add memory traffic beside them: a unit takes a record per chunk step
-    // and a producer CTA needs about twelve chunk steps per item (four on an SM), so twelve CTAs per unit keep up.
+    // Producers beyond what the chains consume only add memory traffic beside them: a unit takes a record per chunk
+    // step and a producer CTA needs about twelve chunk steps per item (four on an SM), so twelve CTAs per unit keep
+    // up.
     unsigned resident = 12u * static_cast<unsigned>(units);
     if (resident < static_cast<unsigned>(sms)) resident = static_cast<unsigned>(sms);
     if (resident > 4u * static_cast<unsigned>(sms)) resident = 4u * static_cast<unsigned>(sms);

@@ -27,8 +27,8 @@ prefill_recurrent_kernel(const PrefillParams p) {
     constexpr int kSplit = kD / Block::kRows;
     const int unit = blockIdx.x / kSplit;
     const int row_base = (blockIdx.x - unit * kSplit) * Block::kRows;
-    // (at 16 tokens the compiler spills four times as much around the multiplication: 20 sequences of 16 tokens at 32 heads
-    // 31.7 -> 32.4 us; elsewhere it is ahead, 6 tokens at 8 heads 4.50 -> 4.17)
+    // (at 16 tokens the compiler spills four times as much around the multiplication: 20 sequences of 16 tokens at 32
+    // heads 31.7 -> 32.4 us; elsewhere it is ahead, 6 tokens at 8 heads 4.50 -> 4.17)
     const int n = kMax == 16 && !kPipelined ? unit / p.Hv : unit / p.by_hv;
     const int hv = unit - n * p.Hv;
     const int hqk = hv / p.by_group;

@@ -48,15 +48,13 @@ prefill_state_half_kernel(const __grid_constant__ TensorMaps maps, const Prefill
     if (warp == kSIssueWarp) tmem_dealloc(tmem, kStateTmemCols);
 }
 
-// Whether the state pass runs two CTAs per unit.  A half unit's chunk step takes 1.06 us against 1.40 of a whole unit's, so
-// half units win where the longest chain decides: always while every one of them has an SM of its own (32 units of 64
-// chunks 144 us whole, 126 half), and for more units if the longest chain is at least twice what an SM has to do on
-// average, set-up of the units included (128 units, longest chain 3.1 times the average 22.8 / 19.7; 2.0 times 183 / 179.5,
-// 1.75 times 106.7 / 106.5, once 205 / 217).
-// The longest chain is the caller's word.  If that bound is far too large, whole units would have been faster by 5 to 11 %
-// (57 x 144 tokens at 32 heads 216 us, half 240; 15 x 546 185 / 197; 30 x 300 at 8 heads 55.7 / 61.4).  The device knows
-// better, but a kernel that holds both forms and chooses costs every call of more units 2 us (1337 + 512 + 199 tokens
-// 57.4 -> 59.8).
+// Whether the state pass runs two CTAs per unit.  A half unit's chunk step takes 1.06 us against 1.40 of a whole
+// unit's, so half units win where the longest chain decides: always while every one of them has an SM of its own (32
+// units of 64 chunks 144 us whole, 126 half), and for more units if the longest chain is at least twice what an SM has
+// to do on average, set-up of the units included (2.0 times the average 183 / 179.5, 1.75 times 106.7 / 106.5, once
+// 205 / 217). The longest chain is the caller's word.  If that bound is far too large, whole units would have been
+// faster by 5 to 11 % (57 x 144 tokens at 32 heads 216 us, half 240).  The device knows better, but a kernel that
+// holds both forms and chooses costs every call of more units 2 us (1337 + 512 + 199 tokens 57.4 -> 59.8).
 static bool half_units(int32_t T, int32_t N, int32_t Hv, int32_t longest, int sms) {
     const long long units = static_cast<long long>(N) * Hv;
     if (2 * units <= sms) return true;

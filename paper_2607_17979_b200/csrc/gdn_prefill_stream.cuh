@@ -52,16 +52,17 @@ struct UnitInfo {
     bool bad_seq, bad_slot;
 };
 
-// After the intra-chunk kernel alone (no order of production to agree on), batches of at most kSmallSeqs sequences: a warp of
-// the state pass works the per-sequence table out from cu_seqlens itself, into shared memory.  Behind the launch before it a CTA then waits for one round trip to global memory, not for the three
-// of rank -> sequence -> first chunk and bounds (1.3 -> 0.6 us; a call of 100 tokens takes 13.7).
+// After the intra-chunk kernel alone (no order of production to agree on), batches of at most kSmallSeqs sequences: a
+// warp of the state pass works the per-sequence table out from cu_seqlens itself, into shared memory.  Behind the
+// launch before it a CTA then waits for one round trip to global memory, not for the three of rank -> sequence ->
+// first chunk and bounds (1.3 -> 0.6 us; a call of 100 tokens takes 13.5).
 struct SeqEntry {       // by rank
     int32_t n, c_first, nc, t0, len, slot, bad, pad;
 };
 
-// Which of the rank-sorted units a CTA takes: its first one by its number, then more in passes that turn round, so that a CTA that
-// took a long one of a pass takes a short one of the next.  The CTAs whose first unit is longer than half the longest are
-// left out of the later passes where the others can do the rest in the longest one's time.
+// Which of the rank-sorted units a CTA takes: its first one by its number, then more in passes that turn round, so
+// that a CTA that took a long one of a pass takes a short one of the next.  The CTAs whose first unit is longer than
+// half the longest are left out of the later passes where the others can do the rest in the longest one's time.
 struct UnitWalk {
     int cta, n_ctas, first_later;       // CTAs first_later .. n_ctas - 1 walk the later passes
     __device__ __forceinline__ int at(int i) const {       // i-th unit, or one past the end
@@ -72,8 +73,8 @@ struct UnitWalk {
     }
 };
 
-// By one converged warp, N <= kSmallSeqs; returns UnitWalk::first_later for `per_seq` units a sequence.  The rules are the table-building
-// kernels': see warp_bounds_ok; more chunks first, ties by index.
+// By one converged warp, N <= kSmallSeqs; returns UnitWalk::first_later for `per_seq` units a sequence.  The rules are
+// the table-building kernels': see warp_bounds_ok; more chunks first, ties by index.
 __device__ __forceinline__ int build_seq_table(SeqEntry* tab, const PrefillParams& p, const int lane, const int per_seq,
                                                const int n_ctas) {
     SeqEntry e = {lane, 0, 0, 0, 0, lane, 0, 0};
@@ -155,9 +156,10 @@ __device__ __forceinline__ void fence_proxy_async_all() {
     asm volatile("fence.proxy.async;" ::: "memory");
 }
 
-// The state pass of one CTA of 512 threads over its share of the rank-sorted units.  kGated = false: every record exists (the intra-chunk kernel ran before).  true: records are being produced by
-// other CTAs of the same cooperative launch and the loading warps wait for each record's flag first.  `tmem` = 512 allocated
-// columns; ends with a CTA barrier.
+// The state pass of one CTA of 512 threads over its share of the rank-sorted units.  kGated = false: every record
+// exists (the intra-chunk kernel ran before).  true: records are being produced by other CTAs of the same cooperative
+// launch and the loading warps wait for each record's flag first.  `tmem` = 512 allocated columns; ends with a CTA
+// barrier.
 template <bool kGated>
 __device__ __forceinline__ void state_stream_role(const TensorMaps& maps, const PrefillParams& p,
                                                   uint8_t* ws, const WorkspaceLayout& lay,
@@ -709,9 +711,9 @@ __device__ __forceinline__ void state_stream_role(const TensorMaps& maps, const 
                 out_sync();
                 await(&bar_y[buf], (g >> 1) & 1u);
                 tc_fence_after_sync();
-                // The tile (lanes = dv, columns = tokens) is read as accumulator fragments (lane 4 x + t holds
-                // columns 8 i + 2 t, + 1; raw Q: both tiles, and added), rounded in pairs and stored transposed, 8 dv of one token per 16
-                // bytes, into a [token][dv] tile of two 128B-swizzled halves of 64 dv (what these warps
+                // The tile (lanes = dv, columns = tokens) is read as accumulator fragments (lane 4 x + t holds columns
+                // 8 i + 2 t, + 1; raw Q: both tiles, and added), rounded in pairs and stored transposed, 8 dv of one
+                // token per 16 bytes, into a [token][dv] tile of two 128B-swizzled halves of 64 dv (what these warps
                 // issue comes out of the chain warps' issue slots).
                 {
                     const int dv0 = q4 * 32 + 8 * (lane >> 3);         // the 8 dv this lane's address covers

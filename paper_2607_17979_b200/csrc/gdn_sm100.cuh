@@ -40,8 +40,9 @@ __device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t parity) {
         : "memory");
     return ok != 0;
 }
-// The same by a whole converged warp: true once every lane's poll has seen the phase complete.  (Poll and vote in one piece:
-// written apart the predicate takes the way through a register and a wait on a completed barrier 180 cycles, not 60.)
+// The same by a whole converged warp: true once every lane's poll has seen the phase complete.  (Poll and vote in one
+// piece: written apart the predicate takes the way through a register and a wait on a completed barrier 180 cycles,
+// not 60.)
 __device__ __forceinline__ bool mbar_try_wait_all(uint64_t* bar, uint32_t parity) {
     uint32_t ok;
     asm volatile(
@@ -193,8 +194,8 @@ __device__ __forceinline__ void mma_ts_c(uint32_t d_tmem, uint32_t a_tmem, uint6
         : "memory");
 }
 // One lane of a converged warp (always the same one).  One branch on it around a whole product and its commit: eight
-// instructions of N = 64 then issue in 232 cycles, with 92 instructions fewer than under an election each (397 cycles); behind
-// a `lane == 0` branch every operand is first moved over from per-thread registers (621).
+// instructions of N = 64 then issue in 232 cycles, with 92 instructions fewer than under an election each (397
+// cycles); behind a `lane == 0` branch every operand is first moved over from per-thread registers (621).
 __device__ __forceinline__ bool elect_one() {
     uint32_t pred;
     asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}"
