@@ -26,9 +26,9 @@ EXPORTS = ("gdn_decode", "gdn_prefill_workspace_bytes", "gdn_prefill", "gdn_pref
            "gdn_host_us_per_decode_call", "gdn_host_us_per_prefill_call", "gdn_status_string",
            "gdn_last_cuda_error_string", "gdn_version")
 
-# kernels one call enqueues (for the benchmark's launch count)
+# kernels one call of the benchmark's step enqueues: a decode, and the prefill of four sequences (no table launch)
 LAUNCHES_PER_DECODE = 1
-LAUNCHES_PER_PREFILL = 3
+LAUNCHES_PER_PREFILL = 2
 LAUNCHES_PER_STEP = LAUNCHES_PER_DECODE + LAUNCHES_PER_PREFILL
 
 if not os.path.exists(LIB_PATH):

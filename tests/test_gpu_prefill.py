@@ -160,7 +160,7 @@ def test_chunked_and_recurrent_routes_agree():
 def test_prefill_varlen_benchmark_config_full(trial):
     """4 sequences {512,1024,2048,4096}, 32 v-heads, five seeds: every output against the oracle,
     through the length-routed entry point (the call the benchmark times) and, on the first seed,
-    through the plain three launches, the persistent state pass and the single cooperative launch."""
+    through the three launches under both names and the single cooperative launch."""
     p = I.make_config(3, trial)
     o_ref, S_ref, _ = oracle_prefill(p)
     cu = p["cu_seqlens"]
@@ -189,8 +189,8 @@ def check_long_context(p, o_ref, S_ref, impl, **kw):
 @pytest.mark.parametrize("trial", [0, 1, 2, 3, 4])
 def test_prefill_long_context_benchmark_config_all_heads(trial):
     """The oracle runs the whole 32768-token, 32-head batch; the GPU result is compared head by
-    head through the length-routed entry point (the single cooperative launch for this shape) on
-    five seeds and, on the first seed, through the three launches and the persistent state pass."""
+    head through the routed entry point (the two-part production for this shape) on five seeds
+    and, on the first seed, through the three launches under both names."""
     p = I.make_config(4, trial)
     o_ref, S_ref, _ = oracle_prefill(p)
     for impl in (("auto", "chunked", "stream") if trial == 0 else ("auto",)):
@@ -281,16 +281,18 @@ def test_length_routed_entry_point_small_shapes(lens):
 
 
 @pytest.mark.parametrize("impl", ["auto", "chunked", "stream"])
-@pytest.mark.parametrize("N", [16, 17])
+@pytest.mark.parametrize("N", [16, 17, 32, 33])
 def test_small_batches_without_a_table_launch_and_the_first_batch_beyond(impl, N):
-    """Up to 16 sequences the intra-chunk kernel finds its chunks from cu_seqlens and writes the
-    per-sequence tables (first chunk, validity, rank) itself; 17 sequences take the table-building
-    launch.  Equal chunk counts (ties in the ranking), an empty sequence, a padding slot and an
+    """Up to 32 sequences the intra-chunk kernel finds its chunk and the state pass its units from
+    cu_seqlens, and no table is written; 33 sequences take the table-building launch.  Equal chunk
+    counts (ties in the ranking), an empty sequence, a padding slot, out-of-order bounds and an
     initial state must come out the same on both sides of that boundary."""
-    lens = [70, 130, 64, 0, 200, 65, 1, 128, 129, 64, 70, 33, 192, 5, 100, 66, 90][:N]
+    lens = [70, 130, 64, 0, 200, 65, 1, 128, 129, 64, 70, 33, 192, 5, 100, 66, 90,
+            64, 0, 1, 130, 65, 70, 128, 3, 64, 129, 0, 66, 200, 63, 127, 65][:N]
     p = I.prefill_inputs(lens, 2, 4, seed=900 + N, init="normal")
     slots = np.arange(N, dtype=np.int32)
     slots[2] = -1
+    slots[-1] = -1 if N >= 32 else slots[-1]
     o, S, st = run_prefill(p, impl, slot_idx=slots)
     assert st == 0
     o_ref, S_ref, _ = oracle_prefill(p, slot_idx=slots)
@@ -302,6 +304,13 @@ def test_small_batches_without_a_table_launch_and_the_first_batch_beyond(impl, N
     cu = p["cu_seqlens"].copy()
     cu[5] = cu[4] - 3
     q["cu_seqlens"] = cu
-    _, _, st_bad = run_prefill(q, impl, slot_idx=slots)
-    assert st_bad != 0
+    o_bad, S_bad, st_bad = run_prefill(q, impl, slot_idx=slots, pool_fill=7.0)
+    assert st_bad == 2
+    # sequence 4 runs backwards, 5 starts before 2 and 3 end: skipped; those in front and behind are as before
+    ok = [n for n in range(N) if n not in (4, 5) and slots[n] >= 0]
+    assert (S_bad[[4, 5]] == 7.0).all()
+    assert np.array_equal(S_bad[ok], S[ok])
+    for n in ok:
+        if lens[n]:
+            assert np.array_equal(o_bad[p["cu_seqlens"][n]:p["cu_seqlens"][n + 1]], o[p["cu_seqlens"][n]:p["cu_seqlens"][n + 1]])
 

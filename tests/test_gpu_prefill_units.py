@@ -31,8 +31,8 @@ def test_unit_changes(lens, alias, route):
 
 @pytest.mark.parametrize("n, hv", [(37, 2), (75, 1), (37, 4), (149, 1)])
 def test_record_forms(n, hv):
-    """Half as many units as SMs and one more, as many and one more (148 SMs): the records change form there, in
-    the three launches and in the two-part route alike."""
+    """Half as many units as SMs and one more, as many and one more (148 SMs), where the state pass takes two CTAs
+    per unit and one: the two-part entry point, which runs the three launches for such batches, gives the same bits."""
     p = I.prefill_inputs([130 - i % 67 for i in range(n)], 1, hv, seed=9800 + n + hv, alpha_lo=0.5, init="normal")
     o, S, status = run_prefill(p, "stream")
     o2, S2, status2 = run_prefill(p, "overlap", split_permille=300)

@@ -22,6 +22,7 @@ def launches(graph):
     ([130], 32, 0, "stream", 2), ([2495], 32, 0, "stream", 2), ([40] * 40, 4, 40, "stream", 3),     # with a table launch
     ([2496], 32, 0, "overlap", 5), ([6100, 2000], 32, 6100, "overlap", 5),
     ([4096, 4096], 32, 4096, "stream", 2), ([6100, 2000], 32, 0, "stream", 2),
+    ([512, 1024, 2048, 4096], 32, 4096, "stream", 2),               # the benchmark's
 ])
 def test_route_is_what_runs(lens, hv, hint, route, nodes):
     from paper_2607_17979_b200 import api
@@ -39,3 +40,5 @@ def test_route_is_what_runs(lens, hv, hint, route, nodes):
     with torch.cuda.stream(side), torch.cuda.graph(graph, stream=side):
         api.gdn_prefill(*args, max_seqlen_hint=hint)
     assert launches(graph.raw_cuda_graph()) == nodes
+    if lens == [512, 1024, 2048, 4096]:
+        assert nodes == api.LAUNCHES_PER_PREFILL
