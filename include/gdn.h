@@ -311,9 +311,9 @@ int gdn_prefill_stream(const void* q, const void* k, const void* v,
  * at the same time, which programmatic dependent launch makes the device do
  * but which CUDA does not promise (and a tool that replays kernels one at a
  * time prevents).  If it does not happen the state pass gives up after about
- * 0.15 ms, marks the half (sequence, v-head) units it has finished, and the last
+ * 0.2 ms, marks the half (sequence, v-head) units it has finished, and the last
  * launch runs the others once the records exist: the results are the same, only
- * time is lost (32768 tokens at 32 heads 0.66 -> 1.18 ms, 2560 0.08 -> 0.25; so
+ * time is lost (32768 tokens at 32 heads 0.66 -> 1.27 ms, 2560 0.08 -> 0.34; so
  * profile gdn_prefill_stream instead under such a tool).  With CUDA_LAUNCH_BLOCKING set this is
  * gdn_prefill_stream.
  */

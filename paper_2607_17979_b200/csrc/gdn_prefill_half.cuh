@@ -39,11 +39,13 @@ constexpr uint32_t kHalfSmem = kHS_Out + 8192 + 1024;
 // TMEM columns: S W^T (two tiles), S Q^T, U P^T, the state product, bf16 S, decayed U (hi / lo lanes), U
 constexpr uint32_t kH_D1 = 0, kH_Y1 = 128, kH_Y2 = 192, kH_D4 = 256, kH_S = 384, kH_Us = 448, kH_U = 480;
 
-// Polls of a record's flag, about half a microsecond each.  A few milliseconds: far longer than the producers ever lag
+// Polls of a record's flag, about 0.4 us each.  A few milliseconds: far longer than the producers ever lag
 // when they do run beside the state pass, far shorter than the other roles' mbarrier waits (which would report an
 // error).  And how long to wait if they have not even started: two launches in a row start within some ten
-// microseconds of each other, and what is lost by giving up too early is no more than the chain has done so far.
-constexpr uint32_t kSpinFlagLimitSoft = 1u << 13, kSpinStartLimit = 1u << 8;
+// microseconds of each other unless another stream's kernel holds the SMs between them (32768 tokens beside 57
+// sequences on a second stream: at half this limit the chains give up for that).  What is lost by giving up too early
+// is no more than the chain has done so far.
+constexpr uint32_t kSpinFlagLimitSoft = 1u << 13, kSpinStartLimit = 1u << 9;
 
 // Which records exist when the state pass starts.
 enum HalfMode {

@@ -20,7 +20,7 @@
 //                 for the state pass at its very end, so that the completion of this launch
 //                 implies the state pass's.
 //   rest          an ordinary launch.  CUDA lets a programmatic dependent start early, it does not
-//                 promise to; if the second part has not started when a chain has waited for a record for 0.1 ms or so,
+//                 promise to; if the second part has not started when a chain has waited for a record for 0.2 ms,
 //                 the chain gives up (without an error: a half unit's final state is written only after
 //                 its last record has been loaded, so an unfinished one has left its initial state
 //                 alone), the half units that were finished are marked, and this launch runs the others now that
@@ -209,7 +209,7 @@ cudaError_t launch_prefill_overlap(const ChunkedParams& cp, cudaStream_t stream,
     // SMs everything is produced before the state pass starts.  So it is where launches are known to be serialised:
     // the state pass waits for a launch that comes after it in the stream, the two must be able to run at the same
     // time.  A profiler that replays kernels one at a time cannot be seen from here: under it the state pass gives up
-    // after 0.15 ms and the last launch does the work (2560 tokens at 32 heads 78 us, serialised 249; with waits that
+    // after 0.2 ms and the last launch does the work (2560 tokens at 32 heads 78 us, serialised 343; with waits that
     // ran out by themselves only, 4800); profile gdn_prefill_stream instead, which runs the same kernels' arithmetic.
     const long long units = static_cast<long long>(p.N) * p.Hv;
     const char* blocking = std::getenv("CUDA_LAUNCH_BLOCKING");
