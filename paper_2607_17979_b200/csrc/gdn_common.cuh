@@ -138,6 +138,22 @@ __device__ __forceinline__ float2 fma2(const float2 a, const float2 b, const flo
     return *reinterpret_cast<float2*>(&d);
 }
 
+// The same for a product or a sum of pairs.
+__device__ __forceinline__ float2 mul2(const float2 a, const float2 b) {
+    unsigned long long d;
+    asm("mul.rn.f32x2 %0, %1, %2;"
+        : "=l"(d)
+        : "l"(*reinterpret_cast<const unsigned long long*>(&a)), "l"(*reinterpret_cast<const unsigned long long*>(&b)));
+    return *reinterpret_cast<float2*>(&d);
+}
+__device__ __forceinline__ float2 add2(const float2 a, const float2 b) {
+    unsigned long long d;
+    asm("add.rn.f32x2 %0, %1, %2;"
+        : "=l"(d)
+        : "l"(*reinterpret_cast<const unsigned long long*>(&a)), "l"(*reinterpret_cast<const unsigned long long*>(&b)));
+    return *reinterpret_cast<float2*>(&d);
+}
+
 // sum over the 8 lanes that share a state row (lanes differing in bits 0..2)
 __device__ __forceinline__ float sum8(float x) {
     x += __shfl_xor_sync(0xffffffffu, x, 1);

@@ -1,35 +1,29 @@
 // Chunked prefill on the sm_100a tensor cores (tcgen05 + TMEM, operands staged by TMA): the
 // intra-chunk kernel and the host side shared by the launchers.
 // The algebra and the record layout are described in gdn_prefill_chunk.cuh.
-#include "gdn_prefill_device.cuh"
+#include "gdn_prefill_intra.cuh"
 
 namespace gdn {
 
 // =============================================================================================
-// K1: intra-chunk quantities, one CTA (256 threads) per (chunk, v-head); see intra_item().
+// K1: intra-chunk quantities of every (chunk, v-head) item, one persistent CTA per SM; see gdn_prefill_intra.cuh.
 // =============================================================================================
-// kInlineTable: a batch of at most kSmallSeqs sequences needs no table-building launch in front: every warp finds the
-// CTA's chunk from cu_seqlens, a sequence a lane.
-// Order of the CTAs. In a row (kRow) the heads of a chunk stand next to one another, so that the heads that share Q
-// and K find them in L2, and the last chunks come first, so that what the state pass opens with (the first chunks of
-// the first sequences) was written last and is still there: against all chunks of one head after the other 57 x 144
-// tokens take 214.5 us instead of 219. Few items run all at once, find nothing that an earlier one fetched, and only
-// ask for the same lines at the same time (200 tokens 16.5 instead of 16.3), so those have a grid of chunks x heads.
-// Two kernels: testing for the form inside one costs 0.1 us a call.
-template <bool kInlineTable, bool kRow>
-__global__ void __launch_bounds__(kIntraThreads, 4)
+// kInlineTable: a batch of at most kSmallSeqs sequences needs no table-building launch in front: the warp that hands the
+// items out finds their chunks from cu_seqlens, a sequence a lane.
+template <bool kInlineTable>
+__global__ void __launch_bounds__(kProdThreads, 1)
 prefill_intra_kernel(const __grid_constant__ TensorMaps maps, const PrefillParams p, uint8_t* ws,
                      const WorkspaceLayout lay) {
-    const int at = static_cast<int>(blockIdx.x);
-    int c = at, hv = blockIdx.y;
-    // this CTA's item; false beyond the batch's chunks, which the host can only bound
-    const auto place = [&](int chunks) {
-        if constexpr (!kRow) return c < chunks;
-        const int item = chunks * p.Hv - 1 - at;
-        c = item / p.by_hv;
-        hv = item - c * p.Hv;
-        return item >= 0;
-    };
+    pdl_launch_dependents();
+    produce_cta<kInlineTable ? kItemsInline : kItemsTable>(maps, p, ws, lay);
+}
+
+// The same for few items: a CTA of 256 threads per item, up to four to an SM.
+template <bool kInlineTable>
+__global__ void __launch_bounds__(kIntraThreads, 4)
+prefill_intra_few_kernel(const __grid_constant__ TensorMaps maps, const PrefillParams p, uint8_t* ws,
+                     const WorkspaceLayout lay) {
+    const int c = blockIdx.x, hv = blockIdx.y;
     __shared__ uint32_t tmem_base_s;
     const int tid = threadIdx.x, warp = tid >> 5;
     pdl_launch_dependents();
@@ -63,8 +57,8 @@ prefill_intra_kernel(const __grid_constant__ TensorMaps maps, const PrefillParam
             const int y = __shfl_up_sync(0xffffffffu, incl, d);
             if (lane >= d) incl += y;
         }
-        mine = place(__shfl_sync(0xffffffffu, incl, 31));
-        if (at == 0 && blockIdx.y == 0 && warp == 0 &&
+        mine = c < __shfl_sync(0xffffffffu, incl, 31);      // (the host can only bound the number of chunks)
+        if (c == 0 && blockIdx.y == 0 && warp == 0 &&
             (!ok || (lane == 0 && t0 != 0) || (lane == p.N - 1 && t1 != p.T)))
             report(p.dev_status, kDevBadCuSeqlens);
         const unsigned here = __ballot_sync(0xffffffffu, c < incl && c >= incl - nc);
@@ -75,7 +69,7 @@ prefill_intra_kernel(const __grid_constant__ TensorMaps maps, const PrefillParam
         ci.len = __shfl_sync(0xffffffffu, ci.len, ci.seq & 31);
         ci.pad = 0;
     } else {
-        mine = place(*reinterpret_cast<const int32_t*>(ws));
+        mine = c < *reinterpret_cast<const int32_t*>(ws);
         if (mine) ci = reinterpret_cast<const ChunkInfo*>(ws + lay.chunks)[c];
     }
     if (!mine) {
@@ -86,8 +80,7 @@ prefill_intra_kernel(const __grid_constant__ TensorMaps maps, const PrefillParam
     uint8_t* rec = ws + lay.records + (static_cast<size_t>(c) * p.Hv + hv) * kRecBytes;
 
     extern __shared__ uint8_t smem_raw[];
-    uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
-                                               ~static_cast<uintptr_t>(1023));
+    uint8_t* smem = align_1024(smem_raw);
     __shared__ IntraStatics st;
     intra_item<false>(maps, p, rec, ci, hqk, hv, smem, st, &tmem_base_s, 0, tid, [] { __syncthreads(); });
     tc_fence_before_sync();
@@ -149,16 +142,21 @@ cudaError_t launch_prefill_intra(const TensorMaps& maps, const ChunkedParams& cp
     DeviceInfo di;
     cudaError_t e = device_info(&di);
     if (e != cudaSuccess) return e;
-    // from about two items an SM on the row of items is no slower (13 chunks x 16 heads, 22 x 16, 39 x 8: level)
     const int64_t items = static_cast<int64_t>(cp.lay.max_chunks) * cp.p.Hv;
-    const bool row = items > 2 * di.sms;
-    auto kernel = row ? inline_tables ? prefill_intra_kernel<true, true> : prefill_intra_kernel<false, true>
-                      : inline_tables ? prefill_intra_kernel<true, false> : prefill_intra_kernel<false, false>;
-    e = ensure_dynamic_smem(kernel, kIntraSmem);
+    // Few items run all at once in either form, and there the shorter way through one item counts: a pipeline's warps
+    // fetch eight pieces of code from L2 before the first item is through (us a call, CTA per item / pipeline: 64 items
+    // 13.3 / 15.3, 512 37.1 / 38.5, 672 46.2 / 46.5, 1024 64.6 / 63.8, 1280 in 40 sequences 75.2 / 69.3).
+    if (items <= 5ll * di.sms) {
+        auto kernel = inline_tables ? prefill_intra_few_kernel<true> : prefill_intra_few_kernel<false>;
+        e = ensure_dynamic_smem(kernel, kIntraSmem);
+        if (e != cudaSuccess) return e;
+        return launch_dependent(kernel, dim3(cp.lay.max_chunks, cp.p.Hv), dim3(kIntraThreads), kIntraSmem, stream, maps, cp.p, cp.ws, cp.lay);
+    }
+    auto kernel = inline_tables ? prefill_intra_kernel<true> : prefill_intra_kernel<false>;
+    e = ensure_dynamic_smem(kernel, kProdSmem);
     if (e != cudaSuccess) return e;
-    const dim3 grid = row ? dim3(static_cast<unsigned>(items)) : dim3(cp.lay.max_chunks, cp.p.Hv);
-    return launch_dependent(kernel, grid, dim3(kIntraThreads), kIntraSmem, stream, maps, cp.p, cp.ws,
-                            cp.lay);
+    const dim3 grid(static_cast<unsigned>(items < di.sms ? items : di.sms));
+    return launch_dependent(kernel, grid, dim3(kProdThreads), kProdSmem, stream, maps, cp.p, cp.ws, cp.lay);
 }
 
 // The three-launch path: table-building launch (none for small batches), the intra-chunk kernel

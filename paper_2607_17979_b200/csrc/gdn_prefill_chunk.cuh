@@ -106,7 +106,8 @@ __device__ __forceinline__ bool block_bounds_ok(bool here, int32_t t0, int32_t t
 //   [0,256)                      int32 header: [0] total_chunks, [1] total_items
 //                                (= total_chunks * Hv), [2] item queue head,
 //                                [4] items produced before the state pass starts, [5] 1 once the
-//                                producers of the others run (two-part route)
+//                                producers of the others run, [6] the chunk that the first
+//                                chain has come to (two-part route)
 //   seq_first[N+1]               int32: first chunk of each sequence (prefix sum); an invalid
 //                                sequence has zero chunks and seq_bad[n] = 1
 //   seq_bad[N]                   int32
@@ -129,7 +130,7 @@ struct WorkspaceLayout {
     int32_t max_chunks, max_nc;
 };
 
-constexpr int kHdrTotalChunks = 0, kHdrTotalItems = 1, kHdrItemHead = 2, kHdrSplit = 4, kHdrStarted = 5;
+constexpr int kHdrTotalChunks = 0, kHdrTotalItems = 1, kHdrItemHead = 2, kHdrSplit = 4, kHdrStarted = 5, kHdrProgress = 6;
 
 inline size_t round256(size_t x) { return (x + 255) & ~static_cast<size_t>(255); }
 

@@ -67,8 +67,9 @@ __device__ __forceinline__ void mma_m16n8k8_tf32(float (&c)[4], const uint32_t (
         : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
         : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b[0]), "r"(b[1]));
 }
-// kN tiles side by side: columns 8 nb .. of B and of the output.
-template <int kSteps, int kN>
+// kN tiles side by side: columns 8 nb .. of B and of the output.  kPairs: of a k-step's eight k, 2t and 2t + 1 stand where
+// t and t + 4 do otherwise, as in gdn_prefill_intra.cuh's products of accumulators: the same sums to the last bit.
+template <int kSteps, int kN, bool kPairs = false>
 __device__ __forceinline__ void mma_tile_tf32(const float* A, int lda, const float* B, int ldb,
                                               float (&c)[kN][4], int g, int t) {
     uint32_t a[kSteps][4], b[kSteps][kN][2];
@@ -76,14 +77,15 @@ __device__ __forceinline__ void mma_tile_tf32(const float* A, int lda, const flo
     for (int ks = 0; ks < kSteps; ++ks) {          // every load first, then the products
         const float* a_ = A + 8 * ks;
         const float* b_ = B + (8 * ks) * ldb;
-        a[ks][0] = to_tf32(a_[g * lda + t]);
-        a[ks][1] = to_tf32(a_[(g + 8) * lda + t]);
-        a[ks][2] = to_tf32(a_[g * lda + t + 4]);
-        a[ks][3] = to_tf32(a_[(g + 8) * lda + t + 4]);
+        const int k0 = kPairs ? 2 * t : t, k1 = kPairs ? 2 * t + 1 : t + 4;
+        a[ks][0] = to_tf32(a_[g * lda + k0]);
+        a[ks][1] = to_tf32(a_[(g + 8) * lda + k0]);
+        a[ks][2] = to_tf32(a_[g * lda + k1]);
+        a[ks][3] = to_tf32(a_[(g + 8) * lda + k1]);
 #pragma unroll
         for (int nb = 0; nb < kN; ++nb) {
-            b[ks][nb][0] = to_tf32(b_[t * ldb + 8 * nb + g]);
-            b[ks][nb][1] = to_tf32(b_[(t + 4) * ldb + 8 * nb + g]);
+            b[ks][nb][0] = to_tf32(b_[k0 * ldb + 8 * nb + g]);
+            b[ks][nb][1] = to_tf32(b_[k1 * ldb + 8 * nb + g]);
         }
     }
 #pragma unroll
@@ -104,6 +106,7 @@ struct IntraStatics {
     alignas(16) float s_b2[kChunk];    // b_r log2(e): inclusive log-decay prefix
     alignas(16) float s_beta[kChunk];  // beta_r (0 past the chunk's length)
     alignas(16) float s_bg[kChunk];    // beta_r e^{b_r}
+    alignas(16) float s_fall[32];      // e^{b_31 - b_i}, i < 32
 };
 
 // T = (I + A)^{-1} for the strictly lower-triangular 64x64 A in sA (fp32, row-major, stride kLdA),
@@ -155,7 +158,7 @@ __device__ __forceinline__ void solve_blocks_16_32(float* sA, const int pr, cons
         c[nb][0] = c[nb][1] = c[nb][2] = c[nb][3] = 0.f;
     }
     __syncwarp();
-    mma_tile_tf32<2, 2>(sA + (16 * I) * kLdA + 16 * I, kLdA, X, kLdA, c, g, t);         // T_IJ = -T_II X
+    mma_tile_tf32<2, 2, true>(sA + (16 * I) * kLdA + 16 * I, kLdA, X, kLdA, c, g, t);   // T_IJ = -T_II X
     __syncwarp();                                      // every lane has read A_IJ (above)
 #pragma unroll
     for (int nb = 0; nb < 2; ++nb) {
@@ -189,9 +192,9 @@ __device__ __forceinline__ void solve_merge_64(float* sA, const int w, const int
     asm volatile("bar.sync %0, 128;" ::"r"(bar_id) : "memory");
     // X = -Tb Y; the rows 0-15 of Tb have columns 0-15 only
     if (r0 == 0)
-        mma_tile_tf32<2, 2>(sA + 32 * kLdA + 32, kLdA, Y, kLdA, c, g, t);
+        mma_tile_tf32<2, 2, true>(sA + 32 * kLdA + 32, kLdA, Y, kLdA, c, g, t);
     else
-        mma_tile_tf32<4, 2>(sA + 48 * kLdA + 32, kLdA, Y, kLdA, c, g, t);
+        mma_tile_tf32<4, 2, true>(sA + 48 * kLdA + 32, kLdA, Y, kLdA, c, g, t);
 #pragma unroll
     for (int nb = 0; nb < 2; ++nb) {
         float* dst = sA + (32 + r0) * kLdA + c0 + 8 * nb;
@@ -318,6 +321,11 @@ __device__ __forceinline__ bool intra_item(const TensorMaps& maps, const Prefill
         st.s_beta[2 * lane] = be0; st.s_beta[2 * lane + 1] = be1;
         const float e0 = ex2_approx(b0 * kLog2e), e1 = ex2_approx(b1 * kLog2e);
         st.s_bg[2 * lane] = be0 * e0; st.s_bg[2 * lane + 1] = be1 * e1;
+        const float b31 = __shfl_sync(0xffffffffu, incl, 15);
+        if (lane < 16) {
+            st.s_fall[2 * lane] = ex2_approx((b31 - b0) * kLog2e);
+            st.s_fall[2 * lane + 1] = ex2_approx((b31 - b1) * kLog2e);
+        }
         // the record's vectors: e^{b_C - b_c}, scale e^{b_r}, and e^{b_C}
         *reinterpret_cast<float2*>(rec + kRecDecay + 8 * lane) =
             make_float2(ex2_approx((bC - b0) * kLog2e), ex2_approx((bC - b1) * kLog2e));
@@ -387,6 +395,9 @@ __device__ __forceinline__ bool intra_item(const TensorMaps& maps, const Prefill
         const float br2 = st.s_b2[r];
         const float rowscale = is_p ? p.scale : st.s_beta[r];      // the output scale rides on P
         const int limit = is_p ? r : r - 1;              // keep columns i <= limit
+        // columns 0-31 of rows 32-63: times e^{b_r - b_31} e^{b_31 - b_i}
+        const bool below = (row & 32) != 0 && colhalf == 0;
+        const float rowfall = below ? rowscale * ex2_approx(br2 - st.s_b2[31]) : 0.f;
         // (rows of a half without tokens are not read)
         if ((row & 32) < ci.len)
 #pragma unroll
@@ -405,11 +416,12 @@ __device__ __forceinline__ bool intra_item(const TensorMaps& maps, const Prefill
                 tmem_wait_ld();
 #pragma unroll
                 for (int q4 = 0; q4 < 4; ++q4) {
-                    const float4 bb = *reinterpret_cast<const float4*>(st.s_b2 + cbase + 4 * q4);
+                    const float4 bb = *reinterpret_cast<const float4*>((below ? st.s_fall : st.s_b2) + cbase + 4 * q4);
                     const float bv[4] = {bb.x, bb.y, bb.z, bb.w};
 #pragma unroll
                     for (int e = 0; e < 4; ++e)          // times e^{b_r - b_i} (above the diagonal: discarded)
-                        val[4 * q4 + e] = rowscale * __uint_as_float(x[4 * q4 + e]) * ex2_approx(br2 - bv[e]);
+                        val[4 * q4 + e] = below ? rowfall * __uint_as_float(x[4 * q4 + e]) * bv[e]
+                                                : rowscale * __uint_as_float(x[4 * q4 + e]) * ex2_approx(br2 - bv[e]);
                 }
                 if (cbase + 15 >= (row & 32)) {
 #pragma unroll

@@ -19,11 +19,10 @@ namespace gdn {
 // =============================================================================================
 constexpr int kFPrepThreads = 256;
 // model of the two-part production (see the kernel): items per SM and chunk step, start-up lag of the second part in
-// chunk steps, and a safety margin in items.  (0.3 would be what the producers do, 0.385 leaves 32 chains the small
-// cut although their chains then wait a little: records are read while still in L2, and the machine is at its power
-// limit.  32 chains of 512 chunks 805 -> 696 us, of 188 296 -> 271; 40 chains, which need the larger cut, 233 -> 227.)
+// chunk steps, and a safety margin in items.  (The time is flat around these: 32 chains of 512 chunks 616 us with a lead
+// of 8 steps, 617 of 4; of 41 80.5 and 82.1; 48 chains of 96, 32 and 15 chunks 152 and 153.)
 constexpr int kSplitProdPermille = 385;
-constexpr int kSplitLeadSteps = 4;
+constexpr int kSplitLeadSteps = 8;
 constexpr int kSplitMarginItems = 64;
 
 __global__ void __launch_bounds__(kFPrepThreads)
@@ -63,6 +62,7 @@ prefill_fused_prep_kernel(const int32_t* __restrict__ cu, int32_t T, int32_t N, 
         end_before = 0;
         hdr[kHdrItemHead] = 0;
         hdr[kHdrStarted] = 0;
+        hdr[kHdrProgress] = 0;
         if (cu[0] != 0 || cu[N] != T) report(dev_status, kDevBadCuSeqlens);
     }
     __syncthreads();
@@ -357,8 +357,7 @@ __global__ void __launch_bounds__(kFusedThreads, 1)
 prefill_fused_kernel(const __grid_constant__ TensorMaps maps, const PrefillParams p, uint8_t* ws,
                      const WorkspaceLayout lay, const int n_state) {
     extern __shared__ uint8_t smem_raw[];
-    uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
-                                               ~static_cast<uintptr_t>(1023));
+    uint8_t* smem = align_1024(smem_raw);
     __shared__ IntraStatics intra_statics[kFGroups];
     __shared__ uint32_t tmem_base_s;
     const int warp = threadIdx.x >> 5;

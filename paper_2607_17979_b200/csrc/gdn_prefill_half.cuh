@@ -148,6 +148,8 @@ __device__ __forceinline__ void state_half_role(const TensorMaps& maps, const Pr
         (void)flags;
         (void)pos;
         (void)cut;
+        volatile int32_t* progress = reinterpret_cast<int32_t*>(ws) + kHdrProgress;
+        (void)progress;
         uint32_t started = 0;           // (kHalfGated) the producers have been seen to run
         (void)started;
         bool live = true;
@@ -219,9 +221,11 @@ __device__ __forceinline__ void state_half_role(const TensorMaps& maps, const Pr
                     tma_load_2d(c_at + kHC_K + 8192, &maps.k, u.hqk * kD + 64, tok, &bar_full_c[ring.st]);
                 }
                 ring.next();
+                if (kMode == kHalfGated && cta == 0 && lane == 0) *progress = j;     // (paces the producers)
             }
             gc += u.nc;
         }
+        if (kMode == kHalfGated && cta == 0 && lane == 0) *progress = 0x7fffffff;
         __syncwarp();
     } else if (warp > kHLoadWarp) {
         // one warp to spare

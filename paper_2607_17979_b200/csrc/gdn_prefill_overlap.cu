@@ -9,16 +9,16 @@
 //
 // Five launches in one stream, the first four each a programmatic dependent of the one before:
 //   prep          chunk table, ranking, processing order, cleared flags and done table, the cut
-//   first part    waits for prep; items [0, cut) of the order, 4 CTAs per SM
+//   first part    waits for prep; items [0, cut) of the order, a CTA per SM
 //   state pass    waits for the first part, THEN lets its dependent start, so the second part's
 //                 CTAs are scheduled only once every state-pass CTA is resident: they can never
 //                 take the SMs the chains need, and every chain that waits for a record is
 //                 resident while the producers still have SMs of their own (the launcher keeps
 //                 2 units <= SMs - kOverlapSpareSms, so every CTA has one half unit)
 //   second part   does not wait for the state pass (it only feeds it); items [cut, total), pulled
-//                 from a queue by twelve CTAs per unit (at most four per SM).  Its CTA 0 waits
-//                 for the state pass at its very end, so that the completion of this launch
-//                 implies the state pass's.
+//                 from a queue by a CTA per SM that is, or becomes, free, no further ahead of the
+//                 chains than what stays in L2.  Its CTA 0 waits for the state pass at its very end,
+//                 so that the completion of this launch implies the state pass's.
 //   rest          an ordinary launch.  CUDA lets a programmatic dependent start early, it does not
 //                 promise to; if the second part has not started when a chain has waited for a record for 0.2 ms,
 //                 the chain gives up (without an error: a half unit's final state is written only after
@@ -27,122 +27,40 @@
 //                 every record exists.  Normally every CTA finds its half unit done and returns at
 //                 once.
 #include "gdn_prefill_half.cuh"
+#include "gdn_prefill_intra.cuh"
 #include <algorithm>
 #include <cstdlib>
 
 namespace gdn {
 
-// First part: resident CTAs over the items [0, cut) of the processing order.  (With one CTA per item the grid has to
-// be sized for all of them, the cut being known on the device only, and the CTAs that find nothing to do leave at 4 ns
-// each: 32768 tokens at 32 heads, a fifth of the items first, 52 us of nothing else.)
-__global__ void __launch_bounds__(kIntraThreads, 4)
+// First part: the items [0, cut) of the processing order.
+__global__ void __launch_bounds__(kProdThreads, 1)
 prefill_intra_first_kernel(const __grid_constant__ TensorMaps maps, const PrefillParams p,
                            uint8_t* ws, const WorkspaceLayout lay) {
     pdl_launch_dependents();
-    pdl_wait();                     // the tables are the prep kernel's
-    const int cut = reinterpret_cast<const int32_t*>(ws)[kHdrSplit];
-    if (static_cast<int>(blockIdx.x) >= cut) return;
-
-    extern __shared__ uint8_t smem_raw[];
-    uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
-                                               ~static_cast<uintptr_t>(1023));
-    __shared__ IntraStatics st;
-    __shared__ uint32_t tmem_base_s;
-    const int tid = threadIdx.x, warp = tid >> 5;
-    if (warp == 0) {
-        tmem_alloc(&tmem_base_s, kIntraTmemCols);
-        tmem_relinquish();
-    }
-    tc_fence_before_sync();
-    __syncthreads();
-    tc_fence_after_sync();
-    uint32_t n_done = 0;
-#pragma unroll 1
-    for (int item = blockIdx.x; item < cut; item += gridDim.x) {
-        const int k = item / p.by_hv;
-        const int hv = item - k * p.Hv;
-        const int c = reinterpret_cast<const int32_t*>(ws + lay.order)[k];
-        const ChunkInfo ci = reinterpret_cast<const ChunkInfo*>(ws + lay.chunks)[c];
-        uint8_t* rec = ws + lay.records + (static_cast<size_t>(c) * p.Hv + hv) * kRecBytes;
-        const bool ok = intra_item<false>(maps, p, rec, ci, hv / p.by_group, hv, smem, st, &tmem_base_s, 0, tid,
-                                          [] { __syncthreads(); }, n_done);
-        ++n_done;
-        tc_fence_before_sync();
-        __syncthreads();
-        tc_fence_after_sync();
-        if (!ok) break;
-    }
-    if (warp == 0) tmem_dealloc(tmem_base_s, kIntraTmemCols);
+    produce_cta<kItemsFirst>(maps, p, ws, lay);
 }
 
-// Second part: resident CTAs pull the items [cut, total) from a queue, in the order the chains
-// consume them, and publish each record through its flag.  No wait for the state pass (this kernel
-// feeds it): every state-pass CTA has passed its own wait for the first part, hence for prep,
-// before this kernel's CTAs are scheduled.
-__global__ void __launch_bounds__(kIntraThreads, 4)
+// Second part: the items [cut, total) from a queue, in the order the chains consume them; each record is published
+// through its flag.  No wait for the state pass (this kernel feeds it): every state-pass CTA has passed its own wait for
+// the first part, hence for prep, before this kernel's CTAs are scheduled.
+__global__ void __launch_bounds__(kProdThreads, 1)
 prefill_intra_second_kernel(const __grid_constant__ TensorMaps maps, const PrefillParams p,
                             uint8_t* ws, const WorkspaceLayout lay) {
     int32_t* hdr = reinterpret_cast<int32_t*>(ws);
     if (blockIdx.x == 0 && threadIdx.x == 0) st_release_u32(reinterpret_cast<uint32_t*>(hdr + kHdrStarted), 1u);
-    const int32_t cut = hdr[kHdrSplit], total = hdr[kHdrTotalItems];
-    const int32_t* order = reinterpret_cast<const int32_t*>(ws + lay.order);
-    const ChunkInfo* chunks = reinterpret_cast<const ChunkInfo*>(ws + lay.chunks);
-    uint32_t* flags = reinterpret_cast<uint32_t*>(ws + lay.flags);
-
-    extern __shared__ uint8_t smem_raw[];
-    uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
-                                               ~static_cast<uintptr_t>(1023));
-    __shared__ IntraStatics st;
-    __shared__ uint32_t tmem_base_s;
-    const int tid = threadIdx.x, warp = tid >> 5;
-    if (cut < total) {
-        if (warp == 0) {
-            tmem_alloc(&tmem_base_s, kIntraTmemCols);
-            tmem_relinquish();
-        }
-        tc_fence_before_sync();
-        __syncthreads();
-        tc_fence_after_sync();
-        uint32_t n_done = 0;
-        for (;;) {
-            if (tid == 0) st.item = cut + atomicAdd(&hdr[kHdrItemHead], 1);
-            __syncthreads();
-            const int item = st.item;
-            if (item >= total) break;
-            const int k = item / p.by_hv;
-            const int hv = item - k * p.Hv;
-            const int c = order[k];
-            const ChunkInfo ci = chunks[c];
-            const size_t slot = static_cast<size_t>(c) * p.Hv + hv;
-            uint8_t* rec = ws + lay.records + slot * kRecBytes;
-            const bool ok = intra_item<false>(maps, p, rec, ci, hv / p.by_group, hv, smem, st, &tmem_base_s, 0, tid,
-                                       [] { __syncthreads(); }, n_done);
-            ++n_done;
-            // publish: every thread's own stores first, then the bulk stores, then the flag
-            __threadfence();
-            tc_fence_before_sync();
-            __syncthreads();
-            if (tid == 0) {
-                bulk_wait_all();
-                fence_proxy_async_all();
-                __threadfence();
-                st_release_u32(&flags[slot], ok ? 1u : 2u);      // 2 = produced after a timeout
-            }
-            if (!ok) break;
-        }
-        tc_fence_before_sync();
-        __syncthreads();
-        if (warp == 0) tmem_dealloc(tmem_base_s, kIntraTmemCols);
-    }
+    if (hdr[kHdrSplit] < hdr[kHdrTotalItems]) produce_cta<kItemsQueue>(maps, p, ws, lay);
     if (blockIdx.x == 0) pdl_wait();        // the call is complete when this launch is
 }
 
-__global__ void __launch_bounds__(kStreamThreads, 1)
+// The two halves of a unit run as a cluster, which puts them on the two SMs of one TPC: a chain whose neighbour in the
+// TPC is a producer takes 1.65 us a step instead of 1.2 (32768 tokens at 32 heads: 650 to 1000 us a call, by where the
+// CTAs happened to land; as pairs 617).
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kStreamThreads, 1)
 prefill_state_half_gated_kernel(const __grid_constant__ TensorMaps maps, const PrefillParams p,
                                   uint8_t* ws, const WorkspaceLayout lay) {
     extern __shared__ uint8_t smem_raw[];
-    uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
-                                               ~static_cast<uintptr_t>(1023));
+    uint8_t* smem = align_1024(smem_raw);
     __shared__ uint32_t tmem_base_s;
     const int warp = threadIdx.x >> 5;
     if (warp == kSIssueWarp) {
@@ -171,8 +89,7 @@ prefill_state_half_rest_kernel(const __grid_constant__ TensorMaps maps, const Pr
         if (reinterpret_cast<const uint16_t*>(ws + lay.done)[blockIdx.x] != 0) return;
     }
     extern __shared__ uint8_t smem_raw[];
-    uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
-                                               ~static_cast<uintptr_t>(1023));
+    uint8_t* smem = align_1024(smem_raw);
     __shared__ uint32_t tmem_base_s;
     const int warp = threadIdx.x >> 5;
     if (warp == kSIssueWarp) {
@@ -198,9 +115,9 @@ cudaError_t launch_prefill_overlap(const ChunkedParams& cp, cudaStream_t stream,
     if (e != cudaSuccess) return e;
     e = ensure_dynamic_smem(prefill_state_half_rest_kernel, kHalfSmem);
     if (e != cudaSuccess) return e;
-    e = ensure_dynamic_smem(prefill_intra_first_kernel, kIntraSmem);
+    e = ensure_dynamic_smem(prefill_intra_first_kernel, kProdSmem);
     if (e != cudaSuccess) return e;
-    e = ensure_dynamic_smem(prefill_intra_second_kernel, kIntraSmem);
+    e = ensure_dynamic_smem(prefill_intra_second_kernel, kProdSmem);
     if (e != cudaSuccess) return e;
     TensorMaps maps;
     if (!make_prefill_tensor_maps(&maps, p)) return cudaErrorInvalidValue;
@@ -223,26 +140,21 @@ cudaError_t launch_prefill_overlap(const ChunkedParams& cp, cudaStream_t stream,
     e = launch_prefill_ranked_prep(cp, stream, 2, split_permille, sms);
     if (e != cudaSuccess) return e;
     const dim3 items(static_cast<unsigned>(cp.lay.max_chunks) * static_cast<unsigned>(p.Hv));
-    const dim3 resident_first(std::min(items.x, 4u * static_cast<unsigned>(sms)));
-    e = launch_dependent(prefill_intra_first_kernel, resident_first, dim3(kIntraThreads), kIntraSmem,
+    const dim3 resident_first(std::min(items.x, static_cast<unsigned>(sms)));
+    e = launch_dependent(prefill_intra_first_kernel, resident_first, dim3(kProdThreads), kProdSmem,
                          stream, maps, p, cp.ws, cp.lay);
     if (e != cudaSuccess) return e;
     const int grid = static_cast<int>(2 * units);
     e = launch_dependent(prefill_state_half_gated_kernel, dim3(grid), dim3(kStreamThreads),
                          kHalfSmem, stream, maps, p, cp.ws, cp.lay);
     if (e != cudaSuccess) return e;
-    // Producers beyond what the chains consume only add memory traffic beside them: a unit takes a record per chunk
-    // step and a producer CTA needs about twelve chunk steps per item (four on an SM), so twelve CTAs per unit keep
-    // up.
-    unsigned resident = 12u * static_cast<unsigned>(units);
-    if (resident < static_cast<unsigned>(sms)) resident = static_cast<unsigned>(sms);
-    if (resident > 4u * static_cast<unsigned>(sms)) resident = 4u * static_cast<unsigned>(sms);
+    const unsigned resident = static_cast<unsigned>(sms);
     const dim3 producers(items.x < resident ? items.x : resident);
     if (serialised) {
-        prefill_intra_second_kernel<<<producers, kIntraThreads, kIntraSmem, stream>>>(maps, p, cp.ws, cp.lay);
+        prefill_intra_second_kernel<<<producers, kProdThreads, kProdSmem, stream>>>(maps, p, cp.ws, cp.lay);
         e = cudaGetLastError();
     } else {
-        e = launch_dependent(prefill_intra_second_kernel, producers, dim3(kIntraThreads), kIntraSmem,
+        e = launch_dependent(prefill_intra_second_kernel, producers, dim3(kProdThreads), kProdSmem,
                              stream, maps, p, cp.ws, cp.lay);
     }
     if (e != cudaSuccess) return e;

@@ -9,8 +9,7 @@ __global__ void __launch_bounds__(kStreamThreads, 1)
 prefill_state_stream_kernel(const __grid_constant__ TensorMaps maps, const PrefillParams p,
                             uint8_t* ws, const WorkspaceLayout lay) {
     extern __shared__ uint8_t smem_raw[];
-    uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
-                                               ~static_cast<uintptr_t>(1023));
+    uint8_t* smem = align_1024(smem_raw);
     __shared__ uint32_t tmem_base_s;
     const int warp = threadIdx.x >> 5;
     if (warp == kSIssueWarp) {
@@ -31,8 +30,7 @@ __global__ void __launch_bounds__(kStreamThreads, 1)
 prefill_state_half_kernel(const __grid_constant__ TensorMaps maps, const PrefillParams p, uint8_t* ws,
                           const WorkspaceLayout lay) {
     extern __shared__ uint8_t smem_raw[];
-    uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
-                                               ~static_cast<uintptr_t>(1023));
+    uint8_t* smem = align_1024(smem_raw);
     __shared__ uint32_t tmem_base_s;
     const int warp = threadIdx.x >> 5;
     if (warp == kSIssueWarp) {

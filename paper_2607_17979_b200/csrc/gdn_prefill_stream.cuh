@@ -144,18 +144,6 @@ __device__ __forceinline__ UnitInfo unit_info(const PrefillParams& p, const uint
 
 constexpr uint32_t kSpinFlagLimit = 1u << 22;
 
-__device__ __forceinline__ uint32_t ld_acquire_u32(const uint32_t* p) {
-    uint32_t v;
-    asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
-    return v;
-}
-__device__ __forceinline__ void st_release_u32(uint32_t* p, uint32_t v) {
-    asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
-}
-__device__ __forceinline__ void fence_proxy_async_all() {
-    asm volatile("fence.proxy.async;" ::: "memory");
-}
-
 // The state pass of one CTA of 512 threads over its share of the rank-sorted units.  kGated = false: every record
 // exists (the intra-chunk kernel ran before).  true: records are being produced by other CTAs of the same cooperative
 // launch and the loading warps wait for each record's flag first.  `tmem` = 512 allocated columns; ends with a CTA
