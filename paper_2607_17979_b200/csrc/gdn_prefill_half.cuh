@@ -15,8 +15,8 @@
 //
 // The roles, their barriers and the unit order are those of gdn_prefill_stream.cuh, with these differences: the fp32
 // master state is held as fragments (32 registers a thread), so whole states cross to and from global memory directly,
-// 8 rows of 32 bytes an access; the accumulator of S W^T is double-buffered, so U~ is in place a chunk
-// ahead; and a CTA's list of half units turns round at each pass over the CTAs (a CTA that took a long one of a pass
+// 8 rows of 32 bytes an access; the bf16 state is double-buffered, so the outputs' products may read the last
+// one while the next is stored; and a CTA's list of half units turns round at each pass over the CTAs (a CTA that took a long one of a pass
 // takes a short one of the next).
 #pragma once
 #include "gdn_prefill_stream.cuh"
@@ -34,10 +34,12 @@ constexpr uint32_t kHC_K = 0, kHC_P = 16384, kHCBytes = 24576;
 constexpr uint32_t kHB_U = 0, kHB_Vec = kRecUHalf, kHBBytes = kRecUHalf + 1024;
 static_assert(kHB_Vec + (kRecBytes - kRecDecay) <= kHBBytes, "the vectors fit");
 constexpr uint32_t kHS_A = 0, kHS_C = kHS_A + kHStages * kHABytes, kHS_B = kHS_C + kHStages * kHCBytes;
-constexpr uint32_t kHS_Out = kHS_B + 2 * kHBBytes;              // o staging [64 tokens][64 dv] bf16
-constexpr uint32_t kHalfSmem = kHS_Out + 8192 + 1024;
-// TMEM columns: S W^T (two tiles), S Q^T, U P^T, the state product, bf16 S, decayed U (hi / lo lanes), U
-constexpr uint32_t kH_D1 = 0, kH_Y1 = 128, kH_Y2 = 192, kH_D4 = 256, kH_S = 384, kH_Us = 448, kH_U = 480;
+constexpr uint32_t kHS_Out = kHS_B + 2 * kHBBytes;              // o staging, two tiles [64 tokens][64 dv] bf16
+constexpr uint32_t kHalfSmem = kHS_Out + 2 * 8192 + 1024;
+// TMEM columns: S W^T, S Q^T, U P^T, the state product, bf16 S (of odd chunks, of even ones: the next is stored while S Q^T
+// still reads the last), decayed U (hi / lo lanes), U
+constexpr uint32_t kH_D1 = 0, kH_Y1 = 128, kH_Y2 = 192, kH_D4 = 256, kH_SOdd = 64, kH_SEven = 384, kH_Us = 448, kH_U = 480;
+__device__ __forceinline__ uint32_t half_s_col(uint32_t g) { return g & 1 ? kH_SOdd : kH_SEven; }
 
 // Polls of a record's flag, about 0.4 us each.  A few milliseconds: far longer than the producers ever lag
 // when they do run beside the state pass, far shorter than the other roles' mbarrier waits (which would report an
@@ -64,7 +66,7 @@ __device__ __forceinline__ void state_half_role(const TensorMaps& maps, const Pr
                                                 const WorkspaceLayout& lay, uint8_t* smem, const uint32_t tmem,
                                                 const int cta, const int n_ctas) {
     __shared__ uint64_t bar_full_a[kHStages], bar_full_b[2], bar_full_c[kHStages], bar_free_a[kHStages], bar_free_b[2],
-        bar_free_c[kHStages], bar_y[2], bar_p[2], bar_y_read, bar_y1, bar_d1, bar_d4, bar_s, bar_u,
+        bar_free_c[kHStages], bar_y[2], bar_p[2], bar_y_read, bar_d1, bar_d4[2], bar_s[2], bar_u,
         bar_drain[2];
     __shared__ int abort_flag;
     __shared__ uint32_t armed[3];         // chunks of the CTA's stream whose copies the loader has started, per ring
@@ -87,18 +89,17 @@ __device__ __forceinline__ void state_half_role(const TensorMaps& maps, const Pr
             mbar_init(&bar_y[st], 1);
             mbar_init(&bar_p[st], kSOutThreads / 32); // U~ in the accumulator
             mbar_init(&bar_drain[st], 1);             // an issuer that gave up: its products
+            mbar_init(&bar_d4[st], 1);                // by halves of dk
+            mbar_init(&bar_s[st], kSEpiWarps / 2);    // the bf16 state in TMEM, by halves of dk
         }
         for (int st = 0; st < kHStages; ++st) {
             mbar_init(&bar_full_a[st], 1);
             mbar_init(&bar_full_c[st], 1);
-            mbar_init(&bar_free_a[st], 2);            // one product of either issuer
-            mbar_init(&bar_free_c[st], 2);
+            mbar_init(&bar_free_a[st], 2);            // a product of either issuer
+            mbar_init(&bar_free_c[st], 1);
         }
         mbar_init(&bar_d1, 1);
-        mbar_init(&bar_d4, 1);
-        mbar_init(&bar_y1, 1);
         mbar_init(&bar_y_read, kSOutThreads / 32);
-        mbar_init(&bar_s, kSEpiWarps);                // the bf16 state in TMEM
         mbar_init(&bar_u, kSEpiWarps);
         abort_flag = 0;
         armed[0] = armed[1] = armed[2] = 0;
@@ -230,16 +231,15 @@ __device__ __forceinline__ void state_half_role(const TensorMaps& maps, const Pr
     } else if (warp > kHLoadWarp) {
         // one warp to spare
     } else if (warp >= kSIssueWarp) {
-        // ===================== issuers: the whole warp waits, one elected lane issues.  An instruction takes 29 cycles
-        // to issue at best, so the chain's products (S W^T, the state product) have a warp of their own; the other issues
-        // the outputs' (S Q^T, U P^T), each behind a chain product's completion, so that it never runs in front of the
-        // next or beside it.
+        // ===================== issuers: the whole warp waits, one elected lane issues.  Two warps: S W^T; and, in this order,
+        // the state product, S Q^T and U P^T.  The products run in the order of issue, so the outputs' two run while the
+        // chain warps are at the state, and neither in front of a product of the chain's nor beside it: with S Q^T right
+        // behind S W^T (beside the U phase, which is shorter) the state product came 130 cycles later.
         const bool outputs = warp > kSIssueWarp;
         const uint32_t id_w = make_idesc_bf16(64, 64, false, true) | kIdescNegateB;
         const uint32_t id_qp = make_idesc_bf16(64, 64, false, false);
-        const uint32_t id_k = make_idesc_bf16(128, 128, false, true);
+        const uint32_t id_k = make_idesc_bf16(128, 64, false, true);
         const uint32_t s0 = smem_u32(smem);
-        const uint32_t tS = tmem + kH_S;
         bool live = true;
         UnitInfo nxt = info(at(0));
         for (int i = 0, hu = at(0); hu < total && live; hu = at(++i)) {
@@ -247,17 +247,15 @@ __device__ __forceinline__ void state_half_role(const TensorMaps& maps, const Pr
             nxt = info(at(i + 1));
             if (u.skip || is_done(hu)) continue;
             if (!outputs) {
-                const uint64_t dW0 = make_sdesc_sw128(s0 + kHS_A + kHA_W, 8192, 1024),
-                               dK0 = make_sdesc_sw128(s0 + kHS_C + kHC_K, 8192, 1024);
-                const uint32_t tD4 = tmem + kH_D4, tUs = tmem + kH_Us;
+                const uint64_t dW0 = make_sdesc_sw128(s0 + kHS_A + kHA_W, 8192, 1024);
 #pragma unroll 1
                 for (int j = 0; j < u.nc; ++j, ring.next()) {
                     const uint32_t g = gc + j;
-                    const uint64_t w = sdesc_advance(dW0, ring.st * kHABytes), kk = sdesc_advance(dK0, ring.st * kHCBytes);
-                    const uint32_t tD1 = tmem + kH_D1 + 64 * (g & 1);
+                    const uint64_t w = sdesc_advance(dW0, ring.st * kHABytes);
+                    const uint32_t tD1 = tmem + kH_D1, tS = tmem + half_s_col(g);
                     if (!warp_wait(&bar_full_a[ring.st], ring.par, abortp, kWaitReason) ||
                         !warp_wait(&bar_p[g & 1], (g >> 1) & 1u, abortp, kWaitReason) ||      // U~ in place
-                        !warp_wait(&bar_s, g & 1u, abortp, kWaitReason)) {                    // bf16 S in TMEM
+                        !warp_wait(&bar_s[0], g & 1u, abortp, kWaitReason)) {                 // bf16 S in TMEM, dk 0-63
                         live = false;
                         break;
                     }
@@ -265,40 +263,51 @@ __device__ __forceinline__ void state_half_role(const TensorMaps& maps, const Pr
                     // U = U~ - S W^T; W is MN-major: k-step ks reads 16 dk rows = 2048 bytes
                     if (elect_one()) {
 #pragma unroll
-                        for (int ks = 0; ks < 8; ++ks)
+                        for (int ks = 0; ks < 4; ++ks)
+                            mma_ts_c<true>(tD1, tS + 8 * ks, sdesc_advance(w, 2048 * ks), id_w);
+                    }
+                    if (!warp_wait(&bar_s[1], g & 1u, abortp, kWaitReason)) {                 // dk 64-127
+                        live = false;
+                        break;
+                    }
+                    tc_fence_after_sync();
+                    if (elect_one()) {
+#pragma unroll
+                        for (int ks = 4; ks < 8; ++ks)
                             mma_ts_c<true>(tD1, tS + 8 * ks, sdesc_advance(w, 2048 * ks), id_w);
                         mma_commit(&bar_d1);
                         mma_commit(&bar_free_a[ring.st]);                     // W has been read
                     }
+                }
+            } else {
+                const uint64_t dQ0 = make_sdesc_sw128(s0 + kHS_A + kHA_Q, 16, 1024), dP0 = make_sdesc_sw128(s0 + kHS_C + kHC_P, 16, 1024),
+                               dK0 = make_sdesc_sw128(s0 + kHS_C + kHC_K, 8192, 1024);
+                const uint32_t tY1 = tmem + kH_Y1, tY2 = tmem + kH_Y2, tU = tmem + kH_U, tD4 = tmem + kH_D4, tUs = tmem + kH_Us;
+#pragma unroll 1
+                for (int j = 0; j < u.nc; ++j, ring.next()) {
+                    const uint32_t g = gc + j, tS = tmem + half_s_col(g);
+                    const uint64_t q = sdesc_advance(dQ0, ring.st * kHABytes), pp = sdesc_advance(dP0, ring.st * kHCBytes),
+                                   kk = sdesc_advance(dK0, ring.st * kHCBytes);
                     if (!warp_wait(&bar_full_c[ring.st], ring.par, abortp, kWaitReason) ||
                         !warp_wait(&bar_u, g & 1u, abortp, kWaitReason)) {        // U operands in TMEM
                         live = false;
                         break;
                     }
                     tc_fence_after_sync();
-                    // (U decayed) K, hi and lo terms in the lower and upper lanes (K tile MN-major: 16 tokens = 2048
-                    // bytes)
                     if (elect_one()) {
-                        mma_ts_c<false>(tD4, tUs, kk, id_k);
+                        // (U decayed) K, hi and lo terms in the lower and upper lanes (K tile MN-major: 16 tokens = 2048
+                        // bytes)
 #pragma unroll
-                        for (int ks = 1; ks < 4; ++ks)
-                            mma_ts_c<true>(tD4, tUs + 8 * ks, sdesc_advance(kk, 2048 * ks), id_k);
-                        mma_commit(&bar_d4);
-                        mma_commit(&bar_free_c[ring.st]);                     // the K tile has been read
+                        for (int h = 0; h < 2; ++h) {
+                            mma_ts_c<false>(tD4 + 64 * h, tUs, sdesc_advance(kk, 8192 * h), id_k);
+#pragma unroll
+                            for (int ks = 1; ks < 4; ++ks)
+                                mma_ts_c<true>(tD4 + 64 * h, tUs + 8 * ks, sdesc_advance(kk, 8192 * h + 2048 * ks), id_k);
+                            mma_commit(&bar_d4[h]);
+                        }
                     }
-                }
-            } else {
-                const uint64_t dQ0 = make_sdesc_sw128(s0 + kHS_A + kHA_Q, 16, 1024),
-                               dP0 = make_sdesc_sw128(s0 + kHS_C + kHC_P, 16, 1024);
-                const uint32_t tY1 = tmem + kH_Y1, tY2 = tmem + kH_Y2, tU = tmem + kH_U;
-#pragma unroll 1
-                for (int j = 0; j < u.nc; ++j, ring.next()) {
-                    const uint32_t g = gc + j;
-                    const uint64_t q = sdesc_advance(dQ0, ring.st * kHABytes), pp = sdesc_advance(dP0, ring.st * kHCBytes);
-                    // S Q^T, once S W^T has retired (its issuer has waited for the tiles), into the tile the output
-                    // warps read a chunk ago
-                    if ((g > 0 && !warp_wait(&bar_y_read, (g - 1) & 1u, abortp, kWaitReason)) ||
-                        !warp_wait(&bar_d1, g & 1u, abortp, kWaitReason)) {
+                    // S Q^T (its tile has landed with W's), into the tile that the output warps read a chunk ago
+                    if (g > 0 && !warp_wait(&bar_y_read, (g - 1) & 1u, abortp, kWaitReason)) {
                         live = false;
                         break;
                     }
@@ -308,22 +317,14 @@ __device__ __forceinline__ void state_half_role(const TensorMaps& maps, const Pr
 #pragma unroll
                         for (int ks = 1; ks < 8; ++ks)
                             mma_ts_c<true>(tY1, tS + 8 * ks, sdesc_advance(q, (ks >> 2) * 8192 + (ks & 3) * 32), id_qp);
-                        mma_commit(&bar_y1);
                         mma_commit(&bar_free_a[ring.st]);                     // Q has been read
-                    }
-                    // U P^T, once the state product has retired
-                    if (!warp_wait(&bar_d4, g & 1u, abortp, kWaitReason)) {
-                        live = false;
-                        break;
-                    }
-                    tc_fence_after_sync();
-                    if (elect_one()) {
+                        // U P^T
                         mma_ts_c<false>(tY2, tU, pp, id_qp);
 #pragma unroll
                         for (int ks = 1; ks < 4; ++ks)
                             mma_ts_c<true>(tY2, tU + 8 * ks, sdesc_advance(pp, 32 * ks), id_qp);
                         mma_commit(&bar_y[g & 1]);
-                        mma_commit(&bar_free_c[ring.st]);                     // P has been read
+                        mma_commit(&bar_free_c[ring.st]);                     // K and P have been read
                     }
                 }
             }
@@ -347,11 +348,11 @@ __device__ __forceinline__ void state_half_role(const TensorMaps& maps, const Pr
         };
         // fp32 master state as fragments: S[4 b + 2 r + e] = row q16 + g8 + 8 r, dk 64 ch + 8 b + 2 t4 + e
         float S[32];
-        auto store_state_bf16 = [&] {             // -> bf16 A operand in TMEM
+        auto store_state_bf16 = [&](uint32_t g) {       // -> chunk g's bf16 A operand in TMEM
             uint32_t pk[16];
 #pragma unroll
             for (int k = 0; k < 16; ++k) pk[k] = pack_bf16(S[2 * k], S[2 * k + 1]);
-            tmem_st_16x128b_x8(tmem + kH_S + lane_base + 32 * ch, pk);
+            tmem_st_16x128b_x8(tmem + half_s_col(g) + lane_base + 32 * ch, pk);
         };
         // element offset of a thread's first pair inside a half tile, and of pair (b, r) from there
         const int frag = (q16 + g8) * kD + 64 * ch + 2 * t4;
@@ -410,8 +411,8 @@ __device__ __forceinline__ void state_half_role(const TensorMaps& maps, const Pr
 #pragma unroll
                 for (int k = 0; k < 32; ++k) S[k] = 0.f;
             }
-            store_state_bf16();
-            hand_over(&bar_s);
+            store_state_bf16(gc);
+            hand_over(&bar_s[ch]);
             // the next initial state, towards L2
             if (p.init_state && tid == 0 && nxt.x > 0 && hu_next < total)
                 bulk_prefetch_l2(p.init_state + static_cast<size_t>(nxt.y) * (kHalfRows * kD), kHalfRows * kD * 4);
@@ -428,13 +429,14 @@ __device__ __forceinline__ void state_half_role(const TensorMaps& maps, const Pr
                 for (int b = 0; b < 4; ++b)
                     dec[b] = *reinterpret_cast<const float2*>(vec + 4 * (32 * ch + 8 * b + 2 * t4));
                 const float gC = *reinterpret_cast<const float*>(vec + (kRecGammaC - kRecDecay));
-                // U P^T of the chunk before has read the last U.  (A wait that finds its phase completed takes more
-                // than 100 cycles all the same: this one and S Q^T's below stand where a product is in flight anyway.)
+                // U P^T of the chunk before has read the last U, and S Q^T before it the bf16 state in whose place the next
+                // will be.  (A wait that finds its phase completed takes more than 100 cycles all the same: this one stands
+                // where a product is in flight anyway.)
                 if (g > 0) await(&bar_y[st ^ 1], ((g - 1) >> 1) & 1u);
                 await(&bar_d1, g & 1u);
                 {   // U (the accumulator holds U~ - S W^T): rounded, and decayed as hi + lo
                     uint32_t x[16], pu[8], ph[8], pl[8];
-                    tmem_ld_16x256b_x4(tmem + kH_D1 + 64 * st + lane_base + 32 * ch, x);
+                    tmem_ld_16x256b_x4(tmem + kH_D1 + lane_base + 32 * ch, x);
                     tmem_wait_ld();
 #pragma unroll
                     for (int b = 0; b < 4; ++b)
@@ -454,8 +456,7 @@ __device__ __forceinline__ void state_half_role(const TensorMaps& maps, const Pr
                 }
                 hand_over(&bar_u);
                 if (lane == 0) mbar_arrive(&bar_free_b[st]);    // this warp has read the vectors
-                await(&bar_y1, g & 1u);              // S Q^T has read the bf16 state
-                await(&bar_d4, g & 1u);
+                await(&bar_d4[ch], g & 1u);
                 // S <- e^{b_C} S + (hi + lo terms)
 #pragma unroll
                 for (int c = 0; c < 2; ++c) {
@@ -469,8 +470,8 @@ __device__ __forceinline__ void state_half_role(const TensorMaps& maps, const Pr
                         S[16 * c + k] = fmaf(gC, S[16 * c + k], __uint_as_float(xh[k]) + __uint_as_float(xl[k]));
                 }
                 if (j + 1 < nc) {
-                    store_state_bf16();          // the next chunk's A operand
-                    hand_over(&bar_s);
+                    store_state_bf16(g + 1);     // the next chunk's A operand
+                    hand_over(&bar_s[ch]);
                 }
             }
             // nothing of a unit is written after a failed wait (every record of the unit has been loaded by now: no
@@ -495,7 +496,6 @@ __device__ __forceinline__ void state_half_role(const TensorMaps& maps, const Pr
         const int q4 = warp & 3;
         const int ot = tid - kSOutWarp0 * 32;
         const size_t tok_stride = static_cast<size_t>(p.Hv) * kD;
-        auto out_sync = [] { asm volatile("bar.sync 1, %0;" ::"n"(kSOutThreads) : "memory"); };
         bool ok = true;
         auto await = [&](uint64_t* bar, uint32_t parity) {
             if (!warp_wait(bar, parity, abortp, kWaitReason)) ok = false;
@@ -506,32 +506,61 @@ __device__ __forceinline__ void state_half_role(const TensorMaps& maps, const Pr
             const int sq = gq & 1;
             const uint8_t* base = smem + kHS_B + sq * kHBBytes;
             await(&bar_full_b[sq], (gq >> 1) & 1u);
-            *reinterpret_cast<float2*>(&s_eb[q4][sq][2 * lane]) =
-                *reinterpret_cast<const float2*>(base + kHB_Vec + (kRecEb - kRecDecay) + 8 * lane);
             // tokens 8 b + 2 t4, + 1 of row 16 q + g8 + 8 r: token group 2 b + (t4 >> 1), see rec_u_index
             const float* sU = reinterpret_cast<const float*>(base + kHB_U) + 2 * (t4 & 1);
-            const int nb = *reinterpret_cast<const int*>(base + kHB_Vec + (kRecGammaC + 4 - kRecDecay));
+            uint32_t x[2][16];
 #pragma unroll
-            for (int c = 0; c < 2; ++c) {
-                uint32_t x[16];
+            for (int c = 0; c < 2; ++c)
 #pragma unroll
                 for (int b = 0; b < 4; ++b)
 #pragma unroll
                     for (int r = 0; r < 2; ++r) {
                         const float2 v = *reinterpret_cast<const float2*>(
                             sU + 4 * rec_u_index(8 * c + 2 * b + (t4 >> 1), 16 * q4 + g8 + 8 * r));
-                        x[4 * b + 2 * r] = __float_as_uint(v.x);
-                        x[4 * b + 2 * r + 1] = __float_as_uint(v.y);
+                        x[c][4 * b + 2 * r] = __float_as_uint(v.x);
+                        x[c][4 * b + 2 * r + 1] = __float_as_uint(v.y);
                     }
-                tmem_st_16x256b_x4(tmem + kH_D1 + 64 * sq + lane_base + 32 * c, x);
-            }
+            const float2 eb = *reinterpret_cast<const float2*>(base + kHB_Vec + (kRecEb - kRecDecay) + 8 * lane);
+            const int nb = *reinterpret_cast<const int*>(base + kHB_Vec + (kRecGammaC + 4 - kRecDecay));
+#pragma unroll
+            for (int c = 0; c < 2; ++c) tmem_st_16x256b_x4(tmem + kH_D1 + lane_base + 32 * c, x[c]);
             // blocks without tokens were not copied: whatever was there is replaced
 #pragma unroll 1
-            for (int b = nb; b < 4; ++b) tmem_zero_16x256b_x2(tmem + kH_D1 + 64 * sq + lane_base + 16 * b);
+            for (int b = nb; b < 4; ++b) tmem_zero_16x256b_x2(tmem + kH_D1 + lane_base + 16 * b);
+            *reinterpret_cast<float2*>(&s_eb[q4][sq][2 * lane]) = eb;
             tmem_wait_st();
             tc_fence_before_sync();
             __syncwarp();
             if (lane == 0) mbar_arrive(&bar_p[sq]);
+        };
+        // The rows of a chunk leave their staging tile once the next U~ is in place, for which the next S W^T waits (right
+        // behind the rows they put it off by 200 cycles).  One group barrier a chunk, which every warp runs also after a
+        // failed wait: the tile's rows are complete, and the rows in the other one, sent a chunk ago, have left.
+        struct {
+            bool any = false;
+            int tok, len, hv, half;
+            uint32_t tile;
+        } rows;
+        auto rows_out = [&] {
+            if (ot == 0) bulk_wait_read_all();
+            if constexpr (kMode == kHalfGated) ok = group_all<1, kSOutThreads>(ok);
+            else asm volatile("bar.sync 1, %0;" ::"n"(kSOutThreads) : "memory");
+            if (rows.any && ok) {
+                const uint8_t* tile = smem + rows.tile;
+                if (rows.len == kChunk) {
+                    if (ot == 0) {
+                        tma_store_2d(&maps.o, rows.hv * kD + rows.half * kHalfRows, rows.tok, tile);
+                        bulk_commit();
+                    }
+                } else {                     // a ragged tail: the rows behind it are another sequence's
+                    const int piece = ot & 7;
+                    __nv_bfloat16* og = p.o + (static_cast<size_t>(rows.tok) * p.Hv + rows.hv) * kD + rows.half * kHalfRows + piece * 8;
+                    for (int row = ot >> 3; row < rows.len; row += 16)
+                        *reinterpret_cast<uint4*>(og + row * tok_stride) =
+                            *reinterpret_cast<const uint4*>(tile + sw128_offset(row, piece));
+                }
+            }
+            rows.any = false;
         };
         bool preloaded = false;     // U~ of the chunk about to be processed is already in place
         UnitInfo nxt = info(at(0));
@@ -548,35 +577,29 @@ __device__ __forceinline__ void state_half_role(const TensorMaps& maps, const Pr
             for (int j = 0; j < u.nc; ++j) {
                 const uint32_t g = gc + j;
                 const int buf = g & 1;
-                // The accumulator of the next chunk was last read two products ago (U of chunk g - 1, in front of whose
-                // rows this group has waited), so the next U~ goes in as soon as its record is there.
+                // The next U~ goes into the accumulator as soon as the chain warps have read this chunk's U out of it (where
+                // it was not put in ahead, this group has waited for the products that follow).
                 const bool ahead = j + 1 < u.nc || (hu_next < total && !nxt.skip && !nxt_done);
 #pragma unroll 1
                 for (int k = preloaded ? 1 : 0; k < (ahead ? 2 : 1); ++k) {
                     if (k == 1) await(&bar_u, g & 1u);
+                    tc_fence_after_sync();
                     preload(g + k);
                 }
                 preloaded = ahead;
-                // Every warp runs both group barriers of every chunk, also after a failed wait; where that is no error
-                // they leave together at the first.
-                if (ot == 0) bulk_wait_read_all();       // the last chunk's rows have left the staging tile
-                if constexpr (kMode == kHalfGated) {
-                    ok = group_all<1, kSOutThreads>(ok);
-                    if (!ok) break;
-                } else {
-                    out_sync();
-                }
+                rows_out();
+                if (kMode == kHalfGated && !ok) break;   // (the verdict is the group's)
                 await(&bar_y[buf], (g >> 1) & 1u);
                 // The rows are made once the chain warps have handed the next state over and wait behind the next
                 // product: beside the refresh they take its issue slots (4096 tokens at 8 v-heads 91.5 us, 88.3 this
                 // way).
-                if (j + 1 < u.nc) await(&bar_s, (g + 1) & 1u);
+                if (j + 1 < u.nc) await(&bar_s[1], (g + 1) & 1u);
                 tc_fence_after_sync();
                 {
                     // Fragments (rows = dv, columns = tokens), rounded in pairs and stored transposed into a
                     // [token][dv] tile: lane l gives the address of matrix l / 8: tokens 8 (b + (l >> 4)) .., dv 8 (l
                     // >> 3 & 1) ..
-                    const uint32_t dst = smem_u32(smem + kHS_Out);
+                    const uint32_t dst = smem_u32(smem + kHS_Out + 8192 * buf);
 #pragma unroll
                     for (int c = 0; c < 2; ++c) {
                         uint32_t y1[16], y2[16], pk[8];
@@ -604,23 +627,11 @@ __device__ __forceinline__ void state_half_role(const TensorMaps& maps, const Pr
                 fence_proxy_async_smem();
                 __syncwarp();
                 if (lane == 0) mbar_arrive(&bar_y_read);
-                out_sync();
-                const int len = min(kChunk, u.seq_len - j * kChunk), tok = u.seq_t0 + j * kChunk;
-                if (len == kChunk) {
-                    if (ot == 0 && ok) {
-                        tma_store_2d(&maps.o, u.hv * kD + half * kHalfRows, tok, smem + kHS_Out);
-                        bulk_commit();
-                    }
-                } else if (ok) {             // a ragged tail: the rows behind it are another sequence's
-                    const int piece = ot & 7;
-                    __nv_bfloat16* og = p.o + (static_cast<size_t>(tok) * p.Hv + u.hv) * kD + half * kHalfRows + piece * 8;
-                    for (int row = ot >> 3; row < len; row += 16)
-                        *reinterpret_cast<uint4*>(og + row * tok_stride) =
-                            *reinterpret_cast<const uint4*>(smem + kHS_Out + sw128_offset(row, piece));
-                }
+                rows = {true, u.seq_t0 + j * kChunk, min(kChunk, u.seq_len - j * kChunk), u.hv, half, kHS_Out + 8192 * buf};
             }
             gc += u.nc;
         }
+        rows_out();
         if (ot == 0) bulk_wait_all();        // before the CTA's shared memory goes away
     }
 
