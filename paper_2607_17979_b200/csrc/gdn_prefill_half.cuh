@@ -288,7 +288,11 @@ __device__ __forceinline__ void state_half_role(const TensorMaps& maps, const Pr
                     const uint32_t g = gc + j, tS = tmem + half_s_col(g);
                     const uint64_t q = sdesc_advance(dQ0, ring.st * kHABytes), pp = sdesc_advance(dP0, ring.st * kHCBytes),
                                    kk = sdesc_advance(dK0, ring.st * kHCBytes);
+                    // The output warps are through with the last chunk: they have read the tile of S Q^T, and seen this chunk's
+                    // state handed over, which the next one's must not overtake (a parity cannot tell a phase from the
+                    // one after the next).
                     if (!warp_wait(&bar_full_c[ring.st], ring.par, abortp, kWaitReason) ||
+                        (g > 0 && !warp_wait(&bar_y_read, (g - 1) & 1u, abortp, kWaitReason)) ||
                         !warp_wait(&bar_u, g & 1u, abortp, kWaitReason)) {        // U operands in TMEM
                         live = false;
                         break;
@@ -305,14 +309,7 @@ __device__ __forceinline__ void state_half_role(const TensorMaps& maps, const Pr
                                 mma_ts_c<true>(tD4 + 64 * h, tUs + 8 * ks, sdesc_advance(kk, 8192 * h + 2048 * ks), id_k);
                             mma_commit(&bar_d4[h]);
                         }
-                    }
-                    // S Q^T (its tile has landed with W's), into the tile that the output warps read a chunk ago
-                    if (g > 0 && !warp_wait(&bar_y_read, (g - 1) & 1u, abortp, kWaitReason)) {
-                        live = false;
-                        break;
-                    }
-                    tc_fence_after_sync();
-                    if (elect_one()) {
+                        // S Q^T (its tile has landed with W's)
                         mma_ts_c<false>(tY1, tS, q, id_qp);
 #pragma unroll
                         for (int ks = 1; ks < 8; ++ks)
