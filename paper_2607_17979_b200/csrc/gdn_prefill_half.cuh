@@ -66,7 +66,7 @@ __device__ __forceinline__ void state_half_role(const TensorMaps& maps, const Pr
                                                 const WorkspaceLayout& lay, uint8_t* smem, const uint32_t tmem,
                                                 const int cta, const int n_ctas) {
     __shared__ uint64_t bar_full_a[kHStages], bar_full_b[2], bar_full_c[kHStages], bar_free_a[kHStages], bar_free_b[2],
-        bar_free_c[kHStages], bar_y[2], bar_p[2], bar_y_read, bar_d1, bar_d4[2], bar_s[2], bar_u,
+        bar_free_c[kHStages], bar_y[2], bar_p[2], bar_y_read, bar_d1, bar_d4[2], bar_s[2][2], bar_u,
         bar_drain[2];
     __shared__ int abort_flag;
     __shared__ uint32_t armed[3];         // chunks of the CTA's stream whose copies the loader has started, per ring
@@ -90,7 +90,8 @@ __device__ __forceinline__ void state_half_role(const TensorMaps& maps, const Pr
             mbar_init(&bar_p[st], kSOutThreads / 32); // U~ in the accumulator
             mbar_init(&bar_drain[st], 1);             // an issuer that gave up: its products
             mbar_init(&bar_d4[st], 1);                // by halves of dk
-            mbar_init(&bar_s[st], kSEpiWarps / 2);    // the bf16 state in TMEM, by halves of dk
+            for (int h = 0; h < 2; ++h)               // the bf16 state in TMEM, by odd and even chunks and halves of dk
+                mbar_init(&bar_s[st][h], kSEpiWarps / 2);
         }
         for (int st = 0; st < kHStages; ++st) {
             mbar_init(&bar_full_a[st], 1);
@@ -255,7 +256,7 @@ __device__ __forceinline__ void state_half_role(const TensorMaps& maps, const Pr
                     const uint32_t tD1 = tmem + kH_D1, tS = tmem + half_s_col(g);
                     if (!warp_wait(&bar_full_a[ring.st], ring.par, abortp, kWaitReason) ||
                         !warp_wait(&bar_p[g & 1], (g >> 1) & 1u, abortp, kWaitReason) ||      // U~ in place
-                        !warp_wait(&bar_s[0], g & 1u, abortp, kWaitReason)) {                 // bf16 S in TMEM, dk 0-63
+                        !warp_wait(&bar_s[g & 1][0], (g >> 1) & 1u, abortp, kWaitReason)) {                 // bf16 S in TMEM, dk 0-63
                         live = false;
                         break;
                     }
@@ -266,7 +267,7 @@ __device__ __forceinline__ void state_half_role(const TensorMaps& maps, const Pr
                         for (int ks = 0; ks < 4; ++ks)
                             mma_ts_c<true>(tD1, tS + 8 * ks, sdesc_advance(w, 2048 * ks), id_w);
                     }
-                    if (!warp_wait(&bar_s[1], g & 1u, abortp, kWaitReason)) {                 // dk 64-127
+                    if (!warp_wait(&bar_s[g & 1][1], (g >> 1) & 1u, abortp, kWaitReason)) {                 // dk 64-127
                         live = false;
                         break;
                     }
@@ -288,11 +289,7 @@ __device__ __forceinline__ void state_half_role(const TensorMaps& maps, const Pr
                     const uint32_t g = gc + j, tS = tmem + half_s_col(g);
                     const uint64_t q = sdesc_advance(dQ0, ring.st * kHABytes), pp = sdesc_advance(dP0, ring.st * kHCBytes),
                                    kk = sdesc_advance(dK0, ring.st * kHCBytes);
-                    // The output warps are through with the last chunk: they have read the tile of S Q^T, and seen this chunk's
-                    // state handed over, which the next one's must not overtake (a parity cannot tell a phase from the
-                    // one after the next).
                     if (!warp_wait(&bar_full_c[ring.st], ring.par, abortp, kWaitReason) ||
-                        (g > 0 && !warp_wait(&bar_y_read, (g - 1) & 1u, abortp, kWaitReason)) ||
                         !warp_wait(&bar_u, g & 1u, abortp, kWaitReason)) {        // U operands in TMEM
                         live = false;
                         break;
@@ -309,7 +306,14 @@ __device__ __forceinline__ void state_half_role(const TensorMaps& maps, const Pr
                                 mma_ts_c<true>(tD4 + 64 * h, tUs + 8 * ks, sdesc_advance(kk, 8192 * h + 2048 * ks), id_k);
                             mma_commit(&bar_d4[h]);
                         }
-                        // S Q^T (its tile has landed with W's)
+                    }
+                    // S Q^T (its tile has landed with W's), into the tile that the output warps read a chunk ago
+                    if (g > 0 && !warp_wait(&bar_y_read, (g - 1) & 1u, abortp, kWaitReason)) {
+                        live = false;
+                        break;
+                    }
+                    tc_fence_after_sync();
+                    if (elect_one()) {
                         mma_ts_c<false>(tY1, tS, q, id_qp);
 #pragma unroll
                         for (int ks = 1; ks < 8; ++ks)
@@ -409,7 +413,7 @@ __device__ __forceinline__ void state_half_role(const TensorMaps& maps, const Pr
                 for (int k = 0; k < 32; ++k) S[k] = 0.f;
             }
             store_state_bf16(gc);
-            hand_over(&bar_s[ch]);
+            hand_over(&bar_s[gc & 1][ch]);
             // the next initial state, towards L2
             if (p.init_state && tid == 0 && nxt.x > 0 && hu_next < total)
                 bulk_prefetch_l2(p.init_state + static_cast<size_t>(nxt.y) * (kHalfRows * kD), kHalfRows * kD * 4);
@@ -468,7 +472,7 @@ __device__ __forceinline__ void state_half_role(const TensorMaps& maps, const Pr
                 }
                 if (j + 1 < nc) {
                     store_state_bf16(g + 1);     // the next chunk's A operand
-                    hand_over(&bar_s[ch]);
+                    hand_over(&bar_s[(g + 1) & 1][ch]);
                 }
             }
             // nothing of a unit is written after a failed wait (every record of the unit has been loaded by now: no
@@ -589,8 +593,10 @@ __device__ __forceinline__ void state_half_role(const TensorMaps& maps, const Pr
                 await(&bar_y[buf], (g >> 1) & 1u);
                 // The rows are made once the chain warps have handed the next state over and wait behind the next
                 // product: beside the refresh they take its issue slots (4096 tokens at 8 v-heads 91.5 us, 88.3 this
-                // way).
-                if (j + 1 < u.nc) await(&bar_s[1], (g + 1) & 1u);
+                // way).  The chain warps may by now have handed over the state after that one, but no more: it goes on from
+                // the U~ that these warps put in place after these rows.  So the hand-overs have two barriers, in turn (a
+                // parity cannot tell a phase from the one after the next).
+                if (j + 1 < u.nc) await(&bar_s[(g + 1) & 1][1], ((g + 1) >> 1) & 1u);
                 tc_fence_after_sync();
                 {
                     // Fragments (rows = dv, columns = tokens), rounded in pairs and stored transposed into a

@@ -1,6 +1,5 @@
-"""In the half-unit state pass the state product of a chunk waits for the output warps to be through with the chunk before: they
-have then seen that chunk's successor's state handed over, which the one after must not overtake (a wait by parity cannot tell a
-phase from the one after the next)."""
+"""In the half-unit state pass the hand-over of a state may be overtaken by the next one while output warps still wait for it, by
+one and no more: a wait by parity cannot tell a phase from the one after the next, so the hand-overs have two barriers in turn."""
 import os
 import re
 
@@ -15,16 +14,17 @@ from test_gpu_prefill import oracle_prefill
 CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2607_17979_b200", "csrc")
 
 
-def test_state_product_waits_for_the_rows_before():
+def test_hand_overs_of_the_state_alternate_between_two_barriers():
     s = open(os.path.join(CSRC, "gdn_prefill_half.cuh")).read()
-    issuers = s[s.index("===================== issuers"):s.index("===================== chain warps")]
-    rows = issuers.index("warp_wait(&bar_y_read, (g - 1) & 1u")
-    u = issuers.index("warp_wait(&bar_u, g & 1u")
-    product = issuers.index("mma_ts_c<false>(tD4")
-    assert rows < u < product and issuers.count("&bar_y_read") == 1
+    for wait in ("warp_wait(&bar_s[g & 1][0], (g >> 1) & 1u", "warp_wait(&bar_s[g & 1][1], (g >> 1) & 1u",
+                 "await(&bar_s[(g + 1) & 1][1], ((g + 1) >> 1) & 1u)"):
+        assert s.count(wait) == 1
+    assert len(re.findall(r"(?:wait|await)\(&bar_s\[", s)) == 3
+    arrivals = re.findall(r"hand_over\(&bar_s(\S+)\);", s)
+    assert arrivals == ["[gc & 1][ch]", "[(g + 1) & 1][ch]"]
+    # what bounds the lead: the next U~ is put in place by the warps that wait, behind their rows
     out = s[s.index("===================== output warps"):]
-    assert out.index("await(&bar_s[1], (g + 1) & 1u)") < out.index("mbar_arrive(&bar_y_read)")
-    assert not re.search(r"bar_s\[0\]", out)
+    assert out.index("preload(g + k)") < out.index("await(&bar_s[")
 
 
 @pytest.mark.gpu
