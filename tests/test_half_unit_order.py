@@ -20,7 +20,7 @@ def test_hand_overs_of_the_state_alternate_between_two_barriers():
                  "await(&bar_s[(g + 1) & 1][1], ((g + 1) >> 1) & 1u)"):
         assert s.count(wait) == 1
     assert len(re.findall(r"(?:wait|await)\(&bar_s\[", s)) == 3
-    arrivals = re.findall(r"hand_over\(&bar_s(\S+)\);", s)
+    arrivals = re.findall(r"hand_over\(&bar_s(.+)\);", s)
     assert arrivals == ["[gc & 1][ch]", "[(g + 1) & 1][ch]"]
     # what bounds the lead: the next U~ is put in place by the warps that wait, behind their rows
     out = s[s.index("===================== output warps"):]
