@@ -11,7 +11,7 @@
 //   S' = e^{b_C} S0 + U^T diag(e^{b_C-b}) K
 //
 // Three launches: a prep kernel builds the chunk table from cu_seqlens; the
-// intra-chunk kernel (one CTA per chunk and v-head, all chunks in parallel)
+// intra-chunk kernel (all chunks and v-heads in parallel, a pipeline per SM)
 // computes W, U~, P and b with tcgen05 GEMMs and an fp32 triangular solve and
 // writes them as a record; the state pass (one persistent CTA per SM that takes
 // sequence after sequence of a v-head from a list) walks the chunks in order
