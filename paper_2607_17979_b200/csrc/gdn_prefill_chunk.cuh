@@ -52,6 +52,12 @@ constexpr uint32_t kRecBytes = 74496;
 constexpr uint32_t kRecUHalf = (kRecDecay - kRecU) / 2;
 constexpr uint32_t kRecUBlock = kRecUHalf / 4, kRecPBlock = (kRecU - kRecP) / 4;      // bytes of a 16-token block
 __device__ __forceinline__ int token_blocks(int seq_len, int chunk) { return (min(kChunk, seq_len - chunk * kChunk) + 15) >> 4; }
+// The same by the record's own word.  Where a producer has left after a wait that ran out, that is whatever the workspace
+// held, and what is addressed by it has four blocks.
+__device__ __forceinline__ int record_blocks(const void* word) {
+    const uint32_t n = *reinterpret_cast<const uint32_t*>(word);
+    return static_cast<int>(n < 4u ? n : 4u);
+}
 // Place (in 16-byte units) of a token group and dv within one half of U~.  Odd groups have their dv swapped in fours,
 // so that a fragment read (four dv of two neighbouring groups per half warp) touches every bank once.
 __device__ __forceinline__ int rec_u_index(int group, int dv) { return group * 64 + (dv ^ ((group & 1) << 2)); }

@@ -522,7 +522,7 @@ __device__ __forceinline__ void state_half_role(const TensorMaps& maps, const Pr
                         x[c][4 * b + 2 * r + 1] = __float_as_uint(v.y);
                     }
             const float2 eb = *reinterpret_cast<const float2*>(base + kHB_Vec + (kRecEb - kRecDecay) + 8 * lane);
-            const int nb = *reinterpret_cast<const int*>(base + kHB_Vec + (kRecGammaC + 4 - kRecDecay));
+            const int nb = record_blocks(base + kHB_Vec + (kRecGammaC + 4 - kRecDecay));
 #pragma unroll
             for (int c = 0; c < 2; ++c) tmem_st_16x256b_x4(tmem + kH_D1 + lane_base + 32 * c, x[c]);
             // blocks without tokens were not copied: whatever was there is replaced

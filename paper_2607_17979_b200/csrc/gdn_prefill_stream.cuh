@@ -643,7 +643,7 @@ __device__ __forceinline__ void state_stream_role(const TensorMaps& maps, const 
                     smem + sq * kStageBytes + kS_Rec + kRecEb + 8 * lane);
             const float4* sU = reinterpret_cast<const float4*>(smem + sq * kStageBytes + kS_Rec + kRecU +
                                                                    (odv >> 6) * kRecUHalf);
-            const int nb = *reinterpret_cast<const int*>(smem + sq * kStageBytes + kS_Rec + kRecGammaC + 4);
+            const int nb = record_blocks(smem + sq * kStageBytes + kS_Rec + kRecGammaC + 4);
 #pragma unroll
             for (int c0 = 0; c0 < 64; c0 += 32) {       // eight reads in flight
                 uint32_t r[2][16];
