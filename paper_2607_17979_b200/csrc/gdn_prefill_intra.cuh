@@ -527,13 +527,16 @@ __device__ __forceinline__ void produce_role(const TensorMaps& maps, const Prefi
         for (uint32_t k = 0; item_at(kBItem, k); ++k) {
             const Place<kProdInfos> f(k);
             const ItemInfo& info = infos[f.at];
+            // (read before the wait: should it run out, the item's place may be another's by then)
             const int t0 = info.t0, x = info.hv * kD;
+            const uint32_t p_bytes = ((info.len + 15) >> 4) * kRecPBlock;
+            uint8_t* const rec_p = ws + lay.records + static_cast<size_t>(info.rec) * kRecBytes + kRecP;
             const Place<kProdSlots> s(k);
             wait(kBP, s.at, s.par);
             if (lane == 0) {
                 uint8_t* slot = smem + kPS_Slot + s.at * kPSlotBytes;
                 uint64_t* bar = &bars[kBV + s.at];
-                bulk_store(ws + lay.records + static_cast<size_t>(info.rec) * kRecBytes + kRecP, slot, ((info.len + 15) >> 4) * kRecPBlock);
+                bulk_store(rec_p, slot, p_bytes);
                 bulk_commit();
                 bulk_wait_read_all();
                 armed[1] = k + 1;
