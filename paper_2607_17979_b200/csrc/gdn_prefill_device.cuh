@@ -106,7 +106,6 @@ struct IntraStatics {
     alignas(16) float s_b2[kChunk];    // b_r log2(e): inclusive log-decay prefix
     alignas(16) float s_beta[kChunk];  // beta_r (0 past the chunk's length)
     alignas(16) float s_bg[kChunk];    // beta_r e^{b_r}
-    alignas(16) float s_fall[32];      // e^{b_31 - b_i}, i < 32
 };
 
 // T = (I + A)^{-1} for the strictly lower-triangular 64x64 A in sA (fp32, row-major, stride kLdA),
@@ -321,11 +320,6 @@ __device__ __forceinline__ bool intra_item(const TensorMaps& maps, const Prefill
         st.s_beta[2 * lane] = be0; st.s_beta[2 * lane + 1] = be1;
         const float e0 = ex2_approx(b0 * kLog2e), e1 = ex2_approx(b1 * kLog2e);
         st.s_bg[2 * lane] = be0 * e0; st.s_bg[2 * lane + 1] = be1 * e1;
-        const float b31 = __shfl_sync(0xffffffffu, incl, 15);
-        if (lane < 16) {
-            st.s_fall[2 * lane] = ex2_approx((b31 - b0) * kLog2e);
-            st.s_fall[2 * lane + 1] = ex2_approx((b31 - b1) * kLog2e);
-        }
         // the record's vectors: e^{b_C - b_c}, scale e^{b_r}, and e^{b_C}
         *reinterpret_cast<float2*>(rec + kRecDecay + 8 * lane) =
             make_float2(ex2_approx((bC - b0) * kLog2e), ex2_approx((bC - b1) * kLog2e));
@@ -395,9 +389,6 @@ __device__ __forceinline__ bool intra_item(const TensorMaps& maps, const Prefill
         const float br2 = st.s_b2[r];
         const float rowscale = is_p ? p.scale : st.s_beta[r];      // the output scale rides on P
         const int limit = is_p ? r : r - 1;              // keep columns i <= limit
-        // columns 0-31 of rows 32-63: times e^{b_r - b_31} e^{b_31 - b_i}
-        const bool below = (row & 32) != 0 && colhalf == 0;
-        const float rowfall = below ? rowscale * ex2_approx(br2 - st.s_b2[31]) : 0.f;
         // (rows of a half without tokens are not read)
         if ((row & 32) < ci.len)
 #pragma unroll
@@ -416,12 +407,11 @@ __device__ __forceinline__ bool intra_item(const TensorMaps& maps, const Prefill
                 tmem_wait_ld();
 #pragma unroll
                 for (int q4 = 0; q4 < 4; ++q4) {
-                    const float4 bb = *reinterpret_cast<const float4*>((below ? st.s_fall : st.s_b2) + cbase + 4 * q4);
+                    const float4 bb = *reinterpret_cast<const float4*>(st.s_b2 + cbase + 4 * q4);
                     const float bv[4] = {bb.x, bb.y, bb.z, bb.w};
 #pragma unroll
                     for (int e = 0; e < 4; ++e)          // times e^{b_r - b_i} (above the diagonal: discarded)
-                        val[4 * q4 + e] = below ? rowfall * __uint_as_float(x[4 * q4 + e]) * bv[e]
-                                                : rowscale * __uint_as_float(x[4 * q4 + e]) * ex2_approx(br2 - bv[e]);
+                        val[4 * q4 + e] = rowscale * __uint_as_float(x[4 * q4 + e]) * ex2_approx(br2 - bv[e]);
                 }
                 if (cbase + 15 >= (row & 32)) {
 #pragma unroll

@@ -51,7 +51,6 @@ struct ItemInfo {
     alignas(16) float nb2[kChunk];       // -b_r log2(e), b the inclusive log-decay prefix
     float beta[kChunk];                  // beta_r (0 past the chunk's length)
     float bg[kChunk];                    // beta_r e^{b_r}
-    float fall[32];                      // e^{b_31 - b_i}, i < 32
     int32_t t0, len, hv, hqk;
     int32_t rec;                         // record number, chunk * Hv + hv; < 0: no more items
     int32_t pad[3];
@@ -440,13 +439,10 @@ __device__ __forceinline__ void produce_role(const TensorMaps& maps, const Prefi
                     }
                     const float kLog2e = 1.4426950408889634f;
                     const float b1 = incl, b0 = incl - g.y;
-                    const float bC = __shfl_sync(0xffffffffu, incl, 31), b31 = __shfl_sync(0xffffffffu, incl, 15);
+                    const float bC = __shfl_sync(0xffffffffu, incl, 31);
                     const float e0 = ex2_approx(b0 * kLog2e), e1 = ex2_approx(b1 * kLog2e);
                     *reinterpret_cast<float2*>(&info.nb2[2 * lane]) = make_float2(-b0 * kLog2e, -b1 * kLog2e);
                     *reinterpret_cast<float2*>(&info.bg[2 * lane]) = make_float2(beta.x * e0, beta.y * e1);
-                    if (lane < 16)
-                        *reinterpret_cast<float2*>(&info.fall[2 * lane]) =
-                            make_float2(ex2_approx((b31 - b0) * kLog2e), ex2_approx((b31 - b1) * kLog2e));
                     arrive(kBGates, f.at);
                     // the record's vectors: e^{b_C - b_c}, scale e^{b_r}, and e^{b_C}
                     uint8_t* rec = ws + lay.records + static_cast<size_t>(rec_done) * kRecBytes;
@@ -653,8 +649,9 @@ __device__ __forceinline__ void produce_role(const TensorMaps& maps, const Prefi
         }
     } else if (warp < kPWriteWarp0 || warp == kPMaskWarpP || warp == kPMaskWarpA) {
         // ===================== masks.  Accumulator row of this thread: TMEM lane 32 (warp % 4) + lane; lanes 0-63 hold q.k
-        // rows (-> P), lanes 64-127 k.k rows (-> A).  Warps 0-3 take the 32 columns that hold their rows' diagonal, times
-        // e^{b_r - b_i}, the two others the columns 0-31 of rows 32-63, times e^{b_r - b_31} e^{b_31 - b_i}.
+        // rows (-> P), lanes 64-127 k.k rows (-> A), either times e^{b_r - b_i}, which is one exponential everywhere (split
+        // at b_31 the decay has a larger error, and outputs differ in their last bit).  Warps 0-3 take the 32 columns that
+        // hold their rows' diagonal, the two others the columns 0-31 of rows 32-63.
         const bool below = warp >= kPWriteWarp0;
         const int half = warp & 1, r = 32 * half + lane, c0 = below ? 0 : 32 * half;
         const int last = lane - ((warp >> 1) & 1);               // keep columns i <= r of P, i < r of A
@@ -668,8 +665,7 @@ __device__ __forceinline__ void produce_role(const TensorMaps& maps, const Prefi
             const int len = info.len;
             const Place<kPAs> a(k);
             const float nbr2 = info.nb2[r];
-            float rowscale = is_p ? p.scale : info.beta[r];      // the output scale rides on P
-            if (below) rowscale *= ex2_approx(info.nb2[31] - nbr2);
+            const float rowscale = is_p ? p.scale : info.beta[r];        // the output scale rides on P
             if (!is_p) wait(kBAFree, a.at, a.par ^ 1u);
             wait(kBGram, b.at, b.par);
             tc_fence_after_sync();
@@ -686,14 +682,11 @@ __device__ __forceinline__ void produce_role(const TensorMaps& maps, const Prefi
                     float2 val[8];
 #pragma unroll
                     for (int q4 = 0; q4 < 4; ++q4) {
-                        const float4 f4 = *reinterpret_cast<const float4*>((below ? info.fall : info.nb2) + c + 4 * q4);
+                        const float4 f4 = *reinterpret_cast<const float4*>(info.nb2 + c + 4 * q4);
 #pragma unroll
                         for (int e = 0; e < 2; ++e) {
-                            float2 z = e ? make_float2(f4.z, f4.w) : make_float2(f4.x, f4.y);
-                            if (!below) {
-                                z = add2(make_float2(-nbr2, -nbr2), z);
-                                z = make_float2(ex2_approx(z.x), ex2_approx(z.y));
-                            }
+                            float2 z = add2(make_float2(-nbr2, -nbr2), e ? make_float2(f4.z, f4.w) : make_float2(f4.x, f4.y));
+                            z = make_float2(ex2_approx(z.x), ex2_approx(z.y));
                             const int i = 4 * q4 + 2 * e;
                             val[2 * q4 + e] = mul2(mul2(make_float2(rowscale, rowscale), make_float2(__uint_as_float(x[i]), __uint_as_float(x[i + 1]))), z);
                         }
