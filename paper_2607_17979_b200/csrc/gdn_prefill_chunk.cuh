@@ -124,7 +124,9 @@ __device__ __forceinline__ bool block_bounds_ok(bool here, int32_t t0, int32_t t
 //   order[max_chunks]            int32: chunk ids in processing order: by position inside the
 //                                sequence first, by sequence rank second (so that the records
 //                                every state-pass unit needs next are produced first)
-//   hist, fill, cnt, pos[max_nc+2]  int32 scratch of the counting sort (max_nc = T/64 + 1)
+//   hist, fill, cnt, pos[max_nc+2]  int32 scratch of the counting sort (max_nc = T/64 + 1); in the two-part route hist
+//                                then holds how far in the processing order the second part's producers may go when
+//                                the first chain is at a chunk
 //   flags[max_chunks][Hv]        uint32: 1 once the record is complete and visible
 //   done[N][Hv][2]               uint16: 1 once the two-part route's state pass has finished the half unit
 //                                (rank-major, like the unit list); the rest is left to a last launch

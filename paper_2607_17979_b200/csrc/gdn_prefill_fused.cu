@@ -24,6 +24,42 @@ constexpr int kFPrepThreads = 256;
 constexpr int kSplitProdPermille = 385;
 constexpr int kSplitLeadSteps = 8;
 constexpr int kSplitMarginItems = 64;
+// How many items in processing order the producers of the second part may be ahead of the first chain.  500 records are
+// 29 MB, half of what one die's L2 holds; 32 chains of 512 chunks: 617 us, no bound 727 (the records have left L2 when
+// they are read), 300 more (84 CTAs work on four items each).
+constexpr int kPaceItems = 500;
+// And the items that one of them makes in a chain's chunk step (2.3 and 1.07 us): where all of them together make fewer
+// than the chains read, they have to be further ahead to be done in time.  (The cut reckons with less: it must hold.)
+constexpr float kPaceRate = 0.45f;
+
+// The model of the two-part production, in items of the processing order.  In step j the chains need the Hv pos[j + 1]
+// first ones; a unit holds two SMs, and what the second part has begun kSplitLeadSteps before is ready.
+struct SplitModel {
+    const int32_t* pos;
+    int32_t Hv, sms;
+    // SMs without a half unit, summed over the steps before m
+    __device__ __forceinline__ long long work(int m) const {
+        const long long w = static_cast<long long>(m) * sms - 2ll * Hv * pos[m];
+        return w < 0 ? 0 : w;
+    }
+    __device__ __forceinline__ long long ready_work(int j) const { return work(j > kSplitLeadSteps ? j - kSplitLeadSteps : 0); }
+    __device__ __forceinline__ long long needed(int j) const { return static_cast<long long>(Hv) * pos[j + 1]; }
+    // what step j lacks without a first part: by the cut's cautious rate, and by the producers' own
+    __device__ __forceinline__ long long cut_for(int j) const { return needed(j) - ready_work(j) * kSplitProdPermille / 1000; }
+    __device__ __forceinline__ long long short_of(int j) const {
+        return needed(j) - static_cast<long long>(kPaceRate * ready_work(j));
+    }
+    // How far the producers may go with the first chain at chunk j: the window, and up to the step that lacks most at
+    // least as far as that they are done in time.  (Held to the window there, 64 chains of 128 chunks take 358 us instead
+    // of 290, 48 of 100 220 instead of 203, for the first part alone reaches far beyond it: the producers stood idle first
+    // and were late then.  Not held at all beyond a large first part: 30000 and 1000 tokens at 32 heads 652 instead of 580.)
+    __device__ __forceinline__ int32_t bound(int j, long long short_max, int short_step) const {
+        const long long window = static_cast<long long>(Hv) * pos[j] + kPaceItems;
+        const long long in_time = j <= short_step ? short_max + static_cast<long long>(kPaceRate * work(j)) : 0;
+        const long long b = window > in_time ? window : in_time;
+        return static_cast<int32_t>(b < 0x7fffffff ? b : 0x7fffffff);
+    }
+};
 
 __global__ void __launch_bounds__(kFPrepThreads)
 prefill_fused_prep_kernel(const int32_t* __restrict__ cu, int32_t T, int32_t N, int32_t Hv,
@@ -160,31 +196,30 @@ prefill_fused_prep_kernel(const int32_t* __restrict__ cu, int32_t T, int32_t N, 
     }
     // Two-part production (mode 2).  The items of the processing order before the cut are
     // produced before the state pass starts, the others beside it, on the SMs it leaves free.
-    // The cut is the smallest head start with which the chains never catch up with the
-    // producers, by a simple model: every live (sequence, v-head) unit consumes one item per
-    // chunk step and holds two SMs, the others produce kProdPermille / 1000 items per chunk step
-    // each, and an item started when the state pass starts is ready kLeadSteps chunk steps
-    // later.  In step j the chains need the Hv * pos[j + 1] first items of the order; by then the
-    // second part has produced r * sum_{i < j - lead} (sms - 2 Hv * cnt[i]), and that sum is
-    // m * sms - 2 Hv * pos[m] with m = j - lead.
+    // The cut is the smallest head start with which the chains never catch up with the producers by SplitModel.
     if (for_fused == 2) {
-        __shared__ int32_t need_max;
-        if (tid == 0) need_max = 0;
+        __shared__ int32_t need_max, short_max, short_step;
+        if (tid == 0) need_max = short_max = short_step = 0;
         __syncthreads();
         const long long total_items = hdr[kHdrTotalItems];
+        const SplitModel model = {pos, Hv, sms};
         long long local = 0;
-        const int lead = kSplitLeadSteps, prod = kSplitProdPermille;
+        int32_t short_local = 0, short_at = 0;
         for (int j = tid; j < lay.max_nc; j += kFPrepThreads) {
-            const int m = j > lead ? j - lead : 0;
-            long long produced =
-                (static_cast<long long>(m) * sms - 2ll * Hv * pos[m]) * prod / 1000;
-            if (produced < 0) produced = 0;
-            const long long need = static_cast<long long>(Hv) * pos[j + 1] - produced;
+            const long long need = model.cut_for(j), lacks = model.short_of(j);
             local = need > local ? need : local;
+            if (lacks > short_local) {
+                short_local = static_cast<int32_t>(lacks);
+                short_at = j;
+            }
         }
         if (local > total_items) local = total_items;
         atomicMax(&need_max, static_cast<int32_t>(local));
+        atomicMax(&short_max, short_local);
         __syncthreads();
+        if (short_local == short_max) atomicMax(&short_step, short_at);
+        __syncthreads();
+        for (int j = tid; j < lay.max_nc; j += kFPrepThreads) hist[j] = model.bound(j, short_max, short_step);
         if (tid == 0) {
             long long cut = split_permille >= 0 ? total_items * split_permille / 1000
                                                 : static_cast<long long>(need_max) + kSplitMarginItems;

@@ -63,10 +63,9 @@ constexpr uint32_t kProdTmemCols = 512;
 // TMEM columns, two tiles of 64 each
 constexpr uint32_t kPT_Gram = 0, kPT_U = 128, kPT_W = 256;
 
-// How many items in processing order the producers of the second part may be ahead of the first chain, and how often one
-// asks before it goes on regardless.  500 records are 29 MB, half of what one die's L2 holds; 32 chains of 512 chunks: 617
-// us, no bound 727 (the records have left L2 when they are read), 300 more (84 CTAs work on four items each).
-constexpr int kPaceItems = 500, kPacePolls = 1 << 11;
+// How often a producer of the second part that is as far ahead of the first chain as the tables allow asks again before
+// it goes on regardless.
+constexpr int kPacePolls = 1 << 11;
 
 // Where a CTA's items come from.
 enum ItemSource {
@@ -377,16 +376,15 @@ __device__ __forceinline__ void produce_role(const TensorMaps& maps, const Prefi
             }
         };
         pull();
-        // (kItemsQueue) No further ahead of the chains than that what they read next is still in L2, as far as the first
-        // of them tells; where none seems to come on, no bound.
+        // (kItemsQueue) No further ahead of the chains than that what they read next is still in L2, or than it takes to be
+        // done in time, as far as the first of them tells; where none seems to come on, no bound.
         int allowed = 0;
         auto pace = [&](const int item) {
             if constexpr (kSource == kItemsQueue) {
 #pragma unroll 1
                 for (int n = 0; item >= allowed; ++n) {
                     const int at = *reinterpret_cast<volatile int32_t*>(hdr + kHdrProgress);
-                    allowed = n == kPacePolls || at >= lay.max_nc ? 0x7fffffff
-                                                                  : reinterpret_cast<const int32_t*>(ws + lay.pos)[at] * p.Hv + kPaceItems;
+                    allowed = n == kPacePolls || at >= lay.max_nc ? 0x7fffffff : reinterpret_cast<const int32_t*>(ws + lay.hist)[at];
                     allowed = __shfl_sync(0xffffffffu, allowed, 0);
                 }
             }
