@@ -161,8 +161,12 @@ cudaError_t launch_prefill_intra(const TensorMaps& maps, const ChunkedParams& cp
     const int64_t items = static_cast<int64_t>(cp.lay.max_chunks) * cp.p.Hv;
     // Few items run all at once in either form, and there the shorter way through one item counts: a pipeline's warps
     // fetch eight pieces of code from L2 before the first item is through (us a call, CTA per item / pipeline: 64 items
-    // 13.3 / 15.3, 512 37.1 / 38.5, 672 46.2 / 46.5, 1024 64.6 / 63.8, 1280 in 40 sequences 75.2 / 69.3).
-    if (items <= 5ll * di.sms) {
+    // 13.3 / 15.3, 512 37.1 / 38.5, 672 46.2 / 46.5, 1024 64.6 / 63.8, 1280 in 40 sequences 75.2 / 69.3).  `items` counts a
+    // ragged chunk for each sequence, up to twice what there are.  So a batch whose sequences, were they of equal length,
+    // had at most four items an SM, all of which run at once, has few too (32 heads, 13 x 64 tokens 26.9 / 28.4, 16 x 48
+    // 30.9 / 32.6, 8 x 128 28.2 / 29.5, 18 x 64 33.6 / 34.2; beyond it 20 x 64 40.3 / 39.7, 8 x 130 36.2 / 35.8).
+    const int64_t n = cp.p.N, equal = n * ((cp.p.T + n * kChunk - 1) / (n * kChunk)) * cp.p.Hv;
+    if (items <= 5ll * di.sms || equal <= 4ll * di.sms) {
         const bool row = items > 2ll * di.sms;
         auto kernel = row ? inline_tables ? prefill_intra_few_kernel<true, true> : prefill_intra_few_kernel<false, true>
                           : inline_tables ? prefill_intra_few_kernel<true, false> : prefill_intra_few_kernel<false, false>;

@@ -1,5 +1,6 @@
 """The form in which the intra-chunk kernel is launched, read from a captured call: a grid of chunks x heads up to two items an SM, a
-row of items (the CTAs without a chunk behind all others) from there to where the pipeline's one CTA per SM begins."""
+row of items (the CTAs without a chunk behind all others) from there to where the pipeline's one CTA per SM begins: five items an SM
+by the host's bound, which counts a ragged chunk for each sequence, or four where the sequences would have fewer at equal lengths."""
 import ctypes
 
 import pytest
@@ -35,7 +36,8 @@ def grids(graph):
     ([64 * 9], 8, "grid"),
     ([64] * 32, 8, "row"),               # 32 chunks of the 64 that T and N allow
     ([64 * 9], 32, "row"), ([64 * 20], 32, "row"),
-    ([64 * 60], 32, "pipeline"),
+    ([64] * 13, 32, "row"), ([48] * 16, 32, "row"), ([128] * 8, 32, "row"),      # more than five an SM by the bound, fewer than four in fact
+    ([130] * 8, 32, "pipeline"), ([65] * 17, 32, "pipeline"), ([64 * 60], 32, "pipeline"),
 ])
 def test_form(lens, hv, form):
     from paper_2607_17979_b200 import api
