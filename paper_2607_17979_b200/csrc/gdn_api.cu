@@ -266,10 +266,11 @@ namespace {
 // about 13 us (the tables with the processing order, two more launches) and hide the intra-chunk kernel's time, which
 // grows with the items, as far as the SMs that hold no half unit keep up.  So what decides is the number of (chunk,
 // v-head) items against the units; where the lengths differ, half of the units that have ended on average count as
-// gone (`live`; all units count without a bound on the longest).  The line was fitted to 1351 drawn batches timed in
-// both forms: on average 0.12 % above the faster of the two (three launches always: 5.3 %).  Us in three
-// launches / in two parts on 148 SMs: 32 units of 38 chunks 76.3 / 76.8, of 50 96.0 / 91.2; 64 of 40 115.0 / 123.1, of
-// 86 and 28 180.8 / 174.7.
+// gone (`live`; all units count without a bound on the longest).  The line was fitted to drawn batches timed in both forms
+// while the intra-chunk kernel ran a CTA per item; as a pipeline that kernel costs the three launches less, and they are
+// the faster a little beyond the line too.  Us in three launches / in two parts on 148 SMs: 32 units of 38 chunks 71.3 /
+// 76.0, of 50 89.0 / 89.3, of 128 205 / 171, of 512 774 / 586; 8 units of 60 chunks 86.2 / 94.5, of 240 294.5 / 285.5; but
+// 64 of 40 97.4 / 114.3, of 128 272 / 291.5, 48 of 100 188.6 / 192.6, 40 of 70 126.2 / 131.0, 86 and 28 at 32 heads 160.6 / 163.6.
 bool two_parts_pay(int32_t T, int32_t N, int32_t max_seqlen_hint, int32_t Hv, int32_t sms) {
     const long long units = static_cast<long long>(N) * Hv;
     if (2 * units > sms - gdn::kOverlapSpareSms) return false;     // (gdn_prefill_overlap runs three launches there)

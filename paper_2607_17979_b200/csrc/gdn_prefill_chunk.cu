@@ -161,11 +161,12 @@ cudaError_t launch_prefill_intra(const TensorMaps& maps, const ChunkedParams& cp
     const int64_t items = static_cast<int64_t>(cp.lay.max_chunks) * cp.p.Hv;
     // Few items run all at once in either form, and there the shorter way through one item counts: a pipeline's warps
     // fetch eight pieces of code from L2 before the first item is through (us a call, CTA per item / pipeline: 64 items
-    // 13.3 / 15.3, 512 37.1 / 38.5, 672 46.2 / 46.5, 1024 64.6 / 63.8, 1280 in 40 sequences 75.2 / 69.3).  `items` counts a
-    // ragged chunk for each sequence, up to twice what there are.  So a batch whose sequences, were they of equal length,
-    // had at most four items an SM, all of which run at once, has few too (32 heads, 13 x 64 tokens 26.9 / 28.4, 16 x 48
-    // 30.9 / 32.6, 8 x 128 28.2 / 29.5, 18 x 64 33.6 / 34.2; beyond it 20 x 64 40.3 / 39.7, 8 x 130 36.2 / 35.8).
-    const int64_t n = cp.p.N, equal = n * ((cp.p.T + n * kChunk - 1) / (n * kChunk)) * cp.p.Hv;
+    // 13.4 / 15.8, 512 35.8 / 37.2, 672 43.5 / 43.6, 832 51.1 / 51.2, 1024 61.9 / 61.0, 1280 in 40 sequences 61.8 / 59.7, 3840
+    // 156.5 / 142.4).  `items` counts a ragged chunk for each sequence, up to twice what there are.  So a batch whose
+    // sequences, were they of equal length, had at most four items an SM, all of which run at once, has few too (32 heads,
+    // 13 x 64 tokens 26.9 / 28.4, 16 x 48 30.9 / 32.6, 8 x 128 28.2 / 29.5, 18 x 64 33.6 / 34.2; beyond it 20 x 64 40.3 /
+    // 39.7, 8 x 130 36.2 / 35.8).
+    const int64_t n = cp.p.N, equal = n * (1 + (cp.p.T - 1) / (n * kChunk)) * cp.p.Hv;
     if (items <= 5ll * di.sms || equal <= 4ll * di.sms) {
         const bool row = items > 2ll * di.sms;
         auto kernel = row ? inline_tables ? prefill_intra_few_kernel<true, true> : prefill_intra_few_kernel<false, true>
@@ -178,8 +179,7 @@ cudaError_t launch_prefill_intra(const TensorMaps& maps, const ChunkedParams& cp
     auto kernel = inline_tables ? prefill_intra_kernel<true> : prefill_intra_kernel<false>;
     e = ensure_dynamic_smem(kernel, kProdSmem);
     if (e != cudaSuccess) return e;
-    const dim3 grid(static_cast<unsigned>(items < di.sms ? items : di.sms));
-    return launch_dependent(kernel, grid, dim3(kProdThreads), kProdSmem, stream, maps, cp.p, cp.ws, cp.lay);
+    return launch_dependent(kernel, dim3(static_cast<unsigned>(di.sms)), dim3(kProdThreads), kProdSmem, stream, maps, cp.p, cp.ws, cp.lay);
 }
 
 // The three-launch path: table-building launch (none for small batches), the intra-chunk kernel

@@ -125,7 +125,8 @@ __device__ __forceinline__ void state_half_role(const TensorMaps& maps, const Pr
     auto at = [&](int i) { return walk.at(i); };
     auto info = [&](int hu) { return unit_info(p, ws, lay, seq_tab, min(hu, total - 1) >> 1); };
     // chunks of earlier units of this CTA; chunk j of the current one is chunk g = gc + j of the CTA's stream: stage
-    // g & 1, phase g >> 1 of the barriers that come in pairs, phase g of the others
+    // g & 1, phase g >> 1 of the barriers that come in pairs, phase g of the others and of bar_d4's two, which are halves
+    // of one chunk's product
     uint32_t gc = 0;
 
     // place and parity of a chunk's use in the three-place rings
@@ -573,7 +574,6 @@ __device__ __forceinline__ void state_half_role(const TensorMaps& maps, const Pr
             nxt = info(hu_next);
             nxt_done = is_done(min(hu_next, total - 1));
             if (skip) continue;
-            const int half = hu & 1;
 #pragma unroll 1
             for (int j = 0; j < u.nc; ++j) {
                 const uint32_t g = gc + j;
@@ -630,7 +630,7 @@ __device__ __forceinline__ void state_half_role(const TensorMaps& maps, const Pr
                 fence_proxy_async_smem();
                 __syncwarp();
                 if (lane == 0) mbar_arrive(&bar_y_read);
-                rows = {true, u.seq_t0 + j * kChunk, min(kChunk, u.seq_len - j * kChunk), u.hv, half, kHS_Out + 8192 * buf};
+                rows = {true, u.seq_t0 + j * kChunk, min(kChunk, u.seq_len - j * kChunk), u.hv, hu & 1, kHS_Out + 8192 * buf};
             }
             gc += u.nc;
         }

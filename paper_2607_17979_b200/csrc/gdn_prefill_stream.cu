@@ -46,13 +46,14 @@ prefill_state_half_kernel(const __grid_constant__ TensorMaps maps, const Prefill
     if (warp == kSIssueWarp) tmem_dealloc(tmem, kStateTmemCols);
 }
 
-// Whether the state pass runs two CTAs per unit.  A half unit's chunk step takes 1.06 us against 1.40 of a whole
+// Whether the state pass runs two CTAs per unit.  A half unit's chunk step takes about 1.0 us against 1.40 of a whole
 // unit's, so half units win where the longest chain decides: always while every one of them has an SM of its own (32
-// units of 64 chunks 144 us whole, 126 half), and for more units if the longest chain is at least twice what an SM has
-// to do on average, set-up of the units included (2.0 times the average 183 / 179.5, 1.75 times 106.7 / 106.5, once
-// 205 / 217). The longest chain is the caller's word.  If that bound is far too large, whole units would have been
-// faster by 5 to 11 % (57 x 144 tokens at 32 heads 216 us, half 240).  The device knows better, but a kernel that
-// holds both forms and chooses costs every call of more units 2 us (1337 + 512 + 199 tokens 57.4 -> 59.8).
+// units of 64 chunks 135.8 us whole, 109.3 half), and for more units if the longest chain is at least twice what an SM has
+// to do on average, set-up of the units included (us whole / half, 32 heads: 2.5 times the average 166.9 / 142.9, just
+// below twice 162.2 / 152.5, 1.7 times 152.0 / 157.0, 1.5 times 156.5 / 196.5, once 139.9 / 155.6).  The longest chain is the
+// caller's word.  If that bound is far too large, whole units would have been faster by up to 26 % (57 x 144 tokens at 32 heads 186
+// us, half 220; 3 x 3000).  The device knows better, but a kernel that holds both forms and chooses costs every call of
+// more units 2 us (1337 + 512 + 199 tokens 57.4 -> 59.8).
 static bool half_units(int32_t T, int32_t N, int32_t Hv, int32_t longest, int sms) {
     const long long units = static_cast<long long>(N) * Hv;
     if (2 * units <= sms) return true;
