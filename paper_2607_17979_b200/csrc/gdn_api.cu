@@ -290,8 +290,8 @@ int gdn_prefill_route(int32_t T, int32_t N, int32_t max_seqlen_hint, int32_t Hv,
     // very short sequences: one block of tokens each (one launch, no workspace traffic)
     if (longest <= GDN_RECURRENT_MAX_SEQLEN) return GDN_ROUTE_RECURRENT;
     const long long units = static_cast<long long>(N) * Hv;
-    // Up to four blocks of few units.  Us against the chunked kernels, one sequence: 32 v-heads, 32 tokens 10.0 /
-    // 11.0, 48 13.5 / 12.0; 8 v-heads, 48 10.9 / 11.8, 64 13.6 / 12.1.  The third and fourth block are slower where
+    // Up to four blocks of few units.  Us against the chunked kernels, one sequence: 32 v-heads, 32 tokens 10.1 /
+    // 11.2, 48 13.6 / 12.0; 8 v-heads, 48 11.2 / 11.5, 64 13.8 / 12.0.  The third and fourth block are slower where
     // there are more than a few units and stay: they keep the state to 1e-6, the chunked kernels, whose operands are
     // bf16, to 2e-4. With more units than half the SMs a block takes longer: 4 x 30 tokens (128 units) 18.7 against
     // 18.5 of the chunked kernels as they were.
