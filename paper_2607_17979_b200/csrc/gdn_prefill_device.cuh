@@ -67,9 +67,8 @@ __device__ __forceinline__ void mma_m16n8k8_tf32(float (&c)[4], const uint32_t (
         : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
         : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b[0]), "r"(b[1]));
 }
-// kN tiles side by side: columns 8 nb .. of B and of the output.  kPairs: of a k-step's eight k, 2t and 2t + 1 stand where
-// t and t + 4 do otherwise, as in gdn_prefill_intra.cuh's products of accumulators: the same sums to the last bit.
-template <int kSteps, int kN, bool kPairs = false>
+// kN tiles side by side: columns 8 nb .. of B and of the output.
+template <int kSteps, int kN>
 __device__ __forceinline__ void mma_tile_tf32(const float* A, int lda, const float* B, int ldb,
                                               float (&c)[kN][4], int g, int t) {
     uint32_t a[kSteps][4], b[kSteps][kN][2];
@@ -77,15 +76,14 @@ __device__ __forceinline__ void mma_tile_tf32(const float* A, int lda, const flo
     for (int ks = 0; ks < kSteps; ++ks) {          // every load first, then the products
         const float* a_ = A + 8 * ks;
         const float* b_ = B + (8 * ks) * ldb;
-        const int k0 = kPairs ? 2 * t : t, k1 = kPairs ? 2 * t + 1 : t + 4;
-        a[ks][0] = to_tf32(a_[g * lda + k0]);
-        a[ks][1] = to_tf32(a_[(g + 8) * lda + k0]);
-        a[ks][2] = to_tf32(a_[g * lda + k1]);
-        a[ks][3] = to_tf32(a_[(g + 8) * lda + k1]);
+        a[ks][0] = to_tf32(a_[g * lda + t]);
+        a[ks][1] = to_tf32(a_[(g + 8) * lda + t]);
+        a[ks][2] = to_tf32(a_[g * lda + t + 4]);
+        a[ks][3] = to_tf32(a_[(g + 8) * lda + t + 4]);
 #pragma unroll
         for (int nb = 0; nb < kN; ++nb) {
-            b[ks][nb][0] = to_tf32(b_[k0 * ldb + 8 * nb + g]);
-            b[ks][nb][1] = to_tf32(b_[k1 * ldb + 8 * nb + g]);
+            b[ks][nb][0] = to_tf32(b_[t * ldb + 8 * nb + g]);
+            b[ks][nb][1] = to_tf32(b_[(t + 4) * ldb + 8 * nb + g]);
         }
     }
 #pragma unroll
@@ -157,7 +155,7 @@ __device__ __forceinline__ void solve_blocks_16_32(float* sA, const int pr, cons
         c[nb][0] = c[nb][1] = c[nb][2] = c[nb][3] = 0.f;
     }
     __syncwarp();
-    mma_tile_tf32<2, 2, true>(sA + (16 * I) * kLdA + 16 * I, kLdA, X, kLdA, c, g, t);   // T_IJ = -T_II X
+    mma_tile_tf32<2, 2>(sA + (16 * I) * kLdA + 16 * I, kLdA, X, kLdA, c, g, t);         // T_IJ = -T_II X
     __syncwarp();                                      // every lane has read A_IJ (above)
 #pragma unroll
     for (int nb = 0; nb < 2; ++nb) {
@@ -191,9 +189,9 @@ __device__ __forceinline__ void solve_merge_64(float* sA, const int w, const int
     asm volatile("bar.sync %0, 128;" ::"r"(bar_id) : "memory");
     // X = -Tb Y; the rows 0-15 of Tb have columns 0-15 only
     if (r0 == 0)
-        mma_tile_tf32<2, 2, true>(sA + 32 * kLdA + 32, kLdA, Y, kLdA, c, g, t);
+        mma_tile_tf32<2, 2>(sA + 32 * kLdA + 32, kLdA, Y, kLdA, c, g, t);
     else
-        mma_tile_tf32<4, 2, true>(sA + 48 * kLdA + 32, kLdA, Y, kLdA, c, g, t);
+        mma_tile_tf32<4, 2>(sA + 48 * kLdA + 32, kLdA, Y, kLdA, c, g, t);
 #pragma unroll
     for (int nb = 0; nb < 2; ++nb) {
         float* dst = sA + (32 + r0) * kLdA + c0 + 8 * nb;
